@@ -495,10 +495,7 @@ struct Shot {
   }
 
   __device__ void rot(uint32_t w0, uint32_t ci, const uint64_t *beta, const uint64_t *gamma) {
-    uint32_t pe = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) pe += __popcll(sd[w] & beta[w]) + __popcll(ss[w] & gamma[w]);
-    const uint32_t e = (ev_e0(w0) + 2u * pe) & 3u;
+    const uint32_t e = (ev_e0(w0) + 2u * wpar2<W>(sd, beta, ss, gamma)) & 3u;
     const uint32_t lowbit = ev_lowbit(w0);
     if (ci >= C->n_coef) {
       fail_check(CHK_COEF, ci);
@@ -584,10 +581,7 @@ struct Shot {
 
   // ---- a I + b Z_q, beta == 0: v_a *= a + b xi_a
   __device__ void rot_diag(uint32_t w0, uint32_t ci, const uint64_t *gamma) {
-    uint32_t pe = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) pe += __popcll(ss[w] & gamma[w]);
-    const uint32_t e = (ev_e0(w0) + 2u * pe) & 3u;
+    const uint32_t e = (ev_e0(w0) + 2u * wpar<W>(ss, gamma)) & 3u;
     Cx<R> a, b;
     coef(ci, a, b);
     if (kRegCapable && reg) {
@@ -612,10 +606,7 @@ struct Shot {
 
   // ---- Z measurement, beta = 0: lambda_a = c (-1)^{gamma.a}
   __device__ int meas_a(uint32_t w0, uint32_t ord, const uint64_t *gamma) {
-    uint32_t pe = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) pe += __popcll(ss[w] & gamma[w]);
-    const uint32_t e = (ev_e0(w0) + 2u * pe) & 3u;
+    const uint32_t e = (ev_e0(w0) + 2u * wpar<W>(ss, gamma)) & 3u;
     if (e & 1u) {
       fail_check(CHK_PHASE, e);
       return 1;
