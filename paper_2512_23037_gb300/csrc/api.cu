@@ -28,6 +28,7 @@ int cuda_fail(cudaError_t e, const char *what) {
 
 constexpr uint64_t kDefaultChunk = 1ull << 24;
 using soft::kDefaultFirstCap;
+constexpr uint32_t kAffDim = 8;  // directions of the affine warp passes' maps (256 values per warp)
 using soft::kTauFp32;
 using soft::kTauFp64;
 }  // namespace
@@ -383,15 +384,19 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   // always runs: a lane decides overflow only after pruning, and a map that outgrows the lane
   // before pruning is staged whole by the warp pass, even when the circuit's cap is the lane's.
   const bool lane_grow = lanes16 && lc16 < cap_max;  // maps may outgrow a 16-entry lane
-  const bool two_pass = lanes || cap1 < cap_max;
-  // after lanes, a middle pass (a warp per shot, map up to cap1 entries) takes the shots whose
-  // maps outgrew a lane, and only those that outgrow cap1 go on to the pass at the circuit's
-  // cap. Not when every lane of the run holds 64 entries already: then a shot that outgrew one
-  // goes straight to the circuit's cap (w97 FP32: 44.7 M shots/s against 44.5 M through a
-  // middle pass at 64, and 27.0 M through one at 256, whose larger maps cut its residency).
-  // With smaller lanes in the run it stays for all (many maps that outgrow a 64-entry lane's
-  // six directions still fit 64 entries: batch64 FP32 113 M shots/s when they skipped it)
-  const bool mid_pass = lanes && lc16 < cap1 && cap1 < cap_max && (nbc[0] > 0 || nbc[1] > 0);
+  // the warp-per-shot passes below the circuit's cap keep the map in affine form (affine.cu)
+  // unless the caller shapes them (group size, first_cap, groups per block) or asks for the
+  // sparse form's scheduling (no lanes, no prefix)
+  bool affine = !(o.flags & (SOFT_RUN_NO_LANES | SOFT_RUN_NO_PREFIX)) && o.group_size == 0 && o.first_cap == 0 &&
+                o.groups_per_block == 0;
+  for (uint32_t i = 0; i < n_circ; ++i) affine = affine && circs[i]->d_traj[pk];
+  const bool two_pass = lanes || affine || cap1 < cap_max;
+  // after lanes, a middle pass (a warp per shot) takes the shots whose maps outgrew a lane, and
+  // only those that outgrow it too go on to the pass at the circuit's cap: in affine form, with
+  // room for 2^kAffDim entries, or in sparse form up to cap1 entries. The sparse one is left out
+  // when every lane of the run holds 64 entries already (w97 FP32 ran 44.7 M shots/s without
+  // it, 44.5 M with 64 entries and 27.0 M with 256, whose larger maps cut its residency)
+  const bool mid_pass = lanes && (affine || (lc16 < cap1 && cap1 < cap_max && (nbc[0] > 0 || nbc[1] > 0)));
   const uint32_t g1 = o.group_size ? o.group_size : 32u;
   const uint32_t g2 = 32;
   const size_t smem_limit = 227 * 1024 - 5 * sizeof(unsigned long long) * soft::kMaxCirc;
@@ -592,6 +597,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     q.list = m.rerun;
     q.n_items_dev = m.n_rerun;
   }
+  p.aff_dim = m.aff_dim = kAffDim;
   if (global_rerun) {
     q.gslab = r->d_slab;
     q.gslab_blocks = slab_blocks;
@@ -622,6 +628,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     h.sp = p.sp;
     h.sp_cap = p.sp_cap;
     h.sp_evict_cap = p.sp_evict_cap;
+    if (affine) m.al_cursor = p.al_cursor;  // a shot that starts again has its first error drawn
   }
   soft::LaunchCfg c1{}, c2{}, cm{}, cw{}, cb[2]{};
   p.n_items = std::min(chunk, total);
@@ -636,14 +643,16 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     pb[k].sp_cap = pb[k].sp_evict_cap = 0;
     pb[k].lr = nullptr;
   }
-  if ((e = !lanes ? soft::prepare_shots(p, fp32, W, g1, (int)o.blocks_per_sm, &c1)
+  if ((e = !lanes ? (affine ? soft::prepare_affine(p, fp32, W, (int)o.blocks_per_sm, &c1)
+                            : soft::prepare_shots(p, fp32, W, g1, (int)o.blocks_per_sm, &c1))
                   : lanes16 ? soft::prepare_lanes(p, fp32, W, (int)o.blocks_per_sm, &c1, lc16) : cudaSuccess) !=
           cudaSuccess ||
       (lanes && nbc[1] && (e = soft::prepare_lanes(pb[0], fp32, W, 0, &cb[0], 2 * lc16)) != cudaSuccess) ||
       (lanes && nbc[2] && (e = soft::prepare_lanes(pb[1], fp32, W, 0, &cb[1], 4 * lc16)) != cudaSuccess) ||
       (wide && (e = soft::prepare_lanes(p, fp32, W, 0, &cw, 2 * lc16)) != cudaSuccess) ||
       (two_pass && (e = soft::prepare_shots(q, fp32, W, g2, (int)o.blocks_per_sm, &c2)) != cudaSuccess) ||
-      (mid_pass && (e = soft::prepare_shots(m, fp32, W, g2, (int)o.blocks_per_sm, &cm)) != cudaSuccess)) {
+      (mid_pass && (e = affine ? soft::prepare_affine(m, fp32, W, (int)o.blocks_per_sm, &cm)
+                               : soft::prepare_shots(m, fp32, W, g2, (int)o.blocks_per_sm, &cm)) != cudaSuccess)) {
     soft_run_free(r);
     return cuda_fail(e, "shot kernel configuration");
   }

@@ -94,6 +94,7 @@ struct ShotParams {
   unsigned char *sp;          // spill pool, sp_cap records (layout: lane_spill_bytes): evictions in
   uint32_t sp_cap;            // [0, sp_evict_cap), shots handed from a lane to a warp after that
   uint32_t sp_evict_cap;
+  uint32_t aff_dim;           // affine_kernel: directions of a warp's map (2^aff_dim values)
   unsigned long long *lr;     // [0] eviction records taken, [1] handover records taken;
                               // round r >= 1: [2 + 2r] its first record, [3 + 2r] its count
   CircDev circ[kMaxCirc];
@@ -150,6 +151,11 @@ uint32_t lane_map_dim();  // directions of a first-round lane's affine map (lane
 // on the same stream; stop[3] (zeroed before) receives the largest dimension.
 cudaError_t launch_snap_affine(unsigned char *traj, uint32_t n_snap, uint32_t rw, int fp32, uint32_t W,
                                uint32_t *stop, cudaStream_t st);
+
+// Warp-per-shot kernel with the map in affine form (affine.cu), up to 2^p.aff_dim values; it
+// takes the same work items and lists as the shot kernel. A shot that needs more goes to
+// p.rerun. Starts shots from the noiseless prefix (every circuit needs its traj).
+cudaError_t prepare_affine(const ShotParams &p, int fp32, uint32_t W, int blocks_per_sm, LaunchCfg *cfg);
 
 // Resolve the launch (sets the kernel's shared-memory attribute, queries
 // occupancy). `p.hs_max` must already be hash_slots_for(p.cap). Not a stream
