@@ -19,6 +19,7 @@
 // arithmetic is that kernel's, product by product, so a shot's outcomes do not depend on
 // which of the two runs it (FP64 sums over entries run in slot order).
 #include <algorithm>
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "kernels.cuh"
@@ -44,11 +45,19 @@ __device__ __forceinline__ uint64_t shfl64(uint64_t x, uint32_t src) {
 __device__ __forceinline__ uint64_t xor_all(uint64_t x) {
   return (uint64_t)__reduce_xor_sync(kAll, (uint32_t)x) | ((uint64_t)__reduce_xor_sync(kAll, (uint32_t)(x >> 32)) << 32);
 }
-__device__ __forceinline__ double sum_all(double v) {
+// Both sums over the lanes: the halves of the warp trade one of them first, so that one
+// chain of additions carries both (6 FP64 additions instead of 10).
+__device__ __forceinline__ void sum_both(double &a, double &b) {
+  const bool up = (threadIdx.x & 16u) != 0u;
+  double x = (up ? b : a) + __shfl_xor_sync(kAll, up ? a : b, 16);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kAll, v, off);
-  return v;
+  for (int off = 8; off > 0; off >>= 1) x += __shfl_xor_sync(kAll, x, off);
+  a = __shfl_sync(kAll, x, 0);
+  b = __shfl_sync(kAll, x, 16);
 }
+// acc + |v|^2 as it enters a probability: FP32 norms widened (see pnorm), FP64 fused
+__device__ __forceinline__ double addn(double acc, Cx<float> v) { return acc + pnorm(v); }
+__device__ __forceinline__ double addn(double acc, Cx<double> v) { return __fma_rn(v.x, v.x, __fma_rn(v.y, v.y, acc)); }
 __device__ __forceinline__ uint32_t par32(uint32_t x) { return (uint32_t)__popc(x) & 1u; }
 // i with a zero bit inserted at position q
 __device__ __forceinline__ uint32_t open_bit(uint32_t i, uint32_t q) {
@@ -75,10 +84,19 @@ struct AffShot {
   int status, chain, logical, lastm;
   double fid;
   bool force;
-  PruneTest<R> pt;  // |v|^2 < tau
+  static constexpr bool kScaled = sizeof(R) == 8;  // FP64 maps are scaled (see ScaledPrune)
+  double nrm = 1.0;                                // their squared norm
+  typename std::conditional<kScaled, ScaledPrune, PruneTest<R>>::type pt;  // |v|^2 < tau
 
   __device__ AffShot(const ShotParams &p, unsigned char *base)
       : P(p), lane(threadIdx.x & 31u), v(reinterpret_cast<Cx<R> *>(base)), pt(p.tau) {}
+  // x, or zero where it is below tau
+  __device__ __forceinline__ Cx<R> pruned(Cx<R> x) const {
+    bool sm;
+    if constexpr (kScaled) sm = pt.small(x, nrm);
+    else sm = pt.small(x);
+    return sm ? Cx<R>{0, 0} : x;
+  }
 
   __device__ __forceinline__ uint32_t size() const { return 1u << d; }
   __device__ __forceinline__ static bool nonzero(const Cx<R> &x) { return x.x != (R)0 || x.y != (R)0; }
@@ -145,8 +163,7 @@ struct AffShot {
         s |= (par32(s & g) ^ t) << q;
         x = v[s];
         if (scaled) {
-          x = cscale(x, sc);
-          if (pt.small(x)) x = Cx<R>{0, 0};
+          x = pruned(cscale(x, sc));
         }
       }
       __syncwarp();
@@ -209,24 +226,8 @@ struct AffShot {
       P.diag[3] = value;
     }
   }
-  __device__ double uniform(uint32_t ord) const {
-    const uint4 w = philox(P.seed, shot, 1u, ord);
-    const uint64_t m = ((uint64_t)w.x << 21) ^ (uint64_t)(w.y >> 11);
-    return (double)m * 0x1p-53;
-  }
-  // Outcome +1 iff u < p, p = sp / (sp + sm) snapped to 0 or 1 within 1e-12 (see kernels.cu)
   __device__ __forceinline__ int pick(uint32_t ord, double sp, double sm) {
-    const double tot = sp + sm;
-    if (!(tot > 0.0)) return -1;
-    const bool zero = sp < 1e-12 * tot, one = sp > (1.0 - 1e-12) * tot;
-    if (force) {
-      if (zero) return -1;
-      fid *= one ? 1.0 : sp / tot;
-      return 1;
-    }
-    if (zero) return -1;
-    if (one) return 1;
-    return uniform(ord) * tot < sp ? 1 : -1;
+    return pick_outcome<false>(P.seed, shot, ord, sp, sm, force, fid, nullptr);
   }
   __device__ __forceinline__ static R inv_sqrt(double x) {
     if (sizeof(R) == 4) return (R)rsqrtf((float)x);
@@ -244,6 +245,7 @@ struct AffShot {
     logical = (int)__ldg(&h->logical);
     lastm = (int)__ldg(&h->lastm);
     fid = __ldg(&h->fid);
+    nrm = 1.0;
     recw = lane < C->rw ? __ldg(&r_in[lane]) : 0ull;
     d = __ldg(&a->d);
     if (d > P.aff_dim || d > kSnapDim) {
@@ -278,6 +280,7 @@ struct AffShot {
     kblk = b.z;
     w2 = b.w;
     fid = S.fid[r];
+    if constexpr (kScaled) nrm = S.norm[r];
     recw = lane < C->rw ? S.rec[lane * c + r] : 0ull;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
@@ -368,7 +371,7 @@ struct AffShot {
     apply_pauli(beta, gamma, ((__ldg(&S->c0) >> (2u * code)) + 2u * wordpar(pe)) & 3u);
   }
 
-  // b xi x, xi = i^e (-1)^par
+  // FP32: b xi x, xi = i^e (-1)^par
   __device__ __forceinline__ static Cx<R> bxi(Cx<R> b, Cx<R> bq, uint32_t e, uint32_t par, Cx<R> x) {
     if (kFoldPhase) return cmul(par ? Cx<R>{negr(bq.x), negr(bq.y)} : bq, x);
     return cmul(b, ipow(x, e + 2u * par));
@@ -380,76 +383,116 @@ struct AffShot {
       fail_check(CHK_COEF, ci);
       return;
     }
-    const Coef *cf = C->coef + ci;
-    Cx<R> a, b;
-    if (sizeof(R) == 4) {
-      const float4 f = __ldg(reinterpret_cast<const float4 *>(&cf->fa_re));
-      a = Cx<R>{(R)f.x, (R)f.y};
-      b = Cx<R>{(R)f.z, (R)f.w};
-    } else {
-      const double2 d0 = __ldg(reinterpret_cast<const double2 *>(&cf->a_re));
-      const double2 d1 = __ldg(reinterpret_cast<const double2 *>(&cf->b_re));
-      a = Cx<R>{(R)d0.x, (R)d0.y};
-      b = Cx<R>{(R)d1.x, (R)d1.y};
-    }
-    uint32_t g0, gl = parities(gamma, g0);
-    const Cx<R> bq = ipow(b, e);
-    if (diag) {
-      const Cx<R> c0 = cadd(a, bq), c1 = csub(a, bq);
-      for (uint32_t s = lane; s < size(); s += 32) {
-        const uint32_t par = g0 ^ par32(s & gl);
-        Cx<R> x = v[s];
-        if (kFoldPhase) x = cmul(par ? c1 : c0, x);
-        else x = cadd(cmul(a, x), cmul(b, ipow(x, e + 2u * par)));
-        if (pt.small(x)) x = Cx<R>{0, 0};
-        v[s] = x;
-      }
-      __syncwarp();
-      return;
-    }
+    uint32_t g0, gl = parities(gamma, g0), c = 0;
+    bool fresh = false;
     uint64_t r[W];
-    uint32_t c = coords(beta, r);
-    bool fresh = wnonzero(r);  // beta outside the span: every entry gains a partner
-    if (fresh && d == P.aff_dim) {
-      bool any = false;
-      while (compact_one(gl, g0)) any = true;
-      if (any) {
-        c = coords(beta, r);
-        fresh = wnonzero(r);
-      }
+    if (!diag) {
+      c = coords(beta, r);
+      fresh = wnonzero(r);  // beta outside the span: every entry gains a partner
       if (fresh && d == P.aff_dim) {
-        status = AS_RERUN;
+        bool any = false;
+        while (compact_one(gl, g0)) any = true;
+        if (any) {
+          c = coords(beta, r);
+          fresh = wnonzero(r);
+        }
+        if (fresh && d == P.aff_dim) {
+          status = AS_RERUN;
+          return;
+        }
+      }
+    }
+    const Coef *cf = C->coef + ci;
+    if constexpr (kScaled) {
+      rot_scaled(cf, e, diag, fresh, gl, g0, c, r);
+    } else {
+      const float4 f = __ldg(reinterpret_cast<const float4 *>(&cf->fa_re));
+      const Cx<R> a{(R)f.x, (R)f.y}, b{(R)f.z, (R)f.w};
+      const Cx<R> bq = ipow(b, e);
+      if (diag) {
+        const Cx<R> c0 = cadd(a, bq), c1 = csub(a, bq);
+        for (uint32_t s = lane; s < size(); s += 32) {
+          const uint32_t par = g0 ^ par32(s & gl);
+          const Cx<R> x = v[s];
+          v[s] = pruned(kFoldPhase ? cmul(par ? c1 : c0, x) : cadd(cmul(a, x), cmul(b, ipow(x, e + 2u * par))));
+        }
+        __syncwarp();
         return;
       }
-    }
-    if (fresh) {
-      const uint32_t n = size();
-      add_dim(r);
-      const uint32_t t0 = c | n;  // slot s gains the partner s ^ t0
-      for (uint32_t s = lane; s < n; s += 32) {
-        const Cx<R> x = v[s];
-        Cx<R> ns = cmul(a, x), nt = bxi(b, bq, e, g0 ^ par32(s & gl), x);
-        if (pt.small(ns)) ns = Cx<R>{0, 0};
-        if (pt.small(nt)) nt = Cx<R>{0, 0};
-        v[s] = ns;
-        v[s ^ t0] = nt;
-      }
-    } else {
-      const uint32_t q = (uint32_t)__ffs(c) - 1u, flip = par32(c & gl), np = size() >> 1;
-      for (uint32_t i = lane; i < np; i += 32) {  // a pair of slots per lane
-        const uint32_t s = open_bit(i, q), t = s ^ c;
-        const uint32_t ps = g0 ^ par32(s & gl);
-        const Cx<R> vs = v[s], vt = v[t];
-        Cx<R> ns = cadd(cmul(a, vs), bxi(b, bq, e, ps ^ flip, vt));
-        Cx<R> nt = cadd(cmul(a, vt), bxi(b, bq, e, ps, vs));
-        if (pt.small(ns)) ns = Cx<R>{0, 0};
-        if (pt.small(nt)) nt = Cx<R>{0, 0};
-        v[s] = ns;
-        v[t] = nt;
+      if (fresh) {
+        const uint32_t n = size(), t0 = c | n;  // slot s gains the partner s ^ t0
+        add_dim(r);
+        for (uint32_t s = lane; s < n; s += 32) {
+          const Cx<R> x = v[s];
+          v[s] = pruned(cmul(a, x));
+          v[s ^ t0] = pruned(bxi(b, bq, e, g0 ^ par32(s & gl), x));
+        }
+      } else {
+        const uint32_t q = (uint32_t)__ffs(c) - 1u, flip = par32(c & gl), np = size() >> 1;
+        for (uint32_t i = lane; i < np; i += 32) {  // a pair of slots per lane
+          const uint32_t s = open_bit(i, q), t = s ^ c, ps = g0 ^ par32(s & gl);
+          const Cx<R> vs = v[s], vt = v[t];
+          v[s] = pruned(cadd(cmul(a, vs), bxi(b, bq, e, ps ^ flip, vt)));
+          v[t] = pruned(cadd(cmul(a, vt), bxi(b, bq, e, ps, vs)));
+        }
       }
     }
     __syncwarp();
-    if (size() > C->cap && live_count() > C->cap) status = AS_OVF;
+    if (!diag && size() > C->cap && live_count() > C->cap) status = AS_OVF;
+  }
+  // (rare: many rotations, or very unlikely outcomes, since the last sampled outcome)
+  __device__ __forceinline__ void fit_norm() {
+    for (int k = 0; k < 32 && !ScaledPrune::in_range(nrm); ++k) {  // (bounded: an empty map has norm 0)
+      const double f = ScaledPrune::fit(nrm);
+      for (uint32_t s = lane; s < size(); s += 32) v[s] = cscale(v[s], (R)f);
+      __syncwarp();
+      nrm = nrm * f * f;
+    }
+  }
+  // the scaled form: v' = cm v + i^{e + 3} k (-1)^{gamma.key} v_partner, n2 left to the norm
+  __device__ __forceinline__ void rot_scaled(const Coef *cf, uint32_t e, bool diag, bool fresh, uint32_t gl,
+                                             uint32_t g0, uint32_t c, const uint64_t *r) {
+    const double2 kc = __ldg(reinterpret_cast<const double2 *>(&cf->k));
+    const bool plain = __double2hiint(kc.y) != 0x3FF00000;
+    if (!plain) nrm = mulr(nrm, __ldg(&cf->n2));
+    fit_norm();
+    pt.set(nrm);
+    const ScaledTurn turn(kc.x, (e + 3u) & 3u);
+    auto base = [&](Cx<R> x) { return plain ? cscale(x, (R)kc.y) : x; };
+    if (diag) {
+      for (uint32_t s = lane; s < size(); s += 32) {
+        const Cx<R> x = v[s];
+        v[s] = pruned(turn.add(base(x), x, g0 ^ par32(s & gl)));
+      }
+    } else if (fresh) {  // the old entries stay as they are, but for cm
+      const uint32_t n = size(), t0 = c | n;
+      add_dim(r);
+      for (uint32_t s = lane; s < n; s += 32) {
+        const Cx<R> x = v[s];
+        v[s] = pruned(base(x));
+        v[s ^ t0] = pruned(turn.add(Cx<R>{0, 0}, x, g0 ^ par32(s & gl)));
+      }
+    } else if (size() <= 32u) {
+      // a slot per lane: an FP64 instruction holds its pipe alike for 16 lanes (a pair each,
+      // two outputs one after the other) and for 32
+      const bool in = lane < size();
+      const uint32_t t = lane ^ c;
+      Cx<R> x{0, 0}, y{0, 0};
+      if (in) {
+        x = v[lane];
+        y = v[t];
+      }
+      __syncwarp();
+      if (in) v[lane] = pruned(turn.add(base(x), y, g0 ^ par32(t & gl)));
+    } else {
+      const uint32_t q = (uint32_t)__ffs(c) - 1u, flip = par32(c & gl), np = size() >> 1;
+      for (uint32_t i = lane; i < np; i += 32) {  // a pair of slots per lane
+        const uint32_t s = open_bit(i, q), t = s ^ c, ps = g0 ^ par32(s & gl);
+        const Cx<R> vs = v[s], vt = v[t];
+        v[s] = pruned(turn.add(base(vs), vt, ps ^ flip));
+        v[t] = pruned(turn.add(base(vt), vs, ps));
+      }
+    }
   }
 
   // ---- measurement of P, beta = 0: lambda_a = c (-1)^{gamma.a}
@@ -477,17 +520,25 @@ struct AffShot {
     if (!(h0 && h1)) {  // decided (all eigenvalues equal): integer test only, no scaling
       m = h1 ? -1 : 1;
     } else {
-      double sp = 0.0, sm = 0.0;
-      for (uint32_t s = lane; s < size(); s += 32) {
-        const double a2 = pnorm(v[s]);
-        if (par32(s & gl) ^ sgn) sm += a2;
-        else sp += a2;
+      // a lane's slots 32 apart change sides with the high part of gl: acc[0] takes the rows of
+      // its first slot's side
+      double acc[2] = {0.0, 0.0};
+      for (uint32_t b = 0; b < size(); b += 32) {
+        const uint32_t s = b + lane;
+        const Cx<R> x = s < size() ? v[s] : Cx<R>{0, 0};
+        if (par32(b & gl)) acc[1] = addn(acc[1], x);
+        else acc[0] = addn(acc[0], x);
       }
-      sp = sum_all(sp);
-      sm = sum_all(sm);
+      const bool first_neg = (par32(lane & gl) ^ sgn) != 0u;
+      double sp = first_neg ? acc[1] : acc[0], sm = first_neg ? acc[0] : acc[1];
+      sum_both(sp, sm);
       m = pick(ord, sp, sm);
-      sc = inv_sqrt(m == 1 ? sp : sm);
-      scaled = true;
+      if constexpr (kScaled) {
+        nrm = m == 1 ? sp : sm;
+      } else {
+        sc = inv_sqrt(m == 1 ? sp : sm);
+        scaled = true;
+      }
     }
     __syncwarp();
     // the kept slots share parity(s & gl): one coordinate fewer
@@ -547,26 +598,64 @@ struct AffShot {
       v0 = (lone && hi) ? Cx<R>{0, 0} : v[s];
       x1 = (lone && !hi) ? Cx<R>{0, 0} : ipow(v[t], e2 + 2u * (g20 ^ par32(t & gl2)));
     };
-    double sp = 0.0, sm = 0.0;
-    for (uint32_t i = lane; i < n; i += 32) {
-      uint32_t s, t;
-      Cx<R> v0, x1;
-      pair(i, s, t, v0, x1);
-      sp += 0.5 * pnorm(cadd(v0, x1));
-      sm += 0.5 * pnorm(csub(v0, x1));
-    }
-    sp = sum_all(sp);
-    sm = sum_all(sm);
-    const int m = pick(ord, sp, sm);
-    const R sc = inv_sqrt(2.0 * (m == 1 ? sp : sm));
-    for (uint32_t i = lane; i < n; i += 32) {
-      uint32_t s, t;
-      Cx<R> v0, x1;
-      pair(i, s, t, v0, x1);
-      Cx<R> nv = cscale(m == 1 ? cadd(v0, x1) : csub(v0, x1), sc);
-      if (pt.small(nv)) nv = Cx<R>{0, 0};
-      v[t] = Cx<R>{0, 0};
-      v[s] = nv;  // (t = s when alone)
+    int m;
+    if constexpr (kScaled) {
+      if (lone) {
+        // p = 1/2 exactly: one random bit; the entries with key bit p become m xi v, the norm stays
+        m = force ? 1 : (philox(P.seed, shot, 1u, ord).x >> 31) ? -1 : 1;
+        if (force) fid *= 0.5;
+        for (uint32_t s = lane; s < n; s += 32)
+          if (a0p ^ par32(s & bp)) v[s] = ipow(v[s], e2 + 2u * (g20 ^ par32(s & gl2)) + (m == -1 ? 2u : 0u));
+      } else {
+        // sp, sm = (N +- 2 C) / 2 with N the norm and C = sum Re conj(v0) x1; the kept side's own
+        // norm is summed from the values it keeps
+        double sn = 0.0, cr = 0.0;
+        for (uint32_t i = lane; i < n; i += 32) {
+          uint32_t s, t;
+          Cx<R> v0, x1;
+          pair(i, s, t, v0, x1);
+          sn = addn(addn(sn, v0), x1);
+          cr = fmar((double)v0.x, (double)x1.x, fmar((double)v0.y, (double)x1.y, cr));
+        }
+        sum_both(sn, cr);
+        const double sp = fmar(0.5, sn, cr), sm = fmar(0.5, sn, -cr);
+        m = pick(ord, sp, sm);
+        nrm = 2.0 * (m == 1 ? sp : sm);
+        fit_norm();
+        pt.set(nrm);
+        double kn = 0.0, none = 0.0;
+        for (uint32_t i = lane; i < n; i += 32) {
+          uint32_t s, t;
+          Cx<R> v0, x1;
+          pair(i, s, t, v0, x1);
+          const Cx<R> nv = cadd(v0, m == 1 ? x1 : Cx<R>{negr(x1.x), negr(x1.y)});
+          kn = addn(kn, nv);
+          v[t] = Cx<R>{0, 0};
+          v[s] = pruned(nv);
+        }
+        sum_both(kn, none);
+        nrm = kn;
+      }
+    } else {
+      double sp = 0.0, sm = 0.0;
+      for (uint32_t i = lane; i < n; i += 32) {
+        uint32_t s, t;
+        Cx<R> v0, x1;
+        pair(i, s, t, v0, x1);
+        sp += 0.5 * pnorm(cadd(v0, x1));
+        sm += 0.5 * pnorm(csub(v0, x1));
+      }
+      sum_both(sp, sm);
+      m = pick(ord, sp, sm);
+      const R sc = inv_sqrt(2.0 * (m == 1 ? sp : sm));
+      for (uint32_t i = lane; i < n; i += 32) {
+        uint32_t s, t;
+        Cx<R> v0, x1;
+        pair(i, s, t, v0, x1);
+        const Cx<R> nv = cscale(m == 1 ? cadd(v0, x1) : csub(v0, x1), sc);
+        v[t] = Cx<R>{0, 0};
+        v[s] = pruned(nv);  // (t = s when alone)
+      }
     }
     __syncwarp();
     if (lone) {
@@ -694,6 +783,7 @@ struct AffShot {
     }
     const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C->ev);
     const uint32_t n_events = C->n_events;
+    ev_top = ev;
     if (ev < n_events && status == AS_RUN) {
       uint4 hdr, hn;
       uint64_t body[4 * W], bn[4 * W];
@@ -702,6 +792,7 @@ struct AffShot {
         const uint32_t en = ev + 1u;
         if (en < n_events) load_event(evs + en, hn, bn);
         step(hdr, body, evs + ev);
+        ev_top = en;
         if (en >= n_events || status != AS_RUN) break;
         ev = en;
         hdr = hn;
@@ -735,7 +826,10 @@ struct AffShot {
     if (off < C->out_limit && C->records && lane < C->rw) C->records[off * C->rw + lane] = recw;
     if (ci == 0 && off < P.st_limit) capture(off);
   }
+  uint32_t ev_top;  // the event after the last one that the shot ran
   __device__ void capture(uint64_t off) const {
+    Cx<double> f{1.0, 0.0};
+    if constexpr (kScaled) f = readout(top_phase<W>(C, ev_top), nrm);
     if (lane == 0) {
       P.st_signs[off * 4 + 0] = sd[0];
       P.st_signs[off * 4 + 1] = (W == 2) ? sd[W - 1] : 0ull;
@@ -761,8 +855,10 @@ struct AffShot {
         const size_t o = (size_t)off * P.st_stride + i;
         P.st_keys[2 * o] = k[0];
         P.st_keys[2 * o + 1] = (W == 2) ? k[W - 1] : 0ull;
-        P.st_vals[2 * o] = (double)v[s].x;
-        P.st_vals[2 * o + 1] = (double)v[s].y;
+        Cx<R> x = v[s];
+        if constexpr (kScaled) x = cmul(f, x);
+        P.st_vals[2 * o] = (double)x.x;
+        P.st_vals[2 * o + 1] = (double)x.y;
       }
       n += __popc(m);
     }

@@ -125,7 +125,8 @@ static cudaError_t build_prefixes(soft_circuit *c, cudaStream_t us) {
     p.tau = fp32 ? kTauFp32 : kTauFp64;
     e = soft::launch_prefix(p, fp32, hp.W, c->d_traj[fp32], d_stop + 4 * fp32, ps[fp32]);
     if (e == cudaSuccess)
-      e = soft::launch_snap_affine(c->d_traj[fp32], (uint32_t)n_snap, hp.rw, fp32, hp.W, d_stop + 4 * fp32, ps[fp32]);
+      e = soft::launch_snap_affine(c->d_traj[fp32], (uint32_t)n_snap, hp.rw, fp32, hp.W, d_stop + 4 * fp32, c->d_ev,
+                                   ps[fp32]);
   }
   for (int k = 0; k < 2; ++k)
     if (ps[k]) {

@@ -394,17 +394,22 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
     return true;
   };
 
+  std::vector<int32_t> coef_phase;  // per coefficient: its global phase in units of pi/8
   // fixed angles share entries by value; a parameterised angle gets one entry per (parameter, sign)
-  auto coef_index = [&](double ar, double ai, double br, double bi, int32_t param) -> uint32_t {
+  auto coef_index = [&](double ar, double ai, double br, double bi, double co, double si, int32_t phase,
+                        int32_t param) -> uint32_t {
     for (size_t k = 0; k < P.coefs.size(); ++k) {
       const Coef &c = P.coefs[k];
       if (param >= 0 ? P.coef_param[k] == param
                      : (P.coef_param[k] < 0 && c.a_re == ar && c.a_im == ai && c.b_re == br && c.b_im == bi))
         return (uint32_t)k;
     }
-    Coef c{ar, ai, br, bi, (float)ar, (float)ai, (float)br, (float)bi};
+    const bool scaled = std::fabs(si) <= std::sqrt(3.0) * std::fabs(co);
+    Coef c{ar, ai, br, bi, (float)ar, (float)ai, (float)br, (float)bi, scaled ? si / co : si, scaled ? 1.0 : co,
+           scaled ? 1.0 / (co * co) : 1.0, 0.0};
     P.coefs.push_back(c);
     P.coef_param.push_back(param);
+    coef_phase.push_back(phase);
     return (uint32_t)(P.coefs.size() - 1);
   };
   // records read by OBSERVABLE ops (fidelity measurements of gradient runs)
@@ -561,12 +566,20 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
       uint32_t e0;
       if (!tb.decompose(single(3, o.q0), beta, gamma, &e0)) goto internal;
       bool diag = (beta[0] | beta[1]) == 0;
-      double ar, ai, br, bi;
+      double ar, ai, br, bi, co, si;  // a phase times co I - i si Z
+      int32_t phase = 0;
       if (op == SOFT_RZ) {
-        ar = std::cos(0.5 * o.angle);
+        co = std::cos(0.5 * o.angle);
+        si = std::sin(0.5 * o.angle);
+        ar = co;
         ai = 0.0;
         br = 0.0;
-        bi = -std::sin(0.5 * o.angle);
+        bi = -si;
+        if (co < 0.0) {  // c I - i s Z = e^{i pi} (-c I + i s Z)
+          co = -co;
+          si = -si;
+          phase = 8;
+        }
       } else {
         // diag(1, e^{+-i pi/4}) = (1 + w)/2 I + (1 - w)/2 Z with w = e^{+-i pi/4}
         double c = std::cos(0.25 * M_PI), sn = (op == SOFT_T ? 1.0 : -1.0) * std::sin(0.25 * M_PI);
@@ -574,6 +587,9 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
         ai = 0.5 * sn;
         br = 0.5 * (1.0 - c);
         bi = -0.5 * sn;
+        phase = op == SOFT_T ? 1 : -1;
+        co = std::cos(0.125 * M_PI);
+        si = phase * std::sin(0.125 * M_PI);
       }
       uint32_t lowbit = 0;
       if (!diag) lowbit = beta[0] ? (uint32_t)__builtin_ctzll(beta[0]) : 64u + (uint32_t)__builtin_ctzll(beta[1]);
@@ -582,7 +598,7 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
         param = (int32_t)(((o.pad - 1) << 1) | (o.flags & 1));
         P.n_params = std::max<uint32_t>(P.n_params, o.pad);
       }
-      uint32_t ci = coef_index(ar, ai, br, bi, param);
+      uint32_t ci = coef_index(ar, ai, br, bi, co, si, phase, param);
       Ev<2> &e = new_event(diag ? EV_ROT_DIAG : EV_ROT, 0, e0, lowbit);
       e.a = ci;
       e.b = param >= 0 ? (uint32_t)param : kNoRec;
@@ -638,6 +654,13 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
   }
   new_event(EV_END, 0, 0, 0);
   fuse_events(P.ev);
+  {
+    uint32_t ph = 0;  // (units of pi/8, modulo 16)
+    for (auto &e : P.ev) {
+      if (ev_type(e.w0) == EV_ROT || ev_type(e.w0) == EV_ROT_DIAG) ph += (uint32_t)coef_phase[e.a];
+      e.w0 |= (ph & 15u) << 26;
+    }
+  }
   P.n_records = nrec;
   P.rw = nrec ? (nrec + 63) / 64 : 1;
   if (P.rw > 16) {

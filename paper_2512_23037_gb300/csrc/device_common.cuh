@@ -96,6 +96,75 @@ struct PruneTest {
     return norm2(v) < tau;
   }
 };
+// ---- scaled FP64 maps (the lane kernels and affine_kernel). The map's entries are
+// e^{i phi} v / sqrt(N): a squared norm N per shot, and the circuit's global phase phi (pi/8
+// times the event's ev_phase), which is the same in every shot and only needed when a state
+// is read out. A rotation c I - i s Z is then v' = v - i (s / c) xi v_partner with N / c^2,
+// two fused multiply-adds per entry instead of two complex products (eight operations), and
+// a measurement keeps its outcome's sum as the new N instead of scaling every entry. GB300
+// issues an FP64 instruction per 76 cycles and SM partition whatever its active lanes, and
+// that pipe bounded every FP64 map (random 40-qubit circuit, 0.2 M shots: 2.9 -> 1.8 ms; w97,
+// 0.5 M: 19.1 -> 17.8 ms; w42, 2^22: 12.5 -> 11.3 ms).
+// The sign bit of a 64-bit float as a value to XOR into its high word.
+__device__ __forceinline__ double xor_hi(double x, uint32_t flip) {
+  return __hiloint2double((int)((uint32_t)__double2hiint(x) ^ flip), __double2loint(x));
+}
+// i^(eo) (-1)^neg k: what multiplies the two components of an entry's partner
+struct ScaledTurn {
+  double kx, ky;  // for the new re and im
+  bool swap;      // odd eo: re takes the partner's im
+  __device__ __forceinline__ ScaledTurn(double k, uint32_t eo)
+      : kx(xor_hi(k, ((eo ^ (eo >> 1)) & 1u) << 31)), ky(xor_hi(k, (eo & 2u) << 30)), swap((eo & 1u) != 0u) {}
+  // base + i^eo (-1)^neg k w
+  __device__ __forceinline__ Cx<double> add(Cx<double> base, Cx<double> w, uint32_t neg) const {
+    const double p = swap ? w.y : w.x, q = swap ? w.x : w.y;
+    return {__fma_rn(xor_hi(kx, neg << 31), p, base.x), __fma_rn(xor_hi(ky, neg << 31), q, base.y)};
+  }
+};
+// x >= 0 as a float, rounded toward zero to 21 bits (0 below 2^-125, inf from 2^126), without
+// the FP64 pipe's conversion
+__device__ __forceinline__ float low_float(double x) {
+  const uint32_t h = (uint32_t)__double2hiint(x);
+  return h < (898u << 20) ? 0.0f : h >= (1149u << 20) ? __uint_as_float(0x7F800000u) : __uint_as_float((h - (896u << 20)) << 3);
+}
+// The pruning test |v|^2 < tau N. The bounds of PruneTest, widened to 2^-16 and multiplied by
+// sqrt(N) in FP32 (N truncated to 21 bits), are compared with the high words of |re| and
+// |im|; only values between them compute the norm on the FP64 pipe.
+struct ScaledPrune {
+  double tau;
+  float klo, khi;
+  uint32_t lo = 0, hi = 0;
+  __device__ explicit ScaledPrune(double t)
+      : tau(t), klo((float)(sqrt(0.5 * t) * (1.0 - 0x1p-16))), khi((float)(sqrt(t) * (1.0 + 0x1p-16))) {}
+  __device__ __forceinline__ void set(double N) {  // N in range
+    const float n = low_float(N), r = n * rsqrtf(n);
+    lo = (__float_as_uint(klo * r) >> 3) + (896u << 20);
+    hi = (__float_as_uint(khi * r) >> 3) + (896u << 20) + 1u;
+  }
+  __device__ __forceinline__ bool small(Cx<double> v, double N) const {
+    const uint32_t hx = (uint32_t)__double2hiint(v.x) & 0x7FFFFFFFu, hy = (uint32_t)__double2hiint(v.y) & 0x7FFFFFFFu;
+    if (hx > hi || hy > hi) return false;
+    if (hx < lo && hy < lo) return true;
+    return norm2(v) < mulr(tau, N);
+  }
+  // N within [2^-64, 2^96]: outside, the entries take the factor fit(N) (a power of two:
+  // exact) and N its square
+  __device__ __forceinline__ static bool in_range(double N) {
+    const uint32_t h = (uint32_t)__double2hiint(N);
+    return h >= ((1023u - 64u) << 20) && h < ((1023u + 96u) << 20);
+  }
+  __device__ __forceinline__ static double fit(double N) { return N > 1.0 ? 0x1p-32 : 0x1p32; }
+};
+// e^{i pi ph / 8}
+__device__ __forceinline__ Cx<double> phase_of(uint32_t ph) {
+  double s, c;
+  sincospi(0.125 * (double)ph, &s, &c);
+  return {c, s};
+}
+
+// e^{i pi ph / 8} / sqrt(N): what multiplies a scaled map's entries when they are read out
+__device__ __forceinline__ Cx<double> readout(uint32_t ph, double N) { return cscale(phase_of(ph), rsqrt(N)); }
+
 template <typename R>
 __device__ __forceinline__ double norm2d(Cx<R> v) {
   const double a = (double)v.x, b = (double)v.y;

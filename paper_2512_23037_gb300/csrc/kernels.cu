@@ -904,12 +904,18 @@ struct Shot {
       fail_capacity();
       return a.y;
     }
+    Cx<R> f{(R)1, (R)0};  // FP64 records hold a scaled map: its norm and the circuit's phase here
+    if constexpr (sizeof(R) == 8) f = readout(top_phase<W>(C, a.y), S.norm[r]);
+    auto value = [&](uint32_t i) {
+      const Cx<R> x = S.vals[(size_t)i * c + r];
+      return sizeof(R) == 8 ? cmul(f, x) : x;
+    };
     if (kRegCapable && nnz <= (uint32_t)G) {
       reg = true;
       if (lane < nnz) {
 #pragma unroll
         for (int w = 0; w < W; ++w) rk.w[w] = S.keys[((size_t)lane * W + w) * c + r];
-        rv = S.vals[(size_t)lane * c + r];
+        rv = value(lane);
       }
       t.sync();
     } else {
@@ -918,7 +924,7 @@ struct Shot {
 #pragma unroll
         for (int w = 0; w < W; ++w) k.w[w] = S.keys[((size_t)i * W + w) * c + r];
         set_key(i, k);
-        vals[i] = S.vals[(size_t)i * c + r];
+        vals[i] = value(i);
       }
       t.sync();
       reg = false;

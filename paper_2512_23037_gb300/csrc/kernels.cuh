@@ -149,8 +149,9 @@ uint32_t lane_first_cap(uint32_t max_n, uint32_t max_d, int fp32);
 uint32_t lane_map_dim();  // directions of a first-round lane's affine map (lane_map_cap = 2^lane_map_dim)
 // After launch_prefix: the affine form of each snapshot of the run (events [0, stop[0]]),
 // on the same stream; stop[3] (zeroed before) receives the largest dimension.
+// ev: the circuit's device events (Ev<W>).
 cudaError_t launch_snap_affine(unsigned char *traj, uint32_t n_snap, uint32_t rw, int fp32, uint32_t W,
-                               uint32_t *stop, cudaStream_t st);
+                               uint32_t *stop, const void *ev, cudaStream_t st);
 
 // Warp-per-shot kernel with the map in affine form (affine.cu), up to 2^p.aff_dim values; it
 // takes the same work items and lists as the shot kernel. A shot that needs more goes to

@@ -26,6 +26,8 @@
 // arithmetic, so the results are those of a single round.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "device_common.cuh"
 #include "kernels.cuh"
 #include "shot_common.cuh"
@@ -167,10 +169,12 @@ struct LaneShot {
   int status, chain, logical, lastm;
   double fid;
   bool force;
+  static constexpr bool kScaled = sizeof(R) == 8;  // FP64 maps are scaled (see ScaledPrune)
+  double nrm;  // their squared norm
 
-  PruneTest<R> pt;  // |v|^2 < tau
+  typename std::conditional<kScaled, ScaledPrune, PruneTest<R>>::type pt;  // |v|^2 < tau
 
-  __device__ LaneShot(const ShotParams &p, unsigned char *base) : P(p), C(&p.circ[0]), pt(p.tau) {
+  __device__ LaneShot(const ShotParams &p, unsigned char *base) : P(p), C(&p.circ[0]), nrm(1.0), pt(p.tau) {
     lane = threadIdx.x & 31u;
     const size_t vb = (size_t)Cap * sizeof(Cx<R>) * 32, rb = (size_t)(1 + 2 * kDim) * W * 8 * 32;
     vals = reinterpret_cast<Cx<R> *>(base);
@@ -240,12 +244,10 @@ struct LaneShot {
       }
     return c;
   }
-  // B[d] = r (nonzero, Dual[k] . r = 0 for k < d); its dual e_p ^ XOR_k B[k][p] Dual[k] for
-  // the lowest set bit p of r is orthogonal to every B[k] and has Dual . r = 1, and the
-  // old duals stay dual (Dual[k] . r = 0)
-  __device__ void add_dim(const uint64_t *r) {
+  // z with z . B[k] = 0 for every k and z . r = 1, for a residual r (nonzero, Dual[k] . r = 0):
+  // e_p ^ XOR_k B[k][p] Dual[k] for the lowest set bit p of r
+  __device__ __forceinline__ void co_dual(const uint64_t *r, uint64_t *z) const {
     const uint32_t p = wlow<W>(r);
-    uint64_t z[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) z[w] = ((int)(p >> 6) == w) ? (1ull << (p & 63u)) : 0ull;
 #pragma unroll 1
@@ -254,42 +256,14 @@ struct LaneShot {
 #pragma unroll
         for (int w = 0; w < W; ++w) z[w] ^= row(kRowD + k, w);
       }
+  }
+  // B[d] = r, a residual; the old duals stay dual
+  __device__ void add_dim(const uint64_t *r) {
+    uint64_t z[W];
+    co_dual(r, z);
     put_row(kRowB + d, r);
     put_row(kRowD + d, z);
     ++d;
-  }
-  // The duals of the current basis, built one vector at a time (the same construction as
-  // add_dim, on each vector's residual against the ones before it).
-  __device__ void rebuild_duals() {
-#pragma unroll 1
-    for (uint32_t k = 0; k < d; ++k) {
-      uint64_t r[W];
-      get_row(kRowB + k, r);
-      uint32_t cm = 0;  // Dual[j] . B[k] for j < k
-#pragma unroll 1
-      for (uint32_t j = 0; j < k; ++j)
-        if (row_par(kRowD + j, r)) cm |= 1u << j;
-#pragma unroll 1
-      for (uint32_t j = 0; j < k; ++j)
-        if ((cm >> j) & 1u) {
-#pragma unroll
-          for (int w = 0; w < W; ++w) r[w] ^= row(kRowB + j, w);
-        }
-      const uint32_t p = wlow<W>(r);
-      uint64_t z[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) z[w] = ((int)(p >> 6) == w) ? (1ull << (p & 63u)) : 0ull;
-#pragma unroll 1
-      for (uint32_t j = 0; j < k; ++j)
-        if (row_bit(kRowB + j, p)) {
-#pragma unroll
-          for (int w = 0; w < W; ++w) z[w] ^= row(kRowD + j, w);
-        }
-#pragma unroll 1
-      for (uint32_t j = 0; j < k; ++j)
-        if ((cm >> j) & 1u) xor_row(kRowD + j, z);
-      put_row(kRowD + k, z);
-    }
   }
   // Every live slot s has parity(s & g) = t, and g has bit q set (q < d): bit q of a live
   // slot follows from the others, so the map needs one coordinate less. alpha0 ^= t B[q],
@@ -412,25 +386,8 @@ struct LaneShot {
     }
   }
 
-  __device__ double uniform(uint32_t ord) const {
-    uint4 w = philox<true>(P.seed, shot, 1u, ord);
-    uint64_t m = ((uint64_t)w.x << 21) ^ (uint64_t)(w.y >> 11);
-    return (double)m * 0x1p-53;
-  }
-  // Outcome +1 iff u < p, with p = sp / (sp + sm) snapped to 0 or 1 within 1e-12:
-  // decided as u (sp + sm) < sp, so that only the fidelity mode divides.
   __device__ __forceinline__ int pick(uint32_t ord, double sp, double sm) {
-    const double tot = sp + sm;
-    if (!(tot > 0.0)) return -1;
-    const bool zero = sp < 1e-12 * tot, one = sp > (1.0 - 1e-12) * tot;
-    if (force) {
-      if (zero) return -1;
-      fid *= one ? 1.0 : sp / tot;
-      return 1;
-    }
-    if (zero) return -1;
-    if (one) return 1;
-    return uniform(ord) * tot < sp ? 1 : -1;
+    return pick_outcome<true>(P.seed, shot, ord, sp, sm, force, fid, nullptr);
   }
   __device__ __forceinline__ R inv_sqrt(double x) const {
     if (sizeof(R) == 4) return (R)rsqrtf((float)x);
@@ -444,6 +401,7 @@ struct LaneShot {
     shot = s;
     status = LS_RUN;
     force = false;
+    nrm = 1.0;
     nxt = cursor.x;
     cur = cursor.y;
     kblk = cursor.z;
@@ -501,6 +459,7 @@ struct LaneShot {
                                               (((uint32_t)lastm & 255u) << 8));
     S.hb[r] = make_uint4(nxt, cur, kblk, w2);
     S.fid[r] = fid;
+    if constexpr (kScaled) S.norm[r] = nrm;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       S.sd[w * c + r] = sd[w];
@@ -534,6 +493,7 @@ struct LaneShot {
     kblk = b.z;
     w2 = b.w;
     fid = S.fid[r];
+    if constexpr (kScaled) nrm = S.norm[r];
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       sd[w] = S.sd[w * c + r];
@@ -559,8 +519,11 @@ struct LaneShot {
     if (!ok) fail_capacity();  // (records come from lanes of at most kDim directions)
     return a.x;
   }
-  // ---- the shot's final state (signs, keys, values) for state capture at offset off
-  __device__ void capture(uint64_t off) const {
+  // ---- the shot's final state (signs, keys, values) for state capture at offset off; ph: the
+  // circuit's global phase where it ended
+  __device__ void capture(uint64_t off, uint32_t ph) const {
+    Cx<double> f{1.0, 0.0};
+    if constexpr (kScaled) f = readout(ph, nrm);
     P.st_nnz[off] = nnz();
     P.st_signs[off * 4 + 0] = sd[0];
     P.st_signs[off * 4 + 1] = (W == 2) ? sd[W - 1] : 0ull;
@@ -571,7 +534,8 @@ struct LaneShot {
     for (Mask m = live; m && i < P.st_stride; m &= m - (Mask)1, ++i) {
       const uint32_t s = mffs(m) - 1;
       const Key<W> k = key_of(s);
-      const Cx<R> v = val(s);
+      Cx<R> v = val(s);
+      if constexpr (kScaled) v = cmul(f, v);
       const size_t o = (size_t)off * P.st_stride + i;
       P.st_keys[2 * o] = k.w[0];
       P.st_keys[2 * o + 1] = (W == 2) ? k.w[W - 1] : 0ull;
@@ -628,6 +592,15 @@ struct LaneShot {
     apply_pauli(beta, gamma, ((__ldg(&S->c0) >> (2u * code)) + 2u * wordpar(pe)) & 3u);
   }
 
+  // (rare: many rotations, or very unlikely outcomes, since the last sampled outcome)
+  __device__ __forceinline__ void fit_norm() {
+    for (int k = 0; k < 32 && !ScaledPrune::in_range(nrm); ++k) {  // (bounded: an empty map has norm 0)
+      const double f = ScaledPrune::fit(nrm);
+#pragma unroll 1
+      for (Mask m = live; m; m &= m - (Mask)1) set_val(mffs(m) - 1, cscale(val(mffs(m) - 1), (R)f));
+      nrm = nrm * f * f;
+    }
+  }
   // ---- a I + b Z_q: v'_a = a v_a + b xi_{a^beta} v_{a^beta}; xi = i^e (-1)^{gamma.key}
   // folded into b (b or -b per entry, exact), and a diagonal rotation (beta = 0) is one
   // product (a + b xi) v per entry. gl, g0: gamma's parities with the basis and alpha0 on
@@ -641,27 +614,45 @@ struct LaneShot {
       return;
     }
     const Coef *cf = C->coef + ci;
-    Cx<R> a, b;
-    if (sizeof(R) == 4) {
+    Cx<R> a{0, 0}, bq{0, 0}, bn{0, 0};  // FP32: a, and b with the phase folded in, and its negation
+    double k = 0.0, cm = 1.0;           // FP64: v' = cm v + i^{e + 3} k (-1)^{gamma.key} v_partner
+    if constexpr (!kScaled) {
       const float4 f = __ldg(reinterpret_cast<const float4 *>(&cf->fa_re));
       a = Cx<R>{(R)f.x, (R)f.y};
-      b = Cx<R>{(R)f.z, (R)f.w};
+      bq = ipow(Cx<R>{(R)f.z, (R)f.w}, e);
+      bn = Cx<R>{negr(bq.x), negr(bq.y)};
     } else {
-      const double2 d0 = __ldg(reinterpret_cast<const double2 *>(&cf->a_re));
-      const double2 d1 = __ldg(reinterpret_cast<const double2 *>(&cf->b_re));
-      a = Cx<R>{(R)d0.x, (R)d0.y};
-      b = Cx<R>{(R)d1.x, (R)d1.y};
+      const double2 kc = __ldg(reinterpret_cast<const double2 *>(&cf->k));
+      k = kc.x;
+      cm = kc.y;
     }
-    const Cx<R> bq = ipow(b, e), bn = Cx<R>{negr(bq.x), negr(bq.y)};
+    const bool plain = kScaled && __double2hiint(cm) != 0x3FF00000;
+    const ScaledTurn turn(k, (e + 3u) & 3u);
+    auto base = [&](Cx<R> v) { return plain ? cscale(v, (R)cm) : v; };
+    // the norm takes its factor once the event is certain to happen
+    auto scale = [&]() {
+      if constexpr (kScaled) {
+        if (!plain) nrm = mulr(nrm, __ldg(&cf->n2));
+        fit_norm();
+        pt.set(nrm);
+      }
+    };
+    auto small = [&](Cx<R> v) {
+      if constexpr (kScaled) return pt.small(v, nrm);
+      else return pt.small(v);
+    };
     Mask drop = 0;
     if (diag) {
-      const Cx<R> c0 = cadd(a, bq), c1 = cadd(a, bn);
+      const Cx<R> c0 = kScaled ? a : cadd(a, bq), c1 = kScaled ? a : cadd(a, bn);
       const Mask odd = par_mask(gl, g0);
+      scale();
 #pragma unroll 1
       for (Mask m = live; m; m &= m - (Mask)1) {
         const uint32_t s = mffs(m) - 1;
-        const Cx<R> nv = cmul(in_mask(odd, s) ? c1 : c0, val(s));
-        const bool sm = pt.small(nv);
+        Cx<R> nv = val(s);
+        if constexpr (kScaled) nv = turn.add(base(nv), nv, in_mask(odd, s));
+        else nv = cmul(in_mask(odd, s) ? c1 : c0, nv);
+        const bool sm = small(nv);
         if (!sm) set_val(s, nv);
         drop |= (Mask)sm << s;
       }
@@ -694,24 +685,25 @@ struct LaneShot {
     const Mask odd = par_mask(gl, g0);
     const Mask spread = live | slot_xor_perm<Mask, kDim>(live, c);
     const Mask lead = spread & ~slot_bit_mask<Mask>(__ffs(c) - 1) & cube();  // one member of each pair
+    scale();
 #pragma unroll 1
     for (Mask m = lead; m; m &= m - (Mask)1) {
       const uint32_t s = mffs(m) - 1, t = s ^ c;
       const uint32_t ls = in_mask(live, s), lt = in_mask(live, t);
       const Cx<R> vs = ls ? val(s) : Cx<R>{0, 0}, vt = lt ? val(t) : Cx<R>{0, 0};
-      const Cx<R> bs = in_mask(odd, s) ? bn : bq, bt = in_mask(odd, t) ? bn : bq;
       Cx<R> ns, nt;
-      if (ls && lt) {  // one fused chain per component
+      if constexpr (kScaled) {
+        ns = base(vs);
+        nt = base(vt);
+        if (lt) ns = turn.add(ns, vt, in_mask(odd, t));  // (skipped by a warp whose entries gain partners)
+        if (ls) nt = turn.add(nt, vs, in_mask(odd, s));
+      } else {
+        // one fused chain per component; with a zero partner it rounds as the single product
+        const Cx<R> bs = in_mask(odd, s) ? bn : bq, bt = in_mask(odd, t) ? bn : bq;
         ns = cmad2(a, vs, bt, vt);
         nt = cmad2(a, vt, bs, vs);
-      } else if (ls) {  // an entry without a partner gains one
-        ns = cmul(a, vs);
-        nt = cmul(bs, vs);
-      } else {
-        ns = cmul(bt, vt);
-        nt = cmul(a, vt);
       }
-      const bool ss_ = pt.small(ns), st_ = pt.small(nt);
+      const bool ss_ = small(ns), st_ = small(nt);
       if (!ss_) set_val(s, ns);
       if (!st_) set_val(t, nt);
       drop |= ((Mask)ss_ << s) | ((Mask)st_ << t);
@@ -741,15 +733,30 @@ struct LaneShot {
       if (!gl || !live) return m;
     } else {
       double sp = 0.0, sm = 0.0;
+      if constexpr (kScaled) {  // two fused multiply-adds per entry, one side after the other
 #pragma unroll 1
-      for (Mask mm = live; mm; mm &= mm - (Mask)1) {
-        const uint32_t s = mffs(mm) - 1;
-        const double a2 = pnorm(val(s));
-        if ((neg >> s) & 1u) sm += a2;
-        else sp += a2;
+        for (int side = 0; side < 2; ++side) {
+          double acc = 0.0;
+#pragma unroll 1
+          for (Mask mm = side ? neg : pos; mm; mm &= mm - (Mask)1) {
+            const Cx<R> v = val(mffs(mm) - 1);
+            acc = __fma_rn((double)v.x, (double)v.x, __fma_rn((double)v.y, (double)v.y, acc));
+          }
+          sp = side ? sp : acc;
+          sm = acc;
+        }
+      } else {
+#pragma unroll 1
+        for (Mask mm = live; mm; mm &= mm - (Mask)1) {
+          const uint32_t s = mffs(mm) - 1;
+          const double a2 = pnorm(val(s));
+          if ((neg >> s) & 1u) sm += a2;
+          else sp += a2;
+        }
       }
       m = pick(ord, sp, sm);
-      sc = inv_sqrt(m == 1 ? sp : sm);
+      if constexpr (kScaled) nrm = m == 1 ? sp : sm;
+      else sc = inv_sqrt(m == 1 ? sp : sm);
       keep = (m == 1) ? pos : neg;
     }
     // the kept slots share parity(s & gl) = t, so bit q of their index is redundant; each is
@@ -761,10 +768,15 @@ struct LaneShot {
 #pragma unroll 1
     for (Mask mm = keep; mm; mm &= mm - (Mask)1) {  // ascending: a write lands on a slot already read
       const uint32_t s = mffs(mm) - 1, s2 = (s & lo) | ((s >> (q + 1u)) << q);
-      const Cx<R> v = cscale(val(s), sc);
-      if (!pt.small(v)) {
-        set_val(s2, v);
+      if constexpr (kScaled) {  // (normalising raises every entry: none falls below tau)
+        set_val(s2, val(s));
         nl |= (Mask)1 << s2;
+      } else {
+        const Cx<R> v = cscale(val(s), sc);
+        if (!pt.small(v)) {
+          set_val(s2, v);
+          nl |= (Mask)1 << s2;
+        }
       }
     }
     if (nl) remove_rows(q, gl, t);
@@ -819,53 +831,109 @@ struct LaneShot {
     const bool lone = wnonzero<W>(rr);  // e_p outside the span: no entry has a partner
     const Mask spread = lone ? live : (live | slot_xor_perm<Mask, kDim>(live, c));
     const Mask lead = lone ? live : (spread & ~kb);  // a0 members (lone: every entry)
-    double sp = 0.0, sm = 0.0;
-#pragma unroll 1
-    for (Mask m = lead; m; m &= m - (Mask)1) {
-      const uint32_t s = mffs(m) - 1;
-      Cx<R> v0{0, 0}, x1{0, 0};
-      if (lone) {
-        if ((kb >> s) & 1u) x1 = ipow(val(s), e2 + 2u * in_mask(odd, s));
-        else v0 = val(s);
-      } else {
-        const uint32_t t = s ^ c;
-        if ((live >> s) & 1u) v0 = val(s);
-        if ((live >> t) & 1u) x1 = ipow(val(t), e2 + 2u * in_mask(odd, t));
-      }
-      sp += 0.5 * pnorm(cadd(v0, x1));
-      sm += 0.5 * pnorm(csub(v0, x1));
-    }
-    const int m = pick(ord, sp, sm);
-    const R sc = inv_sqrt(2.0 * (m == 1 ? sp : sm));
+    int m;
     Mask nl = 0;
-#pragma unroll 1
-    for (Mask mm = lead; mm; mm &= mm - (Mask)1) {
-      const uint32_t s = mffs(mm) - 1;
-      Cx<R> v0{0, 0}, x1{0, 0};
+    if constexpr (kScaled) {
       if (lone) {
-        if ((kb >> s) & 1u) x1 = ipow(val(s), e2 + 2u * in_mask(odd, s));
-        else v0 = val(s);
+        // every entry stays, those with key bit p as m xi v: p = 1/2 exactly, so the outcome is
+        // one random bit and the norm stays
+        m = force ? 1 : (philox<true>(P.seed, shot, 1u, ord).x >> 31) ? -1 : 1;
+        if (force) fid *= 0.5;
+#pragma unroll 1
+        for (Mask mm = live & kb; mm; mm &= mm - (Mask)1) {
+          const uint32_t s = mffs(mm) - 1;
+          set_val(s, ipow(val(s), e2 + 2u * in_mask(odd, s) + (m == -1 ? 2u : 0u)));
+        }
+        nl = live;
       } else {
-        const uint32_t t = s ^ c;
-        if ((live >> s) & 1u) v0 = val(s);
-        if ((live >> t) & 1u) x1 = ipow(val(t), e2 + 2u * in_mask(odd, t));
+        // sp, sm = (N +- 2 C) / 2 with N the pairs' norm and C = sum Re conj(v0) x1; the kept
+        // side's own norm is summed from the values it keeps
+        double sn = 0.0, cr = 0.0;
+#pragma unroll 1
+        for (Mask mm = lead; mm; mm &= mm - (Mask)1) {
+          const uint32_t s = mffs(mm) - 1, t = s ^ c;
+          Cx<R> v0{0, 0}, x1{0, 0};
+          if (in_mask(live, s)) v0 = val(s);
+          if (in_mask(live, t)) x1 = ipow(val(t), e2 + 2u * in_mask(odd, t));
+          sn = fmar((double)v0.x, (double)v0.x, fmar((double)v0.y, (double)v0.y, sn));
+          sn = fmar((double)x1.x, (double)x1.x, fmar((double)x1.y, (double)x1.y, sn));
+          cr = fmar((double)v0.x, (double)x1.x, fmar((double)v0.y, (double)x1.y, cr));
+        }
+        const double sp = fmar(0.5, sn, cr), sm = fmar(0.5, sn, -cr);
+        m = pick(ord, sp, sm);
+        nrm = 2.0 * (m == 1 ? sp : sm);
+        fit_norm();
+        pt.set(nrm);
+        const uint32_t flip = m == -1 ? 2u : 0u;
+        double kn = 0.0;
+#pragma unroll 1
+        for (Mask mm = lead; mm; mm &= mm - (Mask)1) {
+          const uint32_t s = mffs(mm) - 1, t = s ^ c;
+          Cx<R> v0{0, 0}, x1{0, 0};
+          if (in_mask(live, s)) v0 = val(s);
+          if (in_mask(live, t)) x1 = ipow(val(t), e2 + flip + 2u * in_mask(odd, t));
+          const Cx<R> nv = cadd(v0, x1);
+          kn = fmar((double)nv.x, (double)nv.x, fmar((double)nv.y, (double)nv.y, kn));
+          if (!pt.small(nv, nrm)) {
+            set_val(s, nv);
+            nl |= (Mask)1 << s;
+          }
+        }
+        nrm = kn;
       }
-      const Cx<R> nv = cscale(m == 1 ? cadd(v0, x1) : csub(v0, x1), sc);
-      if (!pt.small(nv)) {
-        set_val(s, nv);
-        nl |= (Mask)1 << s;
+    } else {
+      double sp = 0.0, sm = 0.0;
+#pragma unroll 1
+      for (Mask mm = lead; mm; mm &= mm - (Mask)1) {
+        const uint32_t s = mffs(mm) - 1;
+        Cx<R> v0{0, 0}, x1{0, 0};
+        if (lone) {
+          if (in_mask(kb, s)) x1 = ipow(val(s), e2 + 2u * in_mask(odd, s));
+          else v0 = val(s);
+        } else {
+          const uint32_t t = s ^ c;
+          if (in_mask(live, s)) v0 = val(s);
+          if (in_mask(live, t)) x1 = ipow(val(t), e2 + 2u * in_mask(odd, t));
+        }
+        sp += 0.5 * pnorm(cadd(v0, x1));
+        sm += 0.5 * pnorm(csub(v0, x1));
+      }
+      m = pick(ord, sp, sm);
+      const R sc = inv_sqrt(2.0 * (m == 1 ? sp : sm));
+#pragma unroll 1
+      for (Mask mm = lead; mm; mm &= mm - (Mask)1) {
+        const uint32_t s = mffs(mm) - 1;
+        Cx<R> v0{0, 0}, x1{0, 0};
+        if (lone) {
+          if (in_mask(kb, s)) x1 = ipow(val(s), e2 + 2u * in_mask(odd, s));
+          else v0 = val(s);
+        } else {
+          const uint32_t t = s ^ c;
+          if (in_mask(live, s)) v0 = val(s);
+          if (in_mask(live, t)) x1 = ipow(val(t), e2 + 2u * in_mask(odd, t));
+        }
+        const Cx<R> nv = cscale(m == 1 ? cadd(v0, x1) : csub(v0, x1), sc);
+        if (!pt.small(nv)) {
+          set_val(s, nv);
+          nl |= (Mask)1 << s;
+        }
       }
     }
     live = nl;
     if (lone) {
       // every key loses bit p (a1 keys become a1 ^ e_p); injective on the space since e_p is
-      // not in the span, so the slots stay, and the basis is rebuilt with new duals
+      // not in the span, so the slots stay. With z . B[k] = 0 for every k and z[p] = 1 (the dual
+      // of e_p's residual), D[k] ^= D[k][p] z clears bit p of the duals and keeps them dual
+      uint64_t z[W];
+      co_dual(rr, z);
+#pragma unroll 1
+      for (uint32_t k = 0; k < d; ++k)
+        if (row_bit(kRowD + k, p)) xor_row(kRowD + k, z);
 #pragma unroll 1
       for (uint32_t k = 0; k <= d; ++k) {
         const uint32_t r2 = k == 0 ? 0u : kRowB + k - 1u;
         if (row_bit(r2, p)) xor_row(r2, ep);
       }
-      rebuild_duals();
     } else {
       restrict_to(bp);  // the kept keys have bit p clear: parity(s & bp) = alpha0[p]
     }
@@ -977,7 +1045,7 @@ struct LaneShot {
 // largest dimension goes to stop[3] (0xFF where a map needs more than kSnapDim)
 template <typename R, int W>
 __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_t stride, uint32_t rw,
-                                   uint32_t *stop) {
+                                   uint32_t *stop, const void *ev) {
   const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_snap || e > stop[0]) return;
   unsigned char *in = traj + (size_t)e * stride;
@@ -991,6 +1059,8 @@ __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_
   for (uint32_t r = 0; r < 1 + 2 * kSnapDim; ++r)
     for (int w = 0; w < W; ++w) rw_[r][w] = 0ull;
   for (uint32_t j = 0; j < (1u << kSnapDim); ++j) out->v[j] = Cx<R>{0, 0};
+  Cx<R> turn{(R)1, (R)0};  // FP64: the circuit's global phase is taken out (scaled maps)
+  if constexpr (sizeof(R) == 8) turn = phase_of(e ? (16u - ev_phase(reinterpret_cast<const Ev<W> *>(ev)[e - 1u].w0)) & 15u : 0u);
   uint32_t d = 0;
   unsigned long long live = 0;
   bool ok = true;
@@ -1024,7 +1094,7 @@ __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_
       c |= 1u << d;
       ++d;
     }
-    out->v[c] = v_in[i];
+    out->v[c] = sizeof(R) == 8 ? cmul(turn, v_in[i]) : v_in[i];
     live |= 1ull << c;
   }
   for (uint32_t r = 0; r < 1 + 2 * kSnapDim; ++r)
@@ -1293,7 +1363,7 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
           if (s.logical) atomicAdd(&wt[warp][4], 1ull);
           if (P.fid_mode && C->fsum) atomicAdd(C->fsum, s.fid);
         }
-        if (!Multi && off < P.st_limit) s.capture(off);
+        if (!Multi && off < P.st_limit) s.capture(off, top_phase<W>(C, e < n_ev ? e + 1u : n_ev));
         if (off < C->out_limit) {
           if (C->status) C->status[off] = (uint8_t)s.status;
           if (C->records)
@@ -1384,14 +1454,14 @@ uint32_t lane_first_cap(uint32_t max_n, uint32_t max_d, int fp32) {
 }
 
 cudaError_t launch_snap_affine(unsigned char *traj, uint32_t n_snap, uint32_t rw, int fp32, uint32_t W,
-                               uint32_t *stop, cudaStream_t st) {
+                               uint32_t *stop, const void *ev, cudaStream_t st) {
   const unsigned grid = (n_snap + 127) / 128;
   if (fp32) {
-    if (W == 1) snap_affine_kernel<float, 1><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<float, 1>(rw), rw, stop);
-    else snap_affine_kernel<float, 2><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<float, 2>(rw), rw, stop);
+    if (W == 1) snap_affine_kernel<float, 1><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<float, 1>(rw), rw, stop, ev);
+    else snap_affine_kernel<float, 2><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<float, 2>(rw), rw, stop, ev);
   } else {
-    if (W == 1) snap_affine_kernel<double, 1><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<double, 1>(rw), rw, stop);
-    else snap_affine_kernel<double, 2><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<double, 2>(rw), rw, stop);
+    if (W == 1) snap_affine_kernel<double, 1><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<double, 1>(rw), rw, stop, ev);
+    else snap_affine_kernel<double, 2><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<double, 2>(rw), rw, stop, ev);
   }
   return cudaGetLastError();
 }

@@ -43,7 +43,9 @@ enum : uint32_t {
   F_COND_REC = 128   // PAULI: apply if parity of records a, b is 1
 };
 
-// Header word 0: type (bits 0-3) | flags (4-11) | e0 (12-13) | lowbit (16-23) | xe0 (24-25).
+// Header word 0: type (bits 0-3) | flags (4-11) | e0 (12-13) | lowbit (16-23) | xe0 (24-25) |
+// phase (26-29): the global phase of the circuit's T gates up to and including this event,
+// in units of pi/8 (T counts 1, T^dag -1; Rz with a negative cosine 8, else none).
 // The gap search's index: bucket b of the top kThrTabBits bits of U holds the
 // first gap g with U < thr[g] for the bucket's lowest U (bucket 2^bits: n_sites).
 constexpr uint32_t kThrTabBits = 12;
@@ -53,6 +55,7 @@ SOFT_HD inline uint32_t ev_flags(uint32_t w0) { return (w0 >> 4) & 255u; }
 SOFT_HD inline uint32_t ev_e0(uint32_t w0) { return (w0 >> 12) & 3u; }
 SOFT_HD inline uint32_t ev_lowbit(uint32_t w0) { return (w0 >> 16) & 255u; }
 SOFT_HD inline uint32_t ev_xe0(uint32_t w0) { return (w0 >> 24) & 3u; }
+SOFT_HD inline uint32_t ev_phase(uint32_t w0) { return (w0 >> 26) & 15u; }
 inline uint32_t ev_pack(uint32_t type, uint32_t flags, uint32_t e0, uint32_t lowbit) {
   return (type & 15u) | ((flags & 255u) << 4) | ((e0 & 3u) << 12) | ((lowbit & 255u) << 16);
 }
@@ -77,10 +80,14 @@ struct alignas(16) Ev {
   uint64_t xbeta[W], xgamma[W];  // MEAS with F_COND_LAST: X_q after the measurement
 };
 
-// a I + b Z_q coefficients, FP64 and the FP32 copies the FP32 kernel uses.
+// a I + b Z_q coefficients, FP64 and the FP32 copies the FP32 kernel uses. Every rotation is
+// a phase times c I - i s Z_q (c, s real); scaled FP64 maps (dev::ScaledPrune) use
+//   cm I - i k Z_q, with a factor n2 on the map's squared norm:
+// k = s / c, cm = 1, n2 = 1 / c^2, unless |s| > sqrt(3) |c|: then k = s, cm = c, n2 = 1.
 struct alignas(16) Coef {
   double a_re, a_im, b_re, b_im;
   float fa_re, fa_im, fb_re, fb_im;
+  double k, cm, n2, pad;
 };
 
 // Constants of a case-B measurement of P (pivot p, J = other rows whose

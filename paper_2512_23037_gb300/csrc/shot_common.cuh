@@ -73,6 +73,11 @@ __device__ __forceinline__ uint32_t first_event(const CircDev *C, int fid_mode, 
 
 // Snapshot of the noiseless run at the top of an event: header, rw record words,
 // kSnapMax keys (W words each), kSnapMax values.
+// The phase of the events before e (Ev::w0, in units of pi/8): the top of event e.
+template <int W>
+__device__ __forceinline__ uint32_t top_phase(const CircDev *C, uint32_t e) {
+  return e ? ev_phase(__ldg(&reinterpret_cast<const Ev<W> *>(C->ev)[e - 1u].w0)) : 0u;
+}
 struct SnapHdr {
   uint32_t nnz, chain, logical, lastm;
   double fid;
@@ -84,7 +89,8 @@ constexpr uint32_t kSnapMax = 64;
 // The snapshot's map in the affine form of the lane kernels (lanes.cu): d directions
 // (0xFFFFFFFF: more than kSnapDim), the live slots (bit s: slot s), rows alpha0,
 // B[0..kSnapDim), Dual[0..kSnapDim), and the values of 2^kSnapDim slots (zero where not
-// live). Computed once per circuit and precision, after the noiseless run.
+// live; FP64: without the global phase, as scaled maps hold them). Computed once per circuit
+// and precision, after the noiseless run.
 constexpr uint32_t kSnapDim = 6;
 template <typename R, int W>
 struct SnapAffine {
@@ -113,9 +119,42 @@ static_assert(kLaneCap >= 2 && kLaneCap <= 16, "lane map capacity (partner indic
 constexpr uint32_t kSpillRef = 0x80000000u;
 constexpr uint32_t kNoRecord = 0xFFFFFFFFu;
 
+// The outcome +1 (or -1) of a measurement with unnormalised probabilities sp and sm: +1 iff
+// u < p, p = sp / (sp + sm) snapped to 0 or 1 within 1e-12, decided as u (sp + sm) < sp. The
+// random words are Philox's for the measurement's ordinal. Sums whose 21-bit truncations
+// settle the snap and the comparison (all but 1 in 10^5) are decided in FP32, which keeps
+// eight instructions off the FP64 pipe; the others exactly. force: fidelity mode, projects
+// onto +1 with weight p in fid. *undecided is set where the outcome depended on u.
+template <bool Rolled>
+__device__ __forceinline__ int pick_outcome(uint64_t seed, uint64_t shot, uint32_t ord, double sp, double sm, bool force,
+                                            double &fid, bool *undecided) {
+  const float a = low_float(sp), t = a + low_float(sm);
+  const bool clear = a > 1e-5f * t && a < (1.0f - 1e-5f) * t;
+  if (!clear || force) {
+    const double tot = sp + sm;
+    if (!(tot > 0.0)) return -1;
+    const bool zero = sp < 1e-12 * tot, one = sp > (1.0 - 1e-12) * tot;
+    if (undecided && !zero && !one) *undecided = true;
+    if (force) {
+      if (zero) return -1;
+      fid *= one ? 1.0 : sp / tot;
+      return 1;
+    }
+    if (zero) return -1;
+    if (one) return 1;
+  }
+  if (undecided) *undecided = true;
+  const uint4 w = philox<Rolled>(seed, shot, 1u, ord);
+  const float diff = (float)w.x * 0x1p-32f * t - a;
+  if (fabsf(diff) > 1e-5f * t) return diff < 0.0f ? 1 : -1;
+  const uint64_t m = ((uint64_t)w.x << 21) ^ (uint64_t)(w.y >> 11);
+  return (double)m * 0x1p-53 * (sp + sm) < sp ? 1 : -1;
+}
+
 // A spill record holds one shot's whole state at the top of an event: item,
 // resume event, n and flags (chain, logical, last outcome); the noise cursor
-// (nxt, cur, kblk, w2); F; the signs; the record words; up to kLaneCap entries.
+// (nxt, cur, kblk, w2); F; the signs; the record words; up to kLaneCap entries (FP64: of a
+// scaled map, and its squared norm).
 // Structure of arrays over `cap` records.
 template <typename R, int W>
 struct Spill {
@@ -123,12 +162,13 @@ struct Spill {
   double *fid;
   uint64_t *sd, *ss, *rec, *keys;
   Cx<R> *vals;
+  double *norm;  // FP64 only
   uint32_t cap;
   __host__ __device__ static size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
   __host__ __device__ static size_t bytes(uint32_t cap, uint32_t rw) {
     const size_t c = cap;
     return 2 * al16(c * 16) + al16(c * 8) + 2 * al16(c * 8 * W) + al16(c * 8 * rw) + al16(c * 8 * W * kLaneCap) +
-           al16(c * sizeof(Cx<R>) * kLaneCap);
+           al16(c * sizeof(Cx<R>) * kLaneCap) + (sizeof(R) == 8 ? al16(c * 8) : 0);
   }
   __device__ Spill(unsigned char *b, uint32_t cap_, uint32_t rw) : cap(cap_) {
     const size_t c = cap;
@@ -147,6 +187,8 @@ struct Spill {
     keys = reinterpret_cast<uint64_t *>(b);
     b += al16(c * 8 * W * kLaneCap);
     vals = reinterpret_cast<Cx<R> *>(b);
+    b += al16(c * sizeof(Cx<R>) * kLaneCap);
+    norm = reinterpret_cast<double *>(b);
   }
 };
 
