@@ -1079,12 +1079,16 @@ struct GradWarp {
     uint64_t sd[2], ss[2];
   };
   __host__ __device__ static constexpr size_t snap_stride(uint32_t rw) {
-    return (sizeof(SnapHdr) + (size_t)rw * 8 + 32 * (size_t)W * 8 + 32 * sizeof(Cx<R>) + 15) & ~(size_t)15;
+    return (snap_keys_off(rw) + 32 * (size_t)W * 8 + 32 * sizeof(Cx<R>) + 15) & ~(size_t)15;
+  }
+  // where the keys start (a multiple of 16, so that the values are aligned)
+  __host__ __device__ static constexpr size_t snap_keys_off(uint32_t rw) {
+    return sizeof(SnapHdr) + (size_t)((rw + 1u) & ~1u) * 8;
   }
   __device__ void save_snapshot(unsigned char *out) {
     SnapHdr *h = reinterpret_cast<SnapHdr *>(out);
     uint64_t *r_out = reinterpret_cast<uint64_t *>(out + sizeof(SnapHdr));
-    uint64_t *k_out = r_out + P.rw;
+    uint64_t *k_out = reinterpret_cast<uint64_t *>(out + snap_keys_off(P.rw));
     Cx<R> *v_out = reinterpret_cast<Cx<R> *>(k_out + 32 * W);
     if (lane == 0) {
       h->nnz = phi.n;
@@ -1113,7 +1117,7 @@ struct GradWarp {
     const unsigned char *in = P.psnap + (size_t)ev0 * P.psnap_stride;
     const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
     const uint64_t *r_in = reinterpret_cast<const uint64_t *>(in + sizeof(SnapHdr));
-    const uint64_t *k_in = r_in + P.rw;
+    const uint64_t *k_in = reinterpret_cast<const uint64_t *>(in + snap_keys_off(P.rw));
     const Cx<R> *v_in = reinterpret_cast<const Cx<R> *>(k_in + 32 * W);
     phi.n = h->nnz;
     r0 = r = h->r;

@@ -8,8 +8,9 @@
 namespace soft {
 namespace dev {
 
+// Aligned to its size, so that both components move in one load or store of 8 or 16 bytes.
 template <typename R>
-struct Cx {
+struct alignas(2 * sizeof(R)) Cx {
   R x, y;
 };
 // Real arithmetic with fixed rounding: explicit round-to-nearest intrinsics, so that no

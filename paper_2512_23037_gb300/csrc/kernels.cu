@@ -758,7 +758,7 @@ struct Shot {
   __device__ void save_snapshot(unsigned char *out) {
     SnapHdr *h = reinterpret_cast<SnapHdr *>(out);
     uint64_t *rw_out = reinterpret_cast<uint64_t *>(out + sizeof(SnapHdr));
-    uint64_t *k_out = rw_out + C->rw;
+    uint64_t *k_out = reinterpret_cast<uint64_t *>(out + snap_keys_off(C->rw));
     Cx<R> *v_out = reinterpret_cast<Cx<R> *>(k_out + kSnapMax * W);
     if (lane == 0) {
       h->nnz = nnz;
@@ -796,7 +796,7 @@ struct Shot {
     const unsigned char *in = C->traj + (size_t)lo * C->traj_stride;
     const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
     const uint64_t *r_in = reinterpret_cast<const uint64_t *>(in + sizeof(SnapHdr));
-    const uint64_t *k_in = r_in + C->rw;
+    const uint64_t *k_in = reinterpret_cast<const uint64_t *>(in + snap_keys_off(C->rw));
     const Cx<R> *v_in = reinterpret_cast<const Cx<R> *>(k_in + kSnapMax * W);
     nnz = __ldg(&h->nnz);
     chain = (int)__ldg(&h->chain);

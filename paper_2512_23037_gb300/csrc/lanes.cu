@@ -1050,7 +1050,7 @@ __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_
   if (e >= n_snap || e > stop[0]) return;
   unsigned char *in = traj + (size_t)e * stride;
   const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
-  const uint64_t *k_in = reinterpret_cast<const uint64_t *>(in + sizeof(SnapHdr)) + rw;
+  const uint64_t *k_in = reinterpret_cast<const uint64_t *>(in + snap_keys_off(rw));
   const Cx<R> *v_in = reinterpret_cast<const Cx<R> *>(k_in + kSnapMax * W);
   SnapAffine<R, W> *out = reinterpret_cast<SnapAffine<R, W> *>(in + snap_affine_off<R, W>(rw));
   const uint32_t n = h->nnz < kSnapMax ? h->nnz : kSnapMax;

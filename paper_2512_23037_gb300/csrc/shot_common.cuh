@@ -82,9 +82,12 @@ struct SnapHdr {
   uint32_t nnz, chain, logical, lastm;
   double fid;
   uint64_t sd[2], ss[2];
-  uint64_t pad[2];
+  uint64_t pad;
 };
+static_assert(sizeof(SnapHdr) == 64, "snapshot header");
 constexpr uint32_t kSnapMax = 64;
+// where the keys start (a multiple of 16, so that FP64 values are aligned)
+__host__ __device__ constexpr size_t snap_keys_off(uint32_t rw) { return sizeof(SnapHdr) + (size_t)((rw + 1u) & ~1u) * 8; }
 
 // The snapshot's map in the affine form of the lane kernels (lanes.cu): d directions
 // (0xFFFFFFFF: more than kSnapDim), the live slots (bit s: slot s), rows alpha0,
@@ -95,13 +98,12 @@ constexpr uint32_t kSnapDim = 6;
 template <typename R, int W>
 struct SnapAffine {
   uint32_t d, live_lo, live_hi, pad;  // live: the slot set, in two words
-  uint64_t rows[1 + 2 * kSnapDim][W];
+  uint64_t rows[2 + 2 * kSnapDim][W];  // (one row of padding: v is 16-byte aligned)
   Cx<R> v[1u << kSnapDim];
 };
 template <typename R, int W>
 __host__ __device__ constexpr size_t snap_affine_off(uint32_t rw) {
-  return (sizeof(SnapHdr) + (size_t)rw * 8 + kSnapMax * (size_t)W * 8 + kSnapMax * sizeof(Cx<R>) + 15) &
-         ~(size_t)15;
+  return (snap_keys_off(rw) + kSnapMax * (size_t)W * 8 + kSnapMax * sizeof(Cx<R>) + 15) & ~(size_t)15;
 }
 template <typename R, int W>
 __host__ __device__ constexpr size_t snap_stride(uint32_t rw) {
