@@ -80,7 +80,7 @@ struct AffShot {
   uint64_t shot;
   uint64_t sd[W], ss[W];
   uint32_t d;
-  uint32_t nxt, cur, kblk, w2;
+  NoiseCursor nc;
   int status, chain, logical, lastm;
   double fid;
   bool force;
@@ -264,66 +264,33 @@ struct AffShot {
     for (uint32_t s = lane; s < size(); s += 32) v[s] = a->v[s];
     __syncwarp();
   }
-  // ---- resumption from a lane's hand-over record: lane i takes entry i; the keys'
-  // differences are reduced against the directions found so far, each new direction the
-  // first nonzero residual. Returns the event to resume at.
+  // ---- resumption from a lane's record (eviction or hand-over), which holds the same form.
+  // Returns the event to resume at.
   __device__ uint32_t load_spill(uint32_t r) {
-    const Spill<R, W> S(P.sp, P.sp_cap, P.rw_max);
-    const size_t c = S.cap;
-    const uint4 a = S.ha[r], b = S.hb[r];
-    const uint32_t n = a.z;
-    chain = (int)(a.w & 1u);
-    logical = (int)((a.w >> 1) & 1u);
-    lastm = (int)(int8_t)((a.w >> 8) & 255u);
-    nxt = b.x;
-    cur = b.y;
-    kblk = b.z;
-    w2 = b.w;
-    fid = S.fid[r];
-    if constexpr (kScaled) nrm = S.norm[r];
-    recw = lane < C->rw ? S.rec[lane * c + r] : 0ull;
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      sd[w] = S.sd[w * c + r];
-      ss[w] = S.ss[w * c + r];
-      B[w] = D[w] = 0ull;
-    }
-    d = 0;
-    if (n > kLaneCap || a.y >= C->n_events) {  // a record never holds more, nor resumes past the end
-      fail_check(CHK_NNZ, n);
+    const Spill<R, W> S(P.sp, P.rw_max, kLaneDim);
+    unsigned char *p = S.at(r);
+    const uint4 a = S.ha(p), b = S.hb(p);
+    d = a.w & 255u;
+    chain = (int)((a.w >> 8) & 1u);
+    logical = (int)((a.w >> 9) & 1u);
+    lastm = (int)(int8_t)((a.w >> 16) & 255u);
+    nc = NoiseCursor{b.x, b.y, b.z};
+    fid = S.fid(p);
+    if constexpr (kScaled) nrm = S.norm(p);
+    recw = lane < C->rw ? S.rec(p)[lane] : 0ull;
+    if (d > kLaneDim || d > P.aff_dim || a.y >= C->n_events) {  // a record never holds more, nor resumes past the end
+      fail_check(CHK_NNZ, d);
       return C->n_events;
     }
-    uint64_t x[W];
-    Cx<R> val{0, 0};
-#pragma unroll
-    for (int w = 0; w < W; ++w) x[w] = lane < n ? S.keys[((size_t)lane * W + w) * c + r] : 0ull;
-    if (lane < n) val = S.vals[(size_t)lane * c + r];
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      a0[w] = shfl64(x[w], 0);
-      x[w] = lane < n ? x[w] ^ a0[w] : 0ull;
+      sd[w] = S.sd(p)[w];
+      ss[w] = S.ss(p)[w];
+      a0[w] = S.rows(p)[w];
+      B[w] = lane < d ? S.rows(p)[(1 + lane) * W + w] : 0ull;
+      D[w] = lane < d ? S.rows(p)[(1 + kLaneDim + lane) * W + w] : 0ull;
     }
-    uint32_t at = 0;  // the entry's slot
-    for (;;) {
-      const uint32_t m = __ballot_sync(kAll, wnonzero(x));
-      if (!m) break;
-      if (d >= P.aff_dim) {  // (records come from lanes of fewer directions)
-        status = AS_RERUN;
-        return a.y;
-      }
-      uint64_t dir[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) dir[w] = shfl64(x[w], (uint32_t)__ffs(m) - 1u);
-      if (wbit<W>(x, wlow(dir))) {
-        at |= 1u << d;
-#pragma unroll
-        for (int w = 0; w < W; ++w) x[w] ^= dir[w];
-      }
-      add_dim(dir);
-    }
-    for (uint32_t s = lane; s < size(); s += 32) v[s] = Cx<R>{0, 0};
-    __syncwarp();
-    if (lane < n) v[at] = val;
+    if (lane < size()) v[lane] = ((a.z >> lane) & 1u) ? S.vals(p)[lane] : Cx<R>{0, 0};
     __syncwarp();
     return a.y;
   }
@@ -344,31 +311,9 @@ struct AffShot {
       fail_check(CHK_SITE, s);
       return;
     }
-    const Site *S = C->sites + s;
-    const uint32_t kind = __ldg(&S->kind);
-    uint32_t code, pa, pb = 0;
-    if ((kind & 3u) == SITE_DEPOL2) {
-      code = (uint32_t)(((uint64_t)w2 * 15u) >> 32) + 1u;
-      pa = code >> 2;
-      pb = code & 3u;
-    } else if ((kind & 3u) == SITE_FLIP) {
-      pa = code = (kind >> 2) & 3u;
-    } else {
-      pa = code = (uint32_t)(((uint64_t)w2 * 3u) >> 32) + 1u;
-    }
-    uint64_t beta[W], gamma[W], pe = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      uint64_t b = 0, g = 0;
-      if (pa == 1u || pa == 2u) { b ^= __ldg(&S->bx[0][w]); g ^= __ldg(&S->gx[0][w]); }
-      if (pa == 3u || pa == 2u) { b ^= __ldg(&S->bz[0][w]); g ^= __ldg(&S->gz[0][w]); }
-      if (pb == 1u || pb == 2u) { b ^= __ldg(&S->bx[1][w]); g ^= __ldg(&S->gx[1][w]); }
-      if (pb == 3u || pb == 2u) { b ^= __ldg(&S->bz[1][w]); g ^= __ldg(&S->gz[1][w]); }
-      beta[w] = b;
-      gamma[w] = g;
-      pe ^= ((sd[w] ^ __ldg(&S->dsd[w])) & b) ^ ((ss[w] ^ __ldg(&S->dss[w])) & g);
-    }
-    apply_pauli(beta, gamma, ((__ldg(&S->c0) >> (2u * code)) + 2u * wordpar(pe)) & 3u);
+    uint64_t beta[W], gamma[W];
+    const uint32_t e = site_pauli<W>(C, s, nc.pair(), sd, ss, beta, gamma);
+    apply_pauli(beta, gamma, e);
   }
 
   // FP32: b xi x, xi = i^e (-1)^par
@@ -690,9 +635,9 @@ struct AffShot {
 
   // one event (header hdr, body: dsd, dss, beta, gamma; E for a fused reset correction's words)
   __device__ void step(const uint4 &hdr, const uint64_t *body, const Ev<W> *E) {
-    while (nxt < hdr.y && status == AS_RUN) {
-      apply_error(nxt);
-      if (!next_site(C, P.seed, shot, cur, kblk, nxt, w2)) status = AS_ERR;
+    while (nc.site() < hdr.y && status == AS_RUN) {
+      apply_error(nc.site());
+      if (!nc.advance(C, P.seed, shot)) status = AS_ERR;
     }
     if (status != AS_RUN) return;
     const uint64_t *beta = body + 2 * W, *gamma = body + 3 * W;
@@ -766,18 +711,19 @@ struct AffShot {
     if (r != kNoRecord) {
       ev = load_spill(r);
     } else {
-      if (P.al_cursor && !C->lanes_off) {  // the bucketing pre-pass drew the first error
+      uint32_t nxt = kAll;
+      if (P.al_cursor && !C->lanes_off) {  // the bucketing pre-pass drew the first errors
         const uint4 k = reinterpret_cast<const uint4 *>(P.al_cursor)[local];
-        nxt = k.x;
-        cur = k.y;
-        kblk = k.z;
-        w2 = k.w;
+        nc = NoiseCursor{k.x, k.y, k.z};
+        if (nc.site() != kMaxPackedSites) nxt = nc.site();
+        if (nc.kblk == kAll) status = AS_ERR;
       } else {
-        cur = kblk = w2 = 0;
-        nxt = kAll;
-        if (!next_site(C, P.seed, shot, cur, kblk, nxt, w2)) kblk = kAll;
+        uint32_t cur = 0, pp = 0;
+        nc.kblk = 0;
+        if (!next_site(C, P.seed, shot, cur, nc.kblk, nxt, pp)) status = AS_ERR;
+        nc.first = pack_error(nxt, pp);
+        nc.second = kNotDrawn;
       }
-      if (kblk == kAll) status = AS_ERR;
       ev = first_event(C, P.fid_mode, nxt);
       load_snapshot(ev);
     }
@@ -888,7 +834,8 @@ __global__ void __launch_bounds__(kAffBlock, sizeof(R) == 4 && W == 1 ? 6 : 5) a
     if (P.list && (local & kSpillRef) && P.sp) {
       rec = local & ~kSpillRef;
       if (rec >= P.sp_cap) break;  // never: records are taken below the pool's capacity
-      local = Spill<R, W>(P.sp, P.sp_cap, P.rw_max).ha[rec].x;
+      const Spill<R, W> S(P.sp, P.rw_max, kLaneDim);
+      local = S.ha(S.at(rec)).x;
     }
     const uint64_t g = item_base + local;
     uint32_t lo = 0, hi = n_circ;  // the circuit of item g

@@ -183,7 +183,7 @@ int soft_compile_circuit(const soft_op *ops, size_t n_ops, uint32_t n_qubits, co
          b_cb = std::max<size_t>(1, hp.cb.size()) * sizeof(soft::CaseB),
          b_st = std::max<size_t>(1, hp.sites.size()) * sizeof(soft::Site),
          b_thr0 = hp.thr.size() * sizeof(uint64_t), b_thr1 = b_thr0 + hp.site_ev.size() * sizeof(uint32_t),
-         b_thr = b_thr1 + hp.thr_tab.size() * sizeof(uint32_t);
+         b_thr2 = b_thr1 + hp.thr_tab.size() * sizeof(uint32_t), b_thr = b_thr2 + hp.site_kind.size();
   cudaError_t e;
   if ((e = cudaMalloc(&c->d_ev, b_ev)) != cudaSuccess || (e = cudaMalloc(&c->d_coef, b_cf)) != cudaSuccess ||
       (e = cudaMalloc(&c->d_cb, b_cb)) != cudaSuccess || (e = cudaMalloc(&c->d_sites, b_st)) != cudaSuccess ||
@@ -209,6 +209,7 @@ int soft_compile_circuit(const soft_op *ops, size_t n_ops, uint32_t n_qubits, co
       (e = up(c->d_thr, hp.thr.data(), b_thr0)) != cudaSuccess ||
       (e = up(thr_b + b_thr0, hp.site_ev.data(), hp.site_ev.size() * sizeof(uint32_t))) != cudaSuccess ||
       (e = up(thr_b + b_thr1, hp.thr_tab.data(), hp.thr_tab.size() * sizeof(uint32_t))) != cudaSuccess ||
+      (e = up(thr_b + b_thr2, hp.site_kind.data(), hp.site_kind.size())) != cudaSuccess ||
       (e = cudaStreamSynchronize(us)) != cudaSuccess) {
     cudaStreamDestroy(us);
     soft_circuit_free(c);
@@ -300,6 +301,7 @@ CircDev circ_desc(const soft_circuit *c, int fp32, bool prefix) {
   soft::CircDev d{};
   d.site_ev = reinterpret_cast<const uint32_t *>(c->d_thr + c->hp.thr.size());
   d.thr_tab = d.site_ev + c->hp.site_ev.size();
+  d.site_kind = reinterpret_cast<const uint8_t *>(d.thr_tab + c->hp.thr_tab.size());
   if (prefix && c->d_traj[fp32]) {
     d.traj = c->d_traj[fp32];
     d.traj_stop = c->traj_stop[fp32];
@@ -373,7 +375,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   uint64_t nbc[3] = {0, 0, 0};         // buckets of the circuits of 16-, 32- and 64-entry lanes
   auto lane_class = [&](uint32_t c) { return c == lc16 ? 0 : c == 2 * lc16 ? 1 : c == 4 * lc16 ? 2 : 3; };
   for (uint32_t i = 0; i < n_circ; ++i) {
-    lcap[i] = circs[i]->d_traj[pk] ? soft::lane_first_cap(circs[i]->traj_max_n[pk], circs[i]->traj_max_d[pk], fp32) : 0u;
+    lcap[i] = circs[i]->d_traj[pk] && circs[i]->hp.n_sites < soft::kMaxPackedSites ? soft::lane_first_cap(circs[i]->traj_max_n[pk], circs[i]->traj_max_d[pk], fp32) : 0u;
     if (lcap[i]) nbc[lane_class(lcap[i])] += circs[i]->hp.ev.size() + 1;
   }
   const uint64_t n_buckets = nbc[0] + nbc[1] + nbc[2];
@@ -390,7 +392,8 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   // sparse form's scheduling (no lanes, no prefix)
   bool affine = !(o.flags & (SOFT_RUN_NO_LANES | SOFT_RUN_NO_PREFIX)) && o.group_size == 0 && o.first_cap == 0 &&
                 o.groups_per_block == 0;
-  for (uint32_t i = 0; i < n_circ; ++i) affine = affine && circs[i]->d_traj[pk];
+  for (uint32_t i = 0; i < n_circ; ++i)
+    affine = affine && circs[i]->d_traj[pk] && circs[i]->hp.n_sites < soft::kMaxPackedSites;
   const bool two_pass = lanes || affine || cap1 < cap_max;
   // after lanes, a middle pass (a warp per shot) takes the shots whose maps outgrew a lane, and
   // only those that outgrow it too go on to the pass at the circuit's cap: in affine form, with
@@ -436,12 +439,12 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     arena_bytes += (bytes + 255) & ~(size_t)255;
   };
   need(&r->d_tally, 5 * n_circ * sizeof(unsigned long long));
-  // lanes: cursors (4 words per item, first: 16-byte aligned), (start event, rank) pairs, order,
-  // bucket starts, counters
-  // then the per-block bucket bases of the block-binned pre-pass
+  // lanes: cursors (4 words per item, 16-byte aligned), the cursors in bucket order, (start
+  // event, rank) pairs, bucket starts, counters, then the per-block bucket bases of the
+  // block-binned pre-pass
   const uint32_t al_grid = lanes ? soft::lane_prepass_grid() : 0u;
   if (lanes)
-    need(&r->d_al, (7 * chunk + (nb + 1) + 2 * (size_t)nb + (size_t)al_grid * (nb + 1)) * sizeof(uint32_t));
+    need(&r->d_al, (10 * chunk + (nb + 1) + 2 * (size_t)nb + (size_t)al_grid * (nb + 1)) * sizeof(uint32_t));
   // spill pool: records for the shots a sparse warp evicts (a quarter of the chunk; when it is
   // full, warps keep their shots), then records for shots a lane hands to a warp (an eighth;
   // when full, the warp reruns them from their start). Entries of the rerun list name a record
@@ -460,7 +463,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   const bool wide = wide_ok && ((o.flags & SOFT_RUN_WIDE_LANES) || std::min(chunk, total) >= (1ull << 23));
   const size_t n_lr = 4 + 2 * ((size_t)rounds + 1);
   if (spill) {
-    need(&r->d_sp, soft::lane_spill_bytes(fp32, W, rw_max, sp_evict + sp_hand));
+    need(&r->d_sp, soft::lane_spill_bytes(fp32, W, rw_max, sp_evict + sp_hand, soft::lane_map_dim()));
     need(&r->d_lr, n_lr * sizeof(unsigned long long));
   }
   r->fid_mode = fid_mode;
@@ -605,10 +608,10 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   }
   if (lanes) {  // start events, order, bucket starts, then the two counter arrays (zeroed per chunk)
     p.al_cursor = r->d_al;
-    p.al_ev = r->d_al + 4 * chunk;
-    p.al_order = r->d_al + 6 * chunk;
-    p.al_start = r->d_al + 7 * chunk;
-    p.al_count = r->d_al + 7 * chunk + (nb + 1);
+    p.al_rec = p.al_order = r->d_al + 4 * chunk;
+    p.al_ev = r->d_al + 8 * chunk;
+    p.al_start = r->d_al + 10 * chunk;
+    p.al_count = r->d_al + 10 * chunk + (nb + 1);
     p.al_next = p.al_count + nb;
     p.al_base = p.al_next + nb;
     p.al_nb = nb;
@@ -623,6 +626,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     p.sp = spill ? r->d_sp : nullptr;
     p.sp_cap = spill ? sp_evict + sp_hand : 0u;
     p.sp_evict_cap = spill ? sp_evict : 0u;
+    p.sp_dim = soft::lane_map_dim();
     p.lr = spill ? r->d_lr : nullptr;
     // the middle pass (or, without one, the pass at the circuit's cap) resumes handed-over shots
     soft::ShotParams &h = mid_pass ? m : q;

@@ -355,6 +355,7 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
         }
       }
       c0 |= (e & 3u) << (2 * code);
+      if (!two) c0 |= (e & 3u) << (8 * code);  // also at code << 2, the site's Pauli pair (see Site)
     }
     s.c0 = c0;
     if (p >= P.pmax) {
@@ -365,6 +366,7 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
       s.thin = (uint32_t)std::floor(std::ldexp(p / P.pmax, 32));
     }
     P.sites.push_back(s);
+    P.site_kind.push_back((uint8_t)(kind | (s.always ? 0u : kSiteThinned)));
     return true;
   };
 

@@ -186,6 +186,16 @@ __device__ __forceinline__ double pnorm(Cx<R> v) {
 __device__ __forceinline__ uint32_t wordpar(uint64_t x) {
   return (uint32_t)__popc((uint32_t)x ^ (uint32_t)(x >> 32)) & 1u;
 }
+// Bytes (4, 8 or 16) from global to shared memory without passing through registers; the
+// thread's own copies are complete after copies_done().
+template <int Bytes>
+__device__ __forceinline__ void copy_async(void *shared, const void *global) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(shared)),
+               "l"(global), "n"(Bytes)
+               : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <int W>
 struct Key {
   uint64_t w[W];

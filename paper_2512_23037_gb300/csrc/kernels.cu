@@ -72,7 +72,8 @@ struct Shot {
   uint64_t shot;
   uint32_t nnz;
   uint64_t sd[W], ss[W];
-  uint32_t nxt, cur, kblk, w2;
+  uint32_t nxt, cur, kblk, pp;     // the next error: its site and Pauli pair
+  uint32_t second = kNotDrawn;     // a handed-over shot: the error after it, if drawn (packed)
   int status, chain, logical, lastm;
   bool force = false;  // fidelity mode: this measurement projects onto +1
   bool undecided = false;  // set when an outcome depended on the uniform (0 < p_+ < 1)
@@ -193,7 +194,14 @@ struct Shot {
 
   // ---- noise: next accepted error site (geometric gaps, then thinning)
   __device__ void draw_next() {
-    if (!next_site(C, P.seed, shot, cur, kblk, nxt, w2)) status = ST_ERR;
+    if (second != kNotDrawn) {
+      nxt = second == 0x0FFFFFFFu ? 0xFFFFFFFFu : second & 0x0FFFFFFFu;
+      pp = second >> 28;
+      cur = nxt == 0xFFFFFFFFu ? C->n_sites : nxt + 1u;
+      second = kNotDrawn;
+      return;
+    }
+    if (!next_site(C, P.seed, shot, cur, kblk, nxt, pp)) status = ST_ERR;
   }
 
   // v'_{a^beta} = i^{e + 2 gamma.a} v_a
@@ -219,36 +227,8 @@ struct Shot {
       fail_check(CHK_SITE, s);
       return;
     }
-    const Site *S = C->sites + s;
-    const uint32_t kind = __ldg(&S->kind);
-    uint32_t code, pa, pb;
-    if ((kind & 3u) == SITE_DEPOL2) {
-      code = (uint32_t)(((uint64_t)w2 * 15u) >> 32) + 1u;
-      pa = code >> 2;
-      pb = code & 3u;
-    } else if ((kind & 3u) == SITE_FLIP) {
-      code = (kind >> 2) & 3u;
-      pa = code;
-      pb = 0;
-    } else {
-      code = (uint32_t)(((uint64_t)w2 * 3u) >> 32) + 1u;
-      pa = code;
-      pb = 0;
-    }
     uint64_t beta[W], gamma[W];
-    uint32_t pe = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      uint64_t b = 0, g = 0;
-      if (pa == 1u || pa == 2u) { b ^= __ldg(&S->bx[0][w]); g ^= __ldg(&S->gx[0][w]); }
-      if (pa == 3u || pa == 2u) { b ^= __ldg(&S->bz[0][w]); g ^= __ldg(&S->gz[0][w]); }
-      if (pb == 1u || pb == 2u) { b ^= __ldg(&S->bx[1][w]); g ^= __ldg(&S->gx[1][w]); }
-      if (pb == 3u || pb == 2u) { b ^= __ldg(&S->bz[1][w]); g ^= __ldg(&S->gz[1][w]); }
-      beta[w] = b;
-      gamma[w] = g;
-      pe += __popcll((sd[w] ^ __ldg(&S->dsd[w])) & b) + __popcll((ss[w] ^ __ldg(&S->dss[w])) & g);
-    }
-    uint32_t e = ((__ldg(&S->c0) >> (2u * code)) + 2u * pe) & 3u;
+    const uint32_t e = site_pauli<W>(C, s, pp, sd, ss, beta, gamma);
     apply_pauli(beta, gamma, e);
   }
 
@@ -871,6 +851,7 @@ struct Shot {
     }
     cur = 0;
     kblk = 0;
+    second = kNotDrawn;
     fid = 1.0;
     force = false;
   }
@@ -878,25 +859,27 @@ struct Shot {
   // A shot handed over by a lane: its whole state at the top of its resume event,
   // which is returned.
   __device__ uint32_t load_spill(uint32_t r) {
-    const Spill<R, W> S(P.sp, P.sp_cap, P.rw_max);
-    const size_t c = S.cap;
-    const uint4 a = S.ha[r], b = S.hb[r];
-    nnz = a.z;
-    chain = (int)(a.w & 1u);
-    logical = (int)((a.w >> 1) & 1u);
-    lastm = (int)(int8_t)((a.w >> 8) & 255u);
-    nxt = b.x;
-    cur = b.y;
+    const Spill<R, W> S(P.sp, P.rw_max, kLaneDim);
+    unsigned char *p = S.at(r);
+    const uint4 a = S.ha(p), b = S.hb(p);
+    nnz = __popc(a.z);
+    const uint32_t rd = a.w & 255u;
+    chain = (int)((a.w >> 8) & 1u);
+    logical = (int)((a.w >> 9) & 1u);
+    lastm = (int)(int8_t)((a.w >> 16) & 255u);
+    nxt = (b.x & 0x0FFFFFFFu) == 0x0FFFFFFFu ? 0xFFFFFFFFu : b.x & 0x0FFFFFFFu;
+    pp = b.x >> 28;
+    cur = nxt == 0xFFFFFFFFu ? C->n_sites : nxt + 1u;
+    second = b.y;
     kblk = b.z;
-    w2 = b.w;
-    fid = S.fid[r];
+    fid = S.fid(p);
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      sd[w] = S.sd[w * c + r];
-      ss[w] = S.ss[w * c + r];
+      sd[w] = S.sd(p)[w];
+      ss[w] = S.ss(p)[w];
     }
-    for (uint32_t w = lane; w < C->rw; w += G) rec[w] = S.rec[w * c + r];
-    if (nnz > kLaneCap || a.y >= C->n_events) {  // a record never holds more, nor resumes past the end
+    for (uint32_t w = lane; w < C->rw; w += G) rec[w] = S.rec(p)[w];
+    if (nnz > kLaneCap || rd > kLaneDim || a.y >= C->n_events) {  // a record never holds more, nor resumes past the end
       fail_check(CHK_NNZ, nnz);
       return C->n_events;
     }
@@ -905,26 +888,28 @@ struct Shot {
       return a.y;
     }
     Cx<R> f{(R)1, (R)0};  // FP64 records hold a scaled map: its norm and the circuit's phase here
-    if constexpr (sizeof(R) == 8) f = readout(top_phase<W>(C, a.y), S.norm[r]);
-    auto value = [&](uint32_t i) {
-      const Cx<R> x = S.vals[(size_t)i * c + r];
-      return sizeof(R) == 8 ? cmul(f, x) : x;
+    if constexpr (sizeof(R) == 8) f = readout(top_phase<W>(C, a.y), S.norm(p));
+    // the sparse form: entry i is the i-th live slot's
+    auto entry = [&](uint32_t i, Key<W> &k, Cx<R> &v) {
+      const uint32_t s = __fns(a.z, 0, (int)i + 1);
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        k.w[w] = S.rows(p)[w];
+        for (uint32_t j = 0; j < rd; ++j)
+          if ((s >> j) & 1u) k.w[w] ^= S.rows(p)[(1 + j) * W + w];
+      }
+      const Cx<R> x = S.vals(p)[s];
+      v = sizeof(R) == 8 ? cmul(f, x) : x;
     };
     if (kRegCapable && nnz <= (uint32_t)G) {
       reg = true;
-      if (lane < nnz) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) rk.w[w] = S.keys[((size_t)lane * W + w) * c + r];
-        rv = value(lane);
-      }
+      if (lane < nnz) entry(lane, rk, rv);
       t.sync();
     } else {
       for (uint32_t i = lane; i < nnz; i += G) {
         Key<W> k;
-#pragma unroll
-        for (int w = 0; w < W; ++w) k.w[w] = S.keys[((size_t)i * W + w) * c + r];
+        entry(i, k, vals[i]);
         set_key(i, k);
-        vals[i] = value(i);
       }
       t.sync();
       reg = false;
@@ -1146,7 +1131,8 @@ __global__ void __launch_bounds__(kBlock, sizeof(R) == 4 ? SOFT_MIN_BLOCKS_F32 :
     if (P.list && (local & kSpillRef) && P.sp) {
       rec = (uint32_t)local & ~kSpillRef;
       if (rec >= P.sp_cap) break;  // never: records are taken below the pool's capacity
-      local = Spill<R, W>(P.sp, P.sp_cap, P.rw_max).ha[rec].x;
+      const Spill<R, W> S(P.sp, P.rw_max, kLaneDim);
+      local = S.ha(S.at(rec)).x;
     }
     const uint64_t g = item_base + local;
     // circuit of item g: the last one whose item range starts at or before g

@@ -35,6 +35,7 @@ struct CircDev {
   uint32_t traj_stop, traj_stride;
   uint32_t traj_fid_stop, pad_traj;  // first fidelity measurement's event (fidelity mode stops there)
   const uint32_t *site_ev;  // per site: the event that applies its error
+  const uint8_t *site_kind; // per site: its kind and kSiteThinned (program.h)
   const uint32_t *thr_tab;  // the gap search's index, 2^kThrTabBits + 1 entries (null: plain search)
 };
 
@@ -78,7 +79,8 @@ struct ShotParams {
   uint32_t *al_ev;  // per item (start event, rank in its bucket), 8-byte aligned
   uint32_t *al_order, *al_start;
   unsigned int *al_count, *al_next;
-  uint32_t *al_cursor;  // per item the noise cursor after its first draw (nxt, cur, kblk, w2), 16-byte aligned
+  uint32_t *al_cursor;  // per item the noise cursor after two draws (NoiseCursor) and the item, 16-byte aligned
+  uint32_t *al_rec;     // those of the items in bucket order (a resume round: al_order)
   uint32_t *al_base;    // per pre-pass block: the block's first rank in each bucket, then its first
                         // slot in the warp pass's list (al_nb + 1 words per block)
   uint32_t al_grid;     // pre-pass blocks (each bins a contiguous range of items)
@@ -94,6 +96,7 @@ struct ShotParams {
   unsigned char *sp;          // spill pool, sp_cap records (layout: lane_spill_bytes): evictions in
   uint32_t sp_cap;            // [0, sp_evict_cap), shots handed from a lane to a warp after that
   uint32_t sp_evict_cap;
+  uint32_t sp_dim;            // directions of the records' maps (the lanes that write them)
   uint32_t aff_dim;           // affine_kernel: directions of a warp's map (2^aff_dim values)
   unsigned long long *lr;     // [0] eviction records taken, [1] handover records taken;
                               // round r >= 1: [2 + 2r] its first record, [3 + 2r] its count
@@ -134,7 +137,8 @@ struct LaunchCfg {
 cudaError_t launch_lane_prepass(const ShotParams &p, cudaStream_t st);
 // round r >= 1: the range of records evicted before it, then their buckets
 cudaError_t launch_lane_resume_prepass(const ShotParams &p, int fp32, uint32_t W, cudaStream_t st);
-size_t lane_spill_bytes(int fp32, uint32_t W, uint32_t rw, uint32_t cap);
+// bytes of `cap` spill records of maps of `dim` directions
+size_t lane_spill_bytes(int fp32, uint32_t W, uint32_t rw, uint32_t cap, uint32_t dim);
 uint32_t lane_rounds();
 uint32_t lane_max_buckets();  // lane-per-shot runs hold at most this many buckets (events + 1 per circuit)
 uint32_t lane_prepass_grid();  // blocks of the bucketing pre-pass (al_base holds this many rows)

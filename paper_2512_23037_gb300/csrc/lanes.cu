@@ -24,6 +24,14 @@
 // the evicted shots by the event they resume at, and packs them into warps again.
 // The last round evicts nothing. Which lane runs a shot does not change its
 // arithmetic, so the results are those of a single round.
+//
+// A warp's time went to waits rather than to the maps (clock counters, w42 FP32: claims 22 %,
+// errors 17 %, finished and evicted shots 13 %, the search for the next bucket 7 %). So the
+// pre-pass draws each shot's first two errors and leaves its cursor in bucket order; a claim
+// issues the snapshot's copies to shared memory before its atomic answers; bucket bounds are
+// read one event ahead; tallies are ballots; and 32 buckets are searched at a time. w42 FP32
+// at 2^24 shots 19.6 -> 16.8 ms, FP64 at 2^22 11.2 -> 9.7 ms, w97 FP32 at 2 M 24.9 -> 21.7 ms,
+// a batch of 64 circuits (7.7 M shots) 31.7 -> 16.6 ms.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -165,7 +173,7 @@ struct LaneShot {
   uint32_t d;
   Mask live;
   uint64_t sd[W], ss[W];
-  uint32_t nxt, cur, kblk, w2;
+  NoiseCursor nc;
   int status, chain, logical, lastm;
   double fid;
   bool force;
@@ -346,36 +354,6 @@ struct LaneShot {
       }
     return k;
   }
-  // The map from explicit entries (a spill record): alpha0 = the first key, each further
-  // key's residual a new direction. False if it needs more than kDim directions.
-  template <typename KeyAt, typename ValAt>
-  __device__ bool load_entries(uint32_t n, KeyAt key_at, ValAt val_at) {
-    d = 0;
-    live = 0;
-    if (n == 0) {
-#pragma unroll
-      for (int w = 0; w < W; ++w) set_row(0, w, 0ull);
-      return true;
-    }
-    const Key<W> k0 = key_at(0);
-    put_row(0, k0.w);
-#pragma unroll 1
-    for (uint32_t i = 0; i < n; ++i) {
-      const Key<W> k = key_at(i);
-      const Key<W> x = kxor(k, k0.w);
-      uint64_t r[W];
-      uint32_t c = coords(x.w, r);
-      if (wnonzero<W>(r)) {
-        if (d == kDim) return false;
-        add_dim(r);
-        c |= 1u << (d - 1u);
-      }
-      set_val(c, val_at(i));
-      live |= (Mask)1 << c;
-    }
-    return true;
-  }
-
   __device__ void fail_capacity() { status = P.small_pass ? LS_RERUN : LS_OVF; }
   __device__ void fail_check(uint32_t code, uint64_t value) {
     status = LS_ERR;
@@ -394,40 +372,38 @@ struct LaneShot {
     return (R)rsqrt(x);
   }
 
-  // ---- start: shot s at event e of the noiseless run (its map in affine form, computed
-  // once per snapshot when the circuit was compiled); the pre-pass drew the shot's first
-  // error: its noise cursor comes with the item
-  __device__ void begin(uint64_t s, uint32_t e, uint4 cursor) {
-    shot = s;
+  __device__ __forceinline__ void fetch_row(uint32_t r, const uint64_t *src) {
+#pragma unroll
+    for (int w = 0; w < W; ++w) copy_async<8>(&rows[((size_t)r * W + w) * 32 + lane], src + w);
+  }
+  __device__ __forceinline__ void fetch_val(uint32_t s, const Cx<R> *src) {
+    copy_async<(int)sizeof(Cx<R>)>(&vals[(size_t)s * 32 + lane], src);
+  }
+  // ---- start at event e of the noiseless run (its map in affine form, computed once per
+  // snapshot when the circuit was compiled): everything but the shot's own cursor. The map
+  // goes to the lane's columns in asynchronous copies (complete after copies_done()), issued
+  // before the claim's atomic has answered
+  __device__ void begin(uint32_t e) {
     status = LS_RUN;
     force = false;
     nrm = 1.0;
-    nxt = cursor.x;
-    cur = cursor.y;
-    kblk = cursor.z;
-    w2 = cursor.w;
-    if (kblk == 0xFFFFFFFFu) {
-      status = LS_ERR;
-      return;
-    }
     const unsigned char *in = C->traj + (size_t)e * C->traj_stride;
     const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
     const uint64_t *r_in = reinterpret_cast<const uint64_t *>(in + sizeof(SnapHdr));
     const SnapAffine<R, W> *a = reinterpret_cast<const SnapAffine<R, W> *>(in + snap_affine_off<R, W>(C->rw));
-    chain = (int)__ldg(&h->chain);
-    logical = (int)__ldg(&h->logical);
-    lastm = (int)__ldg(&h->lastm);
+    const uint2 dl = __ldg(reinterpret_cast<const uint2 *>(&a->d));  // d and the low word of live
+    const uint4 h0 = __ldg(reinterpret_cast<const uint4 *>(h));
+    chain = (int)h0.y;
+    logical = (int)h0.z;
+    lastm = (int)h0.w;
     fid = __ldg(&h->fid);
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       sd[w] = __ldg(&h->sd[w]);
       ss[w] = __ldg(&h->ss[w]);
     }
-#pragma unroll 1
-    for (uint32_t w = 0; w < C->rw; ++w) rec[(size_t)w * 32 + lane] = __ldg(&r_in[w]);
-    const uint2 dl = __ldg(reinterpret_cast<const uint2 *>(&a->d));  // d and the low word of live
-    d = 0;
     live = 0;
+    d = 0;
     if (dl.x > kDim) {
       fail_capacity();
       return;
@@ -435,88 +411,90 @@ struct LaneShot {
     d = dl.x;
     live = (Mask)dl.y;  // (no slot at or above 2^kDim is live)
     if (sizeof(Mask) == 8) live |= (Mask)__ldg(&a->live_hi) << 16 << 16;
-#pragma unroll
-    for (int w = 0; w < W; ++w) set_row(0, w, __ldg(&a->rows[0][w]));
 #pragma unroll 1
-    for (uint32_t k = 0; k < d; ++k)
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        set_row(kRowB + k, w, __ldg(&a->rows[1 + k][w]));
-        set_row(kRowD + k, w, __ldg(&a->rows[1 + kSnapDim + k][w]));
-      }
+    for (uint32_t s = 0; s < (1u << d); ++s) fetch_val(s, &a->v[s]);
+    fetch_row(0, a->rows[0]);
 #pragma unroll 1
-    for (Mask m = live; m; m &= m - (Mask)1) {
-      const uint32_t j = mffs(m) - 1;
-      set_val(j, a->v[j]);
+    for (uint32_t k = 0; k < d; ++k) {
+      fetch_row(kRowB + k, a->rows[1 + k]);
+      fetch_row(kRowD + k, a->rows[1 + kSnapDim + k]);
     }
+#pragma unroll 1
+    for (uint32_t w = 0; w < C->rw; ++w) copy_async<8>(&rec[(size_t)w * 32 + lane], &r_in[w]);
+  }
+  __device__ __forceinline__ void start(uint64_t s, const uint4 &cursor) {
+    shot = s;
+    nc = NoiseCursor{cursor.x, cursor.y, cursor.z};
+    if (cursor.z == 0xFFFFFFFFu) status = LS_ERR;
   }
 
-  // ---- eviction: the shot's whole state into record r, to resume at event ev (entries
-  // in slot order, at most kLaneCap of them: a first-round lane holds no more)
+  // ---- eviction: the shot's whole state into record r, to resume at event ev
   __device__ void evict(const Spill<R, W> &S, uint32_t r, uint32_t item, uint32_t ev) const {
-    const size_t c = S.cap;
-    S.ha[r] = make_uint4(item, ev, nnz(), (uint32_t)(chain & 1) | ((uint32_t)(logical & 1) << 1) |
-                                              (((uint32_t)lastm & 255u) << 8));
-    S.hb[r] = make_uint4(nxt, cur, kblk, w2);
-    S.fid[r] = fid;
-    if constexpr (kScaled) S.norm[r] = nrm;
+    unsigned char *p = S.at(r);
+    S.ha(p) = make_uint4(item, ev, (uint32_t)live, S.meta(d, chain, logical, lastm));
+    S.hb(p) = make_uint4(nc.first, nc.second, nc.kblk, sizeof(Mask) == 8 ? (uint32_t)((unsigned long long)live >> 32) : 0u);
+    S.fid(p) = fid;
+    if constexpr (kScaled) S.norm(p) = nrm;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      S.sd[w * c + r] = sd[w];
-      S.ss[w * c + r] = ss[w];
+      S.sd(p)[w] = sd[w];
+      S.ss(p)[w] = ss[w];
     }
 #pragma unroll 1
-    for (uint32_t w = 0; w < C->rw; ++w) S.rec[w * c + r] = rec[(size_t)w * 32 + lane];
-    uint32_t i = 0;
+    for (uint32_t w = 0; w < C->rw; ++w) S.rec(p)[w] = rec[(size_t)w * 32 + lane];
+    uint64_t *q = S.rows(p);
 #pragma unroll 1
-    for (Mask m = live; m && i < kLaneCap; m &= m - (Mask)1, ++i) {
-      const uint32_t s = mffs(m) - 1;
-      const Key<W> k = key_of(s);
+    for (uint32_t k = 0; k <= d; ++k)
 #pragma unroll
-      for (int w = 0; w < W; ++w) S.keys[((size_t)i * W + w) * c + r] = k.w[w];
-      S.vals[(size_t)i * c + r] = val(s);
-    }
+      for (int w = 0; w < W; ++w) {
+        q[k * W + w] = row(k, w);
+        if (k < d) q[(1 + S.dim + k) * W + w] = row(kRowD + k, w);
+      }
+    Cx<R> *qv = S.vals(p);
+#pragma unroll 1
+    for (Mask m = live; m; m &= m - (Mask)1) qv[mffs(m) - 1] = val(mffs(m) - 1);
   }
-  // ---- resumption from record r; returns the shot's item (chunk-local index)
+  // ---- resumption from record r (asynchronous copies, as begin); returns the shot's item
+  // (chunk-local index)
   __device__ uint32_t resume(const Spill<R, W> &S, uint32_t r, uint64_t first) {
-    const size_t c = S.cap;
-    const uint4 a = S.ha[r], b = S.hb[r];
+    unsigned char *p = S.at(r);
+    const uint4 a = S.ha(p), b = S.hb(p);
     shot = first + a.x;
     status = LS_RUN;
     force = false;
-    const uint32_t n = a.z;
-    chain = (int)(a.w & 1u);
-    logical = (int)((a.w >> 1) & 1u);
-    lastm = (int)(int8_t)((a.w >> 8) & 255u);
-    nxt = b.x;
-    cur = b.y;
-    kblk = b.z;
-    w2 = b.w;
-    fid = S.fid[r];
-    if constexpr (kScaled) nrm = S.norm[r];
+    chain = (int)((a.w >> 8) & 1u);
+    logical = (int)((a.w >> 9) & 1u);
+    lastm = (int)(int8_t)((a.w >> 16) & 255u);
+    nc = NoiseCursor{b.x, b.y, b.z};
+    fid = S.fid(p);
+    if constexpr (kScaled) nrm = S.norm(p);
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      sd[w] = S.sd[w * c + r];
-      ss[w] = S.ss[w * c + r];
+      sd[w] = S.sd(p)[w];
+      ss[w] = S.ss(p)[w];
     }
 #pragma unroll 1
-    for (uint32_t w = 0; w < C->rw; ++w) rec[(size_t)w * 32 + lane] = S.rec[w * c + r];
+    for (uint32_t w = 0; w < C->rw; ++w) copy_async<8>(&rec[(size_t)w * 32 + lane], S.rec(p) + w);
     d = 0;
     live = 0;
-    if (n > kLaneCap) {  // a record never holds more; checked so that a bad record cannot index past the map
-      fail_check(CHK_NNZ, n);
+    const uint32_t rd = a.w & 255u;
+    if (rd > S.dim || rd > kDim) {  // a record never holds more; checked so that a bad record cannot index past the map
+      fail_check(CHK_NNZ, rd);
       return a.x;
     }
-    const bool ok = load_entries(
-        n,
-        [&](uint32_t i) {
-          Key<W> k;
-#pragma unroll
-          for (int w = 0; w < W; ++w) k.w[w] = S.keys[((size_t)i * W + w) * c + r];
-          return k;
-        },
-        [&](uint32_t i) { return S.vals[(size_t)i * c + r]; });
-    if (!ok) fail_capacity();  // (records come from lanes of at most kDim directions)
+    d = rd;
+    live = (Mask)a.z;
+    if (sizeof(Mask) == 8) live |= (Mask)b.w << 16 << 16;
+    live &= cube();
+    const uint64_t *q = S.rows(p);
+    fetch_row(0, q);
+#pragma unroll 1
+    for (uint32_t k = 0; k < d; ++k) {
+      fetch_row(kRowB + k, q + (1 + k) * W);
+      fetch_row(kRowD + k, q + (1 + S.dim + k) * W);
+    }
+#pragma unroll 1
+    for (Mask m = live; m; m &= m - (Mask)1) fetch_val(mffs(m) - 1, S.vals(p) + (mffs(m) - 1));
     return a.x;
   }
   // ---- the shot's final state (signs, keys, values) for state capture at offset off; ph: the
@@ -561,35 +539,9 @@ struct LaneShot {
       fail_check(CHK_SITE, s);
       return;
     }
-    const Site *S = C->sites + s;
-    const uint32_t kind = __ldg(&S->kind);
-    uint32_t code, pa, pb;
-    if ((kind & 3u) == SITE_DEPOL2) {
-      code = (uint32_t)(((uint64_t)w2 * 15u) >> 32) + 1u;
-      pa = code >> 2;
-      pb = code & 3u;
-    } else if ((kind & 3u) == SITE_FLIP) {
-      code = (kind >> 2) & 3u;
-      pa = code;
-      pb = 0;
-    } else {
-      code = (uint32_t)(((uint64_t)w2 * 3u) >> 32) + 1u;
-      pa = code;
-      pb = 0;
-    }
-    uint64_t beta[W], gamma[W], pe = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      uint64_t b = 0, g = 0;
-      if (pa == 1u || pa == 2u) { b ^= __ldg(&S->bx[0][w]); g ^= __ldg(&S->gx[0][w]); }
-      if (pa == 3u || pa == 2u) { b ^= __ldg(&S->bz[0][w]); g ^= __ldg(&S->gz[0][w]); }
-      if (pb == 1u || pb == 2u) { b ^= __ldg(&S->bx[1][w]); g ^= __ldg(&S->gx[1][w]); }
-      if (pb == 3u || pb == 2u) { b ^= __ldg(&S->bz[1][w]); g ^= __ldg(&S->gz[1][w]); }
-      beta[w] = b;
-      gamma[w] = g;
-      pe ^= ((sd[w] ^ __ldg(&S->dsd[w])) & b) ^ ((ss[w] ^ __ldg(&S->dss[w])) & g);
-    }
-    apply_pauli(beta, gamma, ((__ldg(&S->c0) >> (2u * code)) + 2u * wordpar(pe)) & 3u);
+    uint64_t beta[W], gamma[W];
+    const uint32_t e = site_pauli<W>(C, s, nc.pair(), sd, ss, beta, gamma);
+    apply_pauli(beta, gamma, e);
   }
 
   // (rare: many rotations, or very unlikely outcomes, since the last sampled outcome)
@@ -952,9 +904,9 @@ struct LaneShot {
 
   // one event for this lane's shot
   __device__ void step(uint32_t ev, const uint4 &hdr, const uint64_t *body, const Ev<W> *E) {
-    while (nxt < hdr.y && status == LS_RUN) {
-      apply_error(nxt);
-      if (!next_site<true>(C, P.seed, shot, cur, kblk, nxt, w2)) status = LS_ERR;
+    while (nc.site() < hdr.y && status == LS_RUN) {
+      apply_error(nc.site());
+      if (!nc.template advance<true>(C, P.seed, shot)) status = LS_ERR;
     }
     if (status != LS_RUN) return;
     const uint64_t *dsd = body, *dss = body + W, *beta = body + 2 * W, *gamma = body + 3 * W;
@@ -1187,8 +1139,8 @@ __global__ void __launch_bounds__(256) lane_bin_kernel(const __grid_constant__ S
     uint32_t e;
     const CircDev *C;
     if (Resume) {
-      const Spill<R, W> S(P.sp, P.sp_cap, P.rw_max);
-      const uint4 a = S.ha[P.lr[2 + 2 * P.lane_round] + i];
+      const Spill<R, W> S(P.sp, P.rw_max, P.sp_dim);
+      const uint4 a = S.ha(S.at((uint32_t)(P.lr[2 + 2 * P.lane_round] + i)));
       C = &P.circ[circ_of_item(P, base + a.x)];
       e = a.y < C->n_events ? a.y : C->n_events;  // a record always resumes at an event of its circuit
     } else {
@@ -1197,11 +1149,16 @@ __global__ void __launch_bounds__(256) lane_bin_kernel(const __grid_constant__ S
         reinterpret_cast<uint2 *>(P.al_ev)[i] = make_uint2(kNoRecord, atomicAdd(&hist[nb], 1u));
         continue;
       }
-      uint32_t cur = 0, kblk = 0, nxt = 0, w2 = 0;
-      if (!next_site(C, P.seed, C->first_shot + (base + i - C->item_begin), cur, kblk, nxt, w2))
-        kblk = 0xFFFFFFFFu;  // a failure
+      // the shot's first error and the one after it: nearly every shot applies the first as it
+      // starts, and here all lanes of a warp draw
+      uint32_t cur = 0, kblk = 0, nxt = 0, pp = 0, n2 = 0, p2 = 0;
+      const uint64_t shot = C->first_shot + (base + i - C->item_begin);
+      bool ok = next_site(C, P.seed, shot, cur, kblk, nxt, pp);
+      if (ok && nxt != 0xFFFFFFFFu) ok = next_site(C, P.seed, shot, cur, kblk, n2, p2);
+      else n2 = 0xFFFFFFFFu;
       e = first_event(C, P.fid_mode, nxt);
-      reinterpret_cast<uint4 *>(P.al_cursor)[i] = make_uint4(nxt, cur, kblk, w2);
+      reinterpret_cast<uint4 *>(P.al_cursor)[i] =
+          make_uint4(pack_error(nxt, pp), pack_error(n2, p2), ok ? kblk : 0xFFFFFFFFu, (uint32_t)i);
     }
     e += C->bucket0;
     reinterpret_cast<uint2 *>(P.al_ev)[i] = make_uint2(e, atomicAdd(&hist[e], 1u));
@@ -1229,7 +1186,9 @@ __global__ void __launch_bounds__(256) lane_bin_scatter_kernel(const __grid_cons
       if (slot < P.rerun_cap) P.rerun[slot] = (uint32_t)i;
       continue;
     }
-    P.al_order[P.al_start[er.x] + P.al_base[(size_t)blockIdx.x * (nb + 1) + er.x] + er.y] = (uint32_t)i;
+    const uint32_t at = P.al_start[er.x] + P.al_base[(size_t)blockIdx.x * (nb + 1) + er.x] + er.y;
+    if (Resume) P.al_order[at] = (uint32_t)i;
+    else reinterpret_cast<uint4 *>(P.al_rec)[at] = reinterpret_cast<const uint4 *>(P.al_cursor)[i];
   }
 }
 
@@ -1250,18 +1209,13 @@ constexpr int kLaneMinBlocks() {
 template <typename R, int W, bool Multi, uint32_t Cap>
 __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) lane_kernel(const __grid_constant__ ShotParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
-  // per warp: tallies of its current circuit, added to the circuit's when the warp moves
-  // to another circuit and at the end
-  __shared__ unsigned long long wt[lane_block<Cap>() / 32][5];
   const uint32_t warp = threadIdx.x / 32, lane = threadIdx.x & 31u;
-  if (lane < 5) wt[warp][lane] = 0ull;
-  __syncwarp();
   LaneShot<R, W, Cap> s(P, smem + (size_t)warp * lane_warp_bytes<R, W, Cap>(P.rw_max));
   const unsigned long long base = P.item_base_dev ? *P.item_base_dev : P.item_base;
   const unsigned long long n_items =
       P.lane_round ? P.lr[3 + 2 * P.lane_round] : (P.n_items_dev ? *P.n_items_dev : P.n_items);
   const unsigned long long rec0 = P.lane_round ? P.lr[2 + 2 * P.lane_round] : 0ull;
-  const Spill<R, W> S(P.sp, P.sp_cap, P.rw_max);
+  const Spill<R, W> S(P.sp, P.rw_max, P.sp_dim);
   // a batch's launch serves the buckets [P.al_lo, P.al_hi) of its lane map size's circuits
   // (read from the launch parameters where used, so that no register holds them through the
   // loop); a single circuit's, all of them
@@ -1275,20 +1229,22 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
   uint32_t n_ev = C->n_events, e = Multi ? g - C->bucket0 : g;
   const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C->ev);
   s.C = C;
-  auto flush = [&]() {  // the warp's tallies into its current circuit's
-    __syncwarp();
-    if (lane < 5 && wt[warp][lane]) {
-      atomicAdd(&C->tally[lane], wt[warp][lane]);
-      wt[warp][lane] = 0ull;
-    }
-    __syncwarp();
+  // the warp's tallies of its current circuit, lane k counter k (shots, discarded, overflow,
+  // kept, logical), counted by ballots; added to the circuit's when the warp moves to another
+  // circuit and at the end
+  uint32_t cnt = 0;
+  auto flush = [&]() {
+    if (lane < 5 && cnt) atomicAdd(&C->tally[lane], (unsigned long long)cnt);
+    cnt = 0;
   };
   bool active = false;
   uint32_t item = 0;
+  // the current bucket: its first record, the next bucket's, and its claims as last read (they
+  // only grow, so a bucket that looks empty is)
+  uint32_t b0 = __ldg(&P.al_start[g]), b1 = __ldg(&P.al_start[g + 1]), taken = *(volatile unsigned int *)&P.al_next[g];
   const unsigned long long limit = (n_items + 2ull) * ((Multi ? P.al_hi - P.al_lo : P.al_nb) + 2ull) + 64ull;
   for (unsigned long long guard = 0; guard < limit; ++guard) {
     g = Multi ? C->bucket0 + e : e;
-    // idle lanes claim shots that start at event e of circuit ci (one atomic per warp)
     // the event's header and body, loaded before the claims so that their latency overlaps
     // the claims' (w42 FP32: 710.8 -> 715.0 M shots/s)
     const Ev<W> *E = evs + e;
@@ -1306,63 +1262,63 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
         body[2 * k + 1] = v.y;
       }
     }
+    // idle lanes claim shots that start at event e of circuit ci (one atomic per warp). The
+    // snapshot's copies are issued before the atomic answers: a lane that gets no shot has
+    // only filled columns that nobody reads.
     const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
-    if (idle) {
-      const uint32_t b0 = __ldg(&P.al_start[g]), sz = __ldg(&P.al_start[g + 1]) - b0;
+    if (idle && taken < b1 - b0) {
       uint32_t got0 = 0;
       const uint32_t leader = __ffs(idle) - 1;
-      if (lane == leader) got0 = *(volatile unsigned int *)&P.al_next[g] < sz ? atomicAdd(&P.al_next[g], __popc(idle)) : sz;
+      if (lane == leader) got0 = atomicAdd(&P.al_next[g], __popc(idle));
+      if (!active && !P.lane_round) s.begin(e);
       got0 = __shfl_sync(0xFFFFFFFFu, got0, leader);
       if (!active) {
         const uint32_t k = got0 + __popc(idle & ((1u << lane) - 1u));
-        if (k < sz) {
-          item = __ldg(&P.al_order[b0 + k]);
-          if (item < n_items) {
-            active = true;
-            const uint64_t first = C->first_shot + base - (Multi ? C->item_begin : 0ull);  // shot of item i: first + i
-            if (P.lane_round) item = s.resume(S, (uint32_t)(rec0 + item), first);
-            else s.begin(first + item, e, reinterpret_cast<const uint4 *>(P.al_cursor)[item]);
+        if (k < b1 - b0) {
+          const uint64_t first = C->first_shot + base - (Multi ? C->item_begin : 0ull);  // shot of item i: first + i
+          if (P.lane_round) {
+            item = __ldg(&P.al_order[b0 + k]);
+            if (item < n_items) {
+              active = true;
+              item = s.resume(S, (uint32_t)(rec0 + item), first);
+            }
+          } else {
+            const uint4 rc = __ldg(reinterpret_cast<const uint4 *>(P.al_rec) + (b0 + k));
+            item = rc.w;
+            if (item < n_items) {
+              active = true;
+              s.start(first + item, rc);
+            }
           }
         }
       }
+      copies_done();
     }
     if (e < n_ev && __any_sync(0xFFFFFFFFu, active && s.status == LS_RUN)) {
       if (active && s.status == LS_RUN) s.step(e, hdr, body, E);
     }
+    // the next bucket's bounds and claims, used when the warp walks on (their latency overlaps
+    // the end of this iteration)
+    const uint32_t nb_all = P.al_nb;
+    const uint32_t b2 = __ldg(&P.al_start[g + 2u < nb_all ? g + 2u : nb_all]);
+    const uint32_t taken1 = *(volatile unsigned int *)&P.al_next[g + 1u < nb_all ? g + 1u : g];
     // a spill record to write (a hand-over or an eviction), written once below
     uint32_t ev_r = 0xFFFFFFFFu, ev_e = 0;
     // finish: ended, or past the last event
-    if (active && (s.status != LS_RUN || e + 1u >= n_ev)) {
-      if (s.status == LS_RUN) s.status = LS_KEPT;
-      const uint64_t off = base + item - (Multi ? C->item_begin : 0ull);  // the shot's offset within its circuit
-      uint32_t entry = item;  // a rerun starts the shot again from its start
-      bool listed = true;
-      if (s.status == LS_HAND) {  // or it resumes from its state at the top of event e
-        const unsigned long long h = atomicAdd(&P.lr[1], 1ull);
-        if (h < (unsigned long long)(P.sp_cap - P.sp_evict_cap)) {
-          const uint32_t r = P.sp_evict_cap + (uint32_t)h;
-          ev_r = r;
-          ev_e = e;
-          entry = kSpillRef | r;    // in a warp, from the rerun list,
-          listed = !P.lane_wide;    // or in the wide round, which takes every such record
-        }
-        s.status = LS_RERUN;
+    const bool done = active && (s.status != LS_RUN || e + 1u >= n_ev);
+    if (__any_sync(0xFFFFFFFFu, done)) {
+      if (done && s.status == LS_RUN) s.status = LS_KEPT;
+      const bool out = done && s.status < LS_RERUN;  // (the others run again, or go on, in a later pass)
+      {
+        const uint32_t all = __ballot_sync(0xFFFFFFFFu, out), kept = __ballot_sync(0xFFFFFFFFu, out && s.status == LS_KEPT);
+        const uint32_t disc = __ballot_sync(0xFFFFFFFFu, out && s.status == LS_DISC);
+        const uint32_t ovf = __ballot_sync(0xFFFFFFFFu, out && s.status == LS_OVF);
+        const uint32_t log = __ballot_sync(0xFFFFFFFFu, out && s.status == LS_KEPT && s.logical);
+        cnt += __popc(lane == 0 ? all : lane == 1 ? disc : lane == 2 ? ovf : lane == 3 ? kept : lane == 4 ? log : 0u);
       }
-      if (s.status == LS_RERUN) {
-        if (listed) {
-          const unsigned long long i = atomicAdd(P.n_rerun, 1ull);
-          if (i < P.rerun_cap) P.rerun[i] = entry;
-        }
-        if (P.n_rerun_total) atomicAdd(P.n_rerun_total, 1ull);
-      } else {
-        atomicAdd(&wt[warp][0], 1ull);
-        if (s.status == LS_DISC) atomicAdd(&wt[warp][1], 1ull);
-        else if (s.status == LS_OVF) atomicAdd(&wt[warp][2], 1ull);
-        else if (s.status == LS_KEPT) {
-          atomicAdd(&wt[warp][3], 1ull);
-          if (s.logical) atomicAdd(&wt[warp][4], 1ull);
-          if (P.fid_mode && C->fsum) atomicAdd(C->fsum, s.fid);
-        }
+      if (out) {
+        const uint64_t off = base + item - (Multi ? C->item_begin : 0ull);  // the shot's offset within its circuit
+        if (P.fid_mode && s.status == LS_KEPT && C->fsum) atomicAdd(C->fsum, s.fid);
         if (!Multi && off < P.st_limit) s.capture(off, top_phase<W>(C, e < n_ev ? e + 1u : n_ev));
         if (off < C->out_limit) {
           if (C->status) C->status[off] = (uint8_t)s.status;
@@ -1370,8 +1326,26 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
 #pragma unroll 1
             for (uint32_t w = 0; w < C->rw; ++w) C->records[off * C->rw + w] = s.rec[(size_t)w * 32 + lane];
         }
+      } else if (done) {
+        uint32_t entry = item;  // a rerun starts the shot again from its start
+        bool listed = true;
+        if (s.status == LS_HAND) {  // or it resumes from its state at the top of event e
+          const unsigned long long h = atomicAdd(&P.lr[1], 1ull);
+          if (h < (unsigned long long)(P.sp_cap - P.sp_evict_cap)) {
+            const uint32_t r = P.sp_evict_cap + (uint32_t)h;
+            ev_r = r;
+            ev_e = e;
+            entry = kSpillRef | r;    // in a warp, from the rerun list,
+            listed = !P.lane_wide;    // or in the wide round, which takes every such record
+          }
+        }
+        if (listed) {
+          const unsigned long long i = atomicAdd(P.n_rerun, 1ull);
+          if (i < P.rerun_cap) P.rerun[i] = entry;
+        }
+        if (P.n_rerun_total) atomicAdd(P.n_rerun_total, 1ull);
       }
-      active = false;
+      if (done) active = false;
     }
     // few active lanes: their shots go to the spill pool (when it has room), to resume in
     // the next round packed with others, and the warp moves on to fresh shots
@@ -1394,21 +1368,29 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     }
     if (ev_r != 0xFFFFFFFFu) s.evict(S, ev_r, item, ev_e);
     uint32_t en = e + 1u > n_ev ? 0u : e + 1u;  // (within the circuit, cyclically)
-    if (!__any_sync(0xFFFFFFFFu, active)) {
-      // all lanes idle: the next bucket of any circuit (cyclically) that still has shots, or stop
+    if (__any_sync(0xFFFFFFFFu, active)) {
+      if (en) {
+        b0 = b1;
+        b1 = b2;
+        taken = taken1;
+      }
+    } else {
+      // all lanes idle: the next bucket of any circuit (cyclically) that still has shots, or
+      // stop; 32 buckets per step, one per lane
       uint32_t found = 0xFFFFFFFFu;
-      if (lane == 0) {
-        const uint32_t b_lo = Multi ? P.al_lo : 0u, nb = Multi ? P.al_hi - P.al_lo : P.al_nb;
-        const uint32_t g1 = (Multi ? C->bucket0 : 0u) + en - b_lo;
-        for (uint32_t k = 0; k < nb; ++k) {
-          const uint32_t c = b_lo + (g1 + k) % nb;
-          if (*(volatile unsigned int *)&P.al_next[c] < __ldg(&P.al_start[c + 1]) - __ldg(&P.al_start[c])) {
-            found = c;
-            break;
-          }
+      const uint32_t b_lo = Multi ? P.al_lo : 0u, nb = Multi ? P.al_hi - P.al_lo : P.al_nb;
+      const uint32_t g1 = (Multi ? C->bucket0 : 0u) + en - b_lo;
+      for (uint32_t k = 0; k < nb; k += 32) {
+        uint32_t c = g1 + k + lane;
+        if (c >= nb) c -= nb;  // (g1 < nb, k + lane < nb where it counts)
+        bool has = false;
+        if (k + lane < nb) has = *(volatile unsigned int *)&P.al_next[b_lo + c] < __ldg(&P.al_start[b_lo + c + 1]) - __ldg(&P.al_start[b_lo + c]);
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, has);
+        if (m) {
+          found = __shfl_sync(0xFFFFFFFFu, b_lo + c, __ffs(m) - 1);
+          break;
         }
       }
-      found = __shfl_sync(0xFFFFFFFFu, found, 0);
       if (found == 0xFFFFFFFFu) break;
       if (Multi) {
         const uint32_t cn = circ_of_bucket(P, found);
@@ -1424,6 +1406,12 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
       } else {
         en = found;
       }
+    }
+    if (!en || !__any_sync(0xFFFFFFFFu, active)) {  // not the bucket after the last one
+      const uint32_t gn = Multi ? C->bucket0 + en : en;
+      b0 = __ldg(&P.al_start[gn]);
+      b1 = __ldg(&P.al_start[gn + 1]);
+      taken = *(volatile unsigned int *)&P.al_next[gn];
     }
     e = en;
   }
@@ -1474,9 +1462,9 @@ uint32_t lane_prepass_grid() {
   return (uint32_t)(sms > 0 ? sms : 1) * 8u;
 }
 
-size_t lane_spill_bytes(int fp32, uint32_t W, uint32_t rw, uint32_t cap) {
-  return fp32 ? (W == 1 ? Spill<float, 1>::bytes(cap, rw) : Spill<float, 2>::bytes(cap, rw))
-              : (W == 1 ? Spill<double, 1>::bytes(cap, rw) : Spill<double, 2>::bytes(cap, rw));
+size_t lane_spill_bytes(int fp32, uint32_t W, uint32_t rw, uint32_t cap, uint32_t dim) {
+  return (size_t)cap * (fp32 ? (W == 1 ? Spill<float, 1>::record_bytes(rw, dim) : Spill<float, 2>::record_bytes(rw, dim))
+                             : (W == 1 ? Spill<double, 1>::record_bytes(rw, dim) : Spill<double, 2>::record_bytes(rw, dim)));
 }
 
 // the histogram of all buckets in shared memory (above 48 KB by the opt-in attribute)

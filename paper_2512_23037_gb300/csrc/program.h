@@ -102,15 +102,23 @@ struct alignas(16) CaseB {
 };
 
 // One noise site. X_q / Z_q of the site's qubits (index 0 = q0, 1 = q1)
-// carry beta/gamma words; c0 holds 2 bits per Pauli code (code 1..15).
+// carry beta/gamma words; c0 holds 2 bits per Pauli pair pa << 2 | pb (pb = 0 at a one-qubit
+// site, whose codes 1..3 are there too).
 // kind: bits 0-1 = SITE_DEPOL1 (X, Y, Z uniform), SITE_DEPOL2 (15 Paulis
 // uniform) or SITE_FLIP (the one-qubit Pauli code in bits 2-3).
+// The draws read a byte per site instead (CircDev::site_kind): kind, and kSiteThinned where
+// the site's rate is below the circuit's largest (thin holds its acceptance threshold).
 enum : uint32_t { SITE_DEPOL1 = 0, SITE_DEPOL2 = 1, SITE_FLIP = 2 };
+constexpr uint32_t kSiteThinned = 16;
 struct alignas(16) Site {
   uint64_t dsd[2], dss[2];  // sign XOR since the previous event
   uint64_t bx[2][2], gx[2][2], bz[2][2], gz[2][2];
   uint32_t kind, thin, always, c0;
 };
+
+// Lanes pack a site and its Pauli pair into one word; circuits of this many sites or more run
+// without them.
+constexpr uint32_t kMaxPackedSites = 0x0FFFFFFFu;
 
 constexpr uint32_t kNoRec = 0xFFFFFFFFu;
 

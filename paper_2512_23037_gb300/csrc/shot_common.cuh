@@ -15,11 +15,12 @@ namespace dev {
 
 // The next accepted error site at or after `cur` of shot `shot`: geometric gaps
 // of the noise stream against the thresholds thr (the smallest gap g with
-// U < thr[g]), then thinning. nxt = the site (0xFFFFFFFF if none), w2 = its
-// Pauli choice word. False if the guard ran out (impossible for valid tables).
+// U < thr[g]), then thinning. nxt = the site (0xFFFFFFFF if none), pp = its Pauli
+// pair (pa << 2 | pb, codes 1 X, 2 Y, 3 Z; pb = 0 at a one-qubit site).
+// False if the guard ran out (impossible for valid tables).
 template <bool Rolled = false>
 __device__ __forceinline__ bool next_site(const CircDev *C, uint64_t seed, uint64_t shot, uint32_t &cur,
-                                          uint32_t &kblk, uint32_t &nxt, uint32_t &w2) {
+                                          uint32_t &kblk, uint32_t &nxt, uint32_t &pp) {
   const uint32_t n_sites = C->n_sites;
   const uint64_t *thr = C->thr;
   for (uint32_t guard = 0; guard <= n_sites; ++guard) {
@@ -49,15 +50,67 @@ __device__ __forceinline__ bool next_site(const CircDev *C, uint64_t seed, uint6
     }
     uint32_t s = cur + lo;
     cur = s + 1u;
-    const Site *st = C->sites + s;
-    if (!__ldg(&st->always) && !(w.w < __ldg(&st->thin))) continue;
+    const uint32_t kind = __ldg(&C->site_kind[s]);
+    if ((kind & kSiteThinned) && !(w.w < __ldg(&C->sites[s].thin))) continue;
     nxt = s;
-    w2 = w.z;
+    pp = (kind & 3u) == SITE_DEPOL2 ? __umulhi(w.z, 15u) + 1u
+         : (kind & 3u) == SITE_FLIP ? kind & 12u
+                                    : (__umulhi(w.z, 3u) + 1u) << 2;
     return true;
   }
   nxt = 0xFFFFFFFFu;
   return false;
 }
+
+// The image of the error pp at site s, relative to signs (sd, ss) at the previous event:
+// i^e d_beta s_gamma. Every load is independent of the others.
+template <int W>
+__device__ __forceinline__ uint32_t site_pauli(const CircDev *C, uint32_t s, uint32_t pp, const uint64_t *sd,
+                                               const uint64_t *ss, uint64_t *beta, uint64_t *gamma) {
+  const Site *S = C->sites + s;
+  const uint32_t pa = pp >> 2, pb = pp & 3u;
+  uint64_t pe = 0;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    uint64_t b = 0, g = 0;
+    if (pa == 1u || pa == 2u) { b ^= __ldg(&S->bx[0][w]); g ^= __ldg(&S->gx[0][w]); }
+    if (pa == 3u || pa == 2u) { b ^= __ldg(&S->bz[0][w]); g ^= __ldg(&S->gz[0][w]); }
+    if (pb == 1u || pb == 2u) { b ^= __ldg(&S->bx[1][w]); g ^= __ldg(&S->gx[1][w]); }
+    if (pb == 3u || pb == 2u) { b ^= __ldg(&S->bz[1][w]); g ^= __ldg(&S->gz[1][w]); }
+    beta[w] = b;
+    gamma[w] = g;
+    pe ^= ((sd[w] ^ __ldg(&S->dsd[w])) & b) ^ ((ss[w] ^ __ldg(&S->dss[w])) & g);
+  }
+  return ((__ldg(&S->c0) >> (2u * pp)) + 2u * wordpar(pe)) & 3u;
+}
+
+// A shot's place in its noise stream: the next error, the one after it once drawn (`drawn`;
+// the lanes' pre-pass draws both, whose Philox blocks and searches would run with a few
+// active lanes in the lane kernel), and the next Philox block. Packed: site | pair << 28.
+// (site kMaxPackedSites: no error left)
+constexpr uint32_t kNotDrawn = 0x10000000u;  // (no second error: it would be at site 0)
+__device__ __forceinline__ uint32_t pack_error(uint32_t nxt, uint32_t pp) {
+  return nxt == 0xFFFFFFFFu ? 0x0FFFFFFFu : nxt | (pp << 28);
+}
+struct NoiseCursor {
+  uint32_t first, second, kblk;
+  __device__ __forceinline__ uint32_t site() const { return first & 0x0FFFFFFFu; }
+  __device__ __forceinline__ uint32_t pair() const { return first >> 28; }
+  // past the first error
+  template <bool Rolled = false>
+  __device__ __forceinline__ bool advance(const CircDev *C, uint64_t seed, uint64_t shot) {
+    bool ok = true;
+    if (second == kNotDrawn) {
+      uint32_t cur = site() + 1u, nxt = 0xFFFFFFFFu, pp = 0;
+      ok = next_site<Rolled>(C, seed, shot, cur, kblk, nxt, pp);
+      first = pack_error(nxt, pp);
+    } else {
+      first = second;
+      second = kNotDrawn;
+    }
+    return ok;
+  }
+};
 
 // The event a shot whose first error is at site nxt starts at: the event that
 // applies that error, capped at the last valid event of the noiseless run
@@ -153,46 +206,46 @@ __device__ __forceinline__ int pick_outcome(uint64_t seed, uint64_t shot, uint32
   return (double)m * 0x1p-53 * (sp + sm) < sp ? 1 : -1;
 }
 
-// A spill record holds one shot's whole state at the top of an event: item,
-// resume event, n and flags (chain, logical, last outcome); the noise cursor
-// (nxt, cur, kblk, w2); F; the signs; the record words; up to kLaneCap entries (FP64: of a
-// scaled map, and its squared norm).
-// Structure of arrays over `cap` records.
+// A spill record holds one shot's whole state at the top of an event, with its map in a
+// lane's affine form of `dim` directions: item, resume event, live slots (low word), d and
+// flags (chain, logical, last outcome); the noise cursor and the live slots' high word; F;
+// FP64: the squared norm; the signs; the record words; the rows alpha0, B[0..dim),
+// Dual[0..dim); the values of the 2^dim slots (those of live slots below 2^d, rows below d,
+// are written). A lane or a warp reads a whole record at once, so its words are contiguous.
 template <typename R, int W>
 struct Spill {
-  uint4 *ha, *hb;
-  double *fid;
-  uint64_t *sd, *ss, *rec, *keys;
-  Cx<R> *vals;
-  double *norm;  // FP64 only
-  uint32_t cap;
-  __host__ __device__ static size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
-  __host__ __device__ static size_t bytes(uint32_t cap, uint32_t rw) {
-    const size_t c = cap;
-    return 2 * al16(c * 16) + al16(c * 8) + 2 * al16(c * 8 * W) + al16(c * 8 * rw) + al16(c * 8 * W * kLaneCap) +
-           al16(c * sizeof(Cx<R>) * kLaneCap) + (sizeof(R) == 8 ? al16(c * 8) : 0);
+  unsigned char *base;
+  uint32_t rw, dim;
+  size_t stride;
+  __host__ __device__ static size_t fixed(uint32_t rw) {
+    return 48 + (size_t)2 * W * 8 + (size_t)rw * 8;
   }
-  __device__ Spill(unsigned char *b, uint32_t cap_, uint32_t rw) : cap(cap_) {
-    const size_t c = cap;
-    ha = reinterpret_cast<uint4 *>(b);
-    b += al16(c * 16);
-    hb = reinterpret_cast<uint4 *>(b);
-    b += al16(c * 16);
-    fid = reinterpret_cast<double *>(b);
-    b += al16(c * 8);
-    sd = reinterpret_cast<uint64_t *>(b);
-    b += al16(c * 8 * W);
-    ss = reinterpret_cast<uint64_t *>(b);
-    b += al16(c * 8 * W);
-    rec = reinterpret_cast<uint64_t *>(b);
-    b += al16(c * 8 * rw);
-    keys = reinterpret_cast<uint64_t *>(b);
-    b += al16(c * 8 * W * kLaneCap);
-    vals = reinterpret_cast<Cx<R> *>(b);
-    b += al16(c * sizeof(Cx<R>) * kLaneCap);
-    norm = reinterpret_cast<double *>(b);
+  __host__ __device__ static size_t vals_off(uint32_t rw, uint32_t dim) {
+    return (fixed(rw) + (size_t)(1 + 2 * dim) * W * 8 + 15) & ~(size_t)15;
+  }
+  __host__ __device__ static size_t record_bytes(uint32_t rw, uint32_t dim) {
+    return (vals_off(rw, dim) + (sizeof(Cx<R>) << dim) + 15) & ~(size_t)15;
+  }
+  __device__ Spill(unsigned char *b, uint32_t rw_, uint32_t dim_)
+      : base(b), rw(rw_), dim(dim_), stride(record_bytes(rw_, dim_)) {}
+  __device__ __forceinline__ unsigned char *at(uint32_t r) const { return base + (size_t)r * stride; }
+  __device__ __forceinline__ static uint4 &ha(unsigned char *p) { return reinterpret_cast<uint4 *>(p)[0]; }
+  __device__ __forceinline__ static uint4 &hb(unsigned char *p) { return reinterpret_cast<uint4 *>(p)[1]; }
+  __device__ __forceinline__ static double &fid(unsigned char *p) { return reinterpret_cast<double *>(p)[4]; }
+  __device__ __forceinline__ static double &norm(unsigned char *p) { return reinterpret_cast<double *>(p)[5]; }
+  __device__ __forceinline__ static uint64_t *sd(unsigned char *p) { return reinterpret_cast<uint64_t *>(p + 48); }
+  __device__ __forceinline__ static uint64_t *ss(unsigned char *p) { return sd(p) + W; }
+  __device__ __forceinline__ static uint64_t *rec(unsigned char *p) { return sd(p) + 2 * W; }
+  __device__ __forceinline__ uint64_t *rows(unsigned char *p) const { return reinterpret_cast<uint64_t *>(p + fixed(rw)); }
+  __device__ __forceinline__ Cx<R> *vals(unsigned char *p) const {
+    return reinterpret_cast<Cx<R> *>(p + vals_off(rw, dim));
+  }
+  __device__ __forceinline__ static uint32_t meta(uint32_t d, int chain, int logical, int lastm) {
+    return d | ((uint32_t)(chain & 1) << 8) | ((uint32_t)(logical & 1) << 9) | (((uint32_t)lastm & 255u) << 16);
   }
 };
+constexpr uint32_t kLaneDim = 4;  // directions of a first-round lane's records (kLaneCap = 2^kLaneDim)
+static_assert(kLaneCap == (1u << kLaneDim), "lane map");
 
 }  // namespace dev
 }  // namespace soft
