@@ -35,8 +35,12 @@ constexpr uint32_t kAll = 0xFFFFFFFFu;
 constexpr int kAffBlock = 128;
 constexpr uint32_t kAffRecWords = 32;  // lane w keeps record word w (a circuit has at most 16)
 
-template <typename R>
-__host__ __device__ constexpr size_t aff_warp_bytes(uint32_t dim) { return sizeof(Cx<R>) << dim; }
+// events held ahead of a warp in shared memory
+constexpr uint32_t kRing = 4;
+template <typename R, int W>
+__host__ __device__ constexpr size_t aff_warp_bytes(uint32_t dim) {
+  return (sizeof(Cx<R>) << dim) + kRing * sizeof(Ev<W>);
+}
 
 __device__ __forceinline__ uint64_t shfl64(uint64_t x, uint32_t src) {
   return (uint64_t)__shfl_sync(kAll, (unsigned long long)x, (int)src);
@@ -74,6 +78,7 @@ struct AffShot {
   const CircDev *C = nullptr;
   const uint32_t lane;
   Cx<R> *v;             // 2^aff_dim values (shared memory)
+  unsigned char *ring;  // kRing events (shared memory)
   uint64_t B[W], D[W];  // lane k < d: direction k and its dual; 0 in the other lanes
   uint64_t a0[W];       // alpha0 (every lane)
   uint64_t recw;        // lane w: record word w
@@ -89,7 +94,7 @@ struct AffShot {
   typename std::conditional<kScaled, ScaledPrune, PruneTest<R>>::type pt;  // |v|^2 < tau
 
   __device__ AffShot(const ShotParams &p, unsigned char *base)
-      : P(p), lane(threadIdx.x & 31u), v(reinterpret_cast<Cx<R> *>(base)), pt(p.tau) {}
+      : P(p), lane(threadIdx.x & 31u), v(reinterpret_cast<Cx<R> *>(base)), ring(base + (sizeof(Cx<R>) << p.aff_dim)), pt(p.tau) {}
   // x, or zero where it is below tau
   __device__ __forceinline__ Cx<R> pruned(Cx<R> x) const {
     bool sm;
@@ -211,11 +216,41 @@ struct AffShot {
     }
     return false;
   }
-  __device__ uint32_t live_count() const {
+  // live slots, and the last of them
+  __device__ uint32_t live_count(uint32_t *last = nullptr) const {
     uint32_t n = 0;
-    for (uint32_t b = 0; b < size(); b += 32)
-      n += __popc(__ballot_sync(kAll, b + lane < size() && nonzero(v[b + lane])));
+    for (uint32_t b = 0; b < size(); b += 32) {
+      const uint32_t m = __ballot_sync(kAll, b + lane < size() && nonzero(v[b + lane]));
+      n += __popc(m);
+      if (last && m) *last = b + 31u - __clz(m);
+    }
     return n;
+  }
+  // Before the map grows: where half the slots or more are empty, drop the coordinates that the
+  // live ones do not need. Rotations that undo earlier ones (the T^dag after a T) leave such
+  // maps, down to a single entry; compacting only at the map's limit left 75 slots on average
+  // on w97 where 30 do. True if a coordinate went (coordinates and residuals are then stale).
+  __device__ bool compact(uint32_t &gl, uint32_t &g0) {
+    if (d < 3u) return false;
+    uint32_t s0 = 0;
+    const uint32_t n = live_count(&s0);
+    if (n > (size() >> 1) && d < P.aff_dim) return false;
+    if (n == 1u) {  // one entry: alpha0 takes its key
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        a0[w] ^= xor_all(((s0 >> lane) & 1u) ? B[w] : 0ull);
+        B[w] = D[w] = 0ull;
+      }
+      g0 ^= par32(s0 & gl);
+      gl = 0;
+      d = 0;
+      if (s0 && lane == 0) v[0] = v[s0];
+      __syncwarp();
+      return true;
+    }
+    bool any = false;
+    while (compact_one(gl, g0)) any = true;
+    return any;
   }
 
   __device__ void fail_check(uint32_t code, uint64_t value) {
@@ -311,9 +346,23 @@ struct AffShot {
       fail_check(CHK_SITE, s);
       return;
     }
-    uint64_t beta[W], gamma[W];
-    const uint32_t e = site_pauli<W>(C, s, nc.pair(), sd, ss, beta, gamma);
-    apply_pauli(beta, gamma, e);
+    // the site's record, 16 bytes per lane, in one load; its words are combined by reductions
+    // (lanes 0, 1: signs; 2, 3 X's beta and 4, 5 its gamma per qubit; 6-9 Z's; 10: phases)
+    const uint32_t pp = nc.pair(), pa = pp >> 2, pb = pp & 3u;
+    const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(C->sites + s) + (lane < 11u ? lane : 0u));
+    const uint32_t x = ((pa == 1u || pa == 2u) ? 1u : 0u) | ((pb == 1u || pb == 2u) ? 2u : 0u);
+    const uint32_t z = (pa >= 2u ? 1u : 0u) | (pb >= 2u ? 2u : 0u);
+    const bool in_b = (((x << 2) | (z << 6)) >> lane) & 1u, in_g = (((x << 4) | (z << 8)) >> lane) & 1u;
+    uint64_t beta[W], gamma[W], pe = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const uint64_t y = w ? q.y : q.x;
+      beta[w] = xor_all(in_b ? y : 0ull);
+      gamma[w] = xor_all(in_g ? y : 0ull);
+      pe ^= ((sd[w] ^ shfl64(y, 0)) & beta[w]) ^ ((ss[w] ^ shfl64(y, 1)) & gamma[w]);
+    }
+    const uint32_t c0 = __shfl_sync(kAll, (uint32_t)(q.y >> 32), 10);
+    apply_pauli(beta, gamma, ((c0 >> (2u * pp)) + 2u * wordpar(pe)) & 3u);
   }
 
   // FP32: b xi x, xi = i^e (-1)^par
@@ -334,17 +383,13 @@ struct AffShot {
     if (!diag) {
       c = coords(beta, r);
       fresh = wnonzero(r);  // beta outside the span: every entry gains a partner
+      if (fresh && compact(gl, g0)) {
+        c = coords(beta, r);
+        fresh = wnonzero(r);
+      }
       if (fresh && d == P.aff_dim) {
-        bool any = false;
-        while (compact_one(gl, g0)) any = true;
-        if (any) {
-          c = coords(beta, r);
-          fresh = wnonzero(r);
-        }
-        if (fresh && d == P.aff_dim) {
-          status = AS_RERUN;
-          return;
-        }
+        status = AS_RERUN;
+        return;
       }
     }
     const Coef *cf = C->coef + ci;
@@ -633,11 +678,59 @@ struct AffShot {
     return ok ? (uint32_t)((w >> (r & 63)) & 1ull) : 0u;
   }
 
-  // one event (header hdr, body: dsd, dss, beta, gamma; E for a fused reset correction's words)
-  __device__ void step(const uint4 &hdr, const uint64_t *body, const Ev<W> *E) {
+  // past the first error: the one after it, drawn by the warp (next_site of shot_common.cuh with
+  // the candidates of U's bucket compared at once)
+  __device__ __forceinline__ void advance() {
+    if (nc.second != kNotDrawn) {
+      nc.first = nc.second;
+      nc.second = kNotDrawn;
+      return;
+    }
+    uint32_t cur = nc.site() + 1u;
+    draw(cur);
+  }
+  __device__ void draw(uint32_t cur) {
+    const uint32_t n_sites = C->n_sites;
+    for (uint32_t guard = 0; guard <= n_sites; ++guard) {
+      if (cur >= n_sites) {
+        nc.first = pack_error(kAll, 0u);
+        return;
+      }
+      const uint4 w = philox(P.seed, shot, 0u, nc.kblk++);
+      const uint64_t U = (uint64_t)w.x | ((uint64_t)w.y << 32);
+      const uint32_t rem = n_sites - cur, b = (uint32_t)(U >> (64 - kThrTabBits));
+      const uint32_t t0 = __ldg(&C->thr_tab[b]), t1 = __ldg(&C->thr_tab[b + 1]);
+      uint32_t lo = t0 < rem ? t0 : rem;
+      const uint32_t hi = t1 < rem ? t1 : rem;
+      while (lo < hi) {  // (a bucket spans few sites)
+        const uint32_t n = hi - lo < 32u ? hi - lo : 32u;
+        const uint32_t below = __popc(__ballot_sync(kAll, lane < n && !(U < __ldg(&C->thr[lo + (lane < n ? lane : 0u)]))));
+        lo += below;
+        if (below < n) break;
+      }
+      if (lo == rem) {
+        nc.first = pack_error(kAll, 0u);
+        return;
+      }
+      const uint32_t s = cur + lo;
+      cur = s + 1u;
+      const uint32_t kind = __ldg(&C->site_kind[s]);
+      if ((kind & kSiteThinned) && !(w.w < __ldg(&C->sites[s].thin))) continue;
+      nc.first = pack_error(s, (kind & 3u) == SITE_DEPOL2 ? __umulhi(w.z, 15u) + 1u
+                               : (kind & 3u) == SITE_FLIP ? kind & 12u
+                                                          : (__umulhi(w.z, 3u) + 1u) << 2);
+      return;
+    }
+    status = AS_ERR;
+  }
+
+  // one event (its copy in shared memory)
+  __device__ void step(const Ev<W> *ev) {
+    const uint4 hdr = *reinterpret_cast<const uint4 *>(ev);
+    const uint64_t *body = ev->dsd;  // dsd, dss, beta, gamma
     while (nc.site() < hdr.y && status == AS_RUN) {
       apply_error(nc.site());
-      if (!nc.advance(C, P.seed, shot)) status = AS_ERR;
+      advance();
     }
     if (status != AS_RUN) return;
     const uint64_t *beta = body + 2 * W, *gamma = body + 3 * W;
@@ -668,8 +761,8 @@ struct AffShot {
         uint64_t xb[W], xg[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-          xb[w] = __ldg(&E->xbeta[w]);
-          xg[w] = __ldg(&E->xgamma[w]);
+          xb[w] = ev->xbeta[w];
+          xg[w] = ev->xgamma[w];
         }
         apply_pauli(xb, xg, (ev_xe0(w0) + 2u * wpar2<W>(sd, xb, ss, xg)) & 3u);
       }
@@ -691,15 +784,12 @@ struct AffShot {
       }
     }
   }
-  __device__ __forceinline__ static void load_event(const Ev<W> *E, uint4 &hdr, uint64_t *body) {
-    hdr = __ldg(reinterpret_cast<const uint4 *>(E));
-    const ulonglong2 *bp = reinterpret_cast<const ulonglong2 *>(&E->dsd[0]);
-#pragma unroll
-    for (int k = 0; k < 2 * W; ++k) {
-      const ulonglong2 x = __ldg(bp + k);
-      body[2 * k] = x.x;
-      body[2 * k + 1] = x.y;
-    }
+  // event e into its place of the ring, 16 bytes per lane (one copy group per event, empty past
+  // the end, so that the groups count the events)
+  __device__ __forceinline__ void fetch_event(const Ev<W> *evs, uint32_t e, uint32_t n_events) {
+    if (e < n_events && lane < sizeof(Ev<W>) / 16)
+      copy_async<16>(ring + (e % kRing) * sizeof(Ev<W>) + lane * 16u, reinterpret_cast<const unsigned char *>(evs + e) + lane * 16u);
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
   // the shot of item `local` (chunk-local), from spill record r or (kNoRecord) from the
   // event that applies its first error
@@ -718,11 +808,10 @@ struct AffShot {
         if (nc.site() != kMaxPackedSites) nxt = nc.site();
         if (nc.kblk == kAll) status = AS_ERR;
       } else {
-        uint32_t cur = 0, pp = 0;
         nc.kblk = 0;
-        if (!next_site(C, P.seed, shot, cur, nc.kblk, nxt, pp)) status = AS_ERR;
-        nc.first = pack_error(nxt, pp);
         nc.second = kNotDrawn;
+        draw(0);
+        if (nc.site() != kMaxPackedSites) nxt = nc.site();
       }
       ev = first_event(C, P.fid_mode, nxt);
       load_snapshot(ev);
@@ -730,21 +819,17 @@ struct AffShot {
     const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C->ev);
     const uint32_t n_events = C->n_events;
     ev_top = ev;
-    if (ev < n_events && status == AS_RUN) {
-      uint4 hdr, hn;
-      uint64_t body[4 * W], bn[4 * W];
-      load_event(evs + ev, hdr, body);
-      for (;;) {  // the next event's words are loaded while this one runs
-        const uint32_t en = ev + 1u;
-        if (en < n_events) load_event(evs + en, hn, bn);
-        step(hdr, body, evs + ev);
-        ev_top = en;
-        if (en >= n_events || status != AS_RUN) break;
-        ev = en;
-        hdr = hn;
-#pragma unroll
-        for (int k = 0; k < 4 * W; ++k) body[k] = bn[k];
+    if (status == AS_RUN) {
+      for (uint32_t k = 0; k + 1u < kRing; ++k) fetch_event(evs, ev + k, n_events);
+      while (ev < n_events && status == AS_RUN) {  // the events after this one are on their way
+        asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");
+        __syncwarp();
+        fetch_event(evs, ev + kRing - 1u, n_events);
+        step(reinterpret_cast<const Ev<W> *>(ring + (ev % kRing) * sizeof(Ev<W>)));
+        ev_top = ++ev;
       }
+      copies_done();  // (the next shot writes the ring again)
+      __syncwarp();
     }
     if (status == AS_RUN) status = AS_KEPT;
   }
@@ -820,7 +905,7 @@ __global__ void __launch_bounds__(kAffBlock, sizeof(R) == 4 && W == 1 ? 6 : 5) a
   const uint32_t n_circ = P.n_circ < (uint32_t)kMaxCirc ? P.n_circ : (uint32_t)kMaxCirc;
   for (uint32_t i = threadIdx.x; i < 5 * n_circ; i += blockDim.x) btally[i / 5][i % 5] = 0ull;
   __syncthreads();
-  AffShot<R, W> s(P, smem + (threadIdx.x / 32) * aff_warp_bytes<R>(P.aff_dim));
+  AffShot<R, W> s(P, smem + (threadIdx.x / 32) * aff_warp_bytes<R, W>(P.aff_dim));
   const unsigned long long n_items = P.n_items_dev ? *P.n_items_dev : P.n_items;
   const unsigned long long item_base = P.item_base_dev ? *P.item_base_dev : P.item_base;
   for (;;) {
@@ -863,7 +948,9 @@ cudaError_t prepare_affine(const ShotParams &p, int fp32, uint32_t W, int blocks
                                     : reinterpret_cast<const void *>(affine_kernel<float, 2>))
                           : (W == 1 ? reinterpret_cast<const void *>(affine_kernel<double, 1>)
                                     : reinterpret_cast<const void *>(affine_kernel<double, 2>));
-  const size_t smem = (kAffBlock / 32) * (fp32 ? aff_warp_bytes<float>(p.aff_dim) : aff_warp_bytes<double>(p.aff_dim));
+  const size_t smem =
+      (kAffBlock / 32) * (fp32 ? (W == 1 ? aff_warp_bytes<float, 1>(p.aff_dim) : aff_warp_bytes<float, 2>(p.aff_dim))
+                               : (W == 1 ? aff_warp_bytes<double, 1>(p.aff_dim) : aff_warp_bytes<double, 2>(p.aff_dim)));
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, occ = 0;
