@@ -47,6 +47,8 @@ struct soft_run {
   uint32_t *d_al = nullptr;                // lane-per-shot bucketing buffers
   unsigned char *d_sp = nullptr;           // lane-per-shot spill pool (shots evicted between rounds)
   unsigned long long *d_lr = nullptr;      // its record count and each round's record range
+  unsigned char *d_spb[2] = {nullptr, nullptr};       // the same of the 32- and 64-entry lanes
+  unsigned long long *d_lrb[2] = {nullptr, nullptr};
   bool fid_mode = false;
   unsigned long long *d_work = nullptr;    // next1, next2, n_rerun, item_base, diag[4], reruns of all chunks,
                                            // middle pass: next, n_rerun
@@ -466,6 +468,19 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     need(&r->d_sp, soft::lane_spill_bytes(fp32, W, rw_max, sp_evict + sp_hand, soft::lane_map_dim()));
     need(&r->d_lr, n_lr * sizeof(unsigned long long));
   }
+  // the larger lanes' eviction pools: a quarter of their circuits' shots, at most 2^22 records
+  // (a record of a 64-entry lane takes about 0.8 KB)
+  uint32_t sp_big[2] = {0, 0};
+  for (int k = 0; lanes && rounds > 1 && k < 2; ++k) {
+    uint64_t n = 0;
+    for (uint32_t i = 0; i < n_circ; ++i)
+      if (lcap[i] && lane_class(lcap[i]) == 1 + k) n += n_shots[i];
+    n = std::min(n, chunk);
+    if (!nbc[1 + k] || n == 0) continue;
+    sp_big[k] = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(std::min<uint64_t>(n, 1024), n / 4), 1ull << 22);
+    need(&r->d_spb[k], soft::lane_spill_bytes(fp32, W, rw_max, sp_big[k], soft::lane_map_dim() + 1 + k));
+    need(&r->d_lrb[k], n_lr * sizeof(unsigned long long));
+  }
   r->fid_mode = fid_mode;
   if (fid_mode) need(&r->d_fsum, n_circ * sizeof(double));
   need(&r->d_work, 11 * sizeof(unsigned long long));
@@ -638,15 +653,18 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   soft::LaunchCfg c1{}, c2{}, cm{}, cw{}, cb[2]{};
   p.n_items = std::min(chunk, total);
   // the larger lanes (32 and 64 entries): one launch each over their circuits' buckets, after
-  // the 16-entry lanes' first round; they never evict or hand over
+  // the 16-entry lanes' first round, and one more over the shots that it evicts; they never
+  // hand over
   soft::ShotParams pb[2] = {p, p};
   for (int k = 0; k < 2; ++k) {
     pb[k].al_lo = (uint32_t)(nbc[0] + (k ? nbc[1] : 0));
     pb[k].al_hi = pb[k].al_lo + (uint32_t)nbc[1 + k];
-    pb[k].lane_evict = pb[k].lane_hand = pb[k].lane_wide = 0;
-    pb[k].sp = nullptr;
-    pb[k].sp_cap = pb[k].sp_evict_cap = 0;
-    pb[k].lr = nullptr;
+    pb[k].lane_hand = pb[k].lane_wide = 0;
+    pb[k].lane_evict = sp_big[k] ? 1u : 0u;
+    pb[k].sp = r->d_spb[k];
+    pb[k].sp_cap = pb[k].sp_evict_cap = sp_big[k];
+    pb[k].sp_dim = soft::lane_map_dim() + 1 + k;
+    pb[k].lr = r->d_lrb[k];
   }
   if ((e = !lanes ? (affine ? soft::prepare_affine(p, fp32, W, (int)o.blocks_per_sm, &c1)
                             : soft::prepare_shots(p, fp32, W, g1, (int)o.blocks_per_sm, &c1))
@@ -708,6 +726,8 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
         ab.n_items = cnt;
         ab.item_base = base;
         if (dev_base) ab.item_base_dev = r->d_work + 3;
+        if (sp_big[k] && (err = cudaMemsetAsync(r->d_lrb[k], 0, n_lr * sizeof(unsigned long long), st)) != cudaSuccess)
+          return err;
         if ((err = soft::launch_prepared(cb[k], ab, st)) != cudaSuccess) return err;
         r->launches++;
       }
@@ -723,6 +743,20 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
         return err;
       r->launches += 5;
     }
+    for (int k = 0; lanes && k < 2; ++k)
+      if (sp_big[k]) {
+        soft::ShotParams ar = pb[k];
+        ar.item_base = base;
+        if (dev_base) ar.item_base_dev = r->d_work + 3;
+        ar.lane_round = 1;
+        ar.lane_evict = 0;
+        ar.n_items_dev = r->d_lrb[k] + 5;
+        if ((err = cudaMemsetAsync(ar.al_count, 0, 2 * (size_t)nb * sizeof(uint32_t), st)) != cudaSuccess ||
+            (err = soft::launch_lane_resume_prepass(ar, fp32, W, st)) != cudaSuccess ||
+            (err = soft::launch_prepared(cb[k], ar, st)) != cudaSuccess)
+          return err;
+        r->launches += 5;
+      }
     if (wide) {  // the handed-over shots, bucketed by the event they resume at
       soft::ShotParams aw = a;
       aw.lane_round = rounds;
