@@ -645,6 +645,9 @@ struct GradWarp {
   }
 
   // ------------------------------------------------------------- noise
+  __device__ __forceinline__ const SiteDev<W> *site(uint32_t s) const {
+    return reinterpret_cast<const SiteDev<W> *>(P.sites) + s;
+  }
   __device__ void draw_next() {
     for (uint32_t guard = 0; guard <= P.n_sites; ++guard) {
       if (cur >= P.n_sites) {
@@ -672,7 +675,7 @@ struct GradWarp {
       }
       uint32_t s = cur + lo;
       cur = s + 1u;
-      const Site *st = P.sites + s;
+      const SiteDev<W> *st = site(s);
       if (!__ldg(&st->always) && !(w.w < __ldg(&st->thin))) continue;
       nxt = s;
       w2 = w.z;
@@ -683,17 +686,19 @@ struct GradWarp {
   // beta/gamma/e of the error at site s with Pauli code `code`, signs (esd, ess) at the site
   __device__ void error_pauli(uint32_t s, uint32_t code, const uint64_t *esd, const uint64_t *ess, uint64_t *beta,
                               uint64_t *gamma, uint32_t *e) const {
-    const Site *S = P.sites + s;
+    const SiteDev<W> *S = site(s);
     const uint32_t two = (__ldg(&S->kind) & 3u) == SITE_DEPOL2;
-    const uint32_t pa = two ? (code >> 2) : code, pb = two ? (code & 3u) : 0u;
+    const uint32_t need = site_images(two ? code : code << 2);
     uint32_t q = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       uint64_t b = 0, g = 0;
-      if (pa == 1u || pa == 2u) { b ^= __ldg(&S->bx[0][w]); g ^= __ldg(&S->gx[0][w]); }
-      if (pa == 3u || pa == 2u) { b ^= __ldg(&S->bz[0][w]); g ^= __ldg(&S->gz[0][w]); }
-      if (pb == 1u || pb == 2u) { b ^= __ldg(&S->bx[1][w]); g ^= __ldg(&S->gx[1][w]); }
-      if (pb == 3u || pb == 2u) { b ^= __ldg(&S->bz[1][w]); g ^= __ldg(&S->gz[1][w]); }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if ((need >> j) & 1u) {
+          b ^= __ldg(&S->img[j][w]);
+          g ^= __ldg(&S->img[j][W + w]);
+        }
       beta[w] = b;
       gamma[w] = g;
       q += __popcll(esd[w] & b) + __popcll(ess[w] & g);
@@ -889,7 +894,7 @@ struct GradWarp {
       }
       const uint64_t *dsd = body, *dss = body + W, *beta = body + 2 * W, *gamma = body + 3 * W;
       while (nxt < hdr.y && status == G_OK) {
-        const Site *S = P.sites + nxt;
+        const SiteDev<W> *S = site(nxt);
         uint64_t esd[W], ess[W], b[W], g[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) {

@@ -12,7 +12,7 @@ struct GradParams {
   const void *ev;  // Ev<W>
   const Coef *coef;  // coefficients for the current parameter vector
   const CaseB *cb;
-  const Site *sites;
+  const void *sites;  // SiteDev<W>
   const uint64_t *thr;
   const uint32_t *thr_tab;  // the gap search's index (program.h; null: plain search)
   uint32_t n_events, n_sites, rw, n_rot, n_params, blocks;

@@ -347,21 +347,31 @@ struct AffShot {
       return;
     }
     // the site's record, 16 bytes per lane, in one load; its words are combined by reductions
-    // (lanes 0, 1: signs; 2, 3 X's beta and 4, 5 its gamma per qubit; 6-9 Z's; 10: phases)
-    const uint32_t pp = nc.pair(), pa = pp >> 2, pb = pp & 3u;
-    const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(C->sites + s) + (lane < 11u ? lane : 0u));
-    const uint32_t x = ((pa == 1u || pa == 2u) ? 1u : 0u) | ((pb == 1u || pb == 2u) ? 2u : 0u);
-    const uint32_t z = (pa >= 2u ? 1u : 0u) | (pb >= 2u ? 2u : 0u);
-    const bool in_b = (((x << 2) | (z << 6)) >> lane) & 1u, in_g = (((x << 4) | (z << 8)) >> lane) & 1u;
+    const uint32_t pp = nc.pair(), need = site_images(pp);
+    constexpr uint32_t kParts = sizeof(SiteDev<W>) / 16, kSig = W == 1 ? 4u : 8u;  // (lane kSig: the signs)
+    const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(reinterpret_cast<const SiteDev<W> *>(C->sites) + s) +
+                               (lane < kParts ? lane : 0u));
     uint64_t beta[W], gamma[W], pe = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      const uint64_t y = w ? q.y : q.x;
-      beta[w] = xor_all(in_b ? y : 0ull);
-      gamma[w] = xor_all(in_g ? y : 0ull);
-      pe ^= ((sd[w] ^ shfl64(y, 0)) & beta[w]) ^ ((ss[w] ^ shfl64(y, 1)) & gamma[w]);
+      uint64_t esd, ess;
+      if (W == 1) {  // lane j: image j's beta and gamma
+        const bool in = lane < 4u && ((need >> lane) & 1u);
+        beta[w] = xor_all(in ? q.x : 0ull);
+        gamma[w] = xor_all(in ? q.y : 0ull);
+        esd = shfl64(q.x, kSig);
+        ess = shfl64(q.y, kSig);
+      } else {  // lanes 2j, 2j + 1: image j's two words of beta, of gamma
+        const uint64_t y = w ? q.y : q.x;
+        const bool in = lane < 8u && ((need >> (lane >> 1)) & 1u);
+        beta[w] = xor_all(in && !(lane & 1u) ? y : 0ull);
+        gamma[w] = xor_all(in && (lane & 1u) ? y : 0ull);
+        esd = shfl64(y, kSig);
+        ess = shfl64(y, kSig + 1u);
+      }
+      pe ^= ((sd[w] ^ esd) & beta[w]) ^ ((ss[w] ^ ess) & gamma[w]);
     }
-    const uint32_t c0 = __shfl_sync(kAll, (uint32_t)(q.y >> 32), 10);
+    const uint32_t c0 = __shfl_sync(kAll, (uint32_t)(q.y >> 32), (int)kParts - 1);
     apply_pauli(beta, gamma, ((c0 >> (2u * pp)) + 2u * wordpar(pe)) & 3u);
   }
 
@@ -715,7 +725,7 @@ struct AffShot {
       const uint32_t s = cur + lo;
       cur = s + 1u;
       const uint32_t kind = __ldg(&C->site_kind[s]);
-      if ((kind & kSiteThinned) && !(w.w < __ldg(&C->sites[s].thin))) continue;
+      if ((kind & kSiteThinned) && !(w.w < __ldg(&C->site_thin[s]))) continue;
       nc.first = pack_error(s, (kind & 3u) == SITE_DEPOL2 ? __umulhi(w.z, 15u) + 1u
                                : (kind & 3u) == SITE_FLIP ? kind & 12u
                                                           : (__umulhi(w.z, 3u) + 1u) << 2);

@@ -86,6 +86,24 @@ constexpr int kMaxDevices = 64;
 WsCache g_ws[kMaxDevices];
 }  // namespace
 
+template <int W>
+static void site_dev(const soft::Site &s, soft::SiteDev<W> &d) {
+  for (int w = 0; w < W; ++w) {
+    for (int q = 0; q < 2; ++q) {
+      d.img[2 * q][w] = s.bx[q][w];
+      d.img[2 * q][W + w] = s.gx[q][w];
+      d.img[2 * q + 1][w] = s.bz[q][w];
+      d.img[2 * q + 1][W + w] = s.gz[q][w];
+    }
+    d.dsd[w] = s.dsd[w];
+    d.dss[w] = s.dss[w];
+  }
+  d.kind = s.kind;
+  d.thin = s.thin;
+  d.always = s.always;
+  d.c0 = s.c0;
+}
+
 // Records both precisions' noiseless runs of a freshly uploaded circuit (the
 // prefix every shot shares until its first error). Synchronous, but on streams
 // of its own: it waits for no other work on the device.
@@ -183,9 +201,17 @@ int soft_compile_circuit(const soft_op *ops, size_t n_ops, uint32_t n_qubits, co
   }
   size_t b_cf = std::max<size_t>(1, hp.coefs.size()) * sizeof(soft::Coef),
          b_cb = std::max<size_t>(1, hp.cb.size()) * sizeof(soft::CaseB),
-         b_st = std::max<size_t>(1, hp.sites.size()) * sizeof(soft::Site),
+         b_st = std::max<size_t>(1, hp.sites.size()) * (hp.W == 1 ? sizeof(soft::SiteDev<1>) : sizeof(soft::SiteDev<2>)),
          b_thr0 = hp.thr.size() * sizeof(uint64_t), b_thr1 = b_thr0 + hp.site_ev.size() * sizeof(uint32_t),
-         b_thr2 = b_thr1 + hp.thr_tab.size() * sizeof(uint32_t), b_thr = b_thr2 + hp.site_kind.size();
+         b_thr2 = b_thr1 + hp.thr_tab.size() * sizeof(uint32_t),
+         b_thr3 = b_thr2 + hp.sites.size() * sizeof(uint32_t), b_thr = b_thr3 + hp.site_kind.size();
+  std::vector<unsigned char> sites(hp.sites.size() * (hp.W == 1 ? sizeof(soft::SiteDev<1>) : sizeof(soft::SiteDev<2>)));
+  std::vector<uint32_t> thin(hp.sites.size());
+  for (size_t i = 0; i < hp.sites.size(); ++i) {
+    if (hp.W == 1) site_dev(hp.sites[i], reinterpret_cast<soft::SiteDev<1> *>(sites.data())[i]);
+    else site_dev(hp.sites[i], reinterpret_cast<soft::SiteDev<2> *>(sites.data())[i]);
+    thin[i] = hp.sites[i].thin;
+  }
   cudaError_t e;
   if ((e = cudaMalloc(&c->d_ev, b_ev)) != cudaSuccess || (e = cudaMalloc(&c->d_coef, b_cf)) != cudaSuccess ||
       (e = cudaMalloc(&c->d_cb, b_cb)) != cudaSuccess || (e = cudaMalloc(&c->d_sites, b_st)) != cudaSuccess ||
@@ -207,11 +233,12 @@ int soft_compile_circuit(const soft_op *ops, size_t n_ops, uint32_t n_qubits, co
   if ((e = up(c->d_ev, ev_src, b_ev)) != cudaSuccess ||
       (e = up(c->d_coef, hp.coefs.data(), hp.coefs.size() * sizeof(soft::Coef))) != cudaSuccess ||
       (e = up(c->d_cb, hp.cb.data(), hp.cb.size() * sizeof(soft::CaseB))) != cudaSuccess ||
-      (e = up(c->d_sites, hp.sites.data(), hp.sites.size() * sizeof(soft::Site))) != cudaSuccess ||
+      (e = up(c->d_sites, sites.data(), sites.size())) != cudaSuccess ||
       (e = up(c->d_thr, hp.thr.data(), b_thr0)) != cudaSuccess ||
       (e = up(thr_b + b_thr0, hp.site_ev.data(), hp.site_ev.size() * sizeof(uint32_t))) != cudaSuccess ||
       (e = up(thr_b + b_thr1, hp.thr_tab.data(), hp.thr_tab.size() * sizeof(uint32_t))) != cudaSuccess ||
-      (e = up(thr_b + b_thr2, hp.site_kind.data(), hp.site_kind.size())) != cudaSuccess ||
+      (e = up(thr_b + b_thr2, thin.data(), thin.size() * sizeof(uint32_t))) != cudaSuccess ||
+      (e = up(thr_b + b_thr3, hp.site_kind.data(), hp.site_kind.size())) != cudaSuccess ||
       (e = cudaStreamSynchronize(us)) != cudaSuccess) {
     cudaStreamDestroy(us);
     soft_circuit_free(c);
@@ -303,7 +330,8 @@ CircDev circ_desc(const soft_circuit *c, int fp32, bool prefix) {
   soft::CircDev d{};
   d.site_ev = reinterpret_cast<const uint32_t *>(c->d_thr + c->hp.thr.size());
   d.thr_tab = d.site_ev + c->hp.site_ev.size();
-  d.site_kind = reinterpret_cast<const uint8_t *>(d.thr_tab + c->hp.thr_tab.size());
+  d.site_thin = d.thr_tab + c->hp.thr_tab.size();
+  d.site_kind = reinterpret_cast<const uint8_t *>(d.site_thin + c->hp.sites.size());
   if (prefix && c->d_traj[fp32]) {
     d.traj = c->d_traj[fp32];
     d.traj_stop = c->traj_stop[fp32];

@@ -21,7 +21,7 @@ struct soft_circuit {
   void *d_ev = nullptr;  // Ev<W> array, W = hp.W
   soft::Coef *d_coef = nullptr;
   soft::CaseB *d_cb = nullptr;
-  soft::Site *d_sites = nullptr;
+  void *d_sites = nullptr;  // SiteDev<W> array
   uint64_t *d_thr = nullptr;
   uint64_t bytes = 0;
   // the noiseless run's snapshot table per precision (index 0 FP64, 1 FP32),

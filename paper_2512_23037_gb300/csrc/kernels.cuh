@@ -17,7 +17,7 @@ struct CircDev {
   const void *ev;  // Ev<W>
   const Coef *coef;
   const CaseB *cb;
-  const Site *sites;
+  const void *sites;  // SiteDev<W>
   const uint64_t *thr;
   uint32_t n_events, n_sites, rw, cap;  // cap: this circuit's coefficient cap
   uint32_t n_coef, n_cb;
@@ -35,6 +35,7 @@ struct CircDev {
   uint32_t traj_stop, traj_stride;
   uint32_t traj_fid_stop, pad_traj;  // first fidelity measurement's event (fidelity mode stops there)
   const uint32_t *site_ev;  // per site: the event that applies its error
+  const uint32_t *site_thin;
   const uint8_t *site_kind; // per site: its kind and kSiteThinned (program.h)
   const uint32_t *thr_tab;  // the gap search's index, 2^kThrTabBits + 1 entries (null: plain search)
 };

@@ -19,7 +19,7 @@
 //
 // Most shots end at the first detector after their first error, but a few run to
 // the end of the circuit, and they would hold a warp with a few active lanes. So a
-// warp left with at most kEvictBelow active lanes writes their shots' state to a
+// warp left with few active lanes (evict_below) writes their shots' state to a
 // spill pool and moves on to fresh shots. The next round (another launch) buckets
 // the evicted shots by the event they resume at, and packs them into warps again.
 // The last round evicts nothing. Which lane runs a shot does not change its
@@ -57,7 +57,12 @@ constexpr uint32_t kLaneMaxBuckets = 50000;  // the pre-pass histogram of all bu
 #ifndef SOFT_LANE_EVICT
 #define SOFT_LANE_EVICT 10
 #endif
-constexpr uint32_t kEvictBelow = SOFT_LANE_EVICT;  // a warp with this many active lanes or fewer evicts them
+#ifndef SOFT_LANE_EVICT_BIG
+#define SOFT_LANE_EVICT_BIG 12
+#endif
+// a warp with this many active lanes or fewer evicts them
+template <uint32_t Cap>
+__host__ __device__ constexpr uint32_t evict_below() { return Cap <= 16u ? SOFT_LANE_EVICT : SOFT_LANE_EVICT_BIG; }
 #ifndef SOFT_LANE_ROUNDS
 #define SOFT_LANE_ROUNDS 2
 #endif
@@ -1220,6 +1225,10 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
   // (read from the launch parameters where used, so that no register holds them through the
   // loop); a single circuit's, all of them
   if (Multi && P.al_hi <= P.al_lo) return;
+  // one bit per bucket: a warp of this block found it exhausted
+  uint32_t *empty = reinterpret_cast<uint32_t *>(smem + (size_t)(blockDim.x / 32) * lane_warp_bytes<R, W, Cap>(P.rw_max));
+  for (uint32_t k = threadIdx.x; k < (P.al_nb + 31u) / 32u; k += blockDim.x) empty[k] = 0u;
+  __syncthreads();
   // warps start spread evenly over the buckets, so that they meet buckets that still hold shots
   const unsigned long long gw = (unsigned long long)blockIdx.x * (blockDim.x / 32) + warp;
   const unsigned long long nw = (unsigned long long)gridDim.x * (blockDim.x / 32);
@@ -1239,9 +1248,8 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
   };
   bool active = false;
   uint32_t item = 0;
-  // the current bucket: its first record, the next bucket's, and its claims as last read (they
-  // only grow, so a bucket that looks empty is)
-  uint32_t b0 = __ldg(&P.al_start[g]), b1 = __ldg(&P.al_start[g + 1]), taken = *(volatile unsigned int *)&P.al_next[g];
+  // the current bucket: its first record and the next bucket's
+  uint32_t b0 = __ldg(&P.al_start[g]), b1 = __ldg(&P.al_start[g + 1]);
   const unsigned long long limit = (n_items + 2ull) * ((Multi ? P.al_hi - P.al_lo : P.al_nb) + 2ull) + 64ull;
   for (unsigned long long guard = 0; guard < limit; ++guard) {
     g = Multi ? C->bucket0 + e : e;
@@ -1266,7 +1274,12 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     // snapshot's copies are issued before the atomic answers: a lane that gets no shot has
     // only filled columns that nobody reads.
     const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
-    if (idle && taken < b1 - b0) {
+    bool claim = idle && b1 != b0 && !((*(volatile uint32_t *)&empty[g >> 5] >> (g & 31u)) & 1u);
+    if (claim && *(volatile unsigned int *)&P.al_next[g] >= b1 - b0) {  // once per block and bucket
+      if (lane == 0) atomicOr(&empty[g >> 5], 1u << (g & 31u));
+      claim = false;
+    }
+    if (claim) {
       uint32_t got0 = 0;
       const uint32_t leader = __ffs(idle) - 1;
       if (lane == leader) got0 = atomicAdd(&P.al_next[g], __popc(idle));
@@ -1297,11 +1310,8 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     if (e < n_ev && __any_sync(0xFFFFFFFFu, active && s.status == LS_RUN)) {
       if (active && s.status == LS_RUN) s.step(e, hdr, body, E);
     }
-    // the next bucket's bounds and claims, used when the warp walks on (their latency overlaps
-    // the end of this iteration)
-    const uint32_t nb_all = P.al_nb;
-    const uint32_t b2 = __ldg(&P.al_start[g + 2u < nb_all ? g + 2u : nb_all]);
-    const uint32_t taken1 = *(volatile unsigned int *)&P.al_next[g + 1u < nb_all ? g + 1u : g];
+    // the end of the next bucket, used when the warp walks on
+    const uint32_t b2 = __ldg(&P.al_start[g + 2u < P.al_nb ? g + 2u : P.al_nb]);
     // a spill record to write (a hand-over or an eviction), written once below
     uint32_t ev_r = 0xFFFFFFFFu, ev_e = 0;
     // finish: ended, or past the last event
@@ -1351,7 +1361,7 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     // the next round packed with others, and the warp moves on to fresh shots
     if (P.lane_evict) {
       const uint32_t am = __ballot_sync(0xFFFFFFFFu, active);
-      if (am && (uint32_t)__popc(am) <= kEvictBelow && e + 1u < n_ev) {
+      if (am && (uint32_t)__popc(am) <= evict_below<Cap>() && e + 1u < n_ev) {
         const uint32_t leader = __ffs(am) - 1;
         unsigned long long r0 = 0;
         if (lane == leader) r0 = atomicAdd(&P.lr[0], (unsigned long long)__popc(am));
@@ -1372,7 +1382,6 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
       if (en) {
         b0 = b1;
         b1 = b2;
-        taken = taken1;
       }
     } else {
       // all lanes idle: the next bucket of any circuit (cyclically) that still has shots, or
@@ -1411,7 +1420,6 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
       const uint32_t gn = Multi ? C->bucket0 + en : en;
       b0 = __ldg(&P.al_start[gn]);
       b1 = __ldg(&P.al_start[gn + 1]);
-      taken = *(volatile unsigned int *)&P.al_next[gn];
     }
     e = en;
   }
@@ -1513,7 +1521,7 @@ cudaError_t prepare_lanes(const ShotParams &p, int fp32, uint32_t W, int blocks_
                      : cap == kWideCap  ? lane_kernel_for<kWideCap>(fp32, W, multi)
                                         : lane_kernel_for<kLaneCap>(fp32, W, multi);
   if (!kern) return cudaErrorInvalidConfiguration;
-  const size_t smem = lane_smem_bytes(fp32, W, p.rw_max, cap);
+  const size_t smem = lane_smem_bytes(fp32, W, p.rw_max, cap) + (size_t)((p.al_nb + 31u) / 32u) * 4u;
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

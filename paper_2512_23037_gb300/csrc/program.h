@@ -107,7 +107,7 @@ struct alignas(16) CaseB {
 // kind: bits 0-1 = SITE_DEPOL1 (X, Y, Z uniform), SITE_DEPOL2 (15 Paulis
 // uniform) or SITE_FLIP (the one-qubit Pauli code in bits 2-3).
 // The draws read a byte per site instead (CircDev::site_kind): kind, and kSiteThinned where
-// the site's rate is below the circuit's largest (thin holds its acceptance threshold).
+// the site's rate is below the circuit's largest (site_thin: its acceptance threshold).
 enum : uint32_t { SITE_DEPOL1 = 0, SITE_DEPOL2 = 1, SITE_FLIP = 2 };
 constexpr uint32_t kSiteThinned = 16;
 struct alignas(16) Site {
@@ -115,6 +115,19 @@ struct alignas(16) Site {
   uint64_t bx[2][2], gx[2][2], bz[2][2], gz[2][2];
   uint32_t kind, thin, always, c0;
 };
+// The device's copy, W words per vector: the images X_q0, Z_q0, X_q1, Z_q1 (beta words, then
+// gamma words each), so that an error's image is a masked XOR of loads that wait for nothing.
+template <int W>
+struct alignas(16) SiteDev {
+  uint64_t img[4][2 * W];
+  uint64_t dsd[W], dss[W];
+  uint32_t kind, thin, always, c0;
+};
+// The images that the Pauli pair pa << 2 | pb multiplies (bit j: img[j]).
+SOFT_HD inline uint32_t site_images(uint32_t pp) {
+  const uint32_t pa = pp >> 2, pb = pp & 3u;
+  return ((pa == 1u || pa == 2u) ? 1u : 0u) | (pa >= 2u ? 2u : 0u) | ((pb == 1u || pb == 2u) ? 4u : 0u) | (pb >= 2u ? 8u : 0u);
+}
 
 // Lanes pack a site and its Pauli pair into one word; circuits of this many sites or more run
 // without them.

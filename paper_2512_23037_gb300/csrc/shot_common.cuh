@@ -51,7 +51,7 @@ __device__ __forceinline__ bool next_site(const CircDev *C, uint64_t seed, uint6
     uint32_t s = cur + lo;
     cur = s + 1u;
     const uint32_t kind = __ldg(&C->site_kind[s]);
-    if ((kind & kSiteThinned) && !(w.w < __ldg(&C->sites[s].thin))) continue;
+    if ((kind & kSiteThinned) && !(w.w < __ldg(&C->site_thin[s]))) continue;
     nxt = s;
     pp = (kind & 3u) == SITE_DEPOL2 ? __umulhi(w.z, 15u) + 1u
          : (kind & 3u) == SITE_FLIP ? kind & 12u
@@ -67,20 +67,29 @@ __device__ __forceinline__ bool next_site(const CircDev *C, uint64_t seed, uint6
 template <int W>
 __device__ __forceinline__ uint32_t site_pauli(const CircDev *C, uint32_t s, uint32_t pp, const uint64_t *sd,
                                                const uint64_t *ss, uint64_t *beta, uint64_t *gamma) {
-  const Site *S = C->sites + s;
-  const uint32_t pa = pp >> 2, pb = pp & 3u;
+  const SiteDev<W> *S = reinterpret_cast<const SiteDev<W> *>(C->sites) + s;
+  const uint32_t need = site_images(pp);
+#pragma unroll
+  for (int w = 0; w < W; ++w) beta[w] = gamma[w] = 0ull;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint64_t m = 0ull - (uint64_t)((need >> j) & 1u);
+    const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(S->img[j]);
+    const ulonglong2 x = __ldg(p);
+    if (W == 1) {
+      beta[0] ^= x.x & m;
+      gamma[0] ^= x.y & m;
+    } else {
+      const ulonglong2 y = __ldg(p + 1);
+      beta[0] ^= x.x & m;
+      beta[W - 1] ^= x.y & m;
+      gamma[0] ^= y.x & m;
+      gamma[W - 1] ^= y.y & m;
+    }
+  }
   uint64_t pe = 0;
 #pragma unroll
-  for (int w = 0; w < W; ++w) {
-    uint64_t b = 0, g = 0;
-    if (pa == 1u || pa == 2u) { b ^= __ldg(&S->bx[0][w]); g ^= __ldg(&S->gx[0][w]); }
-    if (pa == 3u || pa == 2u) { b ^= __ldg(&S->bz[0][w]); g ^= __ldg(&S->gz[0][w]); }
-    if (pb == 1u || pb == 2u) { b ^= __ldg(&S->bx[1][w]); g ^= __ldg(&S->gx[1][w]); }
-    if (pb == 3u || pb == 2u) { b ^= __ldg(&S->bz[1][w]); g ^= __ldg(&S->gz[1][w]); }
-    beta[w] = b;
-    gamma[w] = g;
-    pe ^= ((sd[w] ^ __ldg(&S->dsd[w])) & b) ^ ((ss[w] ^ __ldg(&S->dss[w])) & g);
-  }
+  for (int w = 0; w < W; ++w) pe ^= ((sd[w] ^ __ldg(&S->dsd[w])) & beta[w]) ^ ((ss[w] ^ __ldg(&S->dss[w])) & gamma[w]);
   return ((__ldg(&S->c0) >> (2u * pp)) + 2u * wordpar(pe)) & 3u;
 }
 
