@@ -370,21 +370,19 @@ struct GradWarp {
     sm_from_stage(m, 2 * n, [&](uint32_t i) { return norm2d(svals[i]) >= thr && norm2d(svals[i]) > 0.0; });
     return true;
   }
-  // <lambda| Z_q |phi> = sum_a conj(lambda_{a^beta}) xi_a phi_a
-  __device__ void zexp(const SMap<R, W> &lam, const SMap<R, W> &ph, const uint64_t *beta, const uint64_t *gamma,
-                       uint32_t e, double *re, double *im) {
-    double cr = 0.0, ci = 0.0;
+  // Im <lambda| Z_q |phi>, <lambda| Z_q |phi> = sum_a conj(lambda_{a^beta}) xi_a phi_a
+  __device__ double zexp(const SMap<R, W> &lam, const SMap<R, W> &ph, const uint64_t *beta, const uint64_t *gamma,
+                         uint32_t e) {
+    double ci = 0.0;
     for (uint32_t i = lane; i < ph.n; i += 32) {
       const Key<W> k = smk(ph, i);
       const int j = sfind(lam, kxor(k, beta));
       if (j < 0) continue;
       const Cx<R> xp = ipow(ph.v[i], e + 2u * kpar(k, gamma));
       const Cx<R> l = lam.v[j];
-      cr += (double)l.x * (double)xp.x + (double)l.y * (double)xp.y;
       ci += (double)l.x * (double)xp.y - (double)l.y * (double)xp.x;
     }
-    *re = wsum(cr);
-    *im = wsum(ci);
+    return wsum(ci);
   }
   __device__ void reset_sides(const SMap<R, W> &m, const uint64_t *gamma, uint32_t sgn, bool &h0, bool &h1) {
     bool a0 = false, a1 = false;
@@ -462,10 +460,32 @@ struct GradWarp {
     }
     t.sync();
   }
-  // drop |v|^2 < tau_rel |map|^2
+  // The larger exponent of re and im (0 for zero), in units of a factor of two.
+  __device__ __forceinline__ static uint32_t top_exp(Cx<double> v) {
+    const uint32_t x = (uint32_t)__double2hiint(v.x) & 0x7FFFFFFFu, y = (uint32_t)__double2hiint(v.y) & 0x7FFFFFFFu;
+    return (x > y ? x : y) >> 20;
+  }
+  __device__ __forceinline__ static uint32_t top_exp(Cx<float> v) {
+    const uint32_t x = __float_as_uint(v.x) & 0x7FFFFFFFu, y = __float_as_uint(v.y) & 0x7FFFFFFFu;
+    return (x > y ? x : y) >> 23;
+  }
+  // drop |v|^2 < tau_rel |map|^2. With E the map's largest exponent, at most 32 entries and
+  // both components below 2^(E + 1), |map|^2 lies in [4^E, 2^8 4^E]: an entry within kKeep
+  // exponents of E stays and one more than kDrop below it goes (tau_rel 1e-20 = 2^-66.4 in
+  // FP64, 1e-10 = 2^-33.2 in FP32). Only entries between compute the norms: the sum over the
+  // lanes alone took 5 FP64 additions of 76 cycles each after every rotation and projection.
+  static constexpr uint32_t kKeep = sizeof(R) == 8 ? 28u : 12u, kDrop = sizeof(R) == 8 ? 35u : 19u;
   __device__ void prune_rel(RMap<R, W> &m) {
+    const bool in = lane < m.n;
+    const uint32_t x = in ? top_exp(m.v) : 0u, E = __reduce_max_sync(0xFFFFFFFFu, x);
+    if (t.all(!in || x + kKeep >= E)) {
+      if (E > kDrop) return;  // (every entry stays; near zero the sums decide)
+    } else if (E > kDrop && t.all(!in || x + kKeep >= E || x + kDrop < E)) {
+      compact(m, in && x + kKeep >= E);
+      return;
+    }
     const double thr = P.tau_rel * norm2_map(m);
-    const bool keep = lane < m.n && norm2d(m.v) >= thr;
+    const bool keep = in && norm2d(m.v) >= thr;
     compact(m, keep);
   }
 
@@ -497,9 +517,23 @@ struct GradWarp {
     const bool has = valid && partner != 0u;
     const bool app = valid && !has;
     const Cx<R> src = has ? vj : m.v;
-    const Cx<R> tb = cmul(b, ipow(src, e + 2u * kpar(has ? pk : m.k, gamma)));
-    Cx<R> nv = cmul(a, m.v);
-    if (has) nv = cadd(nv, tb);
+    const Cx<R> y = ipow(src, e + 2u * kpar(has ? pk : m.k, gamma));
+    Cx<R> nv, tb;
+    if (a.y == (R)0 && b.x == (R)0) {  // an Rz: cos I - i sin Z (FP32 rounds as the products below)
+      const R by = b.y, nby = negr(b.y);
+      nv = cscale(m.v, a.x);
+      if (sizeof(R) == 8 && has) {
+        nv = Cx<R>{fmar(nby, y.y, nv.x), fmar(by, y.x, nv.y)};
+        tb = Cx<R>{0, 0};
+      } else {
+        tb = Cx<R>{mulr(nby, y.y), mulr(by, y.x)};
+        if (has) nv = cadd(nv, tb);
+      }
+    } else {
+      tb = cmul(b, y);
+      nv = cmul(a, m.v);
+      if (has) nv = cadd(nv, tb);
+    }
     const uint32_t ab = t.ballot(app);
     const uint32_t nA = __popc(ab);
     if (m.n + nA > 32u) return false;
@@ -789,15 +823,15 @@ struct GradWarp {
   }
   __device__ ErrRec<W> *errs() const { return reinterpret_cast<ErrRec<W> *>(tape + L.errs); }
 
-  // <lambda| Z_q |phi> for the ROT event (beta, gamma, e): sum_a conj(lambda_{a^beta}) xi_a phi_a
-  __device__ void zexp(const RMap<R, W> &lam, const RMap<R, W> &phi, const uint64_t *beta, const uint64_t *gamma,
-                       uint32_t e, double *re, double *im) {
+  // Im <lambda| Z_q |phi> for the ROT event (beta, gamma, e): sum_a conj(lambda_{a^beta}) xi_a phi_a
+  __device__ double zexp(const RMap<R, W> &lam, const RMap<R, W> &phi, const uint64_t *beta, const uint64_t *gamma,
+                         uint32_t e) {
     if (lane < lam.n) {
       skey_set(lane, lam.k);
       svals[lane] = lam.v;
     }
     t.sync();
-    double cr = 0.0, ci = 0.0;
+    double ci = 0.0;
     if (lane < phi.n) {
       const Key<W> target = kxor(phi.k, beta);
       const Cx<R> xp = ipow(phi.v, e + 2u * kpar(phi.k, gamma));  // xi_a phi_a
@@ -805,15 +839,97 @@ struct GradWarp {
         if (keq(skey(j), target)) {
           const Cx<R> l = svals[j];
           // conj(l) * xp
-          cr = (double)l.x * (double)xp.x + (double)l.y * (double)xp.y;
           ci = (double)l.x * (double)xp.y - (double)l.y * (double)xp.x;
           break;
         }
       }
     }
     t.sync();
-    *re = wsum(cr);
-    *im = wsum(ci);
+    return wsum(ci);
+  }
+
+  // lam -= f m, exact zeros dropped and the rest pruned; false if it needs more entries than a map
+  // holds
+  __device__ bool subtract(RMap<R, W> &lam, const RMap<R, W> &m, R f) {
+    if (lane < lam.n) {
+      skey_set(lane, lam.k);
+      svals[lane] = lam.v;
+    }
+    t.sync();
+    const Cx<R> d = lane < m.n ? Cx<R>{mulr(-f, m.v.x), mulr(-f, m.v.y)} : Cx<R>{0, 0};
+    bool app = lane < m.n;
+    for (uint32_t j = 0; j < lam.n; ++j)
+      if (app && keq(skey(j), m.k)) {
+        svals[j] = cadd(svals[j], d);
+        app = false;
+      }
+    const uint32_t b = t.ballot(app);
+    if (app) {  // (at most 64 staged entries)
+      skey_set(lam.n + lanes_below(b), m.k);
+      svals[lam.n + lanes_below(b)] = d;
+    }
+    t.sync();
+    const uint32_t n = lam.n + __popc(b);
+    const Key<W> k0 = skey(lane), k1 = skey(lane + 32);
+    const Cx<R> v0 = svals[lane], v1 = svals[lane + 32];
+    const bool in0 = lane < n && (v0.x != (R)0 || v0.y != (R)0), in1 = lane + 32 < n && (v1.x != (R)0 || v1.y != (R)0);
+    const uint32_t b0 = t.ballot(in0), b1 = t.ballot(in1);
+    if (__popc(b0) + __popc(b1) > 32) return false;
+    t.sync();
+    if (in0) {
+      skey_set(lanes_below(b0), k0);
+      svals[lanes_below(b0)] = v0;
+    }
+    if (in1) {
+      skey_set(__popc(b0) + lanes_below(b1), k1);
+      svals[__popc(b0) + lanes_below(b1)] = v1;
+    }
+    t.sync();
+    lam.n = __popc(b0) + __popc(b1);
+    if (lane < lam.n) {
+      lam.k = skey(lane);
+      lam.v = svals[lane];
+    }
+    t.sync();
+    if (lam.n) prune_rel(lam);
+    return true;
+  }
+  __device__ bool subtract(SMap<R, W> &lam, const SMap<R, W> &m, R f) {
+    for (uint32_t i = lane; i < lam.n; i += 32) {
+      skey2_set(i, smk(lam, i));
+      svals[i] = lam.v[i];
+    }
+    t.sync();
+    uint32_t n = lam.n;
+    for (uint32_t base = 0; base < m.n; base += 32) {
+      const uint32_t i = base + lane;
+      bool app = false;
+      Key<W> k;
+      Cx<R> d{0, 0};
+      if (i < m.n) {
+        k = smk(m, i);
+        d = Cx<R>{mulr(-f, m.v[i].x), mulr(-f, m.v[i].y)};
+        const int j = sfind(lam, k);
+        app = j < 0;
+        if (j >= 0) svals[j] = cadd(svals[j], d);
+      }
+      const uint32_t b = t.ballot(app);
+      if (app) {  // (at most 2 kWideCap staged entries)
+        skey2_set(n + lanes_below(b), k);
+        svals[n + lanes_below(b)] = d;
+      }
+      n += __popc(b);
+    }
+    t.sync();
+    uint32_t live = 0;
+    for (uint32_t base = 0; base < n; base += 32) {
+      const uint32_t i = base + lane;
+      live += __popc(t.ballot(i < n && (svals[i].x != (R)0 || svals[i].y != (R)0)));
+    }
+    if (live > kWideCap) return false;
+    sm_from_stage(lam, n, [&](uint32_t i) { return svals[i].x != (R)0 || svals[i].y != (R)0; });
+    if (lam.n) prune_rel(lam);
+    return true;
   }
 
   // ------------------------------------------------------------- one pattern
@@ -829,8 +945,6 @@ struct GradWarp {
       for (uint32_t w = lane; w < (P.n_events + 63) / 64; w += 32) bits[w] = 0ull;
     }
     double *grad = P.grad + off * P.n_params;
-    for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] = 0.0;
-    t.sync();
     fwd_init();
     cur = 0;
     kblk = 0;
@@ -849,10 +963,31 @@ struct GradWarp {
       if (!(n_acc > 0.0)) status = G_ZERO;
       else F = n_fid / n_acc;
     }
-    if (status == G_OK && n_fid > 0.0) {  // N_fid = 0: F = 0 and dF/dtheta = 0 exactly
-      // sweep 1: N_fid from the end; sweep 2: N_acc from just before the first fidelity measurement
-      if (!sweep(phi, P.n_events, r, grad, 1.0)) status = kCapFail;
-      if (status == G_OK && !sweep(pre, ev_f, rot_before_f, grad, -F)) status = kCapFail;
+    for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] = 0.0;
+    t.sync();
+    // N_fid = 0: F = 0 and dF/dtheta = 0 exactly; no fidelity measurement: F = 1 at any angles
+    const bool swept = status == G_OK && n_fid > 0.0 && seen_f;
+    if (swept) {
+      // dF = (dN_fid - F dN_acc) / N_acc. The sweep of N_fid starts at the end with phi; at the
+      // first fidelity measurement the one of N_acc joins it, linear in the adjoint state:
+      // lambda - F pre goes on as one sweep. Most kept patterns have F = 1 there with lambda =
+      // pre, and are done (w42rz, 10^5 patterns in FP64: 8.1 -> 2.6 ms, with the norms of
+      // prune_rel left out). Should the joined map need more entries than there are, the two
+      // sweeps run one after the other (mode 1, 2).
+      for (int mode = 0;;) {
+        const bool ok = sweep(mode == 2 ? pre : phi, mode == 2 ? ev_f : P.n_events, mode == 2 ? rot_before_f : r, grad,
+                              mode == 2 ? -F : 1.0, mode == 0 ? ev_f : 0xFFFFFFFFu, (R)F);
+        if (mode == 0 && !ok) {
+          t.sync();
+          for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] = 0.0;
+          t.sync();
+          mode = 1;
+          continue;
+        }
+        if (!ok) status = kCapFail;
+        if (mode != 1 || !ok) break;
+        mode = 2;
+      }
       t.sync();
       for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] /= n_acc;
     }
@@ -873,7 +1008,7 @@ struct GradWarp {
         atomicAdd(&P.sums[2], 1.0);
       }
     }
-    if (status != G_OK)
+    if (status != G_OK && swept)
       for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] = 0.0;
     t.sync();
   }
@@ -1178,8 +1313,10 @@ struct GradWarp {
 
   // Reverse sweep from just before event `ev_end` (its errors included): the
   // adjoint starts as `lam` (the state there) and every parameterised rotation
-  // adds weight * s * Im <lambda| Z_q |phi> to grad[k].
-  __device__ bool sweep(const Map &src, uint32_t ev_end, uint32_t r_end, double *grad, double weight) {
+  // adds weight * s * Im <lambda| Z_q |phi> to grad[k]. Before event ev_join (0xFFFFFFFF: none)
+  // the adjoint becomes lambda - f pre. False if a map would need more entries than there are.
+  __device__ bool sweep(const Map &src, uint32_t ev_end, uint32_t r_end, double *grad, double weight, uint32_t ev_join,
+                        R f) {
     Map lam_local{};
     Map &lam = Wide ? lam_store : lam_local;  // registers, or the warp's shared-memory map
     copy_map(lam, src);
@@ -1210,8 +1347,7 @@ struct GradWarp {
             Map phk_local{};
             Map &phk = Wide ? phk_store : phk_local;
             tape_load_phi(r, phk);
-            double zr, zi;
-            zexp(lam, phk, beta, gamma, e, &zr, &zi);
+            const double zi = zexp(lam, phk, beta, gamma, e);
             const double s = (hdr.w & 1u) ? -1.0 : 1.0;
             if (lane == 0) grad[hdr.w >> 1] += weight * s * zi;
           }
@@ -1274,6 +1410,10 @@ struct GradWarp {
         } else if (type == EV_PAULI) {
           if (tape_bit(ev)) pauli_adj(lam, beta, gamma, (ev_e0(w0) + 2u * pe(beta, gamma)) & 3u);
         }
+      }
+      if (ev == ev_join) {
+        if (!subtract(lam, pre, f)) return false;
+        if (lam.n == 0u) return true;
       }
       // errors applied before this event, newest first
       while (ei >= 0 && errs()[ei].ev == ev) {
