@@ -73,7 +73,7 @@ template <typename R, int W>
 struct AffShot {
   // the products that share a phase take it folded into b, or apply it per entry, as in
   // kernels.cu (Shot::kFoldPhase), so that both kernels round alike
-  static constexpr bool kFoldPhase = sizeof(R) == 8 || W == 1;
+  [[maybe_unused]] static constexpr bool kFoldPhase = sizeof(R) == 8 || W == 1;
   const ShotParams &P;
   const CircDev *C = nullptr;
   const uint32_t lane;
@@ -94,7 +94,7 @@ struct AffShot {
   typename std::conditional<kScaled, ScaledPrune, PruneTest<R>>::type pt;  // |v|^2 < tau
 
   __device__ AffShot(const ShotParams &p, unsigned char *base)
-      : P(p), lane(threadIdx.x & 31u), v(reinterpret_cast<Cx<R> *>(base)), ring(base + (sizeof(Cx<R>) << p.aff_dim)), pt(p.tau) {}
+      : P(p), lane(threadIdx.x & 31u), v(reinterpret_cast<Cx<R> *>(base)), ring(base + (sizeof(Cx<R>) << p.aff_dim)), pt(p.prune) {}
   // x, or zero where it is below tau
   __device__ __forceinline__ Cx<R> pruned(Cx<R> x) const {
     bool sm;
@@ -119,12 +119,9 @@ struct AffShot {
     return __ballot_sync(kAll, in);
   }
   __device__ __forceinline__ static bool wnonzero(const uint64_t *x) { return (x[0] | x[W - 1]) != 0ull; }
-  __device__ __forceinline__ static uint32_t wlow(const uint64_t *x) {
-    return x[0] ? (uint32_t)(__ffsll((long long)x[0]) - 1) : 64u + (uint32_t)(__ffsll((long long)x[W - 1]) - 1);
-  }
   // the vector z with z . B[k] = 0 for every k and z . r = 1, for a residual r
   __device__ __forceinline__ void co_dual(const uint64_t *r, uint64_t *z) const {
-    const uint32_t p = wlow(r);
+    const uint32_t p = wlow<W>(r);
     const bool in = wbit<W>(B, p) != 0u;
 #pragma unroll
     for (int w = 0; w < W; ++w)

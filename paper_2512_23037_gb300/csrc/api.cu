@@ -28,6 +28,7 @@ int cuda_fail(cudaError_t e, const char *what) {
 
 constexpr uint64_t kDefaultChunk = 1ull << 24;
 using soft::kDefaultFirstCap;
+constexpr uint64_t kSmallRun = 32768;  // shots of a chunk up to which evicted shots go to the warp pass
 constexpr uint32_t kAffDim = 8;  // directions of the affine warp passes' maps (256 values per warp)
 using soft::kTauFp32;
 using soft::kTauFp64;
@@ -50,8 +51,10 @@ struct soft_run {
   unsigned char *d_spb[2] = {nullptr, nullptr};       // the same of the 32- and 64-entry lanes
   unsigned long long *d_lrb[2] = {nullptr, nullptr};
   bool fid_mode = false;
-  unsigned long long *d_work = nullptr;    // next1, next2, n_rerun, item_base, diag[4], reruns of all chunks,
-                                           // middle pass: next, n_rerun
+  unsigned long long *d_once = nullptr;    // d_tally, d_work and d_fsum
+  unsigned long long *d_work = nullptr;    // [3] item_base, [4..7] diag, [8] reruns of all chunks
+  unsigned long long *d_chunk = nullptr;   // per chunk: next1, next2, n_rerun, middle pass's next and n_rerun;
+                                           // from [8] the lane rounds' ranges, then the bucket counters
   uint32_t *d_rerun = nullptr;
   unsigned char *d_slab = nullptr;         // global-memory state for large-cap reruns
   uint8_t *d_status = nullptr;             // circuit 0 only
@@ -142,7 +145,7 @@ static cudaError_t build_prefixes(soft_circuit *c, cudaStream_t us) {
     d.n_cb = (uint32_t)hp.cb.size();
     p.cap = std::min(hp.cap, soft::kDefaultFirstCap);
     p.rw_max = hp.rw;
-    p.tau = fp32 ? kTauFp32 : kTauFp64;
+    p.prune = soft::prune_bounds(fp32 ? kTauFp32 : kTauFp64);
     e = soft::launch_prefix(p, fp32, hp.W, c->d_traj[fp32], d_stop + 4 * fp32, ps[fp32]);
     if (e == cudaSuccess)
       e = soft::launch_snap_affine(c->d_traj[fp32], (uint32_t)n_snap, hp.rw, fp32, hp.W, d_stop + 4 * fp32, c->d_ev,
@@ -468,20 +471,31 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     pieces.push_back(Piece{reinterpret_cast<void **>(ptr), bytes});
     arena_bytes += (bytes + 255) & ~(size_t)255;
   };
-  need(&r->d_tally, 5 * n_circ * sizeof(unsigned long long));
+  // cleared once: tallies, fidelity sums, run counters (d_work)
+  const size_t n_lr = 4 + 2 * ((size_t)(lanes ? soft::lane_rounds() : 1u) + 1);
+  const size_t once_words = 5 * (size_t)n_circ + (fid_mode ? n_circ : 0) + 11;
+  need(&r->d_once, once_words * sizeof(unsigned long long));
+  // cleared for every chunk: the chunk's counters and round ranges (of each lane size), then the
+  // bucket counters
+  const size_t chunk_words = 8 + 3 * n_lr;
+  need(&r->d_chunk, chunk_words * sizeof(unsigned long long) + 2 * (size_t)nb * sizeof(uint32_t));
   // lanes: cursors (4 words per item, 16-byte aligned), the cursors in bucket order, (start
   // event, rank) pairs, bucket starts, counters, then the per-block bucket bases of the
   // block-binned pre-pass
-  const uint32_t al_grid = lanes ? soft::lane_prepass_grid() : 0u;
-  if (lanes)
-    need(&r->d_al, (10 * chunk + (nb + 1) + 2 * (size_t)nb + (size_t)al_grid * (nb + 1)) * sizeof(uint32_t));
+  const uint32_t al_grid = lanes ? soft::lane_prepass_grid(std::min(chunk, total)) : 0u;
+  if (lanes) need(&r->d_al, (10 * chunk + (nb + 1) + (size_t)al_grid * (nb + 1)) * sizeof(uint32_t));
   // spill pool: records for the shots a sparse warp evicts (a quarter of the chunk; when it is
   // full, warps keep their shots), then records for shots a lane hands to a warp (an eighth;
   // when full, the warp reruns them from their start). Entries of the rerun list name a record
   // with their top bit, so a chunk stays below 2^31 items for it.
   const uint32_t rounds = lanes ? soft::lane_rounds() : 1u;
+  // few shots: a second round would walk the events with a few warps, each step as slow as a
+  // single lane's loops; the warp pass takes the evicted shots instead (w42 FP32, 4099 shots:
+  // 1.2 -> 0.3 ms)
+  const bool small_run = lanes && affine && !(o.flags & SOFT_RUN_WIDE_LANES) && std::min(chunk, total) <= kSmallRun;
+  const uint64_t evict_want = small_run ? std::min(chunk, total) : std::max<uint64_t>(std::min<uint64_t>(chunk, 1024), chunk / 4);
+  const uint32_t sp_evict = rounds > 1 ? (uint32_t)evict_want : 0u;
   const bool spill = lanes16 && (rounds > 1 || lane_grow) && chunk < (1ull << 31);
-  const uint32_t sp_evict = rounds > 1 ? (uint32_t)std::max<uint64_t>(std::min<uint64_t>(chunk, 1024), chunk / 4) : 0u;
   const uint32_t sp_hand = lane_grow ? (uint32_t)std::max<uint64_t>(std::min<uint64_t>(chunk, 1024), chunk / 8) : 0u;
   // the wide round: the handed-over shots continue in lanes of twice the map (their records
   // are its input), and only those that outgrow it rerun in a warp. Single-circuit runs only
@@ -491,11 +505,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   // FP32 550.0 M against 533.0 M (sparse lanes); FP64 348.2 M against 344.5 M (affine lanes).
   const bool wide_ok = spill && lane_grow && n_circ == 1 && !(o.flags & SOFT_RUN_NO_WIDE_LANES);
   const bool wide = wide_ok && ((o.flags & SOFT_RUN_WIDE_LANES) || std::min(chunk, total) >= (1ull << 23));
-  const size_t n_lr = 4 + 2 * ((size_t)rounds + 1);
-  if (spill) {
-    need(&r->d_sp, soft::lane_spill_bytes(fp32, W, rw_max, sp_evict + sp_hand, soft::lane_map_dim()));
-    need(&r->d_lr, n_lr * sizeof(unsigned long long));
-  }
+  if (spill) need(&r->d_sp, soft::lane_spill_bytes(fp32, W, rw_max, sp_evict + sp_hand, soft::lane_map_dim()));
   // the larger lanes' eviction pools: a quarter of their circuits' shots, at most 2^22 records
   // (a record of a 64-entry lane takes about 0.8 KB)
   uint32_t sp_big[2] = {0, 0};
@@ -504,14 +514,11 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     for (uint32_t i = 0; i < n_circ; ++i)
       if (lcap[i] && lane_class(lcap[i]) == 1 + k) n += n_shots[i];
     n = std::min(n, chunk);
-    if (!nbc[1 + k] || n == 0) continue;
+    if (!nbc[1 + k] || n == 0 || small_run) continue;
     sp_big[k] = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(std::min<uint64_t>(n, 1024), n / 4), 1ull << 22);
     need(&r->d_spb[k], soft::lane_spill_bytes(fp32, W, rw_max, sp_big[k], soft::lane_map_dim() + 1 + k));
-    need(&r->d_lrb[k], n_lr * sizeof(unsigned long long));
   }
   r->fid_mode = fid_mode;
-  if (fid_mode) need(&r->d_fsum, n_circ * sizeof(double));
-  need(&r->d_work, 11 * sizeof(unsigned long long));
   if (two_pass) need(&r->d_rerun, (mid_pass ? 2 : 1) * chunk * sizeof(uint32_t));
   uint32_t slab_blocks = 0;
   if (global_rerun) {
@@ -565,9 +572,12 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     soft_run_free(r);
     return cuda_fail(e, "cudaEventCreate");
   }
-  if ((e = cudaMemsetAsync(r->d_tally, 0, 5 * n_circ * sizeof(unsigned long long), st)) != cudaSuccess ||
-      (e = cudaMemsetAsync(r->d_work, 0, 11 * sizeof(unsigned long long), st)) != cudaSuccess ||
-      (fid_mode && (e = cudaMemsetAsync(r->d_fsum, 0, n_circ * sizeof(double), st)) != cudaSuccess)) {
+  r->d_tally = r->d_once;
+  r->d_work = r->d_tally + 5 * n_circ;
+  if (fid_mode) r->d_fsum = reinterpret_cast<double *>(r->d_work + 11);
+  if (spill) r->d_lr = r->d_chunk + 8;
+  for (int k = 0; k < 2; ++k) r->d_lrb[k] = r->d_chunk + 8 + (k + 1) * n_lr;
+  if ((e = cudaMemsetAsync(r->d_once, 0, once_words * sizeof(unsigned long long), st)) != cudaSuccess) {
     soft_run_free(r);
     return cuda_fail(e, "cudaMemsetAsync");
   }
@@ -604,12 +614,12 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   p.circ[0].records = r->d_records;
   p.circ[0].out_limit = r->out_limit;
   p.rw_max = rw_max;
-  p.tau = fp32 ? kTauFp32 : kTauFp64;
+  p.prune = soft::prune_bounds(fp32 ? kTauFp32 : kTauFp64);
   p.seed = seed;
-  p.next_item = r->d_work;
+  p.next_item = r->d_chunk;
   p.rerun = r->d_rerun;
   p.rerun_cap = two_pass ? (uint32_t)chunk : 0u;
-  p.n_rerun = r->d_work + 2;
+  p.n_rerun = r->d_chunk + 2;
   p.diag = r->d_work + 4;
   p.n_rerun_total = r->d_work + 8;
   p.groups_per_block = o.groups_per_block;
@@ -630,17 +640,17 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   q.hs_max = soft::hash_slots_for(cap_max);
   q.small_pass = 0;
   q.list = r->d_rerun;
-  q.n_items_dev = r->d_work + 2;
-  q.next_item = r->d_work + 1;
+  q.n_items_dev = r->d_chunk + 2;
+  q.next_item = r->d_chunk + 1;
   q.n_rerun_total = nullptr;
   soft::ShotParams m = q;  // middle pass: first list in, second list out
   if (mid_pass) {
     m.cap = cap1;
     m.hs_max = soft::hash_slots_for(cap1);
     m.small_pass = 1;
-    m.next_item = r->d_work + 9;
+    m.next_item = r->d_chunk + 3;
     m.rerun = r->d_rerun + chunk;
-    m.n_rerun = r->d_work + 10;
+    m.n_rerun = r->d_chunk + 4;
     q.list = m.rerun;
     q.n_items_dev = m.n_rerun;
   }
@@ -654,15 +664,16 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     p.al_rec = p.al_order = r->d_al + 4 * chunk;
     p.al_ev = r->d_al + 8 * chunk;
     p.al_start = r->d_al + 10 * chunk;
-    p.al_count = r->d_al + 10 * chunk + (nb + 1);
+    p.al_count = reinterpret_cast<unsigned int *>(r->d_chunk + chunk_words);
     p.al_next = p.al_count + nb;
-    p.al_base = p.al_next + nb;
+    p.al_base = r->d_al + 10 * chunk + (nb + 1);
     p.al_nb = nb;
     p.al_lo = 0;  // the 16-entry lanes' buckets; the larger lanes' launches set their own
     p.al_hi = (uint32_t)nbc[0];
     p.al_grid = al_grid;
     p.lane_round = 0;
     p.lane_evict = spill && rounds > 1 ? 1u : 0u;
+    p.lane_list = small_run ? 1u : 0u;
     p.lane_hand = spill ? 1u : 0u;
     p.lane_wide = wide ? 1u : 0u;
     p.lane_wide_round = 0;
@@ -688,7 +699,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     pb[k].al_lo = (uint32_t)(nbc[0] + (k ? nbc[1] : 0));
     pb[k].al_hi = pb[k].al_lo + (uint32_t)nbc[1 + k];
     pb[k].lane_hand = pb[k].lane_wide = 0;
-    pb[k].lane_evict = sp_big[k] ? 1u : 0u;
+    pb[k].lane_evict = sp_big[k] || small_run ? 1u : 0u;
     pb[k].sp = r->d_spb[k];
     pb[k].sp_cap = pb[k].sp_evict_cap = sp_big[k];
     pb[k].sp_dim = soft::lane_map_dim() + 1 + k;
@@ -726,8 +737,8 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   };
   auto enqueue_chunk = [&](uint64_t base, uint64_t cnt, bool dev_base) -> cudaError_t {
     cudaError_t err;
-    if ((err = cudaMemsetAsync(r->d_work, 0, 3 * sizeof(unsigned long long), st)) != cudaSuccess) return err;
-    if (mid_pass && (err = cudaMemsetAsync(r->d_work + 9, 0, 2 * sizeof(unsigned long long), st)) != cudaSuccess)
+    if ((err = cudaMemsetAsync(r->d_chunk, 0, chunk_words * sizeof(unsigned long long) + 2 * (size_t)nb * sizeof(uint32_t),
+                               st)) != cudaSuccess)
       return err;
     soft::ShotParams a = p, b = q, c = m;
     a.n_items = b.n_items = c.n_items = cnt;
@@ -735,14 +746,10 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     if (dev_base) a.item_base_dev = b.item_base_dev = c.item_base_dev = r->d_work + 3;
     if ((err = mark()) != cudaSuccess) return err;
     if (lanes) {
-      if ((err = cudaMemsetAsync(a.al_count, 0, 2 * (size_t)nb * sizeof(uint32_t), st)) != cudaSuccess ||
-          (err = soft::launch_lane_prepass(a, st)) != cudaSuccess)
-        return err;
-      r->launches += 3;
+      if ((err = soft::launch_lane_prepass(a, st)) != cudaSuccess) return err;
+      r->launches += al_grid > 1 ? 3 : 1;
     }
     if ((err = mark(lanes)) != cudaSuccess) return err;
-    if (spill && (err = cudaMemsetAsync(r->d_lr, 0, n_lr * sizeof(unsigned long long), st)) != cudaSuccess)
-      return err;
     if (!lanes || lanes16) {
       if ((err = soft::launch_prepared(c1, a, st)) != cudaSuccess) return err;
       r->launches++;
@@ -754,13 +761,11 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
         ab.n_items = cnt;
         ab.item_base = base;
         if (dev_base) ab.item_base_dev = r->d_work + 3;
-        if (sp_big[k] && (err = cudaMemsetAsync(r->d_lrb[k], 0, n_lr * sizeof(unsigned long long), st)) != cudaSuccess)
-          return err;
         if ((err = soft::launch_prepared(cb[k], ab, st)) != cudaSuccess) return err;
         r->launches++;
       }
     // later rounds: the evicted shots, bucketed by the event they resume at
-    for (uint32_t rd = 1; spill && rd < rounds; ++rd) {
+    for (uint32_t rd = 1; spill && !small_run && rd < rounds; ++rd) {
       soft::ShotParams ar = a;
       ar.lane_round = rd;
       ar.lane_evict = rd + 1 < rounds ? 1u : 0u;
@@ -769,7 +774,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
           (err = soft::launch_lane_resume_prepass(ar, fp32, W, st)) != cudaSuccess ||
           (err = soft::launch_prepared(c1, ar, st)) != cudaSuccess)
         return err;
-      r->launches += 5;
+      r->launches += al_grid > 1 ? 5 : 2;
     }
     for (int k = 0; lanes && k < 2; ++k)
       if (sp_big[k]) {
@@ -783,7 +788,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
             (err = soft::launch_lane_resume_prepass(ar, fp32, W, st)) != cudaSuccess ||
             (err = soft::launch_prepared(cb[k], ar, st)) != cudaSuccess)
           return err;
-        r->launches += 5;
+        r->launches += al_grid > 1 ? 5 : 2;
       }
     if (wide) {  // the handed-over shots, bucketed by the event they resume at
       soft::ShotParams aw = a;
@@ -797,7 +802,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
           (err = soft::launch_lane_resume_prepass(aw, fp32, W, st)) != cudaSuccess ||
           (err = soft::launch_prepared(cw, aw, st)) != cudaSuccess)
         return err;
-      r->launches += 5;
+      r->launches += al_grid > 1 ? 5 : 2;
     }
     if ((err = mark()) != cudaSuccess) return err;
     if (mid_pass) {

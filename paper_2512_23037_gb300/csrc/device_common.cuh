@@ -5,6 +5,8 @@
 
 #include <cstdint>
 
+#include "kernels.cuh"
+
 namespace soft {
 namespace dev {
 
@@ -82,12 +84,7 @@ template <typename R>
 struct PruneTest {
   R tau;
   uint32_t lo = 0, hi = 0;  // high words of the two bounds above (FP64)
-  __device__ explicit PruneTest(double t) : tau((R)t) {
-    if (sizeof(R) == 8) {
-      lo = (uint32_t)((unsigned long long)__double_as_longlong(sqrt(0.5 * t) * (1.0 - 0x1p-18)) >> 32);
-      hi = (uint32_t)((unsigned long long)__double_as_longlong(sqrt(t) * (1.0 + 0x1p-18)) >> 32);
-    }
-  }
+  __device__ explicit PruneTest(const PruneBounds &b) : tau((R)b.tau), lo(b.lo), hi(b.hi) {}
   __device__ __forceinline__ bool small(Cx<R> v) const {
     if (sizeof(R) == 4) return norm2(v) < tau;
     const uint32_t hx = (uint32_t)((unsigned long long)__double_as_longlong((double)v.x) >> 32) & 0x7FFFFFFFu;
@@ -135,8 +132,7 @@ struct ScaledPrune {
   double tau;
   float klo, khi;
   uint32_t lo = 0, hi = 0;
-  __device__ explicit ScaledPrune(double t)
-      : tau(t), klo((float)(sqrt(0.5 * t) * (1.0 - 0x1p-16))), khi((float)(sqrt(t) * (1.0 + 0x1p-16))) {}
+  __device__ explicit ScaledPrune(const PruneBounds &b) : tau(b.tau), klo(b.klo), khi(b.khi) {}
   __device__ __forceinline__ void set(double N) {  // N in range
     const float n = low_float(N), r = n * rsqrtf(n);
     lo = (__float_as_uint(klo * r) >> 3) + (896u << 20);
@@ -255,6 +251,14 @@ __device__ __forceinline__ uint32_t wpar2(const uint64_t *a, const uint64_t *b, 
 template <int W>
 __device__ __forceinline__ uint32_t wbit(const uint64_t *a, uint32_t i) {
   return (uint32_t)((word_of<W>(a, i) >> (i & 63)) & 1ull);
+}
+// The lowest set bit of a nonzero W-word vector. (Written with a reversal and a leading-zero
+// count: nvcc 13.0 compiled __ffsll of a residual from a warp reduction in affine.cu to a
+// wrong value, -1 for 8, which the random-circuit tests caught.)
+template <int W>
+__device__ __forceinline__ uint32_t wlow(const uint64_t *x) {
+  const bool first = W == 1 || x[0] != 0ull;
+  return (first ? 0u : 64u) + (uint32_t)__clzll((long long)__brevll(first ? x[0] : x[W - 1]));
 }
 template <int W>
 __device__ __forceinline__ void wflip(uint64_t *a, uint32_t i) {

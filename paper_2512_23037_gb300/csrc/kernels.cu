@@ -17,6 +17,9 @@
 //              (Eq. Pi_pm, Theorem 1 (2)); probabilities in FP64.
 #include <cooperative_groups.h>
 
+#include <cmath>
+#include <cstring>
+
 #include "device_common.cuh"
 #include "shot_common.cuh"
 #include "kernels.cuh"
@@ -94,7 +97,7 @@ struct Shot {
   static constexpr bool kFoldPhase = sizeof(R) == 8 || W == 1;
   PruneTest<R> pt;  // |v|^2 < tau (thresholds computed once per thread)
 
-  __device__ Shot(const Tile &tile, const ShotParams &p, unsigned char *base) : t(tile), P(p), pt(p.tau) {
+  __device__ Shot(const Tile &tile, const ShotParams &p, unsigned char *base) : t(tile), P(p), pt(p.prune) {
     cap = P.cap;
     slots = 2 * cap;
     hsmax = P.hs_max;
@@ -417,7 +420,7 @@ struct Shot {
     const R sc = inv_sqrt_as<R>(m == 1 ? sp : sm);
     bool keep = valid && (neg == (m == -1));
     if (keep) rv = cscale(rv, sc);
-    reg_compact(keep && norm2(rv) >= (R)P.tau);
+    reg_compact(keep && norm2(rv) >= (R)P.prune.tau);
     return m;
   }
 
@@ -446,7 +449,7 @@ struct Shot {
       rv = cscale(m == 1 ? cadd(v0, x1) : csub(v0, x1), sc);
       rk = a0;
     }
-    reg_compact(owner && norm2(rv) >= (R)P.tau);
+    reg_compact(owner && norm2(rv) >= (R)P.prune.tau);
     return m;
   }
 
@@ -613,7 +616,7 @@ struct Shot {
     const int m = pick(ord, sp, sm);
     const R sc = inv_sqrt_as<R>(m == 1 ? sp : sm);
     const uint32_t want = (m == 1) ? 0u : 1u;
-    const R tau = (R)P.tau;
+    const R tau = (R)P.prune.tau;
     t.sync();
     nnz = compact(0, nnz, [&](Key<W> &k, Cx<R> &v) {
       if ((kpar(k, gamma) ^ sgn) != want) return false;
@@ -722,7 +725,7 @@ struct Shot {
       vals[cap + i] = nv;
     }
     t.sync();
-    const R tau = (R)P.tau;
+    const R tau = (R)P.prune.tau;
     nnz = compact(cap, nnz, [&](Key<W> &, Cx<R> &v) { return norm2(v) >= tau; });
     rebuild();
     return m;
@@ -1226,6 +1229,16 @@ cudaError_t prepare_t(const ShotParams &p, int blocks_per_sm, LaunchCfg *cfg) {
 }
 
 }  // namespace
+
+PruneBounds prune_bounds(double tau) {
+  auto high = [](double x) {
+    uint64_t u;
+    std::memcpy(&u, &x, sizeof u);
+    return (uint32_t)(u >> 32);
+  };
+  return PruneBounds{tau, high(std::sqrt(0.5 * tau) * (1.0 - 0x1p-18)), high(std::sqrt(tau) * (1.0 + 0x1p-18)),
+                     (float)(std::sqrt(0.5 * tau) * (1.0 - 0x1p-16)), (float)(std::sqrt(tau) * (1.0 + 0x1p-16))};
+}
 
 cudaError_t launch_advance(unsigned long long *item_base, unsigned long long step, cudaStream_t stream) {
   advance_kernel<<<1, 1, 0, stream>>>(item_base, step);

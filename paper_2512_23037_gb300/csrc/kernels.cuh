@@ -40,12 +40,21 @@ struct CircDev {
   const uint32_t *thr_tab;  // the gap search's index, 2^kThrTabBits + 1 entries (null: plain search)
 };
 
+// The bounds of the pruning test |v|^2 < tau (PruneTest and ScaledPrune in device_common.cuh),
+// computed on the host: their square roots cost each thread 2 us at the start of a launch.
+struct PruneBounds {
+  double tau;
+  uint32_t lo, hi;  // high words of sqrt(tau / 2) (1 - 2^-18) and sqrt(tau) (1 + 2^-18)
+  float klo, khi;   // sqrt(tau / 2) (1 - 2^-16) and sqrt(tau) (1 + 2^-16)
+};
+PruneBounds prune_bounds(double tau);
+
 struct ShotParams {
   uint32_t n_circ;
   uint32_t cap;     // capacity of the on-chip map of this launch (first pass: small)
   uint32_t rw_max;  // record words reserved per group
   uint32_t hs_max;  // hash slots per group: power of two >= 4 * cap
-  double tau;
+  PruneBounds prune;
   uint64_t seed;
   // work: global items item_base + [0, n_items) or item_base + list[0 .. n_items)
   uint64_t item_base, n_items;
@@ -91,6 +100,8 @@ struct ShotParams {
   // pool; the next round buckets them by the event they resume at and packs them into warps
   uint32_t lane_round;        // 0: shots from their start buckets; r >= 1: shots evicted before round r
   uint32_t lane_evict;        // 1: this round may evict
+  uint32_t lane_list;         // 1: evicted shots go on the rerun list for the warp pass (with their
+                              // record, or to start again where the lanes keep none)
   uint32_t lane_hand;         // 1: a lane whose map would outgrow it hands the shot over (a spill record)
   uint32_t lane_wide;         // 1: a wide round takes the handed-over shots (records stay off the rerun list)
   uint32_t lane_wide_round;   // 1: this is the wide round (its records: the handed-over ones)
@@ -142,7 +153,9 @@ cudaError_t launch_lane_resume_prepass(const ShotParams &p, int fp32, uint32_t W
 size_t lane_spill_bytes(int fp32, uint32_t W, uint32_t rw, uint32_t cap, uint32_t dim);
 uint32_t lane_rounds();
 uint32_t lane_max_buckets();  // lane-per-shot runs hold at most this many buckets (events + 1 per circuit)
-uint32_t lane_prepass_grid();  // blocks of the bucketing pre-pass (al_base holds this many rows)
+// blocks of the bucketing pre-pass of up to `items` items (al_base holds this many rows); 1: one
+// block does all of it in one launch
+uint32_t lane_prepass_grid(uint64_t items);
 // cap: the lane map's entries: lane_map_cap() for the first rounds, twice that for the wide
 // round, or lane_first_cap()'s answer for circuits of larger maps
 cudaError_t prepare_lanes(const ShotParams &p, int fp32, uint32_t W, int blocks_per_sm, LaunchCfg *cfg,

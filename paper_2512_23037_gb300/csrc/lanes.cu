@@ -34,6 +34,7 @@
 // a batch of 64 circuits (7.7 M shots) 31.7 -> 16.6 ms.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -102,8 +103,9 @@ template <>
 struct SlotSet<64> {
   using T = unsigned long long;
 };
+// (of a nonempty set)
 __device__ __forceinline__ uint32_t mffs(uint32_t m) { return (uint32_t)__ffs(m); }
-__device__ __forceinline__ uint32_t mffs(unsigned long long m) { return (uint32_t)__ffsll((long long)m); }
+__device__ __forceinline__ uint32_t mffs(unsigned long long m) { return 1u + (uint32_t)__clzll((long long)__brevll(m)); }
 __device__ __forceinline__ uint32_t mpopc(uint32_t m) { return (uint32_t)__popc(m); }
 __device__ __forceinline__ uint32_t mpopc(unsigned long long m) { return (uint32_t)__popcll(m); }
 
@@ -155,12 +157,6 @@ __device__ __forceinline__ bool wnonzero(const uint64_t *x) {
   for (int w = 0; w < W; ++w) o |= x[w];
   return o != 0ull;
 }
-// The lowest set bit of a nonzero W-word vector.
-template <int W>
-__device__ __forceinline__ uint32_t wlow(const uint64_t *x) {
-  return x[0] ? (uint32_t)(__ffsll((long long)x[0]) - 1) : 64u + (uint32_t)(__ffsll((long long)x[W - 1]) - 1);
-}
-
 template <typename R, int W, uint32_t Cap>
 struct LaneShot {
   static constexpr uint32_t kDim = lane_dim(Cap);
@@ -187,7 +183,7 @@ struct LaneShot {
 
   typename std::conditional<kScaled, ScaledPrune, PruneTest<R>>::type pt;  // |v|^2 < tau
 
-  __device__ LaneShot(const ShotParams &p, unsigned char *base) : P(p), C(&p.circ[0]), nrm(1.0), pt(p.tau) {
+  __device__ LaneShot(const ShotParams &p, unsigned char *base) : P(p), C(&p.circ[0]), nrm(1.0), pt(p.prune) {
     lane = threadIdx.x & 31u;
     const size_t vb = (size_t)Cap * sizeof(Cx<R>) * 32, rb = (size_t)(1 + 2 * kDim) * W * 8 * 32;
     vals = reinterpret_cast<Cx<R> *>(base);
@@ -1084,33 +1080,38 @@ __device__ __forceinline__ uint32_t circ_of_bucket(const ShotParams &P, uint32_t
   }
   return lo;
 }
-__global__ void lane_scan_kernel(const __grid_constant__ ShotParams P) {
-  __shared__ uint32_t part[1024];
-  const uint32_t nb = P.al_nb, tid = threadIdx.x, nt = blockDim.x;
+// Exclusive scan of the bucket sizes by one block of 1024 threads: each thread sums a contiguous
+// range, the warps scan their sums by shuffles (a serial pass over 1024 partial sums took 7 us).
+__device__ void scan_buckets(const ShotParams &P) {
+  __shared__ uint32_t part[32];
+  const uint32_t nb = P.al_nb, tid = threadIdx.x, nt = blockDim.x, ln = tid & 31u;
   const uint32_t per = (nb + nt - 1) / nt, lo = tid * per < nb ? tid * per : nb, hi = lo + per < nb ? lo + per : nb;
   uint32_t sum = 0;
   for (uint32_t k = lo; k < hi; ++k) sum += P.al_count[k];
-  part[tid] = sum;
-  __syncthreads();
-  if (tid == 0) {
-    uint32_t run = 0;
-    for (uint32_t k = 0; k < nt; ++k) {
-      const uint32_t v = part[k];
-      part[k] = run;
-      run += v;
+  auto scan = [&](uint32_t v) {  // inclusive, over the warp
+#pragma unroll
+    for (uint32_t off = 1; off < 32; off <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, v, off);
+      if (ln >= off) v += u;
     }
-    P.al_start[nb] = run;
-  }
+    return v;
+  };
+  const uint32_t inc = scan(sum);
+  if (ln == 31u) part[tid / 32] = inc;
   __syncthreads();
-  uint32_t run = part[tid];
+  if (tid < 32) part[tid] = scan(tid < nt / 32 ? part[tid] : 0u);
+  __syncthreads();
+  uint32_t run = inc - sum + (tid >= 32 ? part[tid / 32 - 1] : 0u);
+  if (tid == nt - 1) P.al_start[nb] = run + sum;
   for (uint32_t k = lo; k < hi; ++k) {
     P.al_start[k] = run;
     run += P.al_count[k];
   }
 }
+__global__ void __launch_bounds__(1024) lane_scan_kernel(const __grid_constant__ ShotParams P) { scan_buckets(P); }
 // ---- round r >= 1: its records are those taken since round r - 1 began (the pool's
 // count, capped at its capacity: reservations past it were not written)
-__global__ void lane_round_setup_kernel(const __grid_constant__ ShotParams P) {
+__device__ __forceinline__ void round_setup(const ShotParams &P) {
   const uint32_t r = P.lane_round;
   if (P.lane_wide_round) {  // the wide round: the handed-over shots' records
     const unsigned long long cap = P.sp_cap - P.sp_evict_cap;
@@ -1123,6 +1124,7 @@ __global__ void lane_round_setup_kernel(const __grid_constant__ ShotParams P) {
   P.lr[2 + 2 * r] = first;
   P.lr[3 + 2 * r] = used > first ? used - first : 0ull;
 }
+__global__ void lane_round_setup_kernel(const __grid_constant__ ShotParams P) { round_setup(P); }
 // ---- block-binned pre-pass: each block ranks its contiguous range of items per
 // bucket with shared-memory atomics, then takes one global atomic per non-empty
 // bucket for its base. The first errors cluster in a few buckets, and global
@@ -1130,8 +1132,7 @@ __global__ void lane_round_setup_kernel(const __grid_constant__ ShotParams P) {
 // Items of circuits whose maps outgrow a lane go to the warp pass's list instead: the
 // block ranks them too and reserves their slots with one global atomic.
 template <bool Resume, typename R, int W>
-__global__ void __launch_bounds__(256) lane_bin_kernel(const __grid_constant__ ShotParams P) {
-  extern __shared__ uint32_t hist[];  // nb buckets, then the block's count of warp-pass items
+__device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
   const uint32_t nb = P.al_nb;
   for (uint32_t k = threadIdx.x; k <= nb; k += blockDim.x) hist[k] = 0u;
   __syncthreads();
@@ -1176,9 +1177,14 @@ __global__ void __launch_bounds__(256) lane_bin_kernel(const __grid_constant__ S
   if (threadIdx.x == 0)
     P.al_base[(size_t)blockIdx.x * (nb + 1) + nb] = hist[nb] ? (uint32_t)atomicAdd(P.n_rerun, (unsigned long long)hist[nb]) : 0u;
 }
+template <bool Resume, typename R, int W>
+__global__ void __launch_bounds__(256) lane_bin_kernel(const __grid_constant__ ShotParams P) {
+  extern __shared__ uint32_t hist[];  // nb buckets, then the block's count of warp-pass items
+  bin_items<Resume, R, W>(P, hist);
+}
 // (same grid as lane_bin_kernel: it fixes each item's block)
 template <bool Resume>
-__global__ void __launch_bounds__(256) lane_bin_scatter_kernel(const __grid_constant__ ShotParams P) {
+__device__ __forceinline__ void scatter_items(const ShotParams &P) {
   const uint32_t nb = P.al_nb;
   const unsigned long long n_items =
       Resume ? P.lr[3 + 2 * P.lane_round] : (P.n_items_dev ? *P.n_items_dev : P.n_items);
@@ -1195,6 +1201,26 @@ __global__ void __launch_bounds__(256) lane_bin_scatter_kernel(const __grid_cons
     if (Resume) P.al_order[at] = (uint32_t)i;
     else reinterpret_cast<uint4 *>(P.al_rec)[at] = reinterpret_cast<const uint4 *>(P.al_cursor)[i];
   }
+}
+
+template <bool Resume>
+__global__ void __launch_bounds__(256) lane_bin_scatter_kernel(const __grid_constant__ ShotParams P) {
+  scatter_items<Resume>(P);
+}
+// The whole pre-pass in one block, for few items: a launch instead of three (four with the
+// round's setup), which cost more than the work (6-qubit circuit, 4096 shots: 18 + 17 us).
+template <bool Resume, typename R, int W>
+__global__ void __launch_bounds__(1024, 1) lane_bin_one_kernel(const __grid_constant__ ShotParams P) {
+  extern __shared__ uint32_t hist[];
+  if (Resume) {
+    if (threadIdx.x == 0) round_setup(P);
+    __syncthreads();
+  }
+  bin_items<Resume, R, W>(P, hist);
+  __syncthreads();
+  scan_buckets(P);
+  __syncthreads();
+  scatter_items<Resume>(P);
 }
 
 // Register budget: resident blocks per SM the compiler must allow. FP32 16-slot lanes: 8
@@ -1364,15 +1390,23 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
       if (am && (uint32_t)__popc(am) <= evict_below<Cap>() && e + 1u < n_ev) {
         const uint32_t leader = __ffs(am) - 1;
         unsigned long long r0 = 0;
-        if (lane == leader) r0 = atomicAdd(&P.lr[0], (unsigned long long)__popc(am));
+        if (lane == leader) r0 = atomicAdd(P.sp ? &P.lr[0] : P.n_rerun, (unsigned long long)__popc(am));
         r0 = __shfl_sync(0xFFFFFFFFu, r0, leader);
         if (active) {
           const unsigned long long r = r0 + __popc(am & ((1u << lane) - 1u));
-          if (r < P.sp_evict_cap) {
+          if (!P.sp) {  // (only with lane_list) no records: the warp pass runs them from their start
+            if (r < P.rerun_cap) P.rerun[r] = item;
+            active = false;
+          } else if (r < P.sp_evict_cap) {
             ev_r = (uint32_t)r;
             ev_e = e + 1u;
             active = false;
+            if (P.lane_list) {
+              const unsigned long long i = atomicAdd(P.n_rerun, 1ull);
+              if (i < P.rerun_cap) P.rerun[i] = kSpillRef | (uint32_t)r;
+            }
           }
+          if (!active && P.lane_list && P.n_rerun_total) atomicAdd(P.n_rerun_total, 1ull);
         }
       }
     }
@@ -1463,11 +1497,12 @@ cudaError_t launch_snap_affine(unsigned char *traj, uint32_t n_snap, uint32_t rw
 }
 uint32_t lane_rounds() { return kLaneRounds; }
 uint32_t lane_max_buckets() { return kLaneMaxBuckets; }
-uint32_t lane_prepass_grid() {
+uint32_t lane_prepass_grid(uint64_t items) {
+  if (items <= 8192) return 1;
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return (uint32_t)(sms > 0 ? sms : 1) * 8u;
+  return (uint32_t)std::min<uint64_t>((uint64_t)(sms > 0 ? sms : 1) * 8u, (items + 255) / 256);
 }
 
 size_t lane_spill_bytes(int fp32, uint32_t W, uint32_t rw, uint32_t cap, uint32_t dim) {
@@ -1480,9 +1515,14 @@ template <bool Resume, typename R, int W>
 static cudaError_t launch_bin(const ShotParams &p, cudaStream_t st) {
   const size_t sh = ((size_t)p.al_nb + 1) * sizeof(uint32_t);
   if (sh > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(lane_bin_kernel<Resume, R, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    const void *kern = p.al_grid == 1 ? reinterpret_cast<const void *>(lane_bin_one_kernel<Resume, R, W>)
+                                      : reinterpret_cast<const void *>(lane_bin_kernel<Resume, R, W>);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
     if (e != cudaSuccess) return e;
+  }
+  if (p.al_grid == 1) {
+    lane_bin_one_kernel<Resume, R, W><<<1, 1024, sh, st>>>(p);
+    return cudaGetLastError();
   }
   lane_bin_kernel<Resume, R, W><<<p.al_grid, 256, sh, st>>>(p);
   lane_scan_kernel<<<1, 1024, 0, st>>>(p);
@@ -1491,7 +1531,7 @@ static cudaError_t launch_bin(const ShotParams &p, cudaStream_t st) {
 }
 
 cudaError_t launch_lane_resume_prepass(const ShotParams &p, int fp32, uint32_t W, cudaStream_t st) {
-  lane_round_setup_kernel<<<1, 1, 0, st>>>(p);
+  if (p.al_grid > 1) lane_round_setup_kernel<<<1, 1, 0, st>>>(p);
   if (fp32) return W == 1 ? launch_bin<true, float, 1>(p, st) : launch_bin<true, float, 2>(p, st);
   return W == 1 ? launch_bin<true, double, 1>(p, st) : launch_bin<true, double, 2>(p, st);
 }

@@ -81,7 +81,7 @@ extern "C" int soft_run_shots_noalloc(soft_circuit *c, uint64_t n_shots, uint64_
   d.records = d_records;
   d.out_limit = (d_status || d_records) ? n_shots : 0;
   p.rw_max = hp.rw;
-  p.tau = fp32 ? soft::kTauFp32 : soft::kTauFp64;
+  p.prune = soft::prune_bounds(fp32 ? soft::kTauFp32 : soft::kTauFp64);
   p.seed = seed;
   p.n_items = n_shots;
   p.next_item = work;
