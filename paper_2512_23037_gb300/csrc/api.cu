@@ -28,7 +28,11 @@ int cuda_fail(cudaError_t e, const char *what) {
 
 constexpr uint64_t kDefaultChunk = 1ull << 24;
 using soft::kDefaultFirstCap;
-constexpr uint64_t kSmallRun = 32768;  // shots of a chunk up to which evicted shots go to the warp pass
+// Shots of a chunk up to which evicted shots go to the warp pass instead of a second lane round.
+// Both ways, in ms: w42 FP32 65 k shots 0.66 / 1.59, 262 k 1.08 / 1.35, 400 k 1.59 / 1.57, 700 k
+// 2.14 / 1.79; w97 FP32 130 k 2.55 / 3.17, 400 k 5.44 / 4.93; random 40-qubit circuit 130 k 1.05 /
+// 1.25, 400 k 2.50 / 2.71.
+constexpr uint64_t kSmallRun = 5ull << 16;
 constexpr uint32_t kAffDim = 8;  // directions of the affine warp passes' maps (256 values per warp)
 using soft::kTauFp32;
 using soft::kTauFp64;

@@ -102,8 +102,18 @@ GateTab make_tab(L2 iXa, L2 iZa, L2 iXb, L2 iZb) {
 
 struct Tabs {
   GateTab g[8];
+  L2 back[8][4];  // U^dag Q U for Q = X_a, Z_a, X_b, Z_b
   Tabs() {
     const L2 Xa{1, 0, 0}, Za{0, 1, 0}, Xb{2, 0, 0}, Zb{0, 2, 0};
+    const L2 inv[8][4] = {{Za, Xa, Xb, Zb},                       // H
+                          {L2{1, 1, 3}, Za, Xb, Zb},              // S: X -> -Y backwards
+                          {L2{1, 1, 1}, Za, Xb, Zb},              // S^dag: X -> Y backwards
+                          {Xa, L2{0, 1, 2}, Xb, Zb},              // X
+                          {L2{1, 0, 2}, L2{0, 1, 2}, Xb, Zb},     // Y
+                          {L2{1, 0, 2}, Za, Xb, Zb},              // Z
+                          {L2{3, 0, 0}, Za, Xb, L2{0, 3, 0}},     // CX
+                          {L2{1, 2, 0}, Za, L2{2, 1, 0}, Zb}};    // CZ
+    std::memcpy(back, inv, sizeof back);
     g[SOFT_H] = make_tab(Za, Xa, Xb, Zb);
     g[SOFT_S] = make_tab(L2{1, 1, 1}, Za, Xb, Zb);       // X -> Y
     g[SOFT_S_DAG] = make_tab(L2{1, 1, 3}, Za, Xb, Zb);   // X -> -Y
@@ -119,49 +129,222 @@ const Tabs &tabs() {
   return t;
 }
 
+// 64 x 64 bit matrix, transposed in place (exchanging blocks of 32, 16, ... 1 bits).
+void transpose64(uint64_t a[64]) {
+  uint64_t m = 0x00000000FFFFFFFFull;
+  for (uint32_t j = 32; j; j >>= 1, m ^= m << j)
+    for (uint32_t k = 0; k < 64; k = (k + j + 1) & ~j) {
+      const uint64_t t = ((a[k] >> j) ^ a[k + j]) & m;
+      a[k] ^= t << j;
+      a[k + j] ^= t;
+    }
+}
+
 struct Tableau {
   uint32_t n = 0;
-  std::vector<Row> d, s;
+  // The tableau by columns (per qubit: bit i of xd is row d_i's X bit there): a gate is a few
+  // word operations. Rows are taken from them where products of rows are needed.
+  struct Col {
+    uint64_t xd[2] = {0, 0}, zd[2] = {0, 0}, xs[2] = {0, 0}, zs[2] = {0, 0};
+  };
+  std::vector<Col> col;
+  mutable std::vector<Row> d, s;
+  mutable bool rows_ok = false;
   uint64_t pend_d[2] = {0, 0}, pend_s[2] = {0, 0};  // sign XOR since the last event
+  // X_q and Z_q as i^e d_beta s_gamma, kept through the Clifford gates: with the rows' signs
+  // of the gates so far (all_d, all_s) a gate changes only its own qubits' images, to products
+  // of them. A noise site takes its images from here; decomposing over the rows for each site
+  // was most of the compile time, and
+  // the rows' updates by gates most of the rest (soft_compile_circuit: w42 3.1 -> 1.0 ms,
+  // w97 22.4 -> 3.1 ms; the same programs byte for byte).
+  struct Image {
+    uint64_t b[2] = {0, 0}, g[2] = {0, 0};
+    uint32_t e = 0;
+  };
+  std::vector<Image> ix, iz;
+  uint64_t all_d[2] = {0, 0}, all_s[2] = {0, 0};
+
+  static Image times(const Image &p, const Image &q) {
+    Image o;
+    o.e = (p.e + q.e + 2u * (uint32_t)(pc(p.g[0] & q.b[0]) + pc(p.g[1] & q.b[1]))) & 3u;
+    for (int w = 0; w < 2; ++w) {
+      o.b[w] = p.b[w] ^ q.b[w];
+      o.g[w] = p.g[w] ^ q.g[w];
+    }
+    return o;
+  }
+  uint32_t gate_signs(const Image &i) const {
+    return (uint32_t)(pc(all_d[0] & i.b[0]) + pc(all_d[1] & i.b[1]) + pc(all_s[0] & i.g[0]) + pc(all_s[1] & i.g[1]));
+  }
+  void gate_images(int op, uint32_t a, uint32_t b, bool two) {
+    const L2 *to = tabs().back[op];
+    const Image xa = ix[a], za = iz[a], xb = two ? ix[b] : Image{}, zb = two ? iz[b] : Image{};
+    auto image = [&](const L2 &l) {
+      Image o;
+      o.e = (uint32_t)l.e & 3u;
+      if (l.x & 1u) o = times(o, xa);
+      if (l.x & 2u) o = times(o, xb);
+      if (l.z & 1u) o = times(o, za);
+      if (l.z & 2u) o = times(o, zb);
+      return o;
+    };
+    ix[a] = image(to[0]);
+    iz[a] = image(to[1]);
+    if (two) {
+      ix[b] = image(to[2]);
+      iz[b] = image(to[3]);
+    }
+  }
+  // X_q (code 1), Y_q = i X_q Z_q (2) or Z_q (3) at zero signs
+  void image(int code, uint32_t q, uint64_t beta[2], uint64_t gamma[2], uint32_t *e0) const {
+    Image i = code == 3 ? iz[q] : ix[q];
+    if (code == 2) {
+      i = times(i, iz[q]);
+      i.e += 1u;
+    }
+    for (int w = 0; w < 2; ++w) {
+      beta[w] = i.b[w];
+      gamma[w] = i.g[w];
+    }
+    *e0 = (i.e + 2u * gate_signs(i)) & 3u;
+  }
+
+  // any i^e X^x Z^z at zero signs
+  void image(const Pz &p, uint64_t beta[2], uint64_t gamma[2], uint32_t *e0) const {
+    Image o;
+    for (uint32_t q = 0; q < n; ++q)
+      if (bit(p.x, q)) o = times(o, ix[q]);
+    for (uint32_t q = 0; q < n; ++q)
+      if (bit(p.z, q)) o = times(o, iz[q]);
+    for (int w = 0; w < 2; ++w) {
+      beta[w] = o.b[w];
+      gamma[w] = o.g[w];
+    }
+    *e0 = (o.e + (uint32_t)p.e + 2u * gate_signs(o)) & 3u;
+  }
 
   void init(uint32_t nq) {
     n = nq;
+    ix.assign(n, Image{});
+    iz.assign(n, Image{});
+    for (uint32_t q = 0; q < n; ++q) {
+      flip(ix[q].b, q);
+      flip(iz[q].g, q);
+    }
+    col.assign(n, Col{});
+    for (uint32_t i = 0; i < n; ++i) {
+      flip(col[i].xd, i);
+      flip(col[i].zs, i);
+    }
+    rows_ok = false;
+  }
+  // one part of the rows (X or Z words of d or s) from the columns', or back
+  template <typename Get, typename Set>
+  static void transpose(uint32_t rows_in, uint32_t rows_out, Get get, Set set) {
+    for (uint32_t ob = 0; ob < rows_out; ob += 64)
+      for (uint32_t ib = 0; ib < rows_in; ib += 64) {
+        uint64_t m[64];
+        for (uint32_t k = 0; k < 64; ++k) m[k] = ib + k < rows_in ? get(ib + k, ob >> 6) : 0ull;
+        transpose64(m);
+        for (uint32_t k = 0; k < 64 && ob + k < rows_out; ++k) set(ob + k, ib >> 6, m[k]);
+      }
+  }
+  void rows() const {
+    if (rows_ok) return;
     d.assign(n, Row{});
     s.assign(n, Row{});
-    for (uint32_t i = 0; i < n; ++i) {
-      flip(d[i].x, i);
-      flip(s[i].z, i);
+    transpose(n, n, [&](uint32_t q, uint32_t w) { return col[q].xd[w]; }, [&](uint32_t i, uint32_t w, uint64_t v) { d[i].x[w] = v; });
+    transpose(n, n, [&](uint32_t q, uint32_t w) { return col[q].zd[w]; }, [&](uint32_t i, uint32_t w, uint64_t v) { d[i].z[w] = v; });
+    transpose(n, n, [&](uint32_t q, uint32_t w) { return col[q].xs[w]; }, [&](uint32_t i, uint32_t w, uint64_t v) { s[i].x[w] = v; });
+    transpose(n, n, [&](uint32_t q, uint32_t w) { return col[q].zs[w]; }, [&](uint32_t i, uint32_t w, uint64_t v) { s[i].z[w] = v; });
+    rows_ok = true;
+  }
+  // the columns of changed rows
+  void rows_changed() {
+    transpose(n, n, [&](uint32_t i, uint32_t w) { return d[i].x[w]; }, [&](uint32_t q, uint32_t w, uint64_t v) { col[q].xd[w] = v; });
+    transpose(n, n, [&](uint32_t i, uint32_t w) { return d[i].z[w]; }, [&](uint32_t q, uint32_t w, uint64_t v) { col[q].zd[w] = v; });
+    transpose(n, n, [&](uint32_t i, uint32_t w) { return s[i].x[w]; }, [&](uint32_t q, uint32_t w, uint64_t v) { col[q].xs[w] = v; });
+    transpose(n, n, [&](uint32_t i, uint32_t w) { return s[i].z[w]; }, [&](uint32_t q, uint32_t w, uint64_t v) { col[q].zs[w] = v; });
+  }
+  // The images after a case-B measurement of P. The row operations (s_j = +-s'_j s_p for j in J,
+  // d_p = +-d'_p prod d_J) keep d's and s's apart; then s_p becomes d''_p, d'_j (j in G)
+  // +-d''_j d''_p, and d'_p = i^-e0b P s_gamma2 with P = +-s''_p.
+  void case_b_images(const CaseB &B) {
+    const uint32_t p = B.p;
+    auto without_p = [&](uint64_t v[2]) { v[p >> 6] &= ~(1ull << (p & 63)); };
+    auto par = [](const uint64_t *a, const uint64_t *b) { return (uint32_t)(pc(a[0] & b[0]) + pc(a[1] & b[1])); };
+    Image dp, sp;  // d'_p and s_p in the new rows
+    flip(sp.b, p);
+    for (int w = 0; w < 2; ++w) dp.g[w] = B.gamma2[w];
+    without_p(dp.g);
+    flip(dp.g, p);
+    dp.e = (4u - (B.e0b & 3u) + 2u * B.rP) & 3u;
+    if (bit(B.gamma2, p)) dp = times(dp, sp);
+    for (uint32_t q = 0; q < 2 * n; ++q) {
+      Image &im = q < n ? ix[q] : iz[q - n];
+      uint32_t e = im.e + 2u * gate_signs(im);  // at zero signs
+      uint64_t b[2] = {im.b[0], im.b[1]}, g[2] = {im.g[0], im.g[1]};
+      const bool bp = bit(b, p) != 0;
+      if (bp) {
+        for (int w = 0; w < 2; ++w) b[w] ^= B.J[w];
+        e += 2u * B.hdp;
+      }
+      e += 2u * par(g, B.Hs);
+      if (par(g, B.J) & 1u) flip(g, p);
+      const bool gp = bit(g, p) != 0;
+      Image o, sg;
+      for (int w = 0; w < 2; ++w) {
+        o.b[w] = b[w];
+        sg.g[w] = g[w];
+      }
+      without_p(o.b);
+      without_p(sg.g);
+      e += 2u * par(o.b, B.Hd);
+      if (par(o.b, B.G) & 1u) flip(o.b, p);
+      o.e = e & 3u;
+      if (bp) o = times(o, dp);
+      o = times(o, sg);
+      if (gp) o = times(o, sp);
+      o.e = (o.e + 2u * gate_signs(o)) & 3u;
+      im = o;
     }
   }
 
-  // (bits replaced and sign flips applied without data-dependent branches)
-  static int apply_row(const GateTab &t, Row &r, uint32_t a, uint32_t b, bool two) {
-    const uint32_t wa = a >> 6, sa = a & 63, wb = b >> 6, sb = b & 63;
-    uint32_t in = (uint32_t)((r.x[wa] >> sa) & 1u) | ((uint32_t)((r.z[wa] >> sa) & 1u) << 1);
-    if (two) in |= ((uint32_t)((r.x[wb] >> sb) & 1u) << 2) | ((uint32_t)((r.z[wb] >> sb) & 1u) << 3);
-    const uint64_t o = t.out[in];
-    r.x[wa] = (r.x[wa] & ~(1ull << sa)) | ((o & 1u) << sa);
-    r.z[wa] = (r.z[wa] & ~(1ull << sa)) | (((o >> 1) & 1u) << sa);
-    if (two) {
-      r.x[wb] = (r.x[wb] & ~(1ull << sb)) | (((o >> 2) & 1u) << sb);
-      r.z[wb] = (r.z[wb] & ~(1ull << sb)) | (((o >> 3) & 1u) << sb);
-    }
-    return t.flipb[in];
-  }
-
-  // false if a row met an odd phase (impossible for a valid tableau; the compile stops)
-  bool gate(int op, uint32_t a, uint32_t b) {
+  // Rows by rows of the table: which inputs flip the sign, and the (linear) outputs, as word
+  // operations on the qubits' columns.
+  void gate(int op, uint32_t a, uint32_t b) {
     const GateTab &t = tabs().g[op];
     const bool two = (op == SOFT_CX || op == SOFT_CZ);
-    int bad = 0;
-    for (uint32_t i = 0; i < n; ++i) {
-      const int fd = apply_row(t, d[i], a, b, two);
-      const int fs = apply_row(t, s[i], a, b, two);
-      bad |= fd | fs;
-      pend_d[i >> 6] ^= (uint64_t)(fd & 1) << (i & 63);
-      pend_s[i >> 6] ^= (uint64_t)(fs & 1) << (i & 63);
-    }
-    return !(bad & 0x80);
+    rows_ok = false;
+    const uint32_t nw = (n + 63u) / 64u;
+    auto part = [&](uint64_t *xa, uint64_t *za, uint64_t *xb, uint64_t *zb, uint64_t *pend, uint64_t *all) {
+      for (uint32_t w = 0; w < nw; ++w) {
+        const uint64_t v[4] = {xa[w], za[w], two ? xb[w] : 0ull, two ? zb[w] : 0ull};
+        uint64_t f = 0;
+        for (uint32_t in = 1; in < (two ? 16u : 4u); ++in)
+          if (t.flipb[in] & 1u) {
+            uint64_t m = ~0ull;
+            for (uint32_t k = 0; k < (two ? 4u : 2u); ++k) m &= ((in >> k) & 1u) ? v[k] : ~v[k];
+            f |= m;
+          }
+        uint64_t o[4] = {0, 0, 0, 0};
+        for (uint32_t k = 0; k < (two ? 4u : 2u); ++k)
+          for (uint32_t j = 0; j < 4; ++j)
+            if ((t.out[1u << k] >> j) & 1u) o[j] ^= v[k];
+        xa[w] = o[0];
+        za[w] = o[1];
+        if (two) {
+          xb[w] = o[2];
+          zb[w] = o[3];
+        }
+        pend[w] ^= f;
+        all[w] ^= f;
+      }
+    };
+    Col &ca = col[a], &cb = col[two ? b : a];
+    part(ca.xd, ca.zd, cb.xd, cb.zd, pend_d, all_d);
+    part(ca.xs, ca.zs, cb.xs, cb.zs, pend_s, all_s);
+    gate_images(op, a, b, two);
   }
 
   // Q = i^e0 d_beta s_gamma at zero signs. NW: the 64-bit words in use. Bits are set
@@ -200,6 +383,7 @@ struct Tableau {
     return true;
   }
   bool decompose(const Pz &q, uint64_t beta[2], uint64_t gamma[2], uint32_t *e0) const {
+    rows();
     return n <= 64 ? decompose_w<1>(q, beta, gamma, e0) : decompose_w<2>(q, beta, gamma, e0);
   }
 };
@@ -219,8 +403,9 @@ bool is1q(int op) {
 bool is2q(int op) { return op == SOFT_CX || op == SOFT_CZ; }
 bool isclifford(int op) { return op <= SOFT_CZ; }
 
-uint64_t gap_thr(double p, uint64_t g) {
-  double q = -std::expm1((double)(g + 1) * std::log1p(-p));
+// log_q: log1p(-p)
+uint64_t gap_thr(double log_q, uint64_t g) {
+  double q = -std::expm1((double)(g + 1) * log_q);
   if (!(q > 0.0)) return 0;
   if (q >= 1.0) return UINT64_MAX;
   double t = std::ldexp(q, 64);
@@ -314,48 +499,36 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
     uint32_t ex[2] = {0, 0}, ez[2] = {0, 0};
     for (int k = 0; k < (two ? 2 : 1); ++k) {
       uint32_t q = k == 0 ? q0 : q1;
-      if (!tb.decompose(single(1, q), s.bx[k], s.gx[k], &ex[k])) return false;
-      if (!tb.decompose(single(3, q), s.bz[k], s.gz[k], &ez[k])) return false;
+      tb.image(1, q, s.bx[k], s.gx[k], &ex[k]);
+      tb.image(3, q, s.bz[k], s.gz[k], &ez[k]);
     }
     // Phases of the other Paulis by composition. With P = i^a d_b s_c and
     // Q = i^a' d_b' s_c', PQ = i^(a + a' + 2 |c & b'|) d_(b^b') s_(c^c'): s_j
     // anticommutes with d_j only, and the d's (and the s's) commute and square to I.
-    auto comp = [&](uint32_t a, const uint64_t *c, const uint64_t *b2, uint32_t a2) {
-      return (a + a2 + 2u * (uint32_t)(pc(c[0] & b2[0]) + pc(c[1] & b2[1]))) & 3u;
-    };
-    struct One {
-      uint64_t b[2], g[2];
-      uint32_t e;
-    };
-    auto one = [&](int code, int k) -> One {  // 1 X, 2 Y = i X Z, 3 Z on site qubit k
-      One o{};
-      if (code == 1) o = One{{s.bx[k][0], s.bx[k][1]}, {s.gx[k][0], s.gx[k][1]}, ex[k]};
-      else if (code == 3) o = One{{s.bz[k][0], s.bz[k][1]}, {s.gz[k][0], s.gz[k][1]}, ez[k]};
-      else if (code == 2) {
-        for (int w = 0; w < 2; ++w) {
-          o.b[w] = s.bx[k][w] ^ s.bz[k][w];
-          o.g[w] = s.gx[k][w] ^ s.gz[k][w];
-        }
-        o.e = comp(1u + ex[k], s.gx[k], s.bz[k], ez[k]);
-      }
-      return o;
-    };
+    // |c & b'| counts modulo 2 and is linear in either operand, so four parities per pair of
+    // qubits give all 15 codes.
+    auto dot = [&](const uint64_t *c, const uint64_t *b2) { return (uint32_t)(pc(c[0] & b2[0]) + pc(c[1] & b2[1])); };
+    uint32_t e1[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};  // phases of 1 X, 2 Y = i X Z, 3 Z per qubit
+    for (int k = 0; k < (two ? 2 : 1); ++k) {
+      e1[k][1] = ex[k];
+      e1[k][2] = 1u + ex[k] + ez[k] + 2u * dot(s.gx[k], s.bz[k]);
+      e1[k][3] = ez[k];
+    }
     uint32_t c0 = 0;
-    for (int code = 1; code <= (two ? 15 : 3); ++code) {
-      uint32_t e;
-      if (!two) {
-        e = one(code, 0).e;
-      } else {
-        const int pa = code >> 2, pb = code & 3;
-        if (!pa) e = one(pb, 1).e;
-        else if (!pb) e = one(pa, 0).e;
-        else {
-          const One A = one(pa, 0), B = one(pb, 1);
-          e = comp(A.e, A.g, B.b, B.e);
-        }
+    if (!two) {
+      for (int code = 1; code <= 3; ++code) {
+        c0 |= (e1[0][code] & 3u) << (2 * code);
+        c0 |= (e1[0][code] & 3u) << (8 * code);  // also at code << 2, the site's Pauli pair (see Site)
       }
-      c0 |= (e & 3u) << (2 * code);
-      if (!two) c0 |= (e & 3u) << (8 * code);  // also at code << 2, the site's Pauli pair (see Site)
+    } else {
+      const uint32_t cr[2][2] = {{dot(s.gx[0], s.bx[1]), dot(s.gx[0], s.bz[1])}, {dot(s.gz[0], s.bx[1]), dot(s.gz[0], s.bz[1])}};
+      for (int code = 1; code <= 15; ++code) {
+        const int pa = code >> 2, pb = code & 3;
+        const int ax = pa == 1 || pa == 2, az = pa >= 2, bx = pb == 1 || pb == 2, bz = pb >= 2;
+        const uint32_t x = (ax && bx ? cr[0][0] : 0u) + (ax && bz ? cr[0][1] : 0u) + (az && bx ? cr[1][0] : 0u) +
+                           (az && bz ? cr[1][1] : 0u);
+        c0 |= ((e1[0][pa] + e1[1][pb] + 2u * x) & 3u) << (2 * code);
+      }
     }
     s.c0 = c0;
     if (p >= P.pmax) {
@@ -384,10 +557,10 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
     return P.ev.back();
   };
 
-  auto pauli_event = [&](const Pz &Q, uint32_t flags, int32_t r0, int32_t r1) -> bool {
+  auto pauli_event = [&](int code, uint32_t q, uint32_t flags, int32_t r0, int32_t r1) -> bool {
     uint64_t beta[2], gamma[2];
     uint32_t e0;
-    if (!tb.decompose(Q, beta, gamma, &e0)) return false;
+    tb.image(code, q, beta, gamma, &e0);
     Ev<2> &e = new_event(EV_PAULI, flags, e0, 0);
     e.a = (uint32_t)r0;
     e.b = (uint32_t)r1;
@@ -433,10 +606,11 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
   // One Pauli measurement of P (Theorem 1 (2)): case A when P commutes with
   // every stabilizer row, else case B with its row operations and
   // replacement constants. Returns false on an internal inconsistency.
-  auto meas_event = [&](const Pz &Pm, bool recd) -> bool {
+  auto meas_event = [&](const Pz &Pm, int zq, bool recd) -> bool {  // zq: P is Z on this qubit (-1: not)
     uint64_t beta[2], gamma[2];
     uint32_t e0;
-    if (!tb.decompose(Pm, beta, gamma, &e0)) return false;
+    if (zq >= 0) tb.image(3, (uint32_t)zq, beta, gamma, &e0);
+    else tb.image(Pm, beta, gamma, &e0);
     const uint32_t fidf = (recd && nrec < observed.size() && observed[nrec]) ? F_FIDELITY : 0u;
     if ((beta[0] | beta[1]) == 0) {
       Ev<2> &e = new_event(EV_MEAS_A, (recd ? F_RECORD : 0) | fidf, e0, 0);
@@ -446,6 +620,7 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
       return true;
     }
     CaseB cb{};
+    tb.rows();
     uint32_t p = beta[0] ? (uint32_t)__builtin_ctzll(beta[0]) : 64u + (uint32_t)__builtin_ctzll(beta[1]);
     cb.p = p;
     cb.J[0] = beta[0];
@@ -494,6 +669,8 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
     e.b = recd ? nrec : 0;
     e.beta[0] = P.cb.size();
     P.cb.push_back(cb);
+    tb.rows_changed();
+    tb.case_b_images(cb);
     return true;
   };
 
@@ -562,11 +739,11 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
     }
 
     if (isclifford(op)) {
-      if (!tb.gate(op, o.q0, o.q1)) goto internal;
+      tb.gate(op, o.q0, o.q1);
     } else if (op == SOFT_T || op == SOFT_T_DAG || op == SOFT_RZ) {
       uint64_t beta[2], gamma[2];
       uint32_t e0;
-      if (!tb.decompose(single(3, o.q0), beta, gamma, &e0)) goto internal;
+      tb.image(3, o.q0, beta, gamma, &e0);
       bool diag = (beta[0] | beta[1]) == 0;
       double ar, ai, br, bi, co, si;  // a phase times co I - i si Z
       int32_t phase = 0;
@@ -610,11 +787,11 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
     } else if (op == SOFT_M || op == SOFT_R || op == SOFT_MR) {
       bool recd = (op != SOFT_R);
       if (recd && nrec < observed.size() && observed[nrec]) seen_observed = true;
-      if (!meas_event(single(3, o.q0), recd)) goto internal;
+      if (!meas_event(single(3, o.q0), (int)o.q0, recd)) goto internal;
       ord++;
       if (recd) nrec++;
       if (op == SOFT_R || op == SOFT_MR)
-        if (!pauli_event(single(1, o.q0), F_COND_LAST, -1, -1)) goto internal;
+        if (!pauli_event(1, o.q0, F_COND_LAST, -1, -1)) goto internal;
     } else if (op == SOFT_MPP) {
       if (!mpp_open) mpp_acc = Pz{};
       mpp_acc = pmul(mpp_acc, single(o.flags & 3, o.q0));
@@ -627,14 +804,14 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
       if (!mpp_open) {
         mpp_q[0] = mpp_q[1] = 0;
         if (nrec < observed.size() && observed[nrec]) seen_observed = true;
-        if (!meas_event(mpp_acc, true)) goto internal;
+        if (!meas_event(mpp_acc, -1, true)) goto internal;
         ord++;
         nrec++;
       }
     } else if (op == SOFT_CPAULI) {
       int code = o.flags & 3;
       if (code) {
-        if (!pauli_event(single(code, o.q0), F_COND_REC, o.rec[0], o.rec[1])) goto internal;
+        if (!pauli_event(code, o.q0, F_COND_REC, o.rec[0], o.rec[1])) goto internal;
       }
     } else if (op == SOFT_DETECTOR || op == SOFT_OBSERVABLE) {
       uint32_t fl = (op == SOFT_DETECTOR ? F_DETECTOR : F_OBSERVABLE) | ((o.flags & SOFT_FLAG_CHAIN) ? F_CHAIN : 0) |
@@ -671,13 +848,17 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
   }
   P.n_sites = (uint32_t)P.sites.size();
   P.thr.resize(P.n_sites ? P.n_sites : 1);
-  for (uint32_t g = 0; g < P.n_sites; ++g) P.thr[g] = gap_thr(P.pmax, g);
+  {
+    const double log_q = std::log1p(-P.pmax);
+    for (uint32_t g = 0; g < P.n_sites; ++g) P.thr[g] = gap_thr(log_q, g);
+  }
   // thr increases with g, so the first g with U < thr[g] for every U of a bucket of the top
   // bits lies between the bucket's entry and the next one's
   P.thr_tab.assign((1u << kThrTabBits) + 1u, P.n_sites);
-  for (uint32_t b = 0; b < (1u << kThrTabBits); ++b) {
+  for (uint32_t b = 0, at = 0; b < (1u << kThrTabBits); ++b) {
     const uint64_t U = (uint64_t)b << (64 - kThrTabBits);
-    P.thr_tab[b] = (uint32_t)(std::upper_bound(P.thr.begin(), P.thr.begin() + P.n_sites, U) - P.thr.begin());
+    while (at < P.n_sites && P.thr[at] <= U) ++at;  // (both increase)
+    P.thr_tab[b] = at;
   }
   P.site_ev.assign(P.thr.size(), (uint32_t)P.ev.size());
   {
@@ -687,6 +868,7 @@ int compile_program(const soft_op *ops, size_t n_ops, uint32_t n, const soft_noi
       P.site_ev[s] = e;
     }
   }
+  tb.rows();
   P.fin_x.assign(4 * (size_t)n, 0);
   P.fin_z.assign(4 * (size_t)n, 0);
   for (uint32_t i = 0; i < n; ++i)
