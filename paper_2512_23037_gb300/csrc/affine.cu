@@ -369,7 +369,7 @@ struct AffShot {
       pe ^= ((sd[w] ^ esd) & beta[w]) ^ ((ss[w] ^ ess) & gamma[w]);
     }
     const uint32_t c0 = __shfl_sync(kAll, (uint32_t)(q.y >> 32), (int)kParts - 1);
-    apply_pauli(beta, gamma, ((c0 >> (2u * pp)) + 2u * wordpar(pe)) & 3u);
+    apply_pauli(beta, gamma, nc.phase(((c0 >> (2u * pp)) + 2u * wordpar(pe)) & 3u));
   }
 
   // FP32: b xi x, xi = i^e (-1)^par
@@ -798,9 +798,9 @@ struct AffShot {
       copy_async<16>(ring + (e % kRing) * sizeof(Ev<W>) + lane * 16u, reinterpret_cast<const unsigned char *>(evs + e) + lane * 16u);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  // the shot of item `local` (chunk-local), from spill record r or (kNoRecord) from the
-  // event that applies its first error
-  __device__ void run(uint64_t s, uint32_t local, uint32_t r) {
+  // the shot of item `local` (chunk-local), from spill record r or (kNoRecord) from its start
+  // event (ahead: see start_event)
+  __device__ void run(uint64_t s, uint32_t local, uint32_t r, bool ahead) {
     shot = s;
     status = AS_RUN;
     force = false;
@@ -808,19 +808,12 @@ struct AffShot {
     if (r != kNoRecord) {
       ev = load_spill(r);
     } else {
-      uint32_t nxt = kAll;
-      if (P.al_cursor && !C->lanes_off) {  // the bucketing pre-pass drew the first errors
-        const uint4 k = reinterpret_cast<const uint4 *>(P.al_cursor)[local];
-        nc = NoiseCursor{k.x, k.y, k.z};
-        if (nc.site() != kMaxPackedSites) nxt = nc.site();
-        if (nc.kblk == kAll) status = AS_ERR;
-      } else {
-        nc.kblk = 0;
-        nc.second = kNotDrawn;
-        draw(0);
-        if (nc.site() != kMaxPackedSites) nxt = nc.site();
-      }
-      ev = first_event(C, P.fid_mode, nxt);
+      // the pre-pass drew the first errors (and put the shot on this pass's list, or a lane did)
+      const uint4 k = reinterpret_cast<const uint4 *>(P.al_cursor)[local];
+      nc = NoiseCursor{k.x, k.y, k.z == kAll ? k.z : k.z & kBlockMask};
+      if (nc.kblk == kAll) status = AS_ERR;
+      bool resolved;  // (never: those did not leave the pre-pass)
+      ev = start_event(C, P.fid_mode, nc, ahead, resolved);
       load_snapshot(ev);
     }
     const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C->ev);
@@ -938,7 +931,7 @@ __global__ void __launch_bounds__(kAffBlock, sizeof(R) == 4 && W == 1 ? 6 : 5) a
     }
     s.C = &P.circ[lo];
     const uint64_t off = g - s.C->item_begin;
-    s.run(s.C->first_shot + off, local, rec);
+    s.run(s.C->first_shot + off, local, rec, !(lo == 0u && off < P.st_limit));
     s.finish(local, off, lo, btally);
     __syncwarp();
   }

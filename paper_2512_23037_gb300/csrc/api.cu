@@ -131,6 +131,10 @@ static cudaError_t build_prefixes(soft_circuit *c, cudaStream_t us) {
     const size_t stride = soft::prefix_stride(fp32, hp.W, hp.rw);
     if ((e = cudaMalloc(&c->d_traj[fp32], n_snap * stride)) != cudaSuccess) break;
     c->traj_stride[fp32] = (uint32_t)stride;
+    // (a circuit of very many sites, or events past the table's 28 bits, does without)
+    if (hp.n_sites && hp.n_sites <= soft::kFateMaxSites && hp.ev.size() < soft::kFateEvent &&
+        (e = cudaMalloc(&c->d_fate[fp32], (size_t)hp.n_sites * 16 * sizeof(uint32_t))) != cudaSuccess)
+      break;
   }
   for (int fp32 = 0; fp32 < 2 && e == cudaSuccess; ++fp32) {
     soft::ShotParams p{};
@@ -151,6 +155,10 @@ static cudaError_t build_prefixes(soft_circuit *c, cudaStream_t us) {
     p.rw_max = hp.rw;
     p.prune = soft::prune_bounds(fp32 ? kTauFp32 : kTauFp64);
     e = soft::launch_prefix(p, fp32, hp.W, c->d_traj[fp32], d_stop + 4 * fp32, ps[fp32]);
+    if (e == cudaSuccess && c->d_fate[fp32]) {
+      soft::CircDev cd = soft::circ_desc(c, fp32, true);
+      e = soft::launch_fate(cd, hp.W, d_stop + 4 * fp32, c->d_fate[fp32], ps[fp32]);
+    }
     if (e == cudaSuccess)
       e = soft::launch_snap_affine(c->d_traj[fp32], (uint32_t)n_snap, hp.rw, fp32, hp.W, d_stop + 4 * fp32, c->d_ev,
                                    ps[fp32]);
@@ -291,6 +299,8 @@ void soft_circuit_free(soft_circuit *c) {
   cudaFree(c->d_thr);
   cudaFree(c->d_traj[0]);
   cudaFree(c->d_traj[1]);
+  cudaFree(c->d_fate[0]);
+  cudaFree(c->d_fate[1]);
   cudaFree(c->d_stop);
   cudaFree(c->d_gcoef);
   cudaFree(c->d_gnext);
@@ -344,6 +354,7 @@ CircDev circ_desc(const soft_circuit *c, int fp32, bool prefix) {
     d.traj_stop = c->traj_stop[fp32];
     d.traj_fid_stop = c->traj_fid_stop[fp32];
     d.traj_stride = c->traj_stride[fp32];
+    d.fate = c->d_fate[fp32];
   }
   d.ev = c->d_ev;
   d.coef = c->d_coef;
@@ -415,15 +426,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     lcap[i] = circs[i]->d_traj[pk] && circs[i]->hp.n_sites < soft::kMaxPackedSites ? soft::lane_first_cap(circs[i]->traj_max_n[pk], circs[i]->traj_max_d[pk], fp32) : 0u;
     if (lcap[i]) nbc[lane_class(lcap[i])] += circs[i]->hp.ev.size() + 1;
   }
-  const uint64_t n_buckets = nbc[0] + nbc[1] + nbc[2];
-  const bool lanes = !(o.flags & SOFT_RUN_NO_LANES) && !(o.flags & SOFT_RUN_NO_PREFIX) && o.group_size == 0 &&
-                     n_buckets > 0 && n_buckets <= soft::lane_max_buckets();
-  const uint32_t nb = lanes ? (uint32_t)n_buckets : 0u;
-  const bool lanes16 = lanes && nbc[0] > 0;  // the lanes that evict, hand over and feed the wide round
-  // a rerun pass finishes the shots whose maps outgrow the first pass (cap1). After lanes it
-  // always runs: a lane decides overflow only after pruning, and a map that outgrows the lane
-  // before pruning is staged whole by the warp pass, even when the circuit's cap is the lane's.
-  const bool lane_grow = lanes16 && lc16 < cap_max;  // maps may outgrow a 16-entry lane
+  uint64_t n_buckets = nbc[0] + nbc[1] + nbc[2];
   // the warp-per-shot passes below the circuit's cap keep the map in affine form (affine.cu)
   // unless the caller shapes them (group size, first_cap, groups per block) or asks for the
   // sparse form's scheduling (no lanes, no prefix)
@@ -431,7 +434,21 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
                 o.groups_per_block == 0;
   for (uint32_t i = 0; i < n_circ; ++i)
     affine = affine && circs[i]->d_traj[pk] && circs[i]->hp.n_sites < soft::kMaxPackedSites;
-  const bool two_pass = lanes || affine || cap1 < cap_max;
+  if (n_buckets > soft::lane_max_buckets()) {  // too many buckets: no lanes
+    n_buckets = nbc[0] = nbc[1] = nbc[2] = 0;
+    std::fill(lcap.begin(), lcap.end(), 0u);
+  }
+  // with the affine warp passes, the pre-pass runs even where no circuit has lanes: it draws the
+  // shots' errors, finishes those that their first error discards, and lists the others
+  const bool lanes = !(o.flags & SOFT_RUN_NO_LANES) && !(o.flags & SOFT_RUN_NO_PREFIX) && o.group_size == 0 &&
+                     (n_buckets > 0 || affine);
+  const uint32_t nb = lanes ? (uint32_t)n_buckets : 0u;
+  const bool lanes16 = lanes && nbc[0] > 0;  // the lanes that evict, hand over and feed the wide round
+  // a rerun pass finishes the shots whose maps outgrow the first pass (cap1). After lanes it
+  // always runs: a lane decides overflow only after pruning, and a map that outgrows the lane
+  // before pruning is staged whole by the warp pass, even when the circuit's cap is the lane's.
+  const bool lane_grow = lanes16 && lc16 < cap_max;  // maps may outgrow a 16-entry lane
+  const bool two_pass = lanes || cap1 < cap_max;
   // after lanes, a middle pass (a warp per shot) takes the shots whose maps outgrew a lane, and
   // only those that outgrow it too go on to the pass at the circuit's cap: in affine form, with
   // room for 2^kAffDim entries, or in sparse form up to cap1 entries. The sparse one is left out
@@ -658,7 +675,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     q.list = m.rerun;
     q.n_items_dev = m.n_rerun;
   }
-  p.aff_dim = m.aff_dim = kAffDim;
+  m.aff_dim = kAffDim;
   if (global_rerun) {
     q.gslab = r->d_slab;
     q.gslab_blocks = slab_blocks;
@@ -709,8 +726,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     pb[k].sp_dim = soft::lane_map_dim() + 1 + k;
     pb[k].lr = r->d_lrb[k];
   }
-  if ((e = !lanes ? (affine ? soft::prepare_affine(p, fp32, W, (int)o.blocks_per_sm, &c1)
-                            : soft::prepare_shots(p, fp32, W, g1, (int)o.blocks_per_sm, &c1))
+  if ((e = !lanes ? soft::prepare_shots(p, fp32, W, g1, (int)o.blocks_per_sm, &c1)
                   : lanes16 ? soft::prepare_lanes(p, fp32, W, (int)o.blocks_per_sm, &c1, lc16) : cudaSuccess) !=
           cudaSuccess ||
       (lanes && nbc[1] && (e = soft::prepare_lanes(pb[0], fp32, W, 0, &cb[0], 2 * lc16)) != cudaSuccess) ||
@@ -750,7 +766,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     if (dev_base) a.item_base_dev = b.item_base_dev = c.item_base_dev = r->d_work + 3;
     if ((err = mark()) != cudaSuccess) return err;
     if (lanes) {
-      if ((err = soft::launch_lane_prepass(a, st)) != cudaSuccess) return err;
+      if ((err = soft::launch_lane_prepass(a, W, st)) != cudaSuccess) return err;
       r->launches += al_grid > 1 ? 3 : 1;
     }
     if ((err = mark(lanes)) != cudaSuccess) return err;

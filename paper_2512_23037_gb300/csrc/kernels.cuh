@@ -22,7 +22,7 @@ struct CircDev {
   uint32_t n_events, n_sites, rw, cap;  // cap: this circuit's coefficient cap
   uint32_t n_coef, n_cb;
   uint32_t bucket0;    // lane-per-shot scheduling: the circuit's first bucket (one per event, plus one)
-  uint32_t lanes_off;  // 1: its maps outgrow a lane; its shots go straight to the warp pass (no buckets)
+  uint32_t lanes_off;  // 1: its maps outgrow a lane; its shots go straight to the warp pass's list (no buckets)
   uint64_t item_begin, n_shots, first_shot;
   unsigned long long *tally;  // [5]: shots, discarded, overflow, kept, logical
   double *fsum;               // fidelity mode: sum of F over kept shots (may be null)
@@ -35,6 +35,7 @@ struct CircDev {
   uint32_t traj_stop, traj_stride;
   uint32_t traj_fid_stop, pad_traj;  // first fidelity measurement's event (fidelity mode stops there)
   const uint32_t *site_ev;  // per site: the event that applies its error
+  const uint32_t *fate;     // per site and Pauli pair (16 words a site): see fate_kernel (null: none)
   const uint32_t *site_thin;
   const uint8_t *site_kind; // per site: its kind and kSiteThinned (program.h)
   const uint32_t *thr_tab;  // the gap search's index, 2^kThrTabBits + 1 entries (null: plain search)
@@ -146,7 +147,7 @@ struct LaunchCfg {
 
 // Lane-per-shot kernel (lanes.cu): the bucketing pre-pass (start events, bucket
 // starts, order), its launch shape, and its map capacity per shot.
-cudaError_t launch_lane_prepass(const ShotParams &p, cudaStream_t st);
+cudaError_t launch_lane_prepass(const ShotParams &p, uint32_t W, cudaStream_t st);
 // round r >= 1: the range of records evicted before it, then their buckets
 cudaError_t launch_lane_resume_prepass(const ShotParams &p, int fp32, uint32_t W, cudaStream_t st);
 // bytes of `cap` spill records of maps of `dim` directions
@@ -165,6 +166,9 @@ uint32_t lane_map_cap();
 // whose noiseless run's maps reach max_n entries in max_d directions; 0 if none does.
 uint32_t lane_first_cap(uint32_t max_n, uint32_t max_d, int fp32);
 uint32_t lane_map_dim();  // directions of a first-round lane's affine map (lane_map_cap = 2^lane_map_dim)
+// After launch_prefix: the fate of each site's errors (see fate_kernel in lanes.cu), for circuit c
+// (its program, sites and the snapshots being valid up to event stop[0]).
+cudaError_t launch_fate(const CircDev &c, uint32_t W, const uint32_t *stop, uint32_t *fate, cudaStream_t st);
 // After launch_prefix: the affine form of each snapshot of the run (events [0, stop[0]]),
 // on the same stream; stop[3] (zeroed before) receives the largest dimension.
 // ev: the circuit's device events (Ev<W>).

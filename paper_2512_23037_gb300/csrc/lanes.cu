@@ -542,7 +542,7 @@ struct LaneShot {
     }
     uint64_t beta[W], gamma[W];
     const uint32_t e = site_pauli<W>(C, s, nc.pair(), sd, ss, beta, gamma);
-    apply_pauli(beta, gamma, e);
+    apply_pauli(beta, gamma, nc.phase(e));
   }
 
   // (rare: many rotations, or very unlikely outcomes, since the last sampled outcome)
@@ -1058,6 +1058,75 @@ __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_
   atomicMax(&stop[3], ok ? d : 0xFFu);
 }
 
+// ---- the fate of each site's errors, one thread per site and Pauli pair, once per compiled
+// circuit and precision.
+// Before its first error a shot is the noiseless run. An error E commutes past every event that
+// leaves it alone: a rotation whose generator commutes with it, a decided measurement whose
+// outcome it does not flip (its corrections commuting with E too), a parity of unflipped
+// records. Up to such an event the shot is E applied to the noiseless run's state there, bit for
+// bit, since E permutes and phases the entries exactly and the arithmetic rounds alike on values
+// times i^k. So the shot may start at the first event that does not leave E alone, and if that
+// is a measurement with a detector on it, E flips it and the shot ends there, discarded: the
+// pre-pass finishes such shots without running them (60 % of w42's and w97's; the others
+// start 10 to 20 events later; events run per shot: w42 25.7 -> 10.5, w97 46 -> 15).
+// Entry: that event (at most the recorded run's last), kFateDiscard, and E's phase i^e relative to
+// the signed rows, which the Clifford gates in between leave as it is.
+template <int W>
+__global__ void __launch_bounds__(128) fate_kernel(const __grid_constant__ CircDev C, const uint32_t *stop_at, uint32_t *out) {
+  const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x, s = idx >> 4, pp = idx & 15u;
+  if (s >= C.n_sites) return;
+  const SiteDev<W> *S = reinterpret_cast<const SiteDev<W> *>(C.sites) + s;
+  uint32_t e = __ldg(&C.site_ev[s]);
+  const uint32_t stop = *stop_at < C.n_events ? *stop_at : C.n_events;
+  if (e > stop || pp == 0u || ((__ldg(&S->kind) & 3u) != SITE_DEPOL2 && (pp & 3u))) {  // (not an error, or never used)
+    out[idx] = e;
+    return;
+  }
+  const SnapHdr *h = reinterpret_cast<const SnapHdr *>(C.traj + (size_t)e * C.traj_stride);
+  uint64_t b[W], g[W], sd[W], ss[W];
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    sd[w] = h->sd[w];
+    ss[w] = h->ss[w];
+  }
+  const uint32_t ph = site_pauli<W>(&C, s, pp, sd, ss, b, g);
+  const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C.ev);
+  uint32_t kind = 0;
+  for (; e < stop; ++e) {
+    const Ev<W> *E = evs + e;
+    const uint32_t w0 = __ldg(&E->w0), type = ev_type(w0), flags = ev_flags(w0);
+    uint64_t be[W], ga[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      be[w] = __ldg(&E->beta[w]);
+      ga[w] = __ldg(&E->gamma[w]);
+    }
+    if (type == EV_ROT || type == EV_ROT_DIAG) {
+      if (wpar2<W>(be, g, ga, b)) break;  // E anticommutes with the generator
+    } else if (type == EV_MEAS_A) {
+      if (wpar<W>(ga, b)) {  // E flips the outcome
+        if (flags & F_DETECTOR) kind = kFateDiscard;
+        break;
+      }
+      if (flags & F_COND_LAST) {
+        const SnapHdr *hn = reinterpret_cast<const SnapHdr *>(C.traj + (size_t)(e + 1u) * C.traj_stride);
+        if ((int)hn->lastm == -1) {  // the noiseless run applies the correction
+          uint64_t xb[W], xg[W];
+#pragma unroll
+          for (int w = 0; w < W; ++w) {
+            xb[w] = __ldg(&E->xbeta[w]);
+            xg[w] = __ldg(&E->xgamma[w]);
+          }
+          if (wpar2<W>(xb, g, xg, b)) break;
+        }
+      }
+    } else if (type != EV_PARITY && type != EV_END) {
+      break;
+    }
+  }
+  out[idx] = e | kind | (ph << 30);
+}
+
 // ---- bucketing pre-pass. Buckets: per circuit of the run, one per event plus one
 // (shots that start past the end), circuit after circuit from circuit.bucket0.
 // The circuit of item g: the last one whose item range starts at or before g.
@@ -1131,10 +1200,14 @@ __global__ void lane_round_setup_kernel(const __grid_constant__ ShotParams P) { 
 // atomics on one address serialise.
 // Items of circuits whose maps outgrow a lane go to the warp pass's list instead: the
 // block ranks them too and reserves their slots with one global atomic.
+// Shots that their first error discards are finished here (start_event): their status, their
+// record (the noiseless run's, with the failing measurement's bit flipped) and their count.
+constexpr uint32_t kResolved = 0xFFFFFFFEu;  // as a bucket
 template <bool Resume, typename R, int W>
 __device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
   const uint32_t nb = P.al_nb;
-  for (uint32_t k = threadIdx.x; k <= nb; k += blockDim.x) hist[k] = 0u;
+  uint32_t *ended = hist + nb + 1;  // per circuit: shots discarded here
+  for (uint32_t k = threadIdx.x; k <= nb + (Resume ? 0u : P.n_circ); k += blockDim.x) hist[k] = 0u;
   __syncthreads();
   const unsigned long long n_items =
       Resume ? P.lr[3 + 2 * P.lane_round] : (P.n_items_dev ? *P.n_items_dev : P.n_items);
@@ -1150,21 +1223,42 @@ __device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
       C = &P.circ[circ_of_item(P, base + a.x)];
       e = a.y < C->n_events ? a.y : C->n_events;  // a record always resumes at an event of its circuit
     } else {
-      C = &P.circ[circ_of_item(P, base + i)];
+      const uint32_t ci = circ_of_item(P, base + i);
+      C = &P.circ[ci];
+      // the shot's first error and the one after it: nearly every shot applies the first as it
+      // starts, and here all lanes of a warp draw
+      uint32_t cur = 0, nxt = 0, pp = 0, n2 = 0, p2 = 0;
+      NoiseCursor nc{0, 0, 0};
+      const uint64_t off = base + i - C->item_begin, shot = C->first_shot + off;
+      bool ok = next_site(C, P.seed, shot, cur, nc.kblk, nxt, pp);
+      if (ok && nxt != 0xFFFFFFFFu) ok = next_site(C, P.seed, shot, cur, nc.kblk, n2, p2);
+      else n2 = 0xFFFFFFFFu;
+      nc.first = pack_error(nxt, pp);
+      nc.second = pack_error(n2, p2);
+      if (!ok) nc = NoiseCursor{kMaxPackedSites, kMaxPackedSites, 0xFFFFFFFFu};
+      bool resolved = false;
+      e = start_event(C, P.fid_mode, nc, ok && !(ci == 0u && off < P.st_limit), resolved);
+      if (resolved) {
+        reinterpret_cast<uint2 *>(P.al_ev)[i] = make_uint2(kResolved, 0u);
+        atomicAdd(&ended[ci], 1u);
+        if (off < C->out_limit) {
+          if (C->status) C->status[off] = (uint8_t)LS_DISC;
+          if (C->records) {
+            const Ev<W> *E = reinterpret_cast<const Ev<W> *>(C->ev) + e;
+            const uint32_t r = __ldg(&E->b);
+            const uint64_t *rec = reinterpret_cast<const uint64_t *>(C->traj + (size_t)e * C->traj_stride + sizeof(SnapHdr));
+            const bool one = !(ev_flags(__ldg(&E->w0)) & F_INVERT);  // the outcome that fails the detector
+            for (uint32_t w = 0; w < C->rw; ++w)
+              C->records[off * C->rw + w] = __ldg(&rec[w]) | (one && w == (r >> 6) ? 1ull << (r & 63u) : 0ull);
+          }
+        }
+        continue;
+      }
+      reinterpret_cast<uint4 *>(P.al_cursor)[i] = make_uint4(nc.first, nc.second, nc.kblk, (uint32_t)i);
       if (C->lanes_off) {
         reinterpret_cast<uint2 *>(P.al_ev)[i] = make_uint2(kNoRecord, atomicAdd(&hist[nb], 1u));
         continue;
       }
-      // the shot's first error and the one after it: nearly every shot applies the first as it
-      // starts, and here all lanes of a warp draw
-      uint32_t cur = 0, kblk = 0, nxt = 0, pp = 0, n2 = 0, p2 = 0;
-      const uint64_t shot = C->first_shot + (base + i - C->item_begin);
-      bool ok = next_site(C, P.seed, shot, cur, kblk, nxt, pp);
-      if (ok && nxt != 0xFFFFFFFFu) ok = next_site(C, P.seed, shot, cur, kblk, n2, p2);
-      else n2 = 0xFFFFFFFFu;
-      e = first_event(C, P.fid_mode, nxt);
-      reinterpret_cast<uint4 *>(P.al_cursor)[i] =
-          make_uint4(pack_error(nxt, pp), pack_error(n2, p2), ok ? kblk : 0xFFFFFFFFu, (uint32_t)i);
     }
     e += C->bucket0;
     reinterpret_cast<uint2 *>(P.al_ev)[i] = make_uint2(e, atomicAdd(&hist[e], 1u));
@@ -1176,6 +1270,12 @@ __device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
   }
   if (threadIdx.x == 0)
     P.al_base[(size_t)blockIdx.x * (nb + 1) + nb] = hist[nb] ? (uint32_t)atomicAdd(P.n_rerun, (unsigned long long)hist[nb]) : 0u;
+  if (!Resume)
+    for (uint32_t k = threadIdx.x; k < P.n_circ; k += blockDim.x)
+      if (ended[k]) {
+        atomicAdd(&P.circ[k].tally[0], (unsigned long long)ended[k]);
+        atomicAdd(&P.circ[k].tally[1], (unsigned long long)ended[k]);
+      }
 }
 template <bool Resume, typename R, int W>
 __global__ void __launch_bounds__(256) lane_bin_kernel(const __grid_constant__ ShotParams P) {
@@ -1192,6 +1292,7 @@ __device__ __forceinline__ void scatter_items(const ShotParams &P) {
   const unsigned long long i0 = blockIdx.x * per, i1 = i0 + per < n_items ? i0 + per : n_items;
   for (unsigned long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
     const uint2 er = reinterpret_cast<const uint2 *>(P.al_ev)[i];
+    if (er.x == kResolved) continue;
     if (er.x == kNoRecord) {  // a shot of a circuit without lanes: the warp pass's list
       const unsigned long long slot = P.al_base[(size_t)blockIdx.x * (nb + 1) + nb] + er.y;
       if (slot < P.rerun_cap) P.rerun[slot] = (uint32_t)i;
@@ -1495,6 +1596,13 @@ cudaError_t launch_snap_affine(unsigned char *traj, uint32_t n_snap, uint32_t rw
   }
   return cudaGetLastError();
 }
+cudaError_t launch_fate(const CircDev &c, uint32_t W, const uint32_t *stop, uint32_t *fate, cudaStream_t st) {
+  if (!c.n_sites) return cudaSuccess;
+  const unsigned grid = (unsigned)(((size_t)c.n_sites * 16 + 127) / 128);
+  if (W == 1) fate_kernel<1><<<grid, 128, 0, st>>>(c, stop, fate);
+  else fate_kernel<2><<<grid, 128, 0, st>>>(c, stop, fate);
+  return cudaGetLastError();
+}
 uint32_t lane_rounds() { return kLaneRounds; }
 uint32_t lane_max_buckets() { return kLaneMaxBuckets; }
 uint32_t lane_prepass_grid(uint64_t items) {
@@ -1513,7 +1621,7 @@ size_t lane_spill_bytes(int fp32, uint32_t W, uint32_t rw, uint32_t cap, uint32_
 // the histogram of all buckets in shared memory (above 48 KB by the opt-in attribute)
 template <bool Resume, typename R, int W>
 static cudaError_t launch_bin(const ShotParams &p, cudaStream_t st) {
-  const size_t sh = ((size_t)p.al_nb + 1) * sizeof(uint32_t);
+  const size_t sh = ((size_t)p.al_nb + 1 + p.n_circ) * sizeof(uint32_t);
   if (sh > 48 * 1024) {
     const void *kern = p.al_grid == 1 ? reinterpret_cast<const void *>(lane_bin_one_kernel<Resume, R, W>)
                                       : reinterpret_cast<const void *>(lane_bin_kernel<Resume, R, W>);
@@ -1536,7 +1644,9 @@ cudaError_t launch_lane_resume_prepass(const ShotParams &p, int fp32, uint32_t W
   return W == 1 ? launch_bin<true, double, 1>(p, st) : launch_bin<true, double, 2>(p, st);
 }
 
-cudaError_t launch_lane_prepass(const ShotParams &p, cudaStream_t st) { return launch_bin<false, float, 1>(p, st); }
+cudaError_t launch_lane_prepass(const ShotParams &p, uint32_t W, cudaStream_t st) {
+  return W == 1 ? launch_bin<false, float, 1>(p, st) : launch_bin<false, float, 2>(p, st);
+}
 
 template <uint32_t Cap>
 static const void *lane_kernel_for(int fp32, uint32_t W, bool multi) {

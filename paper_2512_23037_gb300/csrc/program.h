@@ -133,6 +133,10 @@ SOFT_HD inline uint32_t site_images(uint32_t pp) {
 // without them.
 constexpr uint32_t kMaxPackedSites = 0x0FFFFFFFu;
 
+// Fate table entry: event (bits 0-27), kFateDiscard, phase of the error (bits 30-31).
+constexpr uint32_t kFateEvent = 0x0FFFFFFFu, kFateDiscard = 0x10000000u;
+constexpr uint32_t kFateMaxSites = 1u << 22;  // (16 words a site)
+
 constexpr uint32_t kNoRec = 0xFFFFFFFFu;
 
 }  // namespace soft

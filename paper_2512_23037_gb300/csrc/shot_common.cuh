@@ -101,8 +101,19 @@ constexpr uint32_t kNotDrawn = 0x10000000u;  // (no second error: it would be at
 __device__ __forceinline__ uint32_t pack_error(uint32_t nxt, uint32_t pp) {
   return nxt == 0xFFFFFFFFu ? 0x0FFFFFFFu : nxt | (pp << 28);
 }
+// kblk carries kPhaseKnown and the first error's phase (bits 30-31) while the shot starts at a
+// later event than the one that applies it.
+constexpr uint32_t kPhaseKnown = 0x20000000u, kBlockMask = 0x1FFFFFFFu;
 struct NoiseCursor {
   uint32_t first, second, kblk;
+  // the first error's phase: that of its site, e, or the one it brought along
+  __device__ __forceinline__ uint32_t phase(uint32_t e) {
+    if (kblk & kPhaseKnown) {
+      e = kblk >> 30;
+      kblk &= kBlockMask;
+    }
+    return e;
+  }
   __device__ __forceinline__ uint32_t site() const { return first & 0x0FFFFFFFu; }
   __device__ __forceinline__ uint32_t pair() const { return first >> 28; }
   // past the first error
@@ -131,6 +142,32 @@ __device__ __forceinline__ uint32_t first_event(const CircDev *C, int fid_mode, 
     return e < stop ? e : stop;
   }
   return stop;
+}
+
+// Where a shot starts whose next two errors nc holds: at the event that applies the first, or
+// later (see fate_kernel), at the latest where its second error comes in or the recorded
+// noiseless run ends. resolved: the shot ends at the returned event, discarded by its detector
+// (whose record is flipped), with nothing left to run. ahead: false for shots whose final
+// state is captured (they run from their first error).
+__device__ __forceinline__ uint32_t start_event(const CircDev *C, int fid_mode, NoiseCursor &nc, bool ahead,
+                                                bool &resolved) {
+  const uint32_t stop = fid_mode && C->traj_fid_stop < C->traj_stop ? C->traj_fid_stop : C->traj_stop;
+  resolved = false;
+  const uint32_t s = nc.site();
+  if (s == kMaxPackedSites) return stop;
+  const uint32_t e1 = __ldg(&C->site_ev[s]);
+  if (e1 > stop) return stop;
+  if (!C->fate || !ahead) return e1;
+  const uint32_t f = __ldg(&C->fate[(size_t)s * 16 + nc.pair()]), s2 = nc.second & kMaxPackedSites;
+  const uint32_t e2 = s2 == kMaxPackedSites ? 0xFFFFFFFFu : __ldg(&C->site_ev[s2]);
+  const uint32_t F = f & kFateEvent;
+  if ((f & kFateDiscard) && F <= stop && e2 > F) {
+    resolved = true;
+    return F;
+  }
+  const uint32_t at = F < e2 ? F : e2;
+  nc.kblk |= kPhaseKnown | (f & 0xC0000000u);
+  return at < stop ? at : stop;
 }
 
 // Snapshot of the noiseless run at the top of an event: header, rw record words,
