@@ -29,10 +29,10 @@ int cuda_fail(cudaError_t e, const char *what) {
 constexpr uint64_t kDefaultChunk = 1ull << 24;
 using soft::kDefaultFirstCap;
 // Shots of a chunk up to which evicted shots go to the warp pass instead of a second lane round.
-// Both ways, in ms: w42 FP32 65 k shots 0.66 / 1.59, 262 k 1.08 / 1.35, 400 k 1.59 / 1.57, 700 k
-// 2.14 / 1.79; w97 FP32 130 k 2.55 / 3.17, 400 k 5.44 / 4.93; random 40-qubit circuit 130 k 1.05 /
-// 1.25, 400 k 2.50 / 2.71.
-constexpr uint64_t kSmallRun = 5ull << 16;
+// Both ways, in ms: w42 FP32 500 k shots 1.15 / 1.42, 1 M 1.70 / 1.77; w42 FP64 520 k 1.41 / 1.68,
+// 1 M 2.12 / 2.12, 2 M 3.43 / 3.05; w97 FP32 400 k 2.93 / 3.56, 1 M 5.43 / 5.20; random 40-qubit
+// circuit 400 k 2.40 / 2.58.
+constexpr uint64_t kSmallRun = 1ull << 20;
 constexpr uint32_t kAffDim = 8;  // directions of the affine warp passes' maps (256 values per warp)
 using soft::kTauFp32;
 using soft::kTauFp64;
@@ -521,11 +521,11 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   // the wide round: the handed-over shots continue in lanes of twice the map (their records
   // are its input), and only those that outgrow it rerun in a warp. Single-circuit runs only
   // (batches measured slower: 125.5 M against 130.3 M shots/s on batch64, before the affine
-  // lanes). By default only for chunks of at least 2^23 shots: its pre-pass and launch cost
-  // more than it saves in small runs (w42 at 2^21 shots: 389.0 M against 412.5 M). w42 at 2^24:
-  // FP32 550.0 M against 533.0 M (sparse lanes); FP64 348.2 M against 344.5 M (affine lanes).
+  // lanes). By default only for the chunks it gains on: it costs a pre-pass and a launch more.
+  // With it / without, w42: FP32 2 M shots 2.26 / 2.51 ms, 8 M 4.87 / 6.45, 16 M 8.44 / 11.9;
+  // FP64 2 M 3.11 / 3.05, 4 M 4.77 / 5.2, 8 M 8.07 / 9.12.
   const bool wide_ok = spill && lane_grow && n_circ == 1 && !(o.flags & SOFT_RUN_NO_WIDE_LANES);
-  const bool wide = wide_ok && ((o.flags & SOFT_RUN_WIDE_LANES) || std::min(chunk, total) >= (1ull << 23));
+  const bool wide = wide_ok && ((o.flags & SOFT_RUN_WIDE_LANES) || std::min(chunk, total) >= (1ull << (fp32 ? 21 : 22)));
   if (spill) need(&r->d_sp, soft::lane_spill_bytes(fp32, W, rw_max, sp_evict + sp_hand, soft::lane_map_dim()));
   // the larger lanes' eviction pools: a quarter of their circuits' shots, at most 2^22 records
   // (a record of a 64-entry lane takes about 0.8 KB)
