@@ -799,8 +799,8 @@ struct AffShot {
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
   // the shot of item `local` (chunk-local), from spill record r or (kNoRecord) from its start
-  // event (ahead: see start_event)
-  __device__ void run(uint64_t s, uint32_t local, uint32_t r, bool ahead) {
+  // event
+  __device__ void run(uint64_t s, uint32_t local, uint32_t r) {
     shot = s;
     status = AS_RUN;
     force = false;
@@ -810,10 +810,9 @@ struct AffShot {
     } else {
       // the pre-pass drew the first errors (and put the shot on this pass's list, or a lane did)
       const uint4 k = reinterpret_cast<const uint4 *>(P.al_cursor)[local];
-      nc = NoiseCursor{k.x, k.y, k.z == kAll ? k.z : k.z & kBlockMask};
+      nc = NoiseCursor{k.x, k.y, k.z};
       if (nc.kblk == kAll) status = AS_ERR;
-      bool resolved;  // (never: those did not leave the pre-pass)
-      ev = start_event(C, P.fid_mode, nc, ahead, resolved);
+      ev = k.w;
       load_snapshot(ev);
     }
     const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C->ev);
@@ -931,7 +930,7 @@ __global__ void __launch_bounds__(kAffBlock, sizeof(R) == 4 && W == 1 ? 6 : 5) a
     }
     s.C = &P.circ[lo];
     const uint64_t off = g - s.C->item_begin;
-    s.run(s.C->first_shot + off, local, rec, !(lo == 0u && off < P.st_limit));
+    s.run(s.C->first_shot + off, local, rec);
     s.finish(local, off, lo, btally);
     __syncwarp();
   }

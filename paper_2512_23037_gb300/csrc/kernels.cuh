@@ -90,7 +90,7 @@ struct ShotParams {
   uint32_t *al_ev;  // per item (start event, rank in its bucket), 8-byte aligned
   uint32_t *al_order, *al_start;
   unsigned int *al_count, *al_next;
-  uint32_t *al_cursor;  // per item the noise cursor after two draws (NoiseCursor) and the item, 16-byte aligned
+  uint32_t *al_cursor;  // per item the noise cursor after two draws (NoiseCursor) and the start event, 16-byte aligned
   uint32_t *al_rec;     // those of the items in bucket order (a resume round: al_order)
   uint32_t *al_base;    // per pre-pass block: the block's first rank in each bucket, then its first
                         // slot in the warp pass's list (al_nb + 1 words per block)

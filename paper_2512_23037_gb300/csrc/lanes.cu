@@ -1068,7 +1068,8 @@ __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_
 // times i^k. So the shot may start at the first event that does not leave E alone, and if that
 // is a measurement with a detector on it, E flips it and the shot ends there, discarded: the
 // pre-pass finishes such shots without running them (60 % of w42's and w97's; the others
-// start 10 to 20 events later; events run per shot: w42 25.7 -> 10.5, w97 46 -> 15).
+// start 10 to 20 events later; events run per shot: w42 25.7 -> 10.7, w97 46 -> 13.4). Two errors
+// are carried to the earlier of their events (start_event).
 // Entry: that event (at most the recorded run's last), kFateDiscard, and E's phase i^e relative to
 // the signed rows, which the Clifford gates in between leave as it is.
 template <int W>
@@ -1200,7 +1201,7 @@ __global__ void lane_round_setup_kernel(const __grid_constant__ ShotParams P) { 
 // atomics on one address serialise.
 // Items of circuits whose maps outgrow a lane go to the warp pass's list instead: the
 // block ranks them too and reserves their slots with one global atomic.
-// Shots that their first error discards are finished here (start_event): their status, their
+// Shots that their first errors discard are finished here (start_event): their status, their
 // record (the noiseless run's, with the failing measurement's bit flipped) and their count.
 constexpr uint32_t kResolved = 0xFFFFFFFEu;  // as a bucket
 template <bool Resume, typename R, int W>
@@ -1237,7 +1238,7 @@ __device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
       nc.second = pack_error(n2, p2);
       if (!ok) nc = NoiseCursor{kMaxPackedSites, kMaxPackedSites, 0xFFFFFFFFu};
       bool resolved = false;
-      e = start_event(C, P.fid_mode, nc, ok && !(ci == 0u && off < P.st_limit), resolved);
+      e = start_event(C, P.fid_mode, P.seed, shot, nc, ok && !(ci == 0u && off < P.st_limit), resolved);
       if (resolved) {
         reinterpret_cast<uint2 *>(P.al_ev)[i] = make_uint2(kResolved, 0u);
         atomicAdd(&ended[ci], 1u);
@@ -1254,7 +1255,7 @@ __device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
         }
         continue;
       }
-      reinterpret_cast<uint4 *>(P.al_cursor)[i] = make_uint4(nc.first, nc.second, nc.kblk, (uint32_t)i);
+      reinterpret_cast<uint4 *>(P.al_cursor)[i] = make_uint4(nc.first, nc.second, nc.kblk, e);
       if (C->lanes_off) {
         reinterpret_cast<uint2 *>(P.al_ev)[i] = make_uint2(kNoRecord, atomicAdd(&hist[nb], 1u));
         continue;
@@ -1300,7 +1301,10 @@ __device__ __forceinline__ void scatter_items(const ShotParams &P) {
     }
     const uint32_t at = P.al_start[er.x] + P.al_base[(size_t)blockIdx.x * (nb + 1) + er.x] + er.y;
     if (Resume) P.al_order[at] = (uint32_t)i;
-    else reinterpret_cast<uint4 *>(P.al_rec)[at] = reinterpret_cast<const uint4 *>(P.al_cursor)[i];
+    else {
+      const uint4 k = reinterpret_cast<const uint4 *>(P.al_cursor)[i];
+      reinterpret_cast<uint4 *>(P.al_rec)[at] = make_uint4(k.x, k.y, k.z, (uint32_t)i);
+    }
   }
 }
 
