@@ -33,7 +33,18 @@ using soft::kDefaultFirstCap;
 // 1 M 2.12 / 2.12, 2 M 3.43 / 3.05; w97 FP32 400 k 2.93 / 3.56, 1 M 5.43 / 5.20; random 40-qubit
 // circuit 400 k 2.40 / 2.58.
 constexpr uint64_t kSmallRun = 1ull << 20;
-constexpr uint32_t kAffDim = 8;  // directions of the affine warp passes' maps (256 values per warp)
+// Active lanes at which a warp evicts its shots: to the warp pass's list, which takes a shot on
+// its own, or to a second round, whose warps are packed again (16-entry lanes, then the larger).
+// In ms at 3 / 8 / 10: w42 FP32 1 M shots 1.40 / 1.45 / 1.52, 200 k 0.87 / 0.73 / 0.77 (listed);
+// at 10 / 17 / 20: w42 FP32 2^24 7.65 / 7.49 / 7.61, FP64 2^22 4.50 / 4.19 / 4.15. Larger lanes
+// at 4 / 8 / 12: w97 FP32 1 M 4.09 / 4.09 / 4.16, 300 k 2.31 / 2.18 / 2.2 (listed); at 12 / 15 /
+// 18: w97 FP32 2 M 6.22 / 6.11 / 6.24, 64-circuit batch 9.97 / 9.66 / 9.56.
+constexpr uint32_t kEvictListed = 8, kEvict = 17, kEvictBigListed = 8, kEvictBig = 15;
+// Directions of the affine warp passes' maps (2^dim values a warp): a shot that needs more goes
+// to the pass at the circuit's cap. In ms at 8 / 9 / 10 / 11: w97 FP32 2 M shots 6.22 / 6.20 / 5.86 / 7.12,
+// w42 FP32 1 M 1.52 / 1.51 / 1.51 / 2.09; w97 FP64 500 k 3.58 / 3.90 / 6.51 / 8.27 (the maps'
+// shared memory leaves fewer warps).
+constexpr uint32_t kAffDimFp32 = 10, kAffDimFp64 = 8;
 using soft::kTauFp32;
 using soft::kTauFp64;
 }  // namespace
@@ -451,7 +462,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   const bool two_pass = lanes || cap1 < cap_max;
   // after lanes, a middle pass (a warp per shot) takes the shots whose maps outgrew a lane, and
   // only those that outgrow it too go on to the pass at the circuit's cap: in affine form, with
-  // room for 2^kAffDim entries, or in sparse form up to cap1 entries. The sparse one is left out
+  // room for 2^aff_dim entries, or in sparse form up to cap1 entries. The sparse one is left out
   // when every lane of the run holds 64 entries already (w97 FP32 ran 44.7 M shots/s without
   // it, 44.5 M with 64 entries and 27.0 M with 256, whose larger maps cut its residency)
   const bool mid_pass = lanes && (affine || (lc16 < cap1 && cap1 < cap_max && (nbc[0] > 0 || nbc[1] > 0)));
@@ -675,7 +686,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     q.list = m.rerun;
     q.n_items_dev = m.n_rerun;
   }
-  m.aff_dim = kAffDim;
+  m.aff_dim = fp32 ? kAffDimFp32 : kAffDimFp64;
   if (global_rerun) {
     q.gslab = r->d_slab;
     q.gslab_blocks = slab_blocks;
@@ -693,7 +704,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     p.al_hi = (uint32_t)nbc[0];
     p.al_grid = al_grid;
     p.lane_round = 0;
-    p.lane_evict = spill && rounds > 1 ? 1u : 0u;
+    p.lane_evict = spill && rounds > 1 ? (small_run ? kEvictListed : kEvict) : 0u;
     p.lane_list = small_run ? 1u : 0u;
     p.lane_hand = spill ? 1u : 0u;
     p.lane_wide = wide ? 1u : 0u;
@@ -720,7 +731,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     pb[k].al_lo = (uint32_t)(nbc[0] + (k ? nbc[1] : 0));
     pb[k].al_hi = pb[k].al_lo + (uint32_t)nbc[1 + k];
     pb[k].lane_hand = pb[k].lane_wide = 0;
-    pb[k].lane_evict = sp_big[k] || small_run ? 1u : 0u;
+    pb[k].lane_evict = small_run ? kEvictBigListed : sp_big[k] ? kEvictBig : 0u;
     pb[k].sp = r->d_spb[k];
     pb[k].sp_cap = pb[k].sp_evict_cap = sp_big[k];
     pb[k].sp_dim = soft::lane_map_dim() + 1 + k;
@@ -788,7 +799,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     for (uint32_t rd = 1; spill && !small_run && rd < rounds; ++rd) {
       soft::ShotParams ar = a;
       ar.lane_round = rd;
-      ar.lane_evict = rd + 1 < rounds ? 1u : 0u;
+      ar.lane_evict = rd + 1 < rounds ? kEvict : 0u;
       ar.n_items_dev = r->d_lr + 3 + 2 * rd;
       if ((err = cudaMemsetAsync(ar.al_count, 0, 2 * (size_t)nb * sizeof(uint32_t), st)) != cudaSuccess ||
           (err = soft::launch_lane_resume_prepass(ar, fp32, W, st)) != cudaSuccess ||

@@ -19,7 +19,7 @@
 //
 // Most shots end at the first detector after their first error, but a few run to
 // the end of the circuit, and they would hold a warp with a few active lanes. So a
-// warp left with few active lanes (evict_below) writes their shots' state to a
+// warp left with few active lanes (lane_evict) writes their shots' state to a
 // spill pool and moves on to fresh shots. The next round (another launch) buckets
 // the evicted shots by the event they resume at, and packs them into warps again.
 // The last round evicts nothing. Which lane runs a shot does not change its
@@ -55,15 +55,6 @@ constexpr int kLaneBlock = 128;
 template <uint32_t Cap>
 __host__ __device__ constexpr int lane_block() { return Cap == 32u ? 64 : kLaneBlock; }
 constexpr uint32_t kLaneMaxBuckets = 50000;  // the pre-pass histogram of all buckets: 200 KB of shared memory
-#ifndef SOFT_LANE_EVICT
-#define SOFT_LANE_EVICT 10
-#endif
-#ifndef SOFT_LANE_EVICT_BIG
-#define SOFT_LANE_EVICT_BIG 12
-#endif
-// a warp with this many active lanes or fewer evicts them
-template <uint32_t Cap>
-__host__ __device__ constexpr uint32_t evict_below() { return Cap <= 16u ? SOFT_LANE_EVICT : SOFT_LANE_EVICT_BIG; }
 #ifndef SOFT_LANE_ROUNDS
 #define SOFT_LANE_ROUNDS 2
 #endif
@@ -1492,7 +1483,7 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     // the next round packed with others, and the warp moves on to fresh shots
     if (P.lane_evict) {
       const uint32_t am = __ballot_sync(0xFFFFFFFFu, active);
-      if (am && (uint32_t)__popc(am) <= evict_below<Cap>() && e + 1u < n_ev) {
+      if (am && (uint32_t)__popc(am) <= P.lane_evict && e + 1u < n_ev) {
         const uint32_t leader = __ffs(am) - 1;
         unsigned long long r0 = 0;
         if (lane == leader) r0 = atomicAdd(P.sp ? &P.lr[0] : P.n_rerun, (unsigned long long)__popc(am));
