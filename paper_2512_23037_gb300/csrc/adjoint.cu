@@ -1373,6 +1373,7 @@ struct GradWarp {
     const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(P.ev);
     uint32_t ev = 0;
     for (; ev <= P.n_events; ++ev) {
+      prefetch_events<W>(evs, P.coef, P.cb, ev, P.n_events, lane);
       save_snapshot(snaps + (size_t)ev * stride);
       if (ev == P.n_events) break;
       const uint32_t w0 = __ldg(&evs[ev].w0), type = ev_type(w0);

@@ -190,6 +190,30 @@ __device__ __forceinline__ void copy_async(void *shared, const void *global) {
                "l"(global), "n"(Bytes)
                : "memory");
 }
+// A hint to bring the line that holds global address p into L1.
+__device__ __forceinline__ void prefetch_line(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+// For a warp that walks the events on its own (the noiseless runs): event `ev` is next. Once per
+// 32 events the lanes ask for the ones after the next 32, an event each, and for the coefficients
+// and case-B constants of those, so that the walk finds them in L1: the loads of a lone warp were
+// a third of its time (with cold caches, w42's noiseless run in FP64 454 -> 389 us, the
+// gradient's 404 -> 329; the events alone gained nothing, each case-B measurement's constants
+// were the long waits).
+template <int W>
+__device__ __forceinline__ void prefetch_events(const Ev<W> *evs, const Coef *coef, const CaseB *cb, uint32_t ev, uint32_t n_events, uint32_t lane) {
+  if (ev & 31u) return;
+  for (uint32_t k = ev ? ev + 32u + lane : lane; k < n_events && k < ev + 64u; k += 32) {
+    const unsigned char *q = reinterpret_cast<const unsigned char *>(evs + k);
+    prefetch_line(q);
+    prefetch_line(q + sizeof(Ev<W>) - 16);
+    const uint32_t type = ev_type(__ldg(&evs[k].w0));
+    if (type == EV_ROT || type == EV_ROT_DIAG) prefetch_line(coef + __ldg(&evs[k].a));
+    if (type == EV_MEAS_B) {
+      const unsigned char *c = reinterpret_cast<const unsigned char *>(cb + (uint32_t)__ldg(&evs[k].beta[0]));
+      for (uint32_t o = 0; o < sizeof(CaseB); o += 128) prefetch_line(c + o);
+      prefetch_line(c + sizeof(CaseB) - 16);
+    }
+  }
+}
 __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <int W>

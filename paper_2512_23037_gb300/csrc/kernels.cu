@@ -950,6 +950,7 @@ struct Shot {
     const uint32_t n_events = C->n_events;
     uint32_t ev = 0, fs = n_events, mx = 0;
     for (; ev <= n_events; ++ev) {
+      prefetch_events<W>(evs, C->coef, C->cb, ev, n_events, lane);
       save_snapshot(out + (size_t)ev * stride);
       mx = nnz > mx ? nnz : mx;
       if (ev == n_events) break;

@@ -985,12 +985,15 @@ struct LaneShot {
 };
 
 // ---- the affine form (SnapAffine) of every valid snapshot of a noiseless run (events
-// [0, stop[0]]), one thread per snapshot, once per compiled circuit and precision; the
-// largest dimension goes to stop[3] (0xFF where a map needs more than kSnapDim)
+// [0, stop[0]]), a warp per snapshot, once per compiled circuit and precision; the
+// largest dimension goes to stop[3] (0xFF where a map needs more than kSnapDim). Each direction is
+// found by all keys at once, their residuals in registers, two a lane (w42 FP64 26 -> 5.6 us, w97
+// 77 -> 7.8 against a thread per snapshot with its rows in local memory).
 template <typename R, int W>
-__global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_t stride, uint32_t rw,
-                                   uint32_t *stop, const void *ev) {
-  const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128) snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_t stride, uint32_t rw,
+                                                          uint32_t *stop, const void *ev) {
+  static_assert(kSnapMax == 64, "two keys a lane");
+  const uint32_t e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u;
   if (e >= n_snap || e > stop[0]) return;
   unsigned char *in = traj + (size_t)e * stride;
   const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
@@ -998,59 +1001,81 @@ __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_
   const Cx<R> *v_in = reinterpret_cast<const Cx<R> *>(k_in + kSnapMax * W);
   SnapAffine<R, W> *out = reinterpret_cast<SnapAffine<R, W> *>(in + snap_affine_off<R, W>(rw));
   const uint32_t n = h->nnz < kSnapMax ? h->nnz : kSnapMax;
-  constexpr uint32_t kB = 1, kD = 1 + kSnapDim;
-  uint64_t rw_[1 + 2 * kSnapDim][W];
-  for (uint32_t r = 0; r < 1 + 2 * kSnapDim; ++r)
-    for (int w = 0; w < W; ++w) rw_[r][w] = 0ull;
-  for (uint32_t j = 0; j < (1u << kSnapDim); ++j) out->v[j] = Cx<R>{0, 0};
   Cx<R> turn{(R)1, (R)0};  // FP64: the circuit's global phase is taken out (scaled maps)
   if constexpr (sizeof(R) == 8) turn = phase_of(e ? (16u - ev_phase(reinterpret_cast<const Ev<W> *>(ev)[e - 1u].w0)) & 15u : 0u);
-  uint32_t d = 0;
-  unsigned long long live = 0;
-  bool ok = true;
-  if (n) {
-    for (int w = 0; w < W; ++w) rw_[0][w] = k_in[w];
+  uint64_t a0[W], B[kSnapDim][W], D[kSnapDim][W], r[2][W];  // r: the keys' residuals
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    a0[w] = n ? k_in[w] : 0ull;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) r[i][w] = lane + 32u * i < n ? k_in[(lane + 32u * i) * W + w] ^ a0[w] : 0ull;
   }
-  for (uint32_t i = 0; i < n && ok; ++i) {
-    uint64_t x[W], r[W];
-    for (int w = 0; w < W; ++w) r[w] = x[w] = k_in[i * W + w] ^ rw_[0][w];
-    uint32_t c = 0;
-    for (uint32_t k = 0; k < d; ++k)
-      if (wpar<W>(rw_[kD + k], x)) {
-        c |= 1u << k;
-        for (int w = 0; w < W; ++w) r[w] ^= rw_[kB + k][w];
-      }
-    if (wnonzero<W>(r)) {
-      if (d == kSnapDim) {
-        ok = false;
-        break;
-      }
-      const uint32_t p = wlow<W>(r);  // the new direction's dual (as in LaneShot::add_dim)
-      uint64_t z[W];
-      for (int w = 0; w < W; ++w) z[w] = ((int)(p >> 6) == w) ? (1ull << (p & 63u)) : 0ull;
-      for (uint32_t k = 0; k < d; ++k)
-        if (wbit<W>(rw_[kB + k], p))
-          for (int w = 0; w < W; ++w) z[w] ^= rw_[kD + k][w];
-      for (int w = 0; w < W; ++w) {
-        rw_[kB + d][w] = r[w];
-        rw_[kD + d][w] = z[w];
-      }
-      c |= 1u << d;
-      ++d;
+  uint32_t d = 0, c[2] = {0, 0};
+  bool done = false, ok = true;
+  // the first key outside the span, in the map's order, is the next direction
+#pragma unroll
+  for (uint32_t j = 0; j <= kSnapDim; ++j) {
+    const uint32_t m0 = __ballot_sync(0xFFFFFFFFu, wnonzero<W>(r[0])), m1 = __ballot_sync(0xFFFFFFFFu, wnonzero<W>(r[1]));
+    const uint32_t m = m0 ? m0 : m1, src = m ? 31u - (uint32_t)__clz((int)(m & (0u - m))) : 0u;
+    done = done || !m;
+    if (j == kSnapDim) {
+      ok = done;
+      break;
     }
-    out->v[c] = sizeof(R) == 8 ? cmul(turn, v_in[i]) : v_in[i];
-    live |= 1ull << c;
+    uint64_t x[W], z[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) x[w] = __shfl_sync(0xFFFFFFFFu, (unsigned long long)(m0 ? r[0][w] : r[1][w]), src);
+    const uint32_t p = done ? 0u : wlow<W>(x);  // its dual (as in LaneShot::add_dim)
+#pragma unroll
+    for (int w = 0; w < W; ++w) z[w] = !done && (int)(p >> 6) == w ? 1ull << (p & 63u) : 0ull;
+#pragma unroll
+    for (uint32_t k = 0; k < j; ++k)
+      if (!done && wbit<W>(B[k], p))
+#pragma unroll
+        for (int w = 0; w < W; ++w) z[w] ^= D[k][w];
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      B[j][w] = x[w];  // (zero once done)
+      D[j][w] = z[w];
+    }
+    d += done ? 0u : 1u;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)  // (residuals lie outside the span so far: its duals are zero on them)
+      if (wpar<W>(z, r[i])) {
+        c[i] |= 1u << j;
+#pragma unroll
+        for (int w = 0; w < W; ++w) r[i][w] ^= x[w];
+      }
   }
-  for (uint32_t r = 0; r < 1 + 2 * kSnapDim; ++r)
-    for (int w = 0; w < W; ++w) out->rows[r][w] = rw_[r][w];
-  out->d = ok ? d : 0xFFFFFFFFu;
-  out->live_lo = (uint32_t)live;
-  out->live_hi = (uint32_t)(live >> 32);
-  atomicMax(&stop[3], ok ? d : 0xFFu);
+  uint32_t live[2] = {0, 0};
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    out->v[lane + 32u * i] = Cx<R>{0, 0};
+    if (lane + 32u * i < n) live[c[i] >> 5] |= 1u << (c[i] & 31u);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (lane + 32u * i < n) out->v[c[i]] = sizeof(R) == 8 ? cmul(turn, v_in[lane + 32u * i]) : v_in[lane + 32u * i];
+  const uint32_t lo = __reduce_or_sync(0xFFFFFFFFu, live[0]), hi = __reduce_or_sync(0xFFFFFFFFu, live[1]);
+  if (lane == 0) {
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      out->rows[0][w] = a0[w];
+#pragma unroll
+      for (uint32_t k = 0; k < kSnapDim; ++k) {
+        out->rows[1 + k][w] = B[k][w];
+        out->rows[1 + kSnapDim + k][w] = D[k][w];
+      }
+    }
+    out->d = ok ? d : 0xFFFFFFFFu;
+    out->live_lo = lo;
+    out->live_hi = hi;
+    atomicMax(&stop[3], ok ? d : 0xFFu);
+  }
 }
 
-// ---- the fate of each site's errors, one thread per site and Pauli pair, once per compiled
-// circuit and precision.
+// ---- the fate of each site's errors, once per compiled circuit and precision.
 // Before its first error a shot is the noiseless run. An error E commutes past every event that
 // leaves it alone: a rotation whose generator commutes with it, a decided measurement whose
 // outcome it does not flip (its corrections commuting with E too), a parity of unflipped
@@ -1063,60 +1088,86 @@ __global__ void snap_affine_kernel(unsigned char *traj, uint32_t n_snap, uint32_
 // are carried to the earlier of their events (start_event).
 // Entry: that event (at most the recorded run's last), kFateDiscard, and E's phase i^e relative to
 // the signed rows, which the Clifford gates in between leave as it is.
+// A warp takes a site and tests 32 events at once, a lane each: whether the event leaves an error
+// alone is linear in its generators' images, so one look at an event serves all 15 pairs (w42: 70 ->
+// 15 us against a thread per site and pair that walks event by event, each step a load's latency;
+// w97 141 -> 46).
 template <int W>
 __global__ void __launch_bounds__(128) fate_kernel(const __grid_constant__ CircDev C, const uint32_t *stop_at, uint32_t *out) {
-  const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x, s = idx >> 4, pp = idx & 15u;
+  const uint32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u, pp = lane & 15u;
   if (s >= C.n_sites) return;
   const SiteDev<W> *S = reinterpret_cast<const SiteDev<W> *>(C.sites) + s;
-  uint32_t e = __ldg(&C.site_ev[s]);
-  const uint32_t stop = *stop_at < C.n_events ? *stop_at : C.n_events;
-  if (e > stop || pp == 0u || ((__ldg(&S->kind) & 3u) != SITE_DEPOL2 && (pp & 3u))) {  // (not an error, or never used)
-    out[idx] = e;
-    return;
-  }
-  const SnapHdr *h = reinterpret_cast<const SnapHdr *>(C.traj + (size_t)e * C.traj_stride);
-  uint64_t b[W], g[W], sd[W], ss[W];
-#pragma unroll
-  for (int w = 0; w < W; ++w) {
-    sd[w] = h->sd[w];
-    ss[w] = h->ss[w];
-  }
-  const uint32_t ph = site_pauli<W>(&C, s, pp, sd, ss, b, g);
-  const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C.ev);
-  uint32_t kind = 0;
-  for (; e < stop; ++e) {
-    const Ev<W> *E = evs + e;
-    const uint32_t w0 = __ldg(&E->w0), type = ev_type(w0), flags = ev_flags(w0);
-    uint64_t be[W], ga[W];
+  const uint32_t at = __ldg(&C.site_ev[s]), stop = *stop_at < C.n_events ? *stop_at : C.n_events;
+  // lane pp: its pair's event and kind, and the errors' phase (others are no errors, or never used)
+  const bool error = lane < 16u && pp && ((__ldg(&S->kind) & 3u) == SITE_DEPOL2 || !(pp & 3u)) && at <= stop;
+  uint32_t e = error ? stop : at, kind = 0;
+  if (error) {
+    const SnapHdr *h = reinterpret_cast<const SnapHdr *>(C.traj + (size_t)at * C.traj_stride);
+    uint64_t b[W], g[W], sd[W], ss[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      be[w] = __ldg(&E->beta[w]);
-      ga[w] = __ldg(&E->gamma[w]);
+      sd[w] = h->sd[w];
+      ss[w] = h->ss[w];
     }
-    if (type == EV_ROT || type == EV_ROT_DIAG) {
-      if (wpar2<W>(be, g, ga, b)) break;  // E anticommutes with the generator
-    } else if (type == EV_MEAS_A) {
-      if (wpar<W>(ga, b)) {  // E flips the outcome
-        if (flags & F_DETECTOR) kind = kFateDiscard;
-        break;
+    kind = site_pauli<W>(&C, s, pp, sd, ss, b, g) << 30;
+  }
+  uint64_t img[4][2 * W];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w) img[j][w] = __ldg(&S->img[j][w]);
+  const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(C.ev);
+  uint32_t open = __ballot_sync(0xFFFFFFFFu, error);
+  for (uint32_t base = at; base < stop && open; base += 32) {
+    const uint32_t k = base + lane;
+    uint32_t flip = 0, turn = 0;  // per generator: it anticommutes with the event, with its correction
+    bool halt = false, ends = false;
+    if (k < stop) {
+      const Ev<W> *E = evs + k;
+      const uint32_t w0 = __ldg(&E->w0), type = ev_type(w0), flags = ev_flags(w0);
+      uint64_t be[W], ga[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        be[w] = __ldg(&E->beta[w]);
+        ga[w] = __ldg(&E->gamma[w]);
       }
-      if (flags & F_COND_LAST) {
-        const SnapHdr *hn = reinterpret_cast<const SnapHdr *>(C.traj + (size_t)(e + 1u) * C.traj_stride);
-        if ((int)hn->lastm == -1) {  // the noiseless run applies the correction
+      if (type == EV_ROT || type == EV_ROT_DIAG) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) flip |= wpar2<W>(be, img[j] + W, ga, img[j]) << j;
+      } else if (type == EV_MEAS_A) {
+        ends = (flags & F_DETECTOR) != 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) flip |= wpar<W>(ga, img[j]) << j;
+        if ((flags & F_COND_LAST) &&  // the noiseless run applies the correction
+            (int)reinterpret_cast<const SnapHdr *>(C.traj + (size_t)(k + 1u) * C.traj_stride)->lastm == -1) {
           uint64_t xb[W], xg[W];
 #pragma unroll
           for (int w = 0; w < W; ++w) {
             xb[w] = __ldg(&E->xbeta[w]);
             xg[w] = __ldg(&E->xgamma[w]);
           }
-          if (wpar2<W>(xb, g, xg, b)) break;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) turn |= wpar2<W>(xb, img[j] + W, xg, img[j]) << j;
         }
+      } else {
+        halt = type != EV_PARITY && type != EV_END;
       }
-    } else if (type != EV_PARITY && type != EV_END) {
-      break;
+    }
+    for (uint32_t m = open; m; m &= m - 1u) {
+      const uint32_t q = 31u - (uint32_t)__clz((int)(m & (0u - m))), need = site_images(q);
+      const bool f = (__popc(flip & need) & 1) != 0;
+      const uint32_t hit = __ballot_sync(0xFFFFFFFFu, halt || f || (__popc(turn & need) & 1)), end = __ballot_sync(0xFFFFFFFFu, ends && f);
+      if (hit) {
+        const uint32_t first = hit & (0u - hit);
+        if (lane == q) {
+          e = base + (31u - (uint32_t)__clz((int)first));
+          kind |= (end & first) ? kFateDiscard : 0u;
+        }
+        open &= ~(1u << q);
+      }
     }
   }
-  out[idx] = e | kind | (ph << 30);
+  if (lane < 16u) out[(size_t)s * 16 + pp] = e | kind;
 }
 
 // ---- bucketing pre-pass. Buckets: per circuit of the run, one per event plus one
@@ -1581,7 +1632,7 @@ uint32_t lane_first_cap(uint32_t max_n, uint32_t max_d, int fp32) {
 
 cudaError_t launch_snap_affine(unsigned char *traj, uint32_t n_snap, uint32_t rw, int fp32, uint32_t W,
                                uint32_t *stop, const void *ev, cudaStream_t st) {
-  const unsigned grid = (n_snap + 127) / 128;
+  const unsigned grid = (n_snap + 3) / 4;
   if (fp32) {
     if (W == 1) snap_affine_kernel<float, 1><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<float, 1>(rw), rw, stop, ev);
     else snap_affine_kernel<float, 2><<<grid, 128, 0, st>>>(traj, n_snap, (uint32_t)snap_stride<float, 2>(rw), rw, stop, ev);
@@ -1593,7 +1644,7 @@ cudaError_t launch_snap_affine(unsigned char *traj, uint32_t n_snap, uint32_t rw
 }
 cudaError_t launch_fate(const CircDev &c, uint32_t W, const uint32_t *stop, uint32_t *fate, cudaStream_t st) {
   if (!c.n_sites) return cudaSuccess;
-  const unsigned grid = (unsigned)(((size_t)c.n_sites * 16 + 127) / 128);
+  const unsigned grid = (c.n_sites + 3u) / 4u;
   if (W == 1) fate_kernel<1><<<grid, 128, 0, st>>>(c, stop, fate);
   else fate_kernel<2><<<grid, 128, 0, st>>>(c, stop, fate);
   return cudaGetLastError();
