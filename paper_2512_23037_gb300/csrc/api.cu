@@ -45,6 +45,7 @@ constexpr uint32_t kEvictListed = 8, kEvict = 17, kEvictBigListed = 8, kEvictBig
 // w42 FP32 1 M 1.52 / 1.51 / 1.51 / 2.09; w97 FP64 500 k 3.58 / 3.90 / 6.51 / 8.27 (the maps'
 // shared memory leaves fewer warps).
 constexpr uint32_t kAffDimFp32 = 10, kAffDimFp64 = 8;
+constexpr uint64_t kSideRounds = 1ull << 21;  // see each_size in run_many
 using soft::kTauFp32;
 using soft::kTauFp64;
 }  // namespace
@@ -83,6 +84,9 @@ struct soft_run {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  // batches of several lane sizes: their launches run side by side (see each_size in run_many)
+  cudaStream_t side[2] = {nullptr, nullptr};
+  cudaEvent_t fork_ev = nullptr, join_ev[2] = {nullptr, nullptr};
   std::vector<cudaEvent_t> pass_ev;        // SOFT_RUN_TIME_PASSES: 4 per chunk around pre-pass, first, rerun
   uint32_t launches = 0;
   // every device buffer above that the run owns lives in one arena, borrowed from
@@ -325,6 +329,14 @@ void soft_run_free(soft_run *r) {
   if (!r) return;
   if (r->stream) cudaStreamSynchronize(r->stream);
   else cudaDeviceSynchronize();
+  for (int k = 0; k < 2; ++k) {
+    if (r->side[k]) {
+      cudaStreamSynchronize(r->side[k]);
+      cudaStreamDestroy(r->side[k]);
+    }
+    if (r->join_ev[k]) cudaEventDestroy(r->join_ev[k]);
+  }
+  if (r->fork_ev) cudaEventDestroy(r->fork_ev);
   // the arena goes back to the circuit's slot (unless the circuit is gone, or keeps a
   // larger one), else it is freed
   if (r->arena) {
@@ -749,6 +761,39 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     soft_run_free(r);
     return cuda_fail(e, "shot kernel configuration");
   }
+  // The lane sizes of a batch have circuits, buckets and spill pools of their own, and each round
+  // of each ends with a few warps that walk the last shots' events. So the sizes' launches run side
+  // by side: the first on the run's stream, the others on streams that start after it got here and
+  // that it waits for. FP32 batches, in ms, one after the other / side by side: 4 circuits of 30 k
+  // shots 1.31 / 0.80, 16 of 8 k 1.39 / 1.07, 32 of 60 k 5.63 / 4.63, 48 of 60 k 6.87 / 6.48, 64 of
+  // 8 k 3.57 / 3.77. The second rounds too up to kSideRounds shots: 24 circuits of 60 k 4.28 ->
+  // 3.63; but the largest batch has enough warps for each (64 circuits, 9.0 -> 9.8).
+  bool sized[3] = {lanes16, lanes && nbc[1] > 0, lanes && nbc[2] > 0};
+  for (int k = 0, n = -1; k < 3; ++k) {
+    if (!sized[k] || ++n == 0) continue;
+    if ((!r->fork_ev && (e = cudaEventCreateWithFlags(&r->fork_ev, cudaEventDisableTiming)) != cudaSuccess) ||
+        (e = cudaStreamCreateWithFlags(&r->side[n - 1], cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&r->join_ev[n - 1], cudaEventDisableTiming)) != cudaSuccess) {
+      soft_run_free(r);
+      return cuda_fail(e, "stream creation");
+    }
+  }
+  auto each_size = [&](bool par, auto &&launch) -> cudaError_t {
+    cudaError_t err = par && r->fork_ev ? cudaEventRecord(r->fork_ev, st) : cudaSuccess;
+    for (int k = 0, n = -1; k < 3; ++k) {
+      if (!sized[k]) continue;
+      cudaStream_t s = ++n && par ? r->side[n - 1] : st;
+      if (n && par && err == cudaSuccess) err = cudaStreamWaitEvent(s, r->fork_ev, 0);
+      if (err == cudaSuccess) err = launch(k, s);
+    }
+    for (int n = 0; n < 2; ++n) {  // (also after an error: nothing stays behind)
+      if (!r->side[n] || !par) continue;
+      cudaError_t je = cudaEventRecord(r->join_ev[n], r->side[n]);
+      if (je == cudaSuccess) je = cudaStreamWaitEvent(st, r->join_ev[n], 0);
+      if (err == cudaSuccess) err = je;
+    }
+    return err;
+  };
   cudaEventRecord(r->ev0, st);
   // one chunk of items [base, base + cnt): clear counters, first pass, rerun pass
   const bool time_passes = (o.flags & SOFT_RUN_TIME_PASSES) && !use_graph;
@@ -781,46 +826,52 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
       r->launches += al_grid > 1 ? 3 : 1;
     }
     if ((err = mark(lanes)) != cudaSuccess) return err;
-    if (!lanes || lanes16) {
+    if (!lanes) {
       if ((err = soft::launch_prepared(c1, a, st)) != cudaSuccess) return err;
       r->launches++;
+    } else if ((err = each_size(true, [&](int k, cudaStream_t s) -> cudaError_t {
+                  soft::ShotParams ab = k ? pb[k - 1] : a;
+                  ab.n_items = cnt;
+                  ab.item_base = base;
+                  if (dev_base) ab.item_base_dev = r->d_work + 3;
+                  r->launches++;
+                  return soft::launch_prepared(k ? cb[k - 1] : c1, ab, s);
+                })) != cudaSuccess) {
+      return err;
     }
-    // the larger lanes, before any later round re-buckets (it clears every bucket's counters)
-    for (int k = 0; lanes && k < 2; ++k)
-      if (nbc[1 + k]) {
-        soft::ShotParams ab = pb[k];
-        ab.n_items = cnt;
-        ab.item_base = base;
-        if (dev_base) ab.item_base_dev = r->d_work + 3;
-        if ((err = soft::launch_prepared(cb[k], ab, st)) != cudaSuccess) return err;
-        r->launches++;
-      }
-    // later rounds: the evicted shots, bucketed by the event they resume at
-    for (uint32_t rd = 1; spill && !small_run && rd < rounds; ++rd) {
+    // later rounds: the evicted shots of every size, bucketed by the event they resume at (the
+    // larger sizes have one such round)
+    for (uint32_t rd = 1; rd < rounds && !small_run; ++rd) {
       soft::ShotParams ar = a;
       ar.lane_round = rd;
-      ar.lane_evict = rd + 1 < rounds ? kEvict : 0u;
-      ar.n_items_dev = r->d_lr + 3 + 2 * rd;
+      ar.rs_n = 0;
+      auto pool = [&](const soft::ShotParams &q) {
+        ar.rs_sp[ar.rs_n] = q.sp;
+        ar.rs_lr[ar.rs_n] = q.lr;
+        ar.rs_dim[ar.rs_n] = q.sp_dim;
+        ar.rs_cap[ar.rs_n++] = q.sp_evict_cap;
+      };
+      if (spill) pool(a);
+      for (int k = 0; k < 2 && rd == 1; ++k)
+        if (sp_big[k]) pool(pb[k]);
+      if (!ar.rs_n) break;
       if ((err = cudaMemsetAsync(ar.al_count, 0, 2 * (size_t)nb * sizeof(uint32_t), st)) != cudaSuccess ||
-          (err = soft::launch_lane_resume_prepass(ar, fp32, W, st)) != cudaSuccess ||
-          (err = soft::launch_prepared(c1, ar, st)) != cudaSuccess)
+          (err = soft::launch_lane_resume_prepass(ar, fp32, W, st)) != cudaSuccess)
         return err;
-      r->launches += al_grid > 1 ? 5 : 2;
+      r->launches += al_grid > 1 ? 4 : 1;
+      err = each_size(cnt <= kSideRounds, [&](int k, cudaStream_t s) -> cudaError_t {
+        if (k ? rd > 1 || !sp_big[k - 1] : !spill) return cudaSuccess;
+        soft::ShotParams as = k ? pb[k - 1] : a;
+        as.item_base = base;
+        if (dev_base) as.item_base_dev = r->d_work + 3;
+        as.lane_round = rd;
+        as.lane_evict = !k && rd + 1 < rounds ? kEvict : 0u;
+        as.n_items_dev = as.lr + 3 + 2 * rd;
+        r->launches++;
+        return soft::launch_prepared(k ? cb[k - 1] : c1, as, s);
+      });
+      if (err != cudaSuccess) return err;
     }
-    for (int k = 0; lanes && k < 2; ++k)
-      if (sp_big[k]) {
-        soft::ShotParams ar = pb[k];
-        ar.item_base = base;
-        if (dev_base) ar.item_base_dev = r->d_work + 3;
-        ar.lane_round = 1;
-        ar.lane_evict = 0;
-        ar.n_items_dev = r->d_lrb[k] + 5;
-        if ((err = cudaMemsetAsync(ar.al_count, 0, 2 * (size_t)nb * sizeof(uint32_t), st)) != cudaSuccess ||
-            (err = soft::launch_lane_resume_prepass(ar, fp32, W, st)) != cudaSuccess ||
-            (err = soft::launch_prepared(cb[k], ar, st)) != cudaSuccess)
-          return err;
-        r->launches += al_grid > 1 ? 5 : 2;
-      }
     if (wide) {  // the handed-over shots, bucketed by the event they resume at
       soft::ShotParams aw = a;
       aw.lane_round = rounds;
@@ -829,6 +880,11 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
       aw.lane_hand = 0;
       aw.n_rerun_total = nullptr;  // (counted when they left the first rounds)
       aw.n_items_dev = r->d_lr + 3 + 2 * rounds;
+      aw.rs_n = 1;
+      aw.rs_sp[0] = aw.sp;
+      aw.rs_lr[0] = aw.lr;
+      aw.rs_dim[0] = aw.sp_dim;
+      aw.rs_cap[0] = aw.sp_evict_cap;
       if ((err = cudaMemsetAsync(aw.al_count, 0, 2 * (size_t)nb * sizeof(uint32_t), st)) != cudaSuccess ||
           (err = soft::launch_lane_resume_prepass(aw, fp32, W, st)) != cudaSuccess ||
           (err = soft::launch_prepared(cw, aw, st)) != cudaSuccess)

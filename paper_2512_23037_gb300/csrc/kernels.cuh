@@ -113,6 +113,12 @@ struct ShotParams {
   uint32_t aff_dim;           // affine_kernel: directions of a warp's map (2^aff_dim values)
   unsigned long long *lr;     // [0] eviction records taken, [1] handover records taken;
                               // round r >= 1: [2 + 2r] its first record, [3 + 2r] its count
+  // the resume pre-pass buckets the records of up to three pools at once (one per lane size, each
+  // with its own counters): pool k's records take the item numbers after those of pool k - 1
+  uint32_t rs_n;
+  uint32_t rs_dim[3], rs_cap[3];  // directions of its records' maps, records that evictions may take
+  unsigned char *rs_sp[3];
+  unsigned long long *rs_lr[3];
   CircDev circ[kMaxCirc];
 };
 

@@ -1231,10 +1231,25 @@ __device__ __forceinline__ void round_setup(const ShotParams &P) {
     P.lr[3 + 2 * r] = P.lr[1] < cap ? P.lr[1] : cap;
     return;
   }
-  const unsigned long long used = P.lr[0] < P.sp_evict_cap ? P.lr[0] : P.sp_evict_cap;
-  const unsigned long long first = r == 1 ? 0ull : P.lr[2 + 2 * (r - 1)] + P.lr[3 + 2 * (r - 1)];
-  P.lr[2 + 2 * r] = first;
-  P.lr[3 + 2 * r] = used > first ? used - first : 0ull;
+  for (uint32_t k = 0; k < P.rs_n; ++k) {
+    unsigned long long *lr = P.rs_lr[k];
+    const unsigned long long used = lr[0] < P.rs_cap[k] ? lr[0] : P.rs_cap[k];
+    const unsigned long long first = r == 1 ? 0ull : lr[2 + 2 * (r - 1)] + lr[3 + 2 * (r - 1)];
+    lr[2 + 2 * r] = first;
+    lr[3 + 2 * r] = used > first ? used - first : 0ull;
+  }
+}
+// the items of a resume pre-pass: the round's records of every pool
+__device__ __forceinline__ unsigned long long resumed_items(const ShotParams &P) {
+  unsigned long long n = 0;
+  for (uint32_t k = 0; k < P.rs_n; ++k) n += P.rs_lr[k][3 + 2 * P.lane_round];
+  return n;
+}
+// item i's pool; i becomes its number within the pool
+__device__ __forceinline__ uint32_t resumed_pool(const ShotParams &P, unsigned long long &i) {
+  uint32_t k = 0;
+  while (k + 1u < P.rs_n && i >= P.rs_lr[k][3 + 2 * P.lane_round]) i -= P.rs_lr[k++][3 + 2 * P.lane_round];
+  return k;
 }
 __global__ void lane_round_setup_kernel(const __grid_constant__ ShotParams P) { round_setup(P); }
 // ---- block-binned pre-pass: each block ranks its contiguous range of items per
@@ -1253,7 +1268,7 @@ __device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
   for (uint32_t k = threadIdx.x; k <= nb + (Resume ? 0u : P.n_circ); k += blockDim.x) hist[k] = 0u;
   __syncthreads();
   const unsigned long long n_items =
-      Resume ? P.lr[3 + 2 * P.lane_round] : (P.n_items_dev ? *P.n_items_dev : P.n_items);
+      Resume ? resumed_items(P) : (P.n_items_dev ? *P.n_items_dev : P.n_items);
   const unsigned long long per = (n_items + gridDim.x - 1) / gridDim.x;
   const unsigned long long i0 = blockIdx.x * per, i1 = i0 + per < n_items ? i0 + per : n_items;
   const unsigned long long base = P.item_base_dev ? *P.item_base_dev : P.item_base;
@@ -1261,8 +1276,10 @@ __device__ __forceinline__ void bin_items(const ShotParams &P, uint32_t *hist) {
     uint32_t e;
     const CircDev *C;
     if (Resume) {
-      const Spill<R, W> S(P.sp, P.rw_max, P.sp_dim);
-      const uint4 a = S.ha(S.at((uint32_t)(P.lr[2 + 2 * P.lane_round] + i)));
+      unsigned long long j = i;
+      const uint32_t k = resumed_pool(P, j);
+      const Spill<R, W> S(P.rs_sp[k], P.rw_max, P.rs_dim[k]);
+      const uint4 a = S.ha(S.at((uint32_t)(P.rs_lr[k][2 + 2 * P.lane_round] + j)));
       C = &P.circ[circ_of_item(P, base + a.x)];
       e = a.y < C->n_events ? a.y : C->n_events;  // a record always resumes at an event of its circuit
     } else {
@@ -1330,7 +1347,7 @@ template <bool Resume>
 __device__ __forceinline__ void scatter_items(const ShotParams &P) {
   const uint32_t nb = P.al_nb;
   const unsigned long long n_items =
-      Resume ? P.lr[3 + 2 * P.lane_round] : (P.n_items_dev ? *P.n_items_dev : P.n_items);
+      Resume ? resumed_items(P) : (P.n_items_dev ? *P.n_items_dev : P.n_items);
   const unsigned long long per = (n_items + gridDim.x - 1) / gridDim.x;
   const unsigned long long i0 = blockIdx.x * per, i1 = i0 + per < n_items ? i0 + per : n_items;
   for (unsigned long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
@@ -1342,8 +1359,11 @@ __device__ __forceinline__ void scatter_items(const ShotParams &P) {
       continue;
     }
     const uint32_t at = P.al_start[er.x] + P.al_base[(size_t)blockIdx.x * (nb + 1) + er.x] + er.y;
-    if (Resume) P.al_order[at] = (uint32_t)i;
-    else {
+    if (Resume) {
+      unsigned long long j = i;
+      resumed_pool(P, j);
+      P.al_order[at] = (uint32_t)j;
+    } else {
       const uint4 k = reinterpret_cast<const uint4 *>(P.al_cursor)[i];
       reinterpret_cast<uint4 *>(P.al_rec)[at] = make_uint4(k.x, k.y, k.z, (uint32_t)i);
     }
