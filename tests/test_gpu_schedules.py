@@ -122,15 +122,15 @@ def test_batch_of_every_lane_size(soft, precision, shots, graph):
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
-@pytest.mark.parametrize("cap", [16, 256, 2048])
-def test_affine_maps_at_their_limits(soft, precision, cap):
+@pytest.mark.parametrize("cap,first_cap", [(16, 0), (256, 0), (2048, 0), (2048, 64)])
+def test_affine_maps_at_their_limits(soft, precision, cap, first_cap):
     """Maps that outgrow the lanes, the affine warps (1024 values in FP32, 256
     in FP64: the pass at the cap takes over) and the cap."""
     S = soft
     circ, noise = C.windowed(31, n_data=32, n_anc=4, blocks=4, w=6, p=1e-2)
     n = 1200
     c = S.soft_compile_circuit(circ.array(), circ.n, noise, cap)
-    r = S.soft_run_shots(c, n, 0, 6, precision=precision, record_mode=S.REC_ALL)
+    r = S.soft_run_shots(c, n, 0, 6, precision=precision, record_mode=S.REC_ALL, first_cap=first_cap)
     rec, st = S.soft_get_records(r, n)
     ref = oracle.run(circ, circ.n, noise, cap, 6, 0, n, threads=8)
     assert compare_records(circ, noise, 6, 0, rec, st, ref, precision) <= 1 + n // 500
