@@ -179,10 +179,13 @@ typedef struct {
  * own shot's map (up to 16 entries, whose keys a lane keeps as an affine space
  * of at most 4 directions). A shot whose map outgrows its lane is
  * handed over at that event (its whole state in a spill record): to the wide
- * round's lanes (see below), or to a warp with a register map of up to
- * first_cap entries (default 64); shots beyond that rerun from their start at
- * the circuit's cap. A warp left with few active lanes moves their shots to a
- * second round that packs them into full warps again. In a
+ * round's lanes (see below), or to a warp (with its map in the same form, of up
+ * to 1024 values in FP32 and 256 in FP64; of up to first_cap entries where the
+ * caller sets first_cap or groups_per_block); shots beyond that rerun from
+ * their start at the circuit's cap. A warp left with few active lanes moves
+ * their shots to a second round that packs them into full warps again, or in
+ * small runs to the warps. Shots that their first errors discard end before
+ * any of this. In a
  * batch each circuit has its own buckets, and a warp serves one circuit at a
  * time. It applies to runs without a forced group size (state capture
  * included: a captured shot's state is written wherever it ends), to
@@ -190,8 +193,8 @@ typedef struct {
  * at most 50 000 events (plus one per circuit) together; otherwise a warp
  * (group) runs each shot. A circuit whose noiseless maps need more than 16
  * entries or 4 directions gets lanes of 32 entries (5 directions) or, with
- * SOFT_FP32 coefficients, of 64 (6 directions): these neither hand over nor
- * evict, and a shot that outgrows one reruns from its start in a warp. The
+ * SOFT_FP32 coefficients, of 64 (6 directions): these do not hand over, and a
+ * shot that outgrows one reruns from its start in a warp. The
  * shots of a batch's other circuits go straight to the warp pass.
  * SOFT_RUN_NO_LANES always uses the warp per shot. Same results either way,
  * another order. */
@@ -199,8 +202,8 @@ typedef struct {
  * (ignored with SOFT_RUN_GRAPH), read back by soft_run_pass_timing. */
 /* The wide round (single-circuit runs; batches never use it): shots whose map
  * outgrows a lane continue in lanes of twice the map before any warp. By
- * default it runs for chunks of at least 2^21 shots (SOFT_FP64: 2^22);
- * SOFT_RUN_WIDE_LANES runs it for any chunk, SOFT_RUN_NO_WIDE_LANES never.
+ * default it runs for chunks of more than 2^20 shots; SOFT_RUN_WIDE_LANES runs
+ * it for any chunk, SOFT_RUN_NO_WIDE_LANES never.
  * Same results either way. */
 enum { SOFT_RUN_GRAPH = 1, SOFT_RUN_FIDELITY = 2, SOFT_RUN_NO_PREFIX = 4, SOFT_RUN_NO_LANES = 8,
        SOFT_RUN_TIME_PASSES = 16, SOFT_RUN_NO_WIDE_LANES = 32, SOFT_RUN_WIDE_LANES = 64 };

@@ -227,8 +227,8 @@ def soft_run_shots(circ: Circuit, n_shots: int, first_shot: int = 0, seed: int =
     the first event instead of from the shared noiseless prefix, lanes=False a
     warp per shot instead of a lane per shot where that applies (same results).
     time_passes=True records events between passes for soft_run_pass_timing.
-    wide: None runs the wide round (single-circuit runs) for chunks of at least
-    2^21 shots (FP64: 2^22), True for any chunk, False never."""
+    wide: None runs the wide round (single-circuit runs) for chunks of more
+    than 2^20 shots, True for any chunk, False never."""
     o = _opts(precision, record_mode, record_k, stream, group_size, blocks_per_sm, chunk_shots, first_cap,
               capture_k, d_records, d_status, groups_per_block, graph, fidelity, prefix, lanes, time_passes, wide)
     out = ctypes.c_void_p()

@@ -40,6 +40,15 @@ constexpr uint64_t kSmallRun = 1ull << 20;
 // at 4 / 8 / 12: w97 FP32 1 M 4.09 / 4.09 / 4.16, 300 k 2.31 / 2.18 / 2.2 (listed); at 12 / 15 /
 // 18: w97 FP32 2 M 6.22 / 6.11 / 6.24, 64-circuit batch 9.97 / 9.66 / 9.56.
 constexpr uint32_t kEvictListed = 8, kEvict = 17, kEvictBigListed = 8, kEvictBig = 15;
+// Sixteenths of a lane launch's warps after whose end the others list all their shots for the warp
+// pass (a launch ends with a few warps that walk the last shots' events, a step as slow as a
+// lane's loops, while the rest of the chip idles). Without / with, in ms: 16-entry lanes of small
+// runs at 15: random 40-qubit circuit 200 k shots 1.45 / 1.30, 100 k 0.97 / 0.71, w42 FP32 1 M 1.46
+// / 1.34, 40 k 0.65 / 0.36, FP64 20 k 0.63 / 0.35 (at 8: random 1.57); larger lanes of small runs at
+// 12, whose shots start again: w97 FP32 400 k 2.22 / 2.03, 20 k 1.00 / 0.65; the second round at 8:
+// w42 FP32 1.5 M 1.98 / 1.66, FP64 2.34 / 2.09; the wide round at 8, whose shots go on from their
+// hand-over: w42 FP32 4 M 2.62 / 2.46, 2^24 7.37 / 7.25, FP64 2^22 4.18 / 3.96.
+constexpr uint32_t kTailListed = 15, kTailBigListed = 12, kTailRound = 8, kTailWide = 8;
 // Directions of the affine warp passes' maps (2^dim values a warp): a shot that needs more goes
 // to the pass at the circuit's cap. In ms at 8 / 9 / 10 / 11: w97 FP32 2 M shots 6.22 / 6.20 / 5.86 / 7.12,
 // w42 FP32 1 M 1.52 / 1.51 / 1.51 / 2.09; w97 FP64 500 k 3.58 / 3.90 / 6.51 / 8.27 (the maps'
@@ -69,7 +78,7 @@ struct soft_run {
   bool fid_mode = false;
   unsigned long long *d_once = nullptr;    // d_tally, d_work and d_fsum
   unsigned long long *d_work = nullptr;    // [3] item_base, [4..7] diag, [8] reruns of all chunks
-  unsigned long long *d_chunk = nullptr;   // per chunk: next1, next2, n_rerun, middle pass's next and n_rerun;
+  unsigned long long *d_chunk = nullptr;   // per chunk: next1, next2, n_rerun, middle pass's next and n_rerun, ended warps of 5 launches;
                                            // from [8] the lane rounds' ranges, then the bucket counters
   uint32_t *d_rerun = nullptr;
   unsigned char *d_slab = nullptr;         // global-memory state for large-cap reruns
@@ -546,11 +555,11 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   // the wide round: the handed-over shots continue in lanes of twice the map (their records
   // are its input), and only those that outgrow it rerun in a warp. Single-circuit runs only
   // (batches measured slower: 125.5 M against 130.3 M shots/s on batch64, before the affine
-  // lanes). By default only for the chunks it gains on: it costs a pre-pass and a launch more.
-  // With it / without, w42: FP32 2 M shots 2.26 / 2.51 ms, 8 M 4.87 / 6.45, 16 M 8.44 / 11.9;
-  // FP64 2 M 3.11 / 3.05, 4 M 4.77 / 5.2, 8 M 8.07 / 9.12.
+  // lanes). By default only for chunks above kSmallRun: it costs a pre-pass and a launch more.
+  // With it / without, w42: FP32 1 M shots 1.36 / 1.32 ms, 2 M 1.68 / 1.95, 8 M 3.99 / 5.78, 16 M
+  // 7.18 / 11.0; FP64 2 M 2.38 / 2.57, 4 M 3.86 / 4.54, 16 M 12.7 / 16.2.
   const bool wide_ok = spill && lane_grow && n_circ == 1 && !(o.flags & SOFT_RUN_NO_WIDE_LANES);
-  const bool wide = wide_ok && ((o.flags & SOFT_RUN_WIDE_LANES) || std::min(chunk, total) >= (1ull << (fp32 ? 21 : 22)));
+  const bool wide = wide_ok && ((o.flags & SOFT_RUN_WIDE_LANES) || std::min(chunk, total) > kSmallRun);
   if (spill) need(&r->d_sp, soft::lane_spill_bytes(fp32, W, rw_max, sp_evict + sp_hand, soft::lane_map_dim()));
   // the larger lanes' eviction pools: a quarter of their circuits' shots, at most 2^22 records
   // (a record of a 64-entry lane takes about 0.8 KB)
@@ -720,6 +729,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     p.lane_round = 0;
     p.lane_evict = spill && rounds > 1 ? (small_run ? kEvictListed : kEvict) : 0u;
     p.lane_list = small_run ? 1u : 0u;
+    p.lane_tail = 0;
     p.lane_hand = spill ? 1u : 0u;
     p.lane_wide = wide ? 1u : 0u;
     p.lane_wide_round = 0;
@@ -813,6 +823,13 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     r->pass_ev.push_back(ev);
     return cudaEventRecord(ev, st);
   };
+  // the launch's last warps list their shots (see kTailListed); its counter is one of the chunk's
+  auto tail = [&](soft::ShotParams &q, const soft::LaunchCfg &cfg, int counter, uint32_t part) {
+    const uint32_t warps = cfg.grid * (cfg.block / 32);
+    q.lane_tail = std::max(1u, (uint32_t)((uint64_t)warps * part / 16u));
+    q.lane_done = reinterpret_cast<unsigned int *>(r->d_chunk + 5) + counter;
+    q.lane_list = 1u;
+  };
   auto enqueue_chunk = [&](uint64_t base, uint64_t cnt, bool dev_base) -> cudaError_t {
     cudaError_t err;
     if ((err = cudaMemsetAsync(r->d_chunk, 0, chunk_words * sizeof(unsigned long long) + 2 * (size_t)nb * sizeof(uint32_t),
@@ -836,6 +853,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
                   ab.n_items = cnt;
                   ab.item_base = base;
                   if (dev_base) ab.item_base_dev = r->d_work + 3;
+                  if (small_run) tail(ab, k ? cb[k - 1] : c1, 2 + k, k ? kTailBigListed : kTailListed);
                   r->launches++;
                   return soft::launch_prepared(k ? cb[k - 1] : c1, ab, s);
                 })) != cudaSuccess) {
@@ -869,6 +887,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
         as.lane_round = rd;
         as.lane_evict = !k && rd + 1 < rounds ? kEvict : 0u;
         as.n_items_dev = as.lr + 3 + 2 * rd;
+        if (!k && rd + 1 == rounds && affine) tail(as, c1, 0, kTailRound);
         r->launches++;
         return soft::launch_prepared(k ? cb[k - 1] : c1, as, s);
       });
@@ -882,6 +901,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
       aw.lane_hand = 0;
       aw.n_rerun_total = nullptr;  // (counted when they left the first rounds)
       aw.n_items_dev = r->d_lr + 3 + 2 * rounds;
+      if (affine) tail(aw, cw, 1, kTailWide);
       aw.rs_n = 1;
       aw.rs_sp[0] = aw.sp;
       aw.rs_lr[0] = aw.lr;

@@ -101,6 +101,8 @@ struct ShotParams {
   // pool; the next round buckets them by the event they resume at and packs them into warps
   uint32_t lane_round;        // 0: shots from their start buckets; r >= 1: shots evicted before round r
   uint32_t lane_evict;        // a warp with this many active lanes or fewer evicts their shots (0: none)
+  uint32_t lane_tail;         // once this many of the launch's warps have ended (counted in lane_done), the
+  unsigned int *lane_done;    // others put all their shots on the rerun list (0: never)
   uint32_t lane_list;         // 1: evicted shots go on the rerun list for the warp pass (with their
                               // record, or to start again where the lanes keep none)
   uint32_t lane_hand;         // 1: a lane whose map would outgrow it hands the shot over (a spill record)

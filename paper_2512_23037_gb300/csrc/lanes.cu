@@ -1,17 +1,17 @@
 // lanes.cu -- shot kernel with one shot per lane, 32 shots per warp, all at the
 // same event.
 //
-// Shots are first bucketed by the event they start at (the event that applies
-// their first error, capped at the end of the circuit's recorded noiseless run).
+// Shots are first bucketed by the event they start at (start_event: where their first
+// errors come to matter, at most the end of the circuit's recorded noiseless run).
 // Every warp then walks the events in order. Its idle lanes claim shots from the
 // bucket of the event it is at, load the noiseless run's state there, and the
 // warp executes each event once for all its lanes: the event is decoded once,
 // and every lane updates its own shot's coefficient map, kept in shared memory
 // (entry i of lane l at row i, column l). A rotation whose map would outgrow
 // kLaneCap entries hands the shot over: its state at the top of that event goes
-// to a spill record, which the warp-per-shot kernel's next pass resumes. The
-// per-shot arithmetic is that of the warp-per-shot kernel (the same formulas,
-// pruning thresholds and outcome rule), entry by entry. In a batch, each circuit
+// to a spill record, which the wide round's lanes or the affine warp pass (affine.cu)
+// resume. The per-shot arithmetic is that of the warp-per-shot kernels (the same
+// formulas, pruning thresholds and outcome rule), entry by entry. In a batch, each circuit
 // has its own range of buckets and a warp serves one circuit at a time. Circuits
 // whose noiseless maps outgrow kLaneCap get lanes of 32 or (FP32) 64 entries, one
 // launch per size over that size's buckets; the shots of circuits beyond those go
@@ -21,8 +21,9 @@
 // the end of the circuit, and they would hold a warp with a few active lanes. So a
 // warp left with few active lanes (lane_evict) writes their shots' state to a
 // spill pool and moves on to fresh shots. The next round (another launch) buckets
-// the evicted shots by the event they resume at, and packs them into warps again.
-// The last round evicts nothing. Which lane runs a shot does not change its
+// the evicted shots by the event they resume at, and packs them into warps again; in
+// small runs the affine warp pass takes them instead. The last round evicts nothing, until
+// most of its warps have ended (lane_tail): the affine pass takes the others' shots. Which lane runs a shot does not change its
 // arithmetic, so the results are those of a single round.
 //
 // A warp's time went to waits rather than to the maps (clock counters, w42 FP32: claims 22 %,
@@ -61,13 +62,12 @@ constexpr uint32_t kLaneMaxBuckets = 50000;  // the pre-pass histogram of all bu
 constexpr uint32_t kLaneRounds = SOFT_LANE_ROUNDS;  // rounds per chunk, the last without eviction
 static_assert(kLaneRounds >= 1 && kLaneRounds <= 8, "lane rounds");
 
-
 // The wide round's lanes: shots handed over by the first rounds continue in lanes
 // of twice the map.
 constexpr uint32_t kWideCap = 2 * kLaneCap;
 // First-pass lanes for circuits whose noiseless maps outgrow kLaneCap: 32 entries (kWideCap)
-// or, with FP32 coefficients, 64 entries. These never evict or hand over: a shot whose map
-// outgrows them runs again from its start in a warp.
+// or, with FP32 coefficients, 64 entries. These never hand over: a shot whose map outgrows
+// them runs again from its start in a warp.
 constexpr uint32_t kLaneBigCap = 4 * kLaneCap;
 
 // Lane map in affine form. The keys of a shot's coefficient map lie in an affine
@@ -1441,6 +1441,7 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
   };
   bool active = false;
   uint32_t item = 0;
+  uint32_t from = kNoRecord;  // wide round: the shot's hand-over record, from which a warp may run it again
   // the current bucket: its first record and the next bucket's
   uint32_t b0 = __ldg(&P.al_start[g]), b1 = __ldg(&P.al_start[g + 1]);
   const unsigned long long limit = (n_items + 2ull) * ((Multi ? P.al_hi - P.al_lo : P.al_nb) + 2ull) + 64ull;
@@ -1486,6 +1487,7 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
             item = __ldg(&P.al_order[b0 + k]);
             if (item < n_items) {
               active = true;
+              if (Cap == kWideCap && P.lane_wide_round) from = (uint32_t)(rec0 + item);
               item = s.resume(S, (uint32_t)(rec0 + item), first);
             }
           } else {
@@ -1530,7 +1532,8 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
             for (uint32_t w = 0; w < C->rw; ++w) C->records[off * C->rw + w] = s.rec[(size_t)w * 32 + lane];
         }
       } else if (done) {
-        uint32_t entry = item;  // a rerun starts the shot again from its start
+        uint32_t entry = item;  // a rerun starts the shot again from its start (or its hand-over)
+        if (Cap == kWideCap && from != kNoRecord) entry = kSpillRef | from;
         bool listed = true;
         if (s.status == LS_HAND) {  // or it resumes from its state at the top of event e
           const unsigned long long h = atomicAdd(&P.lr[1], 1ull);
@@ -1552,17 +1555,20 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     }
     // few active lanes: their shots go to the spill pool (when it has room), to resume in
     // the next round packed with others, and the warp moves on to fresh shots
-    if (P.lane_evict) {
+    if (P.lane_evict || P.lane_tail) {
       const uint32_t am = __ballot_sync(0xFFFFFFFFu, active);
-      if (am && (uint32_t)__popc(am) <= P.lane_evict && e + 1u < n_ev) {
+      bool out = (uint32_t)__popc(am) <= P.lane_evict;  // or few warps are left (every 8th event: the read waits)
+      if ((e & 7u) == 0u && P.lane_tail) out = out || *(volatile unsigned int *)P.lane_done >= P.lane_tail;
+      if (am && out && e + 1u < n_ev) {
         const uint32_t leader = __ffs(am) - 1;
         unsigned long long r0 = 0;
-        if (lane == leader) r0 = atomicAdd(P.sp ? &P.lr[0] : P.n_rerun, (unsigned long long)__popc(am));
+        const bool again = !P.sp || (Cap == kWideCap && P.lane_wide_round);  // no record to write
+        if (lane == leader) r0 = atomicAdd(again ? P.n_rerun : &P.lr[0], (unsigned long long)__popc(am));
         r0 = __shfl_sync(0xFFFFFFFFu, r0, leader);
         if (active) {
           const unsigned long long r = r0 + __popc(am & ((1u << lane) - 1u));
-          if (!P.sp) {  // (only with lane_list) no records: the warp pass runs them from their start
-            if (r < P.rerun_cap) P.rerun[r] = item;
+          if (again) {  // (only with lane_list) the warp pass runs them from their start, or their hand-over
+            if (r < P.rerun_cap) P.rerun[r] = Cap == kWideCap && from != kNoRecord ? kSpillRef | from : item;
             active = false;
           } else if (r < P.sp_evict_cap) {
             ev_r = (uint32_t)r;
@@ -1625,6 +1631,7 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     e = en;
   }
   flush();
+  if (P.lane_tail && lane == 0) atomicAdd(P.lane_done, 1u);
 }
 
 }  // namespace
