@@ -406,7 +406,7 @@ def leg_batch64(S, C, torch, peak_ops, flush):
                      "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                                   "unit": "Tops/s", "frac": achieved / peak_ops,
                                   "equivalent_frac_whole_method": ops_full * n * 2 / (ms_tot / 1000) / peak_ops,
-                                  "traffic": None, "kernel": "lane_kernel + shot_kernel (whole launch sequence)",
+                                  "traffic": None, "kernel": "lane_kernel + affine_kernel (whole launch sequence)",
                                   "ops_per_shot": ops_shot, "ops_per_shot_whole_method": ops_full}}
     for h in hs:
         h.free()
@@ -443,8 +443,8 @@ def leg_w97(S, C, torch, peak_ops, n_chunks):
                                   # the 64-entry lanes' DRAM bytes per 1e8-shot launch (its ncu summary)
                                   "traffic": profile_traffic(kernel_hash(), "lane_kernel_w97.md", chunk) if prec == "fp32" else None,
                                   "kernel": ("lane_kernel (64-entry lanes: the noiseless maps reach 64 entries) + "
-                                             "shot_kernel (shots that outgrow them)") if prec == "fp32" else
-                                            "shot_kernel (warp per shot: 64-entry lanes are FP32 only)",
+                                             "affine_kernel (shots that outgrow them)") if prec == "fp32" else
+                                            "affine_kernel (warp per shot: 64-entry lanes are FP32 only)",
                                   "ops_per_shot": ops_shot, "ops_per_shot_whole_method": ops_full}}
     h.free()
     return out
@@ -692,7 +692,8 @@ def main():
                      "pass_ms_per_step": {"prepass": pass64[0], "first_pass": pass64[1], "rerun": pass64[2]},
                      "flops_per_shot": flops64_shot, "flops_per_shot_whole_method": flops64_full,
                      "work": "FP64 flops of T/Rz output entries (14), diagonal entries (6) and measurement entry "
-                             "visits (4) a shot executes after the shared noiseless prefix (oracle counters)",
+                             "visits (4) of a shot after the shared noiseless prefix (oracle counters), also where an "
+                             "error is carried past it or the shot is finished unrun: an equivalent rate",
                      "peak_basis": "measured: soft_peak_pipe_rate(FP64 FMA) in this run, 2 flops per FMA",
                      "alu_frac": ops_shot * n / (sum(pass64) / 1000) / peak_ops, "equivalent_note": EQUIV_NOTE}
     lane_mode = lane_mode_of(pass_ms)

@@ -86,17 +86,19 @@ def test_prepass_edges(soft, precision, name, n):
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
-@pytest.mark.parametrize("name,n", [("w42", (1 << 20) + 1), ("win5", (1 << 20) + 1), ("win6", (1 << 20) + 1),
-                                    ("w42", 1 << 22)])
-def test_large_runs(soft, precision, name, n):
-    """Above the sizes at which evicted shots go to a second round, and a wide
-    round follows: the counts, and the first shots' records."""
+@pytest.mark.parametrize("name,n,wide", [("w42", (1 << 20) + 1, None), ("w42", (1 << 20) + 1, False),
+                                         ("win5", (1 << 20) + 1, None), ("win6", (1 << 20) + 1, None),
+                                         ("w42", 1 << 22, None)])
+def test_large_runs(soft, precision, name, n, wide):
+    """Above the size at which evicted shots go to a second round, whose last
+    warps list theirs, and a wide round follows, whose shots a warp resumes from
+    their hand-over: the counts, and the first shots' records."""
     S = soft
     circ, noise = _case(name)
     c = S.soft_compile_circuit(circ.array(), circ.n, noise, circ.cap)
     k = 4096
-    runs = [S.soft_run_shots(c, n, 0, 8, precision=precision, record_mode=S.REC_FIRST_K, record_k=k, lanes=lanes)
-            for lanes in (True, False)]
+    runs = [S.soft_run_shots(c, n, 0, 8, precision=precision, record_mode=S.REC_FIRST_K, record_k=k, lanes=lanes,
+                             wide=wide) for lanes in (True, False)]
     (ra, sa), (rb, sb) = (S.soft_get_records(r, k) for r in runs)
     assert np.sum((sa != sb) | np.any(ra != rb, axis=1)) <= _allowed(k, precision)
     _tallies_close(S.soft_tally(runs[0]), S.soft_tally(runs[1]), n, precision)
