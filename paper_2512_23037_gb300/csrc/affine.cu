@@ -18,7 +18,6 @@
 // circuit's cap, which runs it from its start with the sparse form of kernels.cu. FP32
 // arithmetic is that kernel's, product by product, so a shot's outcomes do not depend on
 // which of the two runs it (FP64 sums over entries run in slot order).
-#include <algorithm>
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -905,17 +904,16 @@ __global__ void __launch_bounds__(kAffBlock, sizeof(R) == 4 && W == 1 ? 6 : 5) a
   for (uint32_t i = threadIdx.x; i < 5 * n_circ; i += blockDim.x) btally[i / 5][i % 5] = 0ull;
   __syncthreads();
   AffShot<R, W> s(P, smem + (threadIdx.x / 32) * aff_warp_bytes<R, W>(P.aff_dim));
-  const unsigned long long n_items = P.n_items_dev ? *P.n_items_dev : P.n_items;
+  const unsigned long long n_items = *P.n_items_dev < P.rerun_cap ? *P.n_items_dev : P.rerun_cap;  // the list's entries
   const unsigned long long item_base = P.item_base_dev ? *P.item_base_dev : P.item_base;
   for (;;) {
     unsigned long long item = 0;
     if (s.lane == 0) item = atomicAdd(P.next_item, 1ull);
     item = __shfl_sync(kAll, item, 0);
     if (item >= n_items) break;
-    if (P.list && item >= P.rerun_cap) break;  // a list never holds more than its capacity
-    uint32_t local = P.list ? P.list[item] : (uint32_t)item;
+    uint32_t local = P.list[item];
     uint32_t rec = kNoRecord;  // an entry naming a spill record resumes the shot a lane handed over
-    if (P.list && (local & kSpillRef) && P.sp) {
+    if ((local & kSpillRef) && P.sp) {
       rec = local & ~kSpillRef;
       if (rec >= P.sp_cap) break;  // never: records are taken below the pool's capacity
       const Spill<R, W> S(P.sp, P.rw_max, kLaneDim);
@@ -942,7 +940,7 @@ __global__ void __launch_bounds__(kAffBlock, sizeof(R) == 4 && W == 1 ? 6 : 5) a
 }  // namespace
 
 cudaError_t prepare_affine(const ShotParams &p, int fp32, uint32_t W, int blocks_per_sm, LaunchCfg *cfg) {
-  if (p.aff_dim > 12 || p.rw_max > kAffRecWords) return cudaErrorInvalidConfiguration;
+  if (!p.list || !p.n_items_dev || p.aff_dim > 12 || p.rw_max > kAffRecWords) return cudaErrorInvalidConfiguration;
   const void *kern = fp32 ? (W == 1 ? reinterpret_cast<const void *>(affine_kernel<float, 1>)
                                     : reinterpret_cast<const void *>(affine_kernel<float, 2>))
                           : (W == 1 ? reinterpret_cast<const void *>(affine_kernel<double, 1>)
@@ -958,10 +956,8 @@ cudaError_t prepare_affine(const ShotParams &p, int fp32, uint32_t W, int blocks
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kAffBlock, smem)) != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
   if (blocks_per_sm > 0 && blocks_per_sm < occ) occ = blocks_per_sm;
-  unsigned long long grid = (unsigned long long)occ * sms;
-  if (!p.n_items_dev) grid = std::min(grid, std::max(1ull, (unsigned long long)(p.n_items + kAffBlock / 32 - 1) / (kAffBlock / 32)));
   cfg->kern = kern;
-  cfg->grid = (unsigned)grid;
+  cfg->grid = (unsigned)(occ * sms);
   cfg->block = kAffBlock;
   cfg->smem = smem;
   return cudaSuccess;
