@@ -47,8 +47,10 @@ constexpr uint32_t kEvictListed = 8, kEvict = 17, kEvictBigListed = 8, kEvictBig
 // / 1.34, 40 k 0.65 / 0.36, FP64 20 k 0.63 / 0.35 (at 8: random 1.57); larger lanes of small runs at
 // 12, whose shots start again: w97 FP32 400 k 2.22 / 2.03, 20 k 1.00 / 0.65; the second round at 8:
 // w42 FP32 1.5 M 1.98 / 1.66, FP64 2.34 / 2.09; the wide round at 8, whose shots go on from their
-// hand-over: w42 FP32 4 M 2.62 / 2.46, 2^24 7.37 / 7.25, FP64 2^22 4.18 / 3.96.
-constexpr uint32_t kTailListed = 15, kTailBigListed = 12, kTailRound = 8, kTailWide = 8;
+// hand-over: w42 FP32 4 M 2.62 / 2.46, 2^24 7.37 / 7.25, FP64 2^22 4.18 / 3.96; the larger lanes'
+// second round at 6, whose shots start again: w97 FP32 2 M 5.79 / 5.30 (at 12: 5.54), 4 M 9.70 /
+// 9.25, 64-circuit batch 8.89 / 8.32.
+constexpr uint32_t kTailListed = 15, kTailBigListed = 12, kTailRound = 8, kTailBigRound = 6, kTailWide = 8;
 // Directions of the affine warp passes' maps (2^dim values a warp): a shot that needs more goes
 // to the pass at the circuit's cap. In ms at 8 / 9 / 10 / 11: w97 FP32 2 M shots 6.22 / 6.20 / 5.86 / 7.12,
 // w42 FP32 1 M 1.52 / 1.51 / 1.51 / 2.09; w97 FP64 500 k 3.58 / 3.90 / 6.51 / 8.27 (the maps'
@@ -887,7 +889,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
         as.lane_round = rd;
         as.lane_evict = !k && rd + 1 < rounds ? kEvict : 0u;
         as.n_items_dev = as.lr + 3 + 2 * rd;
-        if (!k && rd + 1 == rounds && affine) tail(as, c1, 0, kTailRound);
+        if (rd + 1 == rounds && affine) tail(as, k ? cb[k - 1] : c1, k ? 2 + k : 0, k ? kTailBigRound : kTailRound);
         r->launches++;
         return soft::launch_prepared(k ? cb[k - 1] : c1, as, s);
       });

@@ -1562,7 +1562,7 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
       if (am && out && e + 1u < n_ev) {
         const uint32_t leader = __ffs(am) - 1;
         unsigned long long r0 = 0;
-        const bool again = !P.sp || (Cap == kWideCap && P.lane_wide_round);  // no record to write
+        const bool again = !P.sp || (Cap > kLaneCap && P.lane_round);  // no record to write
         if (lane == leader) r0 = atomicAdd(again ? P.n_rerun : &P.lr[0], (unsigned long long)__popc(am));
         r0 = __shfl_sync(0xFFFFFFFFu, r0, leader);
         if (active) {
