@@ -35,11 +35,15 @@ using soft::kDefaultFirstCap;
 constexpr uint64_t kSmallRun = 1ull << 20;
 // Active lanes at which a warp evicts its shots: to the warp pass's list, which takes a shot on
 // its own, or to a second round, whose warps are packed again (16-entry lanes, then the larger).
-// In ms at 3 / 8 / 10: w42 FP32 1 M shots 1.40 / 1.45 / 1.52, 200 k 0.87 / 0.73 / 0.77 (listed);
-// at 10 / 17 / 20: w42 FP32 2^24 7.65 / 7.49 / 7.61, FP64 2^22 4.50 / 4.19 / 4.15. Larger lanes
-// at 4 / 8 / 12: w97 FP32 1 M 4.09 / 4.09 / 4.16, 300 k 2.31 / 2.18 / 2.2 (listed); at 12 / 15 /
-// 18: w97 FP32 2 M 6.22 / 6.11 / 6.24, 64-circuit batch 9.97 / 9.66 / 9.56.
-constexpr uint32_t kEvictListed = 8, kEvict = 17, kEvictBigListed = 8, kEvictBig = 15;
+// In ms, listed, at 2 / 4 / 8 / 12: w42 FP32 1 M shots 1.23 / 1.23 / 1.34 / 1.48, 250 k - / 0.64 / 0.62 /
+// 0.65, FP64 700 k 1.29 / 1.27 / 1.34 / 1.43; larger lanes w97 FP32 1 M 3.36 / 3.50 / 3.80, 400 k 1.87 /
+// 1.90 / 2.01, 100 k 1.04 / 1.04 / 1.03. To a second round, at 14 / 17 / 20 / 24: w42 FP32 2^24 7.20 / 7.24 /
+// 7.39 / 7.60, FP64 2^22 3.97 / 3.95 / 3.93 / 3.95; the larger at 11 / 15 / 19 / 23: w97 FP32 2 M 5.38 /
+// 5.28 / 5.30 / 5.45, 64-circuit batch 8.39 / 8.28 / 8.29 / 8.36.
+// The list's threshold is the lower one above kEvictFew shots, where there are enough to keep the
+// lanes full.
+constexpr uint32_t kEvictListed = 8, kEvictListedMany = 4, kEvict = 17, kEvictBigListed = 3, kEvictBig = 15;
+constexpr uint64_t kEvictFew = 1ull << 19;
 // Sixteenths of a lane launch's warps after whose end the others list all their shots for the warp
 // pass (a launch ends with a few warps that walk the last shots' events, a step as slow as a
 // lane's loops, while the rest of the chip idles). Without / with, in ms: 16-entry lanes of small
@@ -729,7 +733,7 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
     p.al_hi = (uint32_t)nbc[0];
     p.al_grid = al_grid;
     p.lane_round = 0;
-    p.lane_evict = spill && rounds > 1 ? (small_run ? kEvictListed : kEvict) : 0u;
+    p.lane_evict = spill && rounds > 1 ? (!small_run ? kEvict : std::min(chunk, total) <= kEvictFew ? kEvictListed : kEvictListedMany) : 0u;
     p.lane_list = small_run ? 1u : 0u;
     p.lane_tail = 0;
     p.lane_hand = spill ? 1u : 0u;
