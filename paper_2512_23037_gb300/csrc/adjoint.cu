@@ -51,15 +51,17 @@ constexpr uint32_t kMaxErr = 256;
 
 template <int W>
 struct ErrRec {
-  uint32_t ev, site, code, pad;
+  uint32_t ev, site, code;
+  uint32_t at;  // an error carried to event ev (load_prefix): the event that applies it << 1 | its phase's lowest bit
   uint64_t sd[W], ss[W];
 };
 
 // Per-warp tape: the map after every rotation (`slot` entries each), the sign
-// words after every event's Clifford XOR, outcome bits, the applied errors.
+// words after every event's Clifford XOR, outcome bits, the applied errors, and the
+// derivatives of the part that both sweeps share (see replay), each with its parameter word.
 template <typename R, int W>
 struct TapeLayout {
-  size_t keys, vals, nnz, signs, bits, errs, total;
+  size_t keys, vals, nnz, signs, bits, errs, z, zk, total;
   uint32_t slot;
   __host__ __device__ TapeLayout(uint32_t n_rot, uint32_t n_events, uint32_t slot_entries = 32) {
     slot = slot_entries;
@@ -76,6 +78,10 @@ struct TapeLayout {
     o += ((size_t)(n_events + 63) / 64) * 8;
     errs = o;
     o += (size_t)kMaxErr * sizeof(ErrRec<W>);
+    z = o;
+    o += (size_t)n_rot * 8;
+    zk = o;
+    o += (size_t)n_rot * 4;
     total = (o + 255) & ~(size_t)255;
   }
 };
@@ -114,6 +120,8 @@ struct GradWarp {
   uint64_t *rec;    // record bits (shared)
   double *terms = nullptr;  // kTerms rows of a rotation's 32 terms (shared; not in wide mode)
   uint32_t n_terms = 0, term_of = 0;  // rows in use; lane i: row i's parameter and sign
+  uint32_t n_z = 0;                   // derivatives on the tape for replay
+  uint32_t n_carried = 0;             // the errors that load_prefix carried
   unsigned char *tape;
   TapeLayout<R, W> L;   // this warp's tape
   TapeLayout<R, W> PL;  // the shared noiseless prefix tape (32-entry slots)
@@ -379,19 +387,27 @@ struct GradWarp {
     sm_from_stage(m, 2 * n, [&](uint32_t i) { return norm2d(svals[i]) >= thr && norm2d(svals[i]) > 0.0; });
     return true;
   }
-  // Im <lambda| Z_q |phi>, <lambda| Z_q |phi> = sum_a conj(lambda_{a^beta}) xi_a phi_a
+  // Im <lambda| Z_q |phi>, <lambda| Z_q |phi> = sum_a conj(lambda_{a^beta}) xi_a phi_a (turned: see term)
   __device__ double zexp(const SMap<R, W> &lam, const SMap<R, W> &ph, const uint64_t *beta, const uint64_t *gamma,
-                         uint32_t e) {
+                         uint32_t e, bool turned) {
     double ci = 0.0;
     for (uint32_t i = lane; i < ph.n; i += 32) {
       const Key<W> k = smk(ph, i);
       const int j = sfind(lam, kxor(k, beta));
       if (j < 0) continue;
-      const Cx<R> xp = ipow(ph.v[i], e + 2u * kpar(k, gamma));
-      const Cx<R> l = lam.v[j];
-      ci += (double)l.x * (double)xp.y - (double)l.y * (double)xp.x;
+      ci += term(lam.v[j], ipow(ph.v[i], e + 2u * kpar(k, gamma)), turned);
     }
     return wsum(ci);
+  }
+  // Im conj(l) x. Errors carried along the noiseless run leave lambda and phi as they are before
+  // them; with the errors applied both would be multiplied by powers of i, which exchanges the two
+  // products when the power is odd (turned) and so moves the last bit of what two cancelling
+  // sweeps leave. The products are taken as they would be with the errors applied.
+  __device__ __forceinline__ static double term(Cx<R> l, Cx<R> x, bool turned) {
+    const double a = turned ? (double)l.y : (double)l.x, b = turned ? (double)x.x : (double)x.y;
+    const double c = turned ? (double)l.x : (double)l.y, d = turned ? (double)x.y : (double)x.x;
+    const double p = fmar(a, b, -mulr(c, d));
+    return turned ? negr(p) : p;
   }
   __device__ void reset_sides(const SMap<R, W> &m, const uint64_t *gamma, uint32_t sgn, bool &h0, bool &h1) {
     bool a0 = false, a1 = false;
@@ -535,21 +551,14 @@ struct GradWarp {
     const Cx<R> src = has ? vj : m.v;
     const Cx<R> y = ipow(src, e + 2u * kpar(has ? pk : m.k, gamma));
     Cx<R> nv, tb;
-    if (a.y == (R)0 && b.x == (R)0) {  // an Rz: cos I - i sin Z (FP32 rounds as the products below)
-      const R by = b.y, nby = negr(b.y);
+    if (a.y == (R)0 && b.x == (R)0) {  // an Rz: cos I - i sin Z (rounds as the products below)
       nv = cscale(m.v, a.x);
-      if (sizeof(R) == 8 && has) {
-        nv = Cx<R>{fmar(nby, y.y, nv.x), fmar(by, y.x, nv.y)};
-        tb = Cx<R>{0, 0};
-      } else {
-        tb = Cx<R>{mulr(nby, y.y), mulr(by, y.x)};
-        if (has) nv = cadd(nv, tb);
-      }
+      tb = Cx<R>{mulr(negr(b.y), y.y), mulr(b.y, y.x)};
     } else {
       tb = cmul(b, y);
       nv = cmul(a, m.v);
-      if (has) nv = cadd(nv, tb);
     }
+    if (has) nv = cadd(nv, tb);
     const uint32_t ab = t.ballot(app);
     const uint32_t nA = __popc(ab);
     if (m.n + nA > 32u) return false;
@@ -867,9 +876,9 @@ struct GradWarp {
   // kTerms rotations (add_terms): on its own it took 5 of the 13 FP64 instructions of a
   // rotation, whose unit was busy for 62 % of an FP32 training step's kernel. The search looks at
   // every key, four loads in flight, instead of stopping at the match. Training step 0.938 -> 0.879
-  // ms, gradient of 10^5 w42rz patterns in FP64 1.94 -> 1.92.
+  // ms.
   __device__ void put_terms(const RMap<R, W> &lam, const RMap<R, W> &phi, const uint64_t *beta, const uint64_t *gamma,
-                            uint32_t e, uint32_t k) {
+                            uint32_t e, uint32_t k, bool turned) {
     skey_set(lane, lam.k);
     if (lane < lam.n) svals[lane] = lam.v;
     t.sync();
@@ -880,131 +889,87 @@ struct GradWarp {
 #pragma unroll
       for (uint32_t i = 0; i < 4; ++i) m |= (keq(skey(j + i), target) ? 1u : 0u) << (j + i);
     m &= vmask(lam.n);
-    if (lane < phi.n && m) {
-      const Cx<R> xp = ipow(phi.v, e + 2u * kpar(phi.k, gamma));  // xi_a phi_a
-      const Cx<R> l = svals[31u - (uint32_t)__clz((int)m)];
-      // conj(l) * xp
-      ci = (double)l.x * (double)xp.y - (double)l.y * (double)xp.x;
-    }
+    if (lane < phi.n && m)
+      ci = term(svals[31u - (uint32_t)__clz((int)m)], ipow(phi.v, e + 2u * kpar(phi.k, gamma)), turned);
     terms[n_terms * 32u + ((lane + n_terms) & 31u)] = ci;
     if (lane == n_terms) term_of = k;
     ++n_terms;
     t.sync();
   }
-  // grad[k] += weight * sign * the sums of the rows of terms: lanes i and 16 + i take the halves of
-  // row i (rotated by i: a bank each)
-  __device__ void add_terms(double *grad, double weight) {
+  // grad[k] += weight * sign * the sums of the rows of terms: lanes i and 16 + i take the even and
+  // the odd terms of row i (rotated by i: a bank each), added in the order of wsum. keep: the sums
+  // go on the tape for replay as well.
+  __device__ void add_terms(double *grad, double weight, bool keep) {
     const uint32_t i = lane & 15u, n = n_terms;
     double v = 0.0;
-    if (i < n)
-#pragma unroll 4
-      for (uint32_t j = 0; j < 16; ++j) v += terms[i * 32u + ((j + (lane & 16u) + i) & 31u)];
-    v += t.shfl_xor(v, 16u);
-    v *= (term_of & 1u) ? -weight : weight;
-    const bool mine = lane < n;
-    const uint32_t same = __match_any_sync(0xFFFFFFFFu, mine ? term_of >> 1 : 0x80000000u | lane);
-    if (t.all(same == 1u << lane)) {  // each parameter once
-      if (mine) grad[term_of >> 1] += v;
-    } else {
-#pragma unroll 1
-      for (uint32_t q = 0; q < n; ++q) {
-        if (lane == q) grad[term_of >> 1] += v;
-        t.sync();
-      }
+    if (i < n) {
+      auto four = [&](uint32_t j) {
+        const double *row = terms + i * 32u;
+        return (row[(j + i) & 31u] + row[(j + 16u + i) & 31u]) + (row[(j + 8u + i) & 31u] + row[(j + 24u + i) & 31u]);
+      };
+      const uint32_t h = lane >> 4;
+      v = (four(h) + four(h + 4u)) + (four(h + 2u) + four(h + 6u));
     }
+    v += t.shfl_xor(v, 16u);
+    if (keep) {
+      if (lane < n) {
+        reinterpret_cast<double *>(tape + L.z)[n_z + lane] = v;
+        reinterpret_cast<uint32_t *>(tape + L.zk)[n_z + lane] = term_of;
+      }
+      n_z += n;
+    }
+    add_each(grad, n, term_of, v, weight);
     n_terms = 0;
     t.sync();
   }
-
-  // lam -= f m, exact zeros dropped and the rest pruned; false if it needs more entries than a map
-  // holds
-  __device__ bool subtract(RMap<R, W> &lam, const RMap<R, W> &m, R f) {
-    if (lane < lam.n) {
-      skey_set(lane, lam.k);
-      svals[lane] = lam.v;
-    }
-    t.sync();
-    const Cx<R> d = lane < m.n ? Cx<R>{mulr(-f, m.v.x), mulr(-f, m.v.y)} : Cx<R>{0, 0};
-    bool app = lane < m.n;
-    for (uint32_t j = 0; j < lam.n; ++j)
-      if (app && keq(skey(j), m.k)) {
-        svals[j] = cadd(svals[j], d);
-        app = false;
+  // grad[k >> 1] += weight * sign * v of lanes [0, n), one after the other where they share a
+  // parameter
+  __device__ __forceinline__ void add_each(double *grad, uint32_t n, uint32_t k, double v, double weight) {
+    const double w = (k & 1u) ? -weight : weight;
+    const bool mine = lane < n;
+    const uint32_t same = __match_any_sync(0xFFFFFFFFu, mine ? k >> 1 : 0x80000000u | lane);
+    if (t.all(same == 1u << lane)) {  // each parameter once
+      if (mine) grad[k >> 1] = fmar(w, v, grad[k >> 1]);
+    } else {
+#pragma unroll 1
+      for (uint32_t q = 0; q < n; ++q) {
+        if (lane == q) grad[k >> 1] = fmar(w, v, grad[k >> 1]);
+        t.sync();
       }
-    const uint32_t b = t.ballot(app);
-    if (app) {  // (at most 64 staged entries)
-      skey_set(lam.n + lanes_below(b), m.k);
-      svals[lam.n + lanes_below(b)] = d;
     }
     t.sync();
-    const uint32_t n = lam.n + __popc(b);
-    const Key<W> k0 = skey(lane), k1 = skey(lane + 32);
-    const Cx<R> v0 = svals[lane], v1 = svals[lane + 32];
-    const bool in0 = lane < n && (v0.x != (R)0 || v0.y != (R)0), in1 = lane + 32 < n && (v1.x != (R)0 || v1.y != (R)0);
-    const uint32_t b0 = t.ballot(in0), b1 = t.ballot(in1);
-    if (__popc(b0) + __popc(b1) > 32) return false;
-    t.sync();
-    if (in0) {
-      skey_set(lanes_below(b0), k0);
-      svals[lanes_below(b0)] = v0;
-    }
-    if (in1) {
-      skey_set(__popc(b0) + lanes_below(b1), k1);
-      svals[__popc(b0) + lanes_below(b1)] = v1;
-    }
-    t.sync();
-    lam.n = __popc(b0) + __popc(b1);
-    if (lane < lam.n) {
-      lam.k = skey(lane);
-      lam.v = svals[lane];
-    }
-    t.sync();
-    if (lam.n) prune_rel(lam, lane < lam.n);
-    return true;
   }
-  __device__ bool subtract(SMap<R, W> &lam, const SMap<R, W> &m, R f) {
-    for (uint32_t i = lane; i < lam.n; i += 32) {
-      skey2_set(i, smk(lam, i));
-      svals[i] = lam.v[i];
-    }
+  // The second sweep where it repeats the first: its derivatives are on the tape, in its order.
+  __device__ void replay(double *grad, double weight) {
     t.sync();
-    uint32_t n = lam.n;
-    for (uint32_t base = 0; base < m.n; base += 32) {
-      const uint32_t i = base + lane;
-      bool app = false;
-      Key<W> k;
-      Cx<R> d{0, 0};
-      if (i < m.n) {
-        k = smk(m, i);
-        d = Cx<R>{mulr(-f, m.v[i].x), mulr(-f, m.v[i].y)};
-        const int j = sfind(lam, k);
-        app = j < 0;
-        if (j >= 0) svals[j] = cadd(svals[j], d);
+    for (uint32_t i = 0; i < n_z; i += 32) {
+      const uint32_t n = n_z - i < 32u ? n_z - i : 32u;
+      double v = 0.0;
+      uint32_t k = 0;
+      if (lane < n) {
+        v = reinterpret_cast<const double *>(tape + L.z)[i + lane];
+        k = reinterpret_cast<const uint32_t *>(tape + L.zk)[i + lane];
       }
-      const uint32_t b = t.ballot(app);
-      if (app) {  // (at most 2 kWideCap staged entries)
-        skey2_set(n + lanes_below(b), k);
-        svals[n + lanes_below(b)] = d;
-      }
-      n += __popc(b);
+      add_each(grad, n, k, v, weight);
     }
-    t.sync();
-    uint32_t live = 0;
-    for (uint32_t base = 0; base < n; base += 32) {
-      const uint32_t i = base + lane;
-      live += __popc(t.ballot(i < n && (svals[i].x != (R)0 || svals[i].y != (R)0)));
-    }
-    if (live > kWideCap) return false;
-    sm_from_stage(lam, n, [&](uint32_t i) { return svals[i].x != (R)0 || svals[i].y != (R)0; });
-    if (lam.n) prune_rel(lam);
-    return true;
+  }
+  // the same entries in the same order
+  __device__ bool same_map(const RMap<R, W> &a, const RMap<R, W> &b) const {
+    if (a.n != b.n) return false;
+    return t.all(lane >= a.n || (keq(a.k, b.k) && a.v.x == b.v.x && a.v.y == b.v.y));
+  }
+  __device__ bool same_map(const SMap<R, W> &a, const SMap<R, W> &b) const {
+    if (a.n != b.n) return false;
+    bool ok = true;
+    for (uint32_t i = lane; i < a.n; i += 32) ok = ok && keq(smk(a, i), smk(b, i)) && a.v[i].x == b.v[i].x && a.v[i].y == b.v[i].y;
+    return t.all(ok);
   }
 
   // ------------------------------------------------------------- one pattern
   __device__ void run(uint64_t pattern, uint64_t off) {
     shot = pattern;
     status = G_OK;
-    n_err = 0;
+    n_err = n_carried = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) sd[w] = ss[w] = 0ull;
     for (uint32_t w = lane; w < P.rw; w += 32) rec[w] = 0ull;
@@ -1033,28 +998,17 @@ struct GradWarp {
     }
     for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] = 0.0;
     t.sync();
-    // N_fid = 0: F = 0 and dF/dtheta = 0 exactly; no fidelity measurement: F = 1 at any angles
-    const bool swept = status == G_OK && n_fid > 0.0 && seen_f;
+    const bool swept = status == G_OK && n_fid > 0.0;  // N_fid = 0: F = 0 and dF/dtheta = 0 exactly
     if (swept) {
-      // dF = (dN_fid - F dN_acc) / N_acc. The sweep of N_fid starts at the end with phi; at the
-      // first fidelity measurement the one of N_acc joins it, linear in the adjoint state:
-      // lambda - F pre goes on as one sweep. Most kept patterns have F = 1 there with lambda =
-      // pre, and are done (w42rz, 10^5 patterns in FP64: 8.1 -> 2.6 ms, with the norms of
-      // prune_rel left out). Should the joined map need more entries than there are, the two
-      // sweeps run one after the other (mode 1, 2).
-      for (int mode = 0;;) {
-        const bool ok = sweep(mode == 2 ? pre : phi, mode == 2 ? ev_f : P.n_events, mode == 2 ? rot_before_f : r, grad,
-                              mode == 2 ? -F : 1.0, mode == 0 ? ev_f : 0xFFFFFFFFu, (R)F);
-        if (mode == 0 && !ok) {
-          t.sync();
-          for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] = 0.0;
-          t.sync();
-          mode = 1;
-          continue;
-        }
-        if (!ok) status = kCapFail;
-        if (mode != 1 || !ok) break;
-        mode = 2;
+      // dF = (dN_fid - F dN_acc) / N_acc. Sweep 1: N_fid from the end; sweep 2: N_acc from just
+      // before the first fidelity measurement. Most kept patterns have F = 1 and the same adjoint
+      // state there in both, entry for entry: sweep 2 then repeats sweep 1 and only its sums are
+      // added again.
+      bool both = false;
+      if (!sweep(phi, P.n_events, r, grad, 1.0, ev_f, both)) status = kCapFail;
+      if (status == G_OK) {
+        if (both) replay(grad, -F);
+        else if (!sweep(pre, ev_f, rot_before_f, grad, -F, 0xFFFFFFFFu, both)) status = kCapFail;
       }
       t.sync();
       for (uint32_t k = lane; k < P.n_params; k += 32) grad[k] /= n_acc;
@@ -1353,8 +1307,7 @@ struct GradWarp {
   }
   // The pattern's start: its errors are carried along the noiseless run to the first event that
   // does not leave one of them alone, as long as the next comes in before it. Most patterns end
-  // there, in a projection onto nothing, after one event (w42rz, 10^5 patterns in FP64: the call
-  // 2.70 -> 2.11 ms). The errors are on record at that event, where the reverse
+  // there, in a projection onto nothing, after one event. The errors are on record at that event, where the reverse
   // sweep takes them back; below it the sweep reads the noiseless run's tape, which they leave
   // alone as well.
   __device__ void load_prefix() {
@@ -1375,8 +1328,10 @@ struct GradWarp {
       error_pauli(nxt, code, esd, ess, b, g, &e);
       ev0 = fate(at, ev0, b, g);
       record_error(0u, code, esd, ess);
+      if (lane == 0) errs()[n_err - 1u].at = at << 1 | (e & 1u);
       draw_next();
     }
+    n_carried = n_err;
     const unsigned char *in = P.psnap + (size_t)ev0 * P.psnap_stride;
     const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
     const uint64_t *r_in = reinterpret_cast<const uint64_t *>(in + sizeof(SnapHdr));
@@ -1451,18 +1406,30 @@ struct GradWarp {
 
   // Reverse sweep from just before event `ev_end` (its errors included): the
   // adjoint starts as `lam` (the state there) and every parameterised rotation
-  // adds weight * s * Im <lambda| Z_q |phi> to grad[k]. Before event ev_join (0xFFFFFFFF: none)
-  // the adjoint becomes lambda - f pre. False if a map would need more entries than there are.
+  // adds weight * s * Im <lambda| Z_q |phi> to grad[k]. both: set where the adjoint equals pre just
+  // before event ev_join (0xFFFFFFFF: none); from there on the sums go on the tape as well. False if
+  // a map would need more entries than there are.
   __device__ bool sweep(const Map &src, uint32_t ev_end, uint32_t r_end, double *grad, double weight, uint32_t ev_join,
-                        R f) {
+                        bool &both) {
     Map lam_local{};
     Map &lam = Wide ? lam_store : lam_local;  // registers, or the warp's shared-memory map
     copy_map(lam, src);
-    n_terms = 0;
+    n_terms = n_z = 0;
+    both = false;
+    auto join = [&]() {
+      if (!same_map(lam, pre)) return;
+      if (!Wide && n_terms) add_terms(grad, weight, false);
+      both = true;
+    };
+    if (ev_join >= P.n_events && ev_join == ev_end) join();  // (no fidelity measurement)
     const Ev<W> *evs = reinterpret_cast<const Ev<W> *>(P.ev);
     int64_t ei = (int64_t)n_err - 1;
     while (ei >= 0 && errs()[ei].ev > ev_end) --ei;  // errors after the sweep's start point
     uint32_t r = r_end;
+    // below ev0 the carried errors are not in the maps: whether their phases turn them by i there
+    uint32_t carried = n_carried;
+    bool turned = false;
+    for (uint32_t i = 0; i < n_carried; ++i) turned ^= (errs()[i].at & 1u) != 0u;
     for (int64_t evi = (int64_t)(ev_end < P.n_events ? ev_end : P.n_events - 1); evi >= 0; --evi) {
       const uint32_t ev = (uint32_t)evi;
       if (ev < ev_end) {
@@ -1484,16 +1451,24 @@ struct GradWarp {
           --r;
           const uint32_t e = (ev_e0(w0) + 2u * pe(beta, gamma)) & 3u;
           if (hdr.w != kNoRec) {
+            for (; carried && errs()[carried - 1u].at >> 1 > ev; --carried) turned ^= (errs()[carried - 1u].at & 1u) != 0u;
             Map phk_local{};
             Map &phk = Wide ? phk_store : phk_local;
             tape_load_phi(r, phk);
             if constexpr (Wide) {
-              const double zi = zexp(lam, phk, beta, gamma, e);
+              const double zi = zexp(lam, phk, beta, gamma, e, ev < ev0 && turned);
               const double s = (hdr.w & 1u) ? -1.0 : 1.0;
-              if (lane == 0) grad[hdr.w >> 1] += weight * s * zi;
+              if (lane == 0) grad[hdr.w >> 1] = fmar(weight * s, zi, grad[hdr.w >> 1]);
+              if (both) {
+                if (lane == 0) {
+                  reinterpret_cast<double *>(tape + L.z)[n_z] = zi;
+                  reinterpret_cast<uint32_t *>(tape + L.zk)[n_z] = hdr.w;
+                }
+                ++n_z;
+              }
             } else {
-              put_terms(lam, phk, beta, gamma, e, hdr.w);
-              if (n_terms == kTerms) add_terms(grad, weight);
+              put_terms(lam, phk, beta, gamma, e, hdr.w, ev < ev0 && turned);
+              if (n_terms == kTerms) add_terms(grad, weight, both);
             }
           }
           const Coef *C = P.coef + hdr.z;
@@ -1560,10 +1535,7 @@ struct GradWarp {
         }
         if (op) settle(lam, in);
       }
-      if (ev == ev_join) {
-        if (!subtract(lam, pre, f)) return false;
-        if (lam.n == 0u) break;
-      }
+      if (ev == ev_join) join();
       // errors applied before this event, newest first
       while (ei >= 0 && errs()[ei].ev == ev) {
         const ErrRec<W> &er = errs()[ei];
@@ -1579,7 +1551,7 @@ struct GradWarp {
         --ei;
       }
     }
-    if (!Wide && n_terms) add_terms(grad, weight);
+    if (!Wide && n_terms) add_terms(grad, weight, both);
     return true;
   }
 };
