@@ -1468,10 +1468,16 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     // snapshot's copies are issued before the atomic answers: a lane that gets no shot has
     // only filled columns that nobody reads.
     const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
-    bool claim = idle && b1 != b0 && !((*(volatile uint32_t *)&empty[g >> 5] >> (g & 31u)) & 1u);
-    if (claim && *(volatile unsigned int *)&P.al_next[g] >= b1 - b0) {  // once per block and bucket
-      if (lane == 0) atomicOr(&empty[g >> 5], 1u << (g & 31u));
-      claim = false;
+    bool claim = idle && b1 != b0;
+    if (claim) {
+      // (other warps change both words meanwhile, so the lanes may read different values: the warp
+      // decides as one, by a vote)
+      bool shut = ((*(volatile uint32_t *)&empty[g >> 5] >> (g & 31u)) & 1u) != 0u;
+      if (!shut && *(volatile unsigned int *)&P.al_next[g] >= b1 - b0) {  // once per block and bucket
+        if (lane == 0) atomicOr(&empty[g >> 5], 1u << (g & 31u));
+        shut = true;
+      }
+      claim = !__any_sync(0xFFFFFFFFu, shut);
     }
     if (claim) {
       uint32_t got0 = 0;
@@ -1558,7 +1564,9 @@ __global__ void __launch_bounds__(lane_block<Cap>(), kLaneMinBlocks<R, Cap>()) l
     if (P.lane_evict || P.lane_tail) {
       const uint32_t am = __ballot_sync(0xFFFFFFFFu, active);
       bool out = (uint32_t)__popc(am) <= P.lane_evict;  // or few warps are left (every 8th event: the read waits)
-      if ((e & 7u) == 0u && P.lane_tail) out = out || *(volatile unsigned int *)P.lane_done >= P.lane_tail;
+      // (a vote: lanes may read different values of the counter)
+      if ((e & 7u) == 0u && P.lane_tail)
+        out = __any_sync(0xFFFFFFFFu, out || *(volatile unsigned int *)P.lane_done >= P.lane_tail);
       if (am && out && e + 1u < n_ev) {
         const uint32_t leader = __ffs(am) - 1;
         unsigned long long r0 = 0;
