@@ -24,7 +24,13 @@
  *   - Handles are owned by the library; free them with the matching *_free.
  *     One handle must not be used from two threads at once.
  *   - Results depend only on (circuit, noise, seed, shot index): splitting a
- *     shot range over calls or GPUs does not change them.
+ *     shot range over calls or GPUs does not change them, nor does the order in
+ *     which shots happen to run. Options that choose other kernels or another
+ *     start (group_size, first_cap, groups_per_block, SOFT_RUN_NO_LANES,
+ *     SOFT_RUN_NO_PREFIX, capture_k) round entries differently: 1e-16 in FP64;
+ *     1e-7 in FP32, where an outcome that close to its probability may change.
+ *     Sums over a map's entries run in an order that may vary (their last FP64
+ *     bit, so the last bits of a captured FP64 state).
  */
 #ifndef SOFT_ABI_H_
 #define SOFT_ABI_H_

@@ -13,11 +13,12 @@
 // its rebuilds after each pruning made the warp-per-shot kernel of kernels.cu 3 to 6 times
 // slower on these shots.
 //
-// A map that needs more than P.aff_dim directions after compaction (of the span of its live
-// slots, so that only maps of more than 2^(aff_dim - 1) entries do) goes to the pass at the
-// circuit's cap, which runs it from its start with the sparse form of kernels.cu. FP32
-// arithmetic is that kernel's, product by product, so a shot's outcomes do not depend on
-// which of the two runs it (FP64 sums over entries run in slot order).
+// A map whose live entries span P.aff_dim directions, however many they are, goes at the next
+// rotation that adds one to the pass at the circuit's cap, which runs it from its start with the
+// sparse form of kernels.cu. The arithmetic is the lane kernel's, product by product, in both
+// precisions: which shots come here from a lane depends on the order of claims and on which warps
+// end first, and no entry may depend on that. Only the FP64 sums over a map's entries run in
+// another order, since this kernel packs a map into fewer slots sooner (their last bit).
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -70,9 +71,6 @@ __device__ __forceinline__ uint32_t open_bit(uint32_t i, uint32_t q) {
 
 template <typename R, int W>
 struct AffShot {
-  // the products that share a phase take it folded into b, or apply it per entry, as in
-  // kernels.cu (Shot::kFoldPhase), so that both kernels round alike
-  [[maybe_unused]] static constexpr bool kFoldPhase = sizeof(R) == 8 || W == 1;
   const ShotParams &P;
   const CircDev *C = nullptr;
   const uint32_t lane;
@@ -371,12 +369,8 @@ struct AffShot {
     apply_pauli(beta, gamma, nc.phase(((c0 >> (2u * pp)) + 2u * wordpar(pe)) & 3u));
   }
 
-  // FP32: b xi x, xi = i^e (-1)^par
-  __device__ __forceinline__ static Cx<R> bxi(Cx<R> b, Cx<R> bq, uint32_t e, uint32_t par, Cx<R> x) {
-    if (kFoldPhase) return cmul(par ? Cx<R>{negr(bq.x), negr(bq.y)} : bq, x);
-    return cmul(b, ipow(x, e + 2u * par));
-  }
-  // ---- a I + b Z_q
+  // ---- a I + b Z_q; FP32 as in LaneShot::rot (lanes.cu): the phase xi folded into b (bq, or its
+  // negation bn), one fused chain per component (with a zero partner it rounds as one product)
   __device__ void rot(uint32_t w0, uint32_t ci, const uint64_t *beta, const uint64_t *gamma, bool diag) {
     const uint32_t e = (ev_e0(w0) + 2u * wpar2<W>(sd, beta, ss, gamma)) & 3u;  // (beta = 0 when diagonal)
     if (ci >= C->n_coef) {
@@ -403,15 +397,10 @@ struct AffShot {
       rot_scaled(cf, e, diag, fresh, gl, g0, c, r);
     } else {
       const float4 f = __ldg(reinterpret_cast<const float4 *>(&cf->fa_re));
-      const Cx<R> a{(R)f.x, (R)f.y}, b{(R)f.z, (R)f.w};
-      const Cx<R> bq = ipow(b, e);
+      const Cx<R> a{(R)f.x, (R)f.y}, bq = ipow(Cx<R>{(R)f.z, (R)f.w}, e), bn{negr(bq.x), negr(bq.y)};
       if (diag) {
-        const Cx<R> c0 = cadd(a, bq), c1 = csub(a, bq);
-        for (uint32_t s = lane; s < size(); s += 32) {
-          const uint32_t par = g0 ^ par32(s & gl);
-          const Cx<R> x = v[s];
-          v[s] = pruned(kFoldPhase ? cmul(par ? c1 : c0, x) : cadd(cmul(a, x), cmul(b, ipow(x, e + 2u * par))));
-        }
+        const Cx<R> c0 = cadd(a, bq), c1 = cadd(a, bn);
+        for (uint32_t s = lane; s < size(); s += 32) v[s] = pruned(cmul(g0 ^ par32(s & gl) ? c1 : c0, v[s]));
         __syncwarp();
         return;
       }
@@ -421,15 +410,15 @@ struct AffShot {
         for (uint32_t s = lane; s < n; s += 32) {
           const Cx<R> x = v[s];
           v[s] = pruned(cmul(a, x));
-          v[s ^ t0] = pruned(bxi(b, bq, e, g0 ^ par32(s & gl), x));
+          v[s ^ t0] = pruned(cmul(g0 ^ par32(s & gl) ? bn : bq, x));
         }
       } else {
         const uint32_t q = (uint32_t)__ffs(c) - 1u, flip = par32(c & gl), np = size() >> 1;
         for (uint32_t i = lane; i < np; i += 32) {  // a pair of slots per lane
           const uint32_t s = open_bit(i, q), t = s ^ c, ps = g0 ^ par32(s & gl);
           const Cx<R> vs = v[s], vt = v[t];
-          v[s] = pruned(cadd(cmul(a, vs), bxi(b, bq, e, ps ^ flip, vt)));
-          v[t] = pruned(cadd(cmul(a, vt), bxi(b, bq, e, ps, vs)));
+          v[s] = pruned(cmad2(a, vs, ps ^ flip ? bn : bq, vt));
+          v[t] = pruned(cmad2(a, vt, ps ? bn : bq, vs));
         }
       }
     }

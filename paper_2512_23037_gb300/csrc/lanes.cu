@@ -23,8 +23,9 @@
 // spill pool and moves on to fresh shots. The next round (another launch) buckets
 // the evicted shots by the event they resume at, and packs them into warps again; in
 // small runs the affine warp pass takes them instead. The last round evicts nothing, until
-// most of its warps have ended (lane_tail): the affine pass takes the others' shots. Which lane runs a shot does not change its
-// arithmetic, so the results are those of a single round.
+// most of its warps have ended (lane_tail): the affine pass takes the others' shots. Which lane or
+// warp runs a shot depends on the order of claims, so all of them share one arithmetic, entry by
+// entry; FP64 sums over a map's entries alone run in another order in the affine pass.
 //
 // A warp's time went to waits rather than to the maps (clock counters, w42 FP32: claims 22 %,
 // errors 17 %, finished and evicted shots 13 %, the search for the next bucket 7 %). So the

@@ -72,3 +72,27 @@ def test_same_batch_again(soft, shots, precision):
         got.append([[S.soft_tally_batch(r, i)[k] for k in KEYS] for i in range(4)])
         r.free()
     assert np.array_equal(np.array(got), np.array([got[0]] * 4)) and [t[0] for t in got[0]] == ns
+
+
+@pytest.mark.parametrize("name", ["w42", "w97", "random40", "win5"])
+def test_entries_do_not_depend_on_the_schedule(soft, name):
+    """FP32: the final map of every shot, bit for bit, whether evicted shots go on
+    in a warp of their own (small runs) or in lanes again (with a wide round),
+    in one chunk or several. (Sums over entries are FP64 and round to FP32
+    alike but where one lies within 1e-16 of a tie.)"""
+    S = soft
+    circ, noise = _case(name)
+    c = S.soft_compile_circuit(circ.array(), circ.n, noise, circ.cap)
+    n, seen = 1500, []
+    for kw in ({}, {"wide": True}, {"chunk_shots": 512}, {}):
+        r = S.soft_run_shots(c, n, 3, 23, precision="fp32", record_mode=S.REC_ALL, capture_k=n, **kw)
+        rec, status = S.soft_get_records(r, n)
+        maps = []
+        for i in range(n):
+            signs, keys, vals = S.soft_get_state(r, i)
+            order = np.lexsort((keys[:, 0], keys[:, 1]))
+            maps.append((signs.tobytes(), keys[order].tobytes(), (vals[order] + 0.0).tobytes()))
+        seen.append((rec, status, maps))
+    for rec, status, maps in seen[1:]:
+        assert np.array_equal(status, seen[0][1]) and np.array_equal(rec, seen[0][0])
+        assert sum(a != b for a, b in zip(maps, seen[0][2])) == 0
