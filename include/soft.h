@@ -150,7 +150,8 @@ typedef struct {
   void *stream;          /* cudaStream_t to launch on; NULL = legacy default stream */
   uint32_t group_size;   /* lanes per shot: 0 = 32, else 16 (two shots per warp) or 32 */
   uint32_t blocks_per_sm;/* 0 = as many as fit */
-  uint64_t chunk_shots;  /* shots per launch; 0 = auto */
+  uint64_t chunk_shots;  /* shots per launch; 0 = auto (fewer where the workspace for that
+                            many, 40 bytes a shot and the spill pools, finds no memory) */
   uint32_t first_cap;    /* capacity of the first pass (0 = auto); shots that exceed
                             it and not coeff_cap are rerun at coeff_cap */
   uint32_t capture_k;    /* keep the final GS state of the first capture_k shots */

@@ -414,9 +414,9 @@ namespace {
 
 using soft::circ_desc;
 
-// Shared launcher of soft_run_shots and soft_run_batch.
-int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t *first_shots, uint32_t n_circ,
-             uint64_t seed, const soft_run_opts *opts, soft_run **out) {
+// One try of run_many; *chunk_out: its chunk, once its workspace is asked for.
+int run_once(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t *first_shots, uint32_t n_circ,
+             uint64_t seed, const soft_run_opts *opts, soft_run **out, uint64_t *chunk_out) {
   if (!circs || !n_shots || !first_shots || !out || n_circ == 0) return fail(SOFT_E_ARG, "null argument or empty batch");
   *out = nullptr;
   if (n_circ > (uint32_t)soft::kMaxCirc) return fail(SOFT_E_ARG, "at most 64 circuits per batch");
@@ -542,19 +542,21 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   need(&r->d_chunk, chunk_words * sizeof(unsigned long long) + 2 * (size_t)nb * sizeof(uint32_t));
   // lanes: cursors (4 words per item, 16-byte aligned), the cursors in bucket order, (start
   // event, rank) pairs, bucket starts, counters, then the per-block bucket bases of the
-  // block-binned pre-pass
+  // block-binned pre-pass: 40 bytes a shot of the chunk
   const uint32_t al_grid = lanes ? soft::lane_prepass_grid(std::min(chunk, total)) : 0u;
   if (lanes) need(&r->d_al, (10 * chunk + (nb + 1) + (size_t)al_grid * (nb + 1)) * sizeof(uint32_t));
   // spill pool: records for the shots a sparse warp evicts (a quarter of the chunk; when it is
   // full, warps keep their shots), then records for shots a lane hands to a warp (an eighth;
   // when full, the warp reruns them from their start). Entries of the rerun list name a record
-  // with their top bit, so a chunk stays below 2^31 items for it.
+  // with their top bit, so a chunk stays below 2^31 items for it. (A record takes 300 to 500
+  // bytes: w42, 2^20 shots, FP64 214 MB in all, FP32 164.)
   const uint32_t rounds = lanes ? soft::lane_rounds() : 1u;
   // few shots: a second round would walk the events with a few warps, each step as slow as a
   // single lane's loops; the warp pass takes the evicted shots instead (w42 FP32, 4099 shots:
   // 1.2 -> 0.3 ms)
   const bool small_run = lanes && affine && !(o.flags & SOFT_RUN_WIDE_LANES) && std::min(chunk, total) <= kSmallRun;
-  const uint64_t evict_want = small_run ? std::min(chunk, total) : std::max<uint64_t>(std::min<uint64_t>(chunk, 1024), chunk / 4);
+  // (where there are few shots to keep the lanes full, more of them leave)
+  const uint64_t evict_want = std::max<uint64_t>(std::min<uint64_t>(chunk, small_run ? 1u << 17 : 1024u), chunk / 4);
   const uint32_t sp_evict = rounds > 1 ? (uint32_t)evict_want : 0u;
   const bool spill = lanes16 && (rounds > 1 || lane_grow) && chunk < (1ull << 31);
   const uint32_t sp_hand = lane_grow ? (uint32_t)std::max<uint64_t>(std::min<uint64_t>(chunk, 1024), chunk / 8) : 0u;
@@ -614,9 +616,11 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
       w.bytes = 0;
     }
   }
+  *chunk_out = chunk;
   if (!r->arena) {
     if ((e = cudaMalloc(&r->arena, arena_bytes)) != cudaSuccess) {
       r->arena = nullptr;
+      cudaGetLastError();  // (not for later launches to report)
       soft_run_free(r);
       return e == cudaErrorMemoryAllocation ? fail(SOFT_E_OOM, "device allocation failed") : cuda_fail(e, "cudaMalloc");
     }
@@ -977,6 +981,21 @@ int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t
   cudaEventRecord(r->ev1, st);
   *out = r;
   return SOFT_OK;
+}
+
+// Shared launcher of soft_run_shots and soft_run_batch. Results do not depend on the chunk, so
+// where a chunk's workspace finds no memory, smaller chunks (down to kLeastChunk) are tried.
+constexpr uint64_t kLeastChunk = 1ull << 16;
+int run_many(soft_circuit *const *circs, const uint64_t *n_shots, const uint64_t *first_shots, uint32_t n_circ,
+             uint64_t seed, const soft_run_opts *opts, soft_run **out) {
+  soft_run_opts o{};
+  if (opts) o = *opts;
+  for (;;) {
+    uint64_t chunk = 0;
+    const int rc = run_once(circs, n_shots, first_shots, n_circ, seed, &o, out, &chunk);
+    if (rc != SOFT_E_OOM || chunk <= kLeastChunk) return rc;
+    o.chunk_shots = std::max(chunk / 2, kLeastChunk);
+  }
 }
 
 }  // namespace
