@@ -161,11 +161,15 @@ static cudaError_t build_prefixes(soft_circuit *c, cudaStream_t us) {
     const size_t stride = soft::prefix_stride(fp32, hp.W, hp.rw);
     if ((e = cudaMalloc(&c->d_traj[fp32], n_snap * stride)) != cudaSuccess) break;
     c->traj_stride[fp32] = (uint32_t)stride;
-    // (a circuit of very many sites, or events past the table's 28 bits, does without)
-    if (hp.n_sites && hp.n_sites <= soft::kFateMaxSites && hp.ev.size() < soft::kFateEvent &&
-        (e = cudaMalloc(&c->d_fate[fp32], (size_t)hp.n_sites * 16 * sizeof(uint32_t))) != cudaSuccess)
-      break;
   }
+  // The fate tables (64 bytes a site each) only save time: a circuit of very many sites, or of
+  // events past the table's 28 bits, does without, and so does one whose table finds no memory.
+  for (int fp32 = 0; fp32 < 2 && e == cudaSuccess; ++fp32)
+    if (hp.n_sites && hp.n_sites <= soft::kFateMaxSites && hp.ev.size() < soft::kFateEvent &&
+        cudaMalloc(&c->d_fate[fp32], (size_t)hp.n_sites * 16 * sizeof(uint32_t)) != cudaSuccess) {
+      c->d_fate[fp32] = nullptr;
+      cudaGetLastError();  // (not for the launches below to report)
+    }
   for (int fp32 = 0; fp32 < 2 && e == cudaSuccess; ++fp32) {
     soft::ShotParams p{};
     p.n_circ = 1;
