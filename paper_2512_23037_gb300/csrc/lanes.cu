@@ -1707,7 +1707,9 @@ static cudaError_t launch_bin(const ShotParams &p, cudaStream_t st) {
   if (sh > 48 * 1024) {
     const void *kern = p.al_grid == 1 ? reinterpret_cast<const void *>(lane_bin_one_kernel<Resume, R, W>)
                                       : reinterpret_cast<const void *>(lane_bin_kernel<Resume, R, W>);
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    // (the largest that any run asks for: see prepare_lanes)
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)((kLaneMaxBuckets + 1 + kMaxCirc) * sizeof(uint32_t)));
     if (e != cudaSuccess) return e;
   }
   if (p.al_grid == 1) {
@@ -1754,8 +1756,12 @@ cudaError_t prepare_lanes(const ShotParams &p, int fp32, uint32_t W, int blocks_
                                         : lane_kernel_for<kLaneCap>(fp32, W, multi);
   if (!kern) return cudaErrorInvalidConfiguration;
   const size_t smem = lane_smem_bytes(fp32, W, p.rw_max, cap) + (size_t)((p.al_nb + 31u) / 32u) * 4u;
-  if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int kSmemLimit = 227 * 1024;
+  if (smem > kSmemLimit) return cudaErrorInvalidConfiguration;
+  // The attribute is the kernel's, not the launch's, and a launch's shared memory depends on its
+  // circuits' events and records: a thread that set its own size could lower it under another's
+  // launch. So every run sets the same.
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
