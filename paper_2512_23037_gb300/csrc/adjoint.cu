@@ -1332,6 +1332,8 @@ struct GradWarp {
       draw_next();
     }
     n_carried = n_err;
+    // one more than a pattern may have, which no event is left to meet
+    if (n_err == kMaxErr && nxt < P.n_sites && ev0 >= P.n_events) status = G_UNSUPPORTED;
     const unsigned char *in = P.psnap + (size_t)ev0 * P.psnap_stride;
     const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
     const uint64_t *r_in = reinterpret_cast<const uint64_t *>(in + sizeof(SnapHdr));

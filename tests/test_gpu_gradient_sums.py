@@ -68,3 +68,22 @@ def test_sums_as_two_sweeps_leave_them(soft, name):
         assert np.linalg.norm((grad - ref)[part]) <= bar * np.linalg.norm(ref[part])
     for got, key in ((fid, "fid"), (pacc, "pacc")):
         assert np.linalg.norm(got - want[key]) <= bar * np.linalg.norm(want[key])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("sites", [255, 256, 257, 300])
+def test_more_errors_than_a_pattern_may_have(soft, sites, precision):
+    """An error at every site (p = 1 - 1e-12), none of which any event meets: a pattern of
+    more than 256 errors is unsupported, one of 256 is not."""
+    S = soft
+    circ = C.Circuit(2, cap=4)
+    circ.noiseless(True)
+    circ.gate(C.RZ, 1, angle=0.3, param=0)
+    circ.noiseless(False)
+    for _ in range(sites):
+        circ.gate(C.H, 0)
+    c = S.soft_compile_circuit(circ.array(), circ.n, C.Noise.uniform(1.0 - 1e-12), circ.cap)
+    assert c.info["n_sites"] == sites
+    fid, pacc, grad, status = [t.cpu().numpy() for t in S.soft_fidelity_grad(c, [0.3], 40, 0, 1, precision)]
+    assert np.all(status == (2 if sites > 256 else 0))
+    assert np.all(fid == (0.0 if sites > 256 else 1.0)) and np.all(grad == 0.0)
