@@ -1296,7 +1296,7 @@ struct GradWarp {
 #pragma unroll
             for (int w = 0; w < W; ++w) c ^= (__ldg(&E->xbeta[w]) & g[w]) ^ (__ldg(&E->xgamma[w]) & b[w]);
         } else {
-          x = type == EV_PARITY || type == EV_END ? 0ull : 1ull;
+          x = type == EV_PARITY ? 0ull : 1ull;
         }
         last = ((__popcll(x) | __popcll(c)) & 1) != 0;
       }
@@ -1309,7 +1309,8 @@ struct GradWarp {
   // does not leave one of them alone, as long as the next comes in before it. Most patterns end
   // there, in a projection onto nothing, after one event. The errors are on record at that event, where the reverse
   // sweep takes them back; below it the sweep reads the noiseless run's tape, which they leave
-  // alone as well.
+  // alone as well. None is carried past the last event, which stands for the circuit's end: the
+  // sweep takes errors back at events only, and counts there those that are too many.
   __device__ void load_prefix() {
     ev0 = *P.pstop;
     while (nxt < P.n_sites && n_err < kMaxErr) {
@@ -1332,8 +1333,6 @@ struct GradWarp {
       draw_next();
     }
     n_carried = n_err;
-    // one more than a pattern may have, which no event is left to meet
-    if (n_err == kMaxErr && nxt < P.n_sites && ev0 >= P.n_events) status = G_UNSUPPORTED;
     const unsigned char *in = P.psnap + (size_t)ev0 * P.psnap_stride;
     const SnapHdr *h = reinterpret_cast<const SnapHdr *>(in);
     const uint64_t *r_in = reinterpret_cast<const uint64_t *>(in + sizeof(SnapHdr));

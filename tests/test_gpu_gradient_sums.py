@@ -28,7 +28,25 @@ SETS = {
     "q4": (706, 8e-3, 2000, 6, 6, "fp64"),
     "q4_fp32": (706, 8e-3, 2000, 6, 6, "fp32"),
     "wide": (703, 2e-2, 400, 3, 3, "fp64"),
+    "unobserved": ("unobserved", 3e-2, 400, 9, 9, "fp64"),
 }
+
+
+def unobserved():
+    """No record is observed (F = 1), and no event is left for most errors to meet."""
+    circ = C.Circuit(5, cap=256)
+    rng = np.random.default_rng(11)
+    for q in range(5):
+        circ.gate(C.H, q)
+    for k in range(30):
+        circ.gate(C.RZ, int(rng.integers(5)), angle=0.0, param=k % 6, negate=bool(k % 3))
+        a, b = (int(v) for v in rng.choice(5, size=2, replace=False))
+        circ.gate(C.CX, a, b)
+        circ.gate(int(rng.choice([C.H, C.S, C.T])), a)
+    circ.detector([circ.measure(0)])
+    for q in range(40):
+        circ.gate(C.X, q % 5)
+    return circ
 
 
 def run_set(S, name):
@@ -36,9 +54,9 @@ def run_set(S, name):
     if which == "w42rz":
         circ, theta = C.workload(which)[0], C.rz_thetas(seed, 72)
     else:
-        q = {705: 3, 706: 4, 703: 6}[which]
-        circ = C.random_param_circuit(which, q, 50 + 6 * q, 6)[0]
-        theta = np.random.default_rng(which).uniform(-np.pi, np.pi, 6)
+        q = {705: 3, 706: 4, 703: 6}.get(which)
+        circ = unobserved() if which == "unobserved" else C.random_param_circuit(which, q, 50 + 6 * q, 6)[0]
+        theta = np.random.default_rng(seed if which == "unobserved" else which).uniform(-np.pi, np.pi, 6)
     c = S.soft_compile_circuit(circ.array(), circ.n, C.Noise.uniform(p), circ.cap)
     return [t.cpu().numpy() for t in S.soft_fidelity_grad(c, theta, n, first, seed, precision)]
 

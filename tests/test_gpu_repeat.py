@@ -58,6 +58,29 @@ def test_same_call_again(soft, name, n, precision):
         assert [t[k] for k in KEYS] == [got[0][2][k] for k in KEYS]
 
 
+@pytest.mark.parametrize("name,n,wide", [("w42", 300007, None), ("w42", (1 << 20) + 1, None),
+                                         ("w42", (1 << 20) + 1, False), ("w97", 200003, None),
+                                         ("random40", 100003, None), ("win5", (1 << 20) + 1, None)])
+def test_every_shot_as_in_a_warp_of_its_own(soft, name, n, wide):
+    """FP64: every record and status byte against the plain schedule, a warp per
+    shot with sparse maps. Both round at 1e-15 and a shot samples some ten
+    outcomes, so that one in 10^14 could differ: none may."""
+    import torch
+    S = soft
+    circ, noise = _case(name)
+    c = S.soft_compile_circuit(circ.array(), circ.n, noise, circ.cap)
+    got = []
+    for kw in ({"wide": wide}, {"lanes": False}):
+        rec = torch.zeros((n, c.info["record_words"]), dtype=torch.int64, device="cuda")
+        status = torch.full((n,), 255, dtype=torch.uint8, device="cuda")
+        r = S.soft_run_shots(c, n, 40, 6, precision="fp64", record_mode=S.REC_ALL, d_records=rec.data_ptr(),
+                             d_status=status.data_ptr(), **kw)
+        S.soft_tally(r)
+        r.free()
+        got.append((rec, status))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("shots", [3000, 100000])
 def test_same_batch_again(soft, shots, precision):
