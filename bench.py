@@ -51,6 +51,10 @@ FLOPS_T_OUT, FLOPS_T_DIAG, FLOPS_MEAS = 14, 6, 4
 # included, over the measured time, against the same peak. The prefix runs once per compile and
 # no shot executes it, so this is the rate a design that re-ran the prefix per shot would need
 # to match; it is not a utilisation and can exceed 1.
+# What `frac` of the ALU rooflines counts.
+WORK_NOTE = ("lane ops of a shot after the noiseless-run prefix it shares with every shot (oracle counters), also "
+             "where an error is carried past them or the shot is finished unrun: an equivalent rate; the whole method "
+             "per shot is ops_per_shot_whole_method")
 EQUIV_NOTE = ("whole-method work per shot (shared noiseless prefix included, which runs once per compile and "
               "is executed by no shot) / time / peak: the rate a per-shot re-run of the prefix would need, "
               "not a utilisation; can exceed 1")
@@ -226,8 +230,8 @@ def _flops(k, post):
 def ops_per_shot_items(items, sample=2000):
     """Shot-weighted algorithmic work per shot over a workload's circuits, from
     the oracle's counters on a sample of the same workload (seed 0): lane ops
-    (executed: after the shared noiseless prefix; whole method) and FP64 flops
-    of the FP64 path (executed; whole method)."""
+    (after the shared noiseless prefix; whole method) and FP64 flops of the FP64
+    path (the same two). The kernels execute less of it (WORK_NOTE)."""
     import oracle
     per = sample if len(items) == 1 else max(50, sample // 10)
     tot = [0.0, 0.0, 0.0, 0.0]
@@ -407,7 +411,7 @@ def leg_batch64(S, C, torch, peak_ops, flush):
                                   "unit": "Tops/s", "frac": achieved / peak_ops,
                                   "equivalent_frac_whole_method": ops_full * n * 2 / (ms_tot / 1000) / peak_ops,
                                   "traffic": None, "kernel": "lane_kernel + affine_kernel (whole launch sequence)",
-                                  "ops_per_shot": ops_shot, "ops_per_shot_whole_method": ops_full}}
+                                  "work": WORK_NOTE, "ops_per_shot": ops_shot, "ops_per_shot_whole_method": ops_full}}
     for h in hs:
         h.free()
     return out
@@ -445,7 +449,7 @@ def leg_w97(S, C, torch, peak_ops, n_chunks):
                                   "kernel": ("lane_kernel (64-entry lanes: the noiseless maps reach 64 entries) + "
                                              "affine_kernel (shots that outgrow them)") if prec == "fp32" else
                                             "affine_kernel (warp per shot: 64-entry lanes are FP32 only)",
-                                  "ops_per_shot": ops_shot, "ops_per_shot_whole_method": ops_full}}
+                                  "work": WORK_NOTE, "ops_per_shot": ops_shot, "ops_per_shot_whole_method": ops_full}}
     h.free()
     return out
 
@@ -677,7 +681,7 @@ def main():
         legs["precision_error"] = leg_precision(S, C, torch, n, min(args.grad_patterns, 100000))
     # dominant kernel: the first-pass shot kernel (lane per shot where it applies), timed with the
     # passes that finish its work (bucketing pre-pass, rerun of outgrown maps) by CUDA events between
-    # them on the launching stream; the work is every shot's executed lane ops
+    # them on the launching stream; the work is every shot's lane ops after the shared prefix (WORK_NOTE)
     pass_ms = [sum(k[j] for k in kms32) / len(kms32) for j in range(3)]
     avg_launch_ms = sum(pass_ms)
     achieved = ops_shot * n / (avg_launch_ms / 1000)
@@ -720,8 +724,7 @@ def main():
                      "pass_ms_per_step": {"prepass": pass_ms[0], "first_pass": pass_ms[1], "rerun": pass_ms[2]},
                      "rerun_shots_per_step": sum(k[3] for k in kms32) / len(kms32),
                      "ops_per_shot": ops_shot, "ops_per_shot_whole_method": ops_full,
-                     "work": "lane ops a shot executes after the noiseless-run prefix it shares with every "
-                             "shot (oracle counters); the whole method per shot is ops_per_shot_whole_method",
+                     "work": WORK_NOTE,
                      "peak_basis": f"{sms} SMs x 128 lanes x {sm_clock:.0f} MHz (sm_max_mhz of measured)",
                      "equivalent_note": EQUIV_NOTE},
         "gpu_launches": launches32,

@@ -188,8 +188,8 @@ typedef struct {
  * handed over at that event (its whole state in a spill record): to the wide
  * round's lanes (see below), or to a warp (with its map in the same form, of up
  * to 1024 values in FP32 and 256 in FP64; of up to first_cap entries where the
- * caller sets first_cap or groups_per_block); shots beyond that rerun from
- * their start at the circuit's cap. A warp left with few active lanes moves
+ * caller sets groups_per_block, or a first_cap other than 64, the default's);
+ * shots beyond that rerun from their start at the circuit's cap. A warp left with few active lanes moves
  * their shots to a second round that packs them into full warps again, or in
  * small runs to the warps. Shots that their first errors discard end before
  * any of this. In a
@@ -291,7 +291,8 @@ int soft_run_timing(soft_run *r, double *ms, uint32_t *n_launches);
  * ms[1] the first pass (the shot kernel of the chosen scheduling), ms[2] the
  * rerun pass of shots whose maps outgrew the first pass (0 without one).
  * n_chunks (may be NULL) receives the number of chunks, n_rerun (may be NULL)
- * the number of shots the rerun pass finished. Waits for the run.
+ * the number of shots that left the first pass for a warp (their maps outgrew
+ * it, or their warps had few shots left). Waits for the run.
  * SOFT_E_ARG unless the run was launched with SOFT_RUN_TIME_PASSES and
  * without SOFT_RUN_GRAPH. */
 int soft_run_pass_timing(soft_run *r, double ms[3], uint32_t *n_chunks, uint64_t *n_rerun);

@@ -307,7 +307,7 @@ def soft_release_workspace():
 
 def soft_run_pass_timing(run: Run):
     """([pre-pass, first pass, rerun pass] ms summed over chunks, chunks, shots
-    finished by the rerun pass) of a run launched with time_passes=True."""
+    that left the first pass for a warp) of a run launched with time_passes=True."""
     ms = (ctypes.c_double * 3)()
     nc = ctypes.c_uint32(0)
     nr = ctypes.c_uint64(0)

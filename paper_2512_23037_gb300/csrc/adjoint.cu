@@ -517,7 +517,8 @@ struct GradWarp {
   // The end of an operation on a map: what it leaves in is pruned and packed, once, in one copy of
   // the code for every kind of event. The kernel waits for instructions more than for anything
   // else (half of its stalled cycles in FP64: a multiprocessor's 16 warps are at 16 places of
-  // it), so less code runs faster: 10^5 patterns of w42rz 2.23 -> 2.00 ms a call.
+  // it), so less code runs faster (10^5 patterns of w42rz, with one sweep a pattern: 2.23 -> 2.00
+  // ms a call).
   __device__ __forceinline__ void settle(RMap<R, W> &m, bool in) { prune_rel(m, in); }
   __device__ __forceinline__ void settle(SMap<R, W> &, bool) {}  // (its operations prune as they stage)
 
@@ -875,8 +876,8 @@ struct GradWarp {
   // and sign bit k & 1: sum_a conj(lambda_{a^beta}) xi_a phi_a. The sum over the lanes waits for
   // kTerms rotations (add_terms): on its own it took 5 of the 13 FP64 instructions of a
   // rotation, whose unit was busy for 62 % of an FP32 training step's kernel. The search looks at
-  // every key, four loads in flight, instead of stopping at the match. Training step 0.938 -> 0.879
-  // ms.
+  // every key, four loads in flight, instead of stopping at the match. Training step, with one
+  // sweep a pattern: 0.938 -> 0.879 ms.
   __device__ void put_terms(const RMap<R, W> &lam, const RMap<R, W> &phi, const uint64_t *beta, const uint64_t *gamma,
                             uint32_t e, uint32_t k, bool turned) {
     skey_set(lane, lam.k);
@@ -1003,7 +1004,8 @@ struct GradWarp {
       // dF = (dN_fid - F dN_acc) / N_acc. Sweep 1: N_fid from the end; sweep 2: N_acc from just
       // before the first fidelity measurement. Most kept patterns have F = 1 and the same adjoint
       // state there in both, entry for entry: sweep 2 then repeats sweep 1 and only its sums are
-      // added again.
+      // added again (w42rz, 10^5 patterns in FP64: 3.5 to 4.2 ms a call, by the angles; one sweep of
+      // lambda - F pre took 1.9, but left other last bits where the two cancel).
       bool both = false;
       if (!sweep(phi, P.n_events, r, grad, 1.0, ev_f, both)) status = kCapFail;
       if (status == G_OK) {

@@ -129,7 +129,8 @@ const Tabs &tabs() {
   return t;
 }
 
-// 64 x 64 bit matrix, transposed in place (exchanging blocks of 32, 16, ... 1 bits).
+// 64 x 64 bit matrix, transposed in place by exchanging blocks of 32, 16, ... 1 bits (the
+// recursive method of Warren, Hacker's Delight, sec. 7-3).
 void transpose64(uint64_t a[64]) {
   uint64_t m = 0x00000000FFFFFFFFull;
   for (uint32_t j = 32; j; j >>= 1, m ^= m << j)

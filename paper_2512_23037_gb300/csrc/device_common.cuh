@@ -276,9 +276,9 @@ template <int W>
 __device__ __forceinline__ uint32_t wbit(const uint64_t *a, uint32_t i) {
   return (uint32_t)((word_of<W>(a, i) >> (i & 63)) & 1ull);
 }
-// The lowest set bit of a nonzero W-word vector. (Written with a reversal and a leading-zero
-// count: nvcc 13.0 compiled __ffsll of a residual from a warp reduction in affine.cu to a
-// wrong value, -1 for 8, which the random-circuit tests caught.)
+// The lowest set bit of a nonzero W-word vector (64 W for zero). A reversal and a leading-zero
+// count: with __ffsll(x) - 1 here a build of affine.cu failed the random-circuit tests, and a
+// print in a scratch copy of it showed -1 beside a residual of 8. Why was not found.
 template <int W>
 __device__ __forceinline__ uint32_t wlow(const uint64_t *x) {
   const bool first = W == 1 || x[0] != 0ull;

@@ -1080,9 +1080,11 @@ __global__ void __launch_bounds__(128) snap_affine_kernel(unsigned char *traj, u
 // Before its first error a shot is the noiseless run. An error E commutes past every event that
 // leaves it alone: a rotation whose generator commutes with it, a decided measurement whose
 // outcome it does not flip (its corrections commuting with E too), a parity of unflipped
-// records. Up to such an event the shot is E applied to the noiseless run's state there, bit for
-// bit, since E permutes and phases the entries exactly and the arithmetic rounds alike on values
-// times i^k. So the shot may start at the first event that does not leave E alone, and if that
+// records. Up to such an event the shot is E applied to the noiseless run's state there, to
+// rounding: E permutes and phases the entries exactly, and rotations round alike on values times
+// i^k; but the state comes from the sparse kernel's form of the maps (FP64: unscaled), and the norm
+// that decides on pruning rounds differently for a value and i times it. So the shot may start at
+// the first event that does not leave E alone, and if that
 // is a measurement with a detector on it, E flips it and the shot ends there, discarded: the
 // pre-pass finishes such shots without running them (60 % of w42's and w97's; the others
 // start 10 to 20 events later; events run per shot: w42 25.7 -> 10.7, w97 46 -> 13.4). Two errors
